@@ -1,6 +1,6 @@
 // mbarrier, cp.async and bulk-copy (TMA) primitives shared by the kernels.  Every wait is
-// bounded by elapsed time on the GPU's global timer: it gives up after `limit_ns` nanoseconds
-// (WAIT_NS_DEFAULT unless the kernel is given another limit) and the caller raises STATUS_TIMEOUT.
+// bounded by elapsed time on the SM's clock: it gives up after `limit_ns` nanoseconds (WAIT_NS_DEFAULT
+// unless the kernel is given another limit) and the caller raises STATUS_TIMEOUT.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -14,6 +14,12 @@ constexpr unsigned long long WAIT_NS_DEFAULT = 20ull * 1000 * 1000;   // 20 ms: 
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+__device__ __forceinline__ unsigned long long sm_cycles() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%clock64;" : "=l"(t));
   return t;
 }
 
@@ -53,13 +59,13 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// Bounded wait on a phase parity; false = gave up after limit_ns.  The clock is read only once
-// a try has failed, so a wait that succeeds at once costs one instruction.
+// Bounded wait on a phase parity; false = gave up after limit_ns (counted as cycles of a 2 GHz clock).  A wait
+// that succeeds at once costs one instruction, and only every 32nd failed try looks at the clock.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
                                           unsigned long long limit_ns = WAIT_NS_DEFAULT) {
   const uint32_t a = smem_u32(bar);
   unsigned long long t0 = 0;
-  for (;;) {
+  for (unsigned n = 1;; ++n) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -67,15 +73,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
         "selp.b32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(a), "r"(parity) : "memory");
     if (ok) return true;
-    const unsigned long long t = global_ns();
+    if ((n & 31u) != 0) continue;
+    const unsigned long long t = sm_cycles();
     if (t0 == 0) t0 = t;
-    else if (t - t0 > limit_ns) return false;
+    else if (t - t0 > 2 * limit_ns) return false;
   }
 }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Arrive on `bar` (counted in its arrivals) once all cp.async copies this thread has issued so far have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }

@@ -7,7 +7,7 @@
 // column ranges:
 //   warps 0-3, 5-8  gather the token rows with 16-byte cp.async into a ring of 128B-swizzled,
 //              K-major shared-memory tiles (64 bf16 of the hidden dimension per stage);
-//   warp  4    allocates TMEM and issues tcgen05.mma (M = 128, N = columns rounded to 16,
+//   warp  4    allocates TMEM and issues tcgen05.mma (elect.sync, M = 128, N = columns rounded to 16,
 //              K = 16 per instruction, fp32 accumulation of exact bf16 products), one per
 //              sub-tile and k-step;
 //   warps 0-3, 5-8  afterwards read TMEM lanes back with tcgen05.ld (warps 0-3 the lower half
@@ -48,18 +48,28 @@ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t saddr) {
 __device__ __forceinline__ uint32_t umma_idesc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(UM >> 4) << 24);
 }
+// umma_bf16 and umma_commit are called by a whole converged warp with uniform arguments; one elected lane
+// issues.  (Called from a branch that only one lane takes, the same instructions cost 74 cycles per MMA and 175
+// per commit to issue, because every operand travels from that lane to the uniform registers; called by the warp
+// they cost 14-37 and 35: with four MMAs and a commit per k-block that was most of the k-loop.)
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
+      "elect.sync _|q, 0xFFFFFFFF;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-               ::"r"(smem_u32(bar)) : "memory");
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xFFFFFFFF;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(smem_u32(bar)) : "memory");
 }
+// The same value in every lane, so that the compiler keeps it in uniform registers.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_sync(0xFFFFFFFFu, x, 0); }
 // 32 consecutive accumulator columns of this thread's TMEM lane; completes at tmem_ld_wait().
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t* r) {
   asm volatile(
@@ -190,7 +200,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   const uint32_t ring = (smem_u32(um_raw) + 1023u) & ~1023u;
 
   if (tid == 0) {
-    for (int s = 0; s < NSTAGE; ++s) { mbar_init(&full_bar[s], 8); mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < NSTAGE; ++s) { mbar_init(&full_bar[s], 256); mbar_init(&empty_bar[s], 1); }
     mbar_init(&acc_bar, 1);
     failed = 0;
     acc_committed = 0;
@@ -259,37 +269,24 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     const uint32_t dsw = (uint32_t)((rsub >> 3) * 1024 + (rsub & 7) * 128 + ((chunk ^ (rsub & 7)) << 4));
     const __nv_bfloat16* tbase = tokens + (size_t)(d.row0 + d.n_cls) * D + chunk * 8;
     bool ok = true;
-    // a stage is published LAG iterations after its copies were issued; LAG < NSTAGE - 1 leaves
-    // the MMA a full iteration to drain a stage before the producer needs it again
-    constexpr int LAG = NSTAGE >= 3 ? NSTAGE - 2 : 1;
-    for (int kb = 0; kb < nkb + LAG; ++kb) {
-      if (kb < nkb) {
-        const int s = kb % NSTAGE;
-        if (kb >= NSTAGE && ok) ok = mbar_wait(&empty_bar[s], ((kb / NSTAGE) - 1) & 1, wait_ns);
-        if (ok) {
-          const uint32_t a0 = ring + (uint32_t)s * stage_bytes + dsw;
-          const uint32_t b0 = a0 + (uint32_t)a_bytes;
-          const __nv_bfloat16* src = tbase + (size_t)kb * UKB;
+    // Each thread's copies of a stage arrive on its barrier when they have landed, so a producer never waits
+    // for its own copies and the whole ring is in flight; the MMA warp orders the two proxies (below).
+    for (int kb = 0; kb < nkb && ok; ++kb) {
+      const int s = kb % NSTAGE;
+      if (kb >= NSTAGE) ok = mbar_wait(&empty_bar[s], ((kb / NSTAGE) - 1) & 1, wait_ns);
+      if (!ok) break;
+      const uint32_t a0 = ring + (uint32_t)s * stage_bytes + dsw;
+      const uint32_t b0 = a0 + (uint32_t)a_bytes;
+      const __nv_bfloat16* src = tbase + (size_t)kb * UKB;
 #pragma unroll
-          for (int i = 0; i < UM * UM_SUB / 32; ++i)
-            if (onA >> i & 1u) cp_async16(a0 + i * 4096, src + offA[i]);
+      for (int i = 0; i < UM * UM_SUB / 32; ++i)
+        if (onA >> i & 1u) cp_async16(a0 + i * 4096, src + offA[i]);
 #pragma unroll
-          for (int i = 0; i < UN_MAX / 32; ++i)
-            if (onB >> i & 1u) cp_async16(b0 + i * 4096, src + offB[i]);
-        }
-      }
-      cp_async_commit();
-      // the group committed LAG iterations ago has landed: publish that stage
-      const int done = kb - LAG;
-      if (done >= 0) {
-        cp_async_wait<LAG>();
-        fence_proxy_async();
-        // one arrival per producer warp: 256 arrivals per stage queue up on the barrier word
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&full_bar[done % NSTAGE]);
-      }
+      for (int i = 0; i < UN_MAX / 32; ++i)
+        if (onB >> i & 1u) cp_async16(b0 + i * 4096, src + offB[i]);
+      cp_async_arrive(&full_bar[s]);
     }
-    cp_async_wait<0>();
+    if (!ok) cp_async_wait_all();
     FICOCO_PHASE(1, 4);
     if (!ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
     bool acc_ok = ok && mbar_wait(&acc_bar, 0, wait_ns);
@@ -419,29 +416,33 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     }
     }
   } else {
-    // ---------------- MMA issuer (one lane) ---------------------------------------------------
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(n_pad);
-      bool ok = true;
-      for (int kb = 0; kb < nkb && ok; ++kb) {
-        const int s = kb % NSTAGE;
-        ok = mbar_wait(&full_bar[s], (kb / NSTAGE) & 1, wait_ns);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t a0 = ring + (uint32_t)s * stage_bytes;
-        const uint64_t ad = umma_smem_desc(a0), bd = umma_smem_desc(a0 + (uint32_t)a_bytes);
+    // ---------------- MMA issuer (the whole warp, one elected lane per instruction) -------------
+    const uint32_t idesc = umma_idesc_bf16(n_pad);
+    const uint32_t u_tmem = warp_uniform(tmem_base), u_ring = warp_uniform(ring);
+    bool m_ok = true;
+    for (int kb = 0; kb < nkb; ++kb) {
+      const int s = kb % NSTAGE;
+      m_ok = __all_sync(0xFFFFFFFFu, mbar_wait(&full_bar[s], (kb / NSTAGE) & 1, wait_ns));
+      if (!m_ok) break;
+      // the operands were written through the generic proxy (cp.async) and are read through the async
+      // proxy: this fence sits between the two on the path that the barrier orders
+      fence_proxy_async();
+      tc_fence_after();
+      const uint32_t a0 = u_ring + (uint32_t)s * stage_bytes;
+      const uint64_t ad = umma_smem_desc(a0), bd = umma_smem_desc(a0 + (uint32_t)a_bytes);
 #pragma unroll
-        for (int k4 = 0; k4 < UKB / 16; ++k4) {
-          umma_bf16(tmem_base, ad + (uint64_t)(k4 * 2), bd + (uint64_t)(k4 * 2), idesc,
-                    (kb > 0 || k4 > 0) ? 1u : 0u);
-          // second row sub-tile: A rows 128.. (UM * 128 bytes further, in 16-byte units), same B
-          if (nsub > 1)
-            umma_bf16(tmem_base + (uint32_t)n_pad, ad + (uint64_t)(UM * 128 / 16) + (uint64_t)(k4 * 2),
-                      bd + (uint64_t)(k4 * 2), idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
-        }
-        umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+      for (int k4 = 0; k4 < UKB / 16; ++k4) {
+        umma_bf16(u_tmem, ad + (uint64_t)(k4 * 2), bd + (uint64_t)(k4 * 2), idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
+        // second row sub-tile: A rows 128.. (UM * 128 bytes further, in 16-byte units), same B
+        if (nsub > 1)
+          umma_bf16(u_tmem + (uint32_t)n_pad, ad + (uint64_t)(UM * 128 / 16) + (uint64_t)(k4 * 2),
+                    bd + (uint64_t)(k4 * 2), idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
       }
-      if (ok) { umma_commit(&acc_bar); acc_committed = 1; }   // accumulator complete
+      umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+    }
+    if (m_ok) umma_commit(&acc_bar);   // accumulator complete
+    if (lane == 0) {
+      if (m_ok) acc_committed = 1;
       else { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
     }
     __syncwarp();
@@ -454,10 +455,8 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   if (warp == 4) {
     if (failed) {
       // MMAs may still be in flight: give them a bounded time to drain before freeing TMEM
-      if (lane == 0) {
-        if (!acc_committed) umma_commit(&acc_bar);
-        mbar_wait(&acc_bar, 0, wait_ns);
-      }
+      if (!acc_committed) umma_commit(&acc_bar);
+      mbar_wait(&acc_bar, 0, wait_ns);
       __syncwarp();
     }
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)tmem_cols)

@@ -323,30 +323,33 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
       cta_sync(1, 256);
     }
   } else {
-    // ---------------- MMA issuer (one lane): six products per k-step, smallest terms first ---------
-    if (lane == 0) {
-      const uint32_t id3 = umma_idesc_bf16(3 * nb), id2 = umma_idesc_bf16(2 * nb), id1 = umma_idesc_bf16(nb);
-      bool ok = true;
-      for (int kb = 0; kb < nkb && ok; ++kb) {
-        const int s = kb % UF_STAGES;
-        ok = mbar_wait(&full_bar[s], (kb / UF_STAGES) & 1, wait_ns);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t a0 = ring + (uint32_t)s * stage_bytes;
-        const uint64_t ah = umma_smem_desc(a0), am = umma_smem_desc(a0 + (uint32_t)a_bytes),
-                       al = umma_smem_desc(a0 + 2u * (uint32_t)a_bytes);
-        const uint64_t bh = umma_smem_desc(a0 + 3u * (uint32_t)a_bytes);   // [h' | m' | l'] start here
+    // ---------------- MMA issuer (the whole warp, one elected lane per instruction): six products per k-step,
+    // smallest terms first --------------------------------------------------------------------------
+    const uint32_t id3 = umma_idesc_bf16(3 * nb), id2 = umma_idesc_bf16(2 * nb), id1 = umma_idesc_bf16(nb);
+    const uint32_t u_tmem = warp_uniform(tmem_base), u_ring = warp_uniform(ring);
+    bool m_ok = true;
+    for (int kb = 0; kb < nkb; ++kb) {
+      const int s = kb % UF_STAGES;
+      m_ok = __all_sync(0xFFFFFFFFu, mbar_wait(&full_bar[s], (kb / UF_STAGES) & 1, wait_ns));
+      if (!m_ok) break;
+      tc_fence_after();
+      const uint32_t a0 = u_ring + (uint32_t)s * stage_bytes;
+      const uint64_t ah = umma_smem_desc(a0), am = umma_smem_desc(a0 + (uint32_t)a_bytes),
+                     al = umma_smem_desc(a0 + 2u * (uint32_t)a_bytes);
+      const uint64_t bh = umma_smem_desc(a0 + 3u * (uint32_t)a_bytes);   // [h' | m' | l'] start here
 #pragma unroll
-        for (int k4 = 0; k4 < UKB / 16; ++k4) {
-          const uint64_t o = (uint64_t)(k4 * 2);
-          const uint32_t acc = (kb > 0 || k4 > 0) ? 1u : 0u;
-          umma_bf16(tmem_base, ah + o, bh + o, id3, acc);                       // h h' | h m' | h l'
-          umma_bf16(tmem_base + (uint32_t)(3 * nb), am + o, bh + o, id2, acc);  // m h' | m m'
-          umma_bf16(tmem_base + (uint32_t)(5 * nb), al + o, bh + o, id1, acc);  // l h'
-        }
-        umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+      for (int k4 = 0; k4 < UKB / 16; ++k4) {
+        const uint64_t o = (uint64_t)(k4 * 2);
+        const uint32_t acc = (kb > 0 || k4 > 0) ? 1u : 0u;
+        umma_bf16(u_tmem, ah + o, bh + o, id3, acc);                       // h h' | h m' | h l'
+        umma_bf16(u_tmem + (uint32_t)(3 * nb), am + o, bh + o, id2, acc);  // m h' | m m'
+        umma_bf16(u_tmem + (uint32_t)(5 * nb), al + o, bh + o, id1, acc);  // l h'
       }
-      if (ok) { umma_commit(&acc_bar); acc_committed = 1; }   // accumulator complete
+      umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+    }
+    if (m_ok) umma_commit(&acc_bar);   // accumulator complete
+    if (lane == 0) {
+      if (m_ok) acc_committed = 1;
       else { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
     }
     __syncwarp();
@@ -358,10 +361,8 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
   if (warp == 4) {
     if (failed) {
       // MMAs may still be in flight: give them a bounded time to drain before freeing TMEM
-      if (lane == 0) {
-        if (!acc_committed) umma_commit(&acc_bar);
-        mbar_wait(&acc_bar, 0, wait_ns);
-      }
+      if (!acc_committed) umma_commit(&acc_bar);
+      mbar_wait(&acc_bar, 0, wait_ns);
       __syncwarp();
     }
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)tmem_cols)

@@ -48,9 +48,9 @@ __device__ __forceinline__ bool poll_count(const int* p, int need, unsigned long
   unsigned long long t0 = 0;
   for (;;) {
     if (ld_acquire(p) >= need) return true;
-    const unsigned long long t = global_ns();
+    const unsigned long long t = sm_cycles();
     if (t0 == 0) t0 = t;
-    else if (t - t0 > limit_ns) return false;
+    else if (t - t0 > 2 * limit_ns) return false;
     if (*reinterpret_cast<const volatile unsigned*>(status) & STATUS_TIMEOUT) return false;
     __nanosleep(32);
   }
