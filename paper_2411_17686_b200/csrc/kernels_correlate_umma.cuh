@@ -103,67 +103,89 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
       : "r"(taddr) : "memory");
 }
 
-// Top-L of one accumulator row over the columns [c_lo, c_hi) (multiples of 16).  The code is
+// Takes t (column c) into a descending list of LCAP entries.  Branch-free: entry k changes when t > v[k], and then
+// to the entry above it where that one changed as well, else to t.  '>' keeps the lower column first among equal
+// values because columns arrive in ascending order; a NaN is never taken.
+template <int LCAP>
+__device__ __forceinline__ void toplist_take(float t, int c, float (&v)[LCAP], int (&ix)[LCAP]) {
+  if constexpr (LCAP > 4) {      // more predicates than there are registers for: the displaced entry moves down
+    bool in = false;
+#pragma unroll
+    for (int k = 0; k < LCAP; ++k) {
+      in = in || t > v[k];
+      const float tv = v[k];
+      const int ti = ix[k];
+      v[k] = in ? t : tv; ix[k] = in ? c : ti;
+      t = in ? tv : t; c = in ? ti : c;
+    }
+    return;
+  }
+  bool p[LCAP];
+#pragma unroll
+  for (int k = 0; k < LCAP; ++k) p[k] = t > v[k];
+#pragma unroll
+  for (int k = LCAP - 1; k > 0; --k) {
+    v[k] = p[k] ? (p[k - 1] ? v[k - 1] : t) : v[k];
+    ix[k] = p[k] ? (p[k - 1] ? ix[k - 1] : c) : ix[k];
+  }
+  v[0] = p[0] ? t : v[0];
+  ix[0] = p[0] ? c : ix[0];
+}
+
+// Top list of one accumulator row over the columns [c_lo, c_hi) (multiples of 16).  The code is
 // kept small on purpose (a rolled loop over 16-column TMEM loads): it runs once per CTA, so a
-// long unrolled body would be paid for in instruction-cache misses.  Insertion is branch-free:
-// once a value is placed the rest of the list shifts down; '>' keeps the lower column first
-// among equal values because columns arrive in ascending order.
+// long unrolled body would be paid for in instruction-cache misses.  What bounds it is the number of
+// instructions per entry: the row's own factor rs > 0 does not change the order of a row's entries and is
+// applied to the list alone, padding columns carry a NaN in rnT instead of being compared with the column
+// count, and the insertion is the one above (about 20 instructions per entry for four-entry lists, 40 before).
 // v / ix: descending list, -inf / INT_MAX in empty slots.  Warp-collective (tcgen05.ld).
 // FiCoCo-L adds the text-bridged term: tS (this row's text->vision weights, element k at
 // tS[k * s_stride]) and tT ([M][t_stride], one row per text token over the CTA's columns) sit in
 // shared memory; C = gamma * cosine + t_scale * sum_k tS_k tT_kc.  tT == nullptr: FiCoCo-V.
 template <int LCAP>
-__device__ __forceinline__ void epilogue_scan(uint32_t tmem_lane, int c_lo, int c_hi, int ncols, int col_begin,
-                                              float rs, const float* rnT, bool row_valid, int L,
-                                              float (&v)[LCAP], int (&ix)[LCAP], const float* tS, int s_stride,
-                                              const float* tT, int t_stride, int M, float gamma, float t_scale) {
+__device__ __forceinline__ void epilogue_scan(uint32_t tmem_lane, int c_lo, int c_hi, int col_begin, float rs,
+                                              const float* rnT, float (&v)[LCAP], int (&ix)[LCAP], const float* tS,
+                                              int s_stride, const float* tT, int t_stride, int M, float gamma,
+                                              float t_scale) {
 #pragma unroll
   for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
-  const int cmax = row_valid ? min(ncols, c_hi) : 0;
-#pragma unroll 1
+  if (tT == nullptr) {
+    #pragma unroll 1
+    for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+      uint32_t r[16];
+      tmem_ld16(tmem_lane + (uint32_t)c0, r);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) toplist_take<LCAP>(rnT[c0 + j] * __uint_as_float(r[j]), col_begin + c0 + j, v, ix);
+    }
+#pragma unroll
+    for (int k = 0; k < LCAP; ++k)
+      if (ix[k] != INT_MAX) v[k] *= rs;
+    return;
+  }
+  #pragma unroll 1
   for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
     uint32_t r[16];
     tmem_ld16_issue(tmem_lane + (uint32_t)c0, r);
     float tx[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) tx[j] = 0.f;
-    if (tT != nullptr) {
-      #pragma unroll 1
-      for (int k = 0; k < M; ++k) {
-        const float a = tS[(size_t)k * s_stride];
-        const float4* q = reinterpret_cast<const float4*>(tT + (size_t)k * t_stride + c0);
+    #pragma unroll 1
+    for (int k = 0; k < M; ++k) {
+      const float a = tS[(size_t)k * s_stride];
+      const float4* q = reinterpret_cast<const float4*>(tT + (size_t)k * t_stride + c0);
 #pragma unroll
-        for (int j4 = 0; j4 < 4; ++j4) {
-          const float4 t4 = q[j4];
-          tx[4 * j4 + 0] = fmaf(a, t4.x, tx[4 * j4 + 0]);
-          tx[4 * j4 + 1] = fmaf(a, t4.y, tx[4 * j4 + 1]);
-          tx[4 * j4 + 2] = fmaf(a, t4.z, tx[4 * j4 + 2]);
-          tx[4 * j4 + 3] = fmaf(a, t4.w, tx[4 * j4 + 3]);
-        }
+      for (int j4 = 0; j4 < 4; ++j4) {
+        const float4 t4 = q[j4];
+        tx[4 * j4 + 0] = fmaf(a, t4.x, tx[4 * j4 + 0]);
+        tx[4 * j4 + 1] = fmaf(a, t4.y, tx[4 * j4 + 1]);
+        tx[4 * j4 + 2] = fmaf(a, t4.z, tx[4 * j4 + 2]);
+        tx[4 * j4 + 3] = fmaf(a, t4.w, tx[4 * j4 + 3]);
       }
     }
     tmem_ld_wait();
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = c0 + j;
-      float cv = gamma * ((rs * rnT[c]) * __uint_as_float(r[j])) + t_scale * tx[j];
-      if (!(c < cmax)) cv = -CUDART_INF_F;           // also drops NaN-free padding columns
-      int ci = col_begin + c;
-      bool ins = false;
-#pragma unroll
-      for (int k = 0; k < LCAP; ++k) {
-        if (k < L) {
-          const bool p = ins || cv > v[k];
-          const float tv = v[k];
-          const int ti = ix[k];
-          v[k] = p ? cv : tv;
-          ix[k] = p ? ci : ti;
-          cv = p ? tv : cv;
-          ci = p ? ti : ci;
-          ins = p;
-        }
-      }
-    }
+    for (int j = 0; j < 16; ++j)
+      toplist_take<LCAP>(gamma * ((rs * rnT[c0 + j]) * __uint_as_float(r[j])) + t_scale * tx[j], col_begin + c0 + j, v, ix);
   }
 }
 
@@ -234,7 +256,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   for (int c = tid; c < UN_MAX; c += UTHREADS) {
     const int p = c < ncols ? checked_index(T_idx[d.tgt0 + col_begin + c], d.np, status) : -1;
     rowT[c] = p;
-    rnT[c] = p >= 0 ? rn[d.patch0 + p] : 0.f;
+    rnT[c] = p >= 0 ? rn[d.patch0 + p] : CUDART_NAN_F;       // a padding column: no list takes its products
   }
   tc_fence_before();
   __syncthreads();
@@ -346,8 +368,8 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
       float v[LCAP];
       int ix[LCAP];
       if (acc_ok && sub * UM + warp * 32 < w.nrows)
-        epilogue_scan<LCAP>(tmem_base + (uint32_t)(sub * n_pad) + ((uint32_t)(warp * 32) << 16), 0, c_mid, ncols,
-                            col_begin, rs, rnT, row_valid, L, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
+        epilogue_scan<LCAP>(tmem_base + (uint32_t)(sub * n_pad) + ((uint32_t)(warp * 32) << 16), 0, c_mid,
+                            col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
                             t_scale);
       else {
 #pragma unroll
@@ -402,8 +424,8 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
       float v[LCAP];
       int ix[LCAP];
       if (acc_ok && sub * UM + grp * 32 < w.nrows)
-        epilogue_scan<LCAP>(tmem_base + (uint32_t)(sub * n_pad) + ((uint32_t)(grp * 32) << 16), c_mid, n_pad, ncols,
-                            col_begin, rs, rnT, row_valid, L, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
+        epilogue_scan<LCAP>(tmem_base + (uint32_t)(sub * n_pad) + ((uint32_t)(grp * 32) << 16), c_mid, n_pad,
+                            col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
                             t_scale);
       else {
 #pragma unroll

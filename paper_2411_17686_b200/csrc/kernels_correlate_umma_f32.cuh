@@ -58,12 +58,10 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
 // being the sum of the six partial products at TMEM columns c + {5, 2, 4, 3, 1, 0} * nb (l h', h l',
 // m m', m h', h m', h h').  Same list discipline as epilogue_scan().  Warp-collective (tcgen05.ld).
 template <int LCAP>
-__device__ __forceinline__ void epilogue_scan_split(uint32_t tmem_lane, int nb, int c_lo, int c_hi, int ncols,
-                                                    int col_begin, float rs, const float* rnT, bool row_valid, int L,
-                                                    float (&v)[LCAP], int (&ix)[LCAP]) {
+__device__ __forceinline__ void epilogue_scan_split(uint32_t tmem_lane, int nb, int c_lo, int c_hi, int col_begin,
+                                                    float rs, const float* rnT, float (&v)[LCAP], int (&ix)[LCAP]) {
 #pragma unroll
   for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
-  const int cmax = row_valid ? min(ncols, c_hi) : 0;
 #pragma unroll 1
   for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
     float a[16];
@@ -78,27 +76,11 @@ __device__ __forceinline__ void epilogue_scan_split(uint32_t tmem_lane, int nb, 
       for (int j = 0; j < 16; ++j) a[j] += __uint_as_float(r[j]);
     }
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = c0 + j;
-      float cv = (rs * rnT[c]) * a[j];
-      if (!(c < cmax)) cv = -CUDART_INF_F;
-      int ci = col_begin + c;
-      bool ins = false;
-#pragma unroll
-      for (int k = 0; k < LCAP; ++k) {
-        if (k < L) {
-          const bool p = ins || cv > v[k];
-          const float tv = v[k];
-          const int ti = ix[k];
-          v[k] = p ? cv : tv;
-          ix[k] = p ? ci : ti;
-          cv = p ? tv : cv;
-          ci = p ? ti : ci;
-          ins = p;
-        }
-      }
-    }
+    for (int j = 0; j < 16; ++j) toplist_take<LCAP>(rnT[c0 + j] * a[j], col_begin + c0 + j, v, ix);
   }
+#pragma unroll
+  for (int k = 0; k < LCAP; ++k)
+    if (ix[k] != INT_MAX) v[k] *= rs;
 }
 
 // Dynamic shared memory: [1024-aligned] two stages of [A_h | A_m | A_l | B_h | B_m | B_l]; an A tile has
@@ -166,7 +148,7 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
     const int c = tid - UM;
     const int p = c < ncols ? checked_index(T_idx[d.tgt0 + col_begin + c], d.np, status) : -1;
     rowT[c] = p;
-    rnT[c] = p >= 0 ? rn[d.patch0 + p] : 0.f;
+    rnT[c] = p >= 0 ? rn[d.patch0 + p] : CUDART_NAN_F;       // a padding column: no list takes its products
   }
   tc_fence_before();
   __syncthreads();
@@ -270,8 +252,7 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
       float v[LCAP];
       int ix[LCAP];
       if (acc_ok && warp * 32 < w.nrows)
-        epilogue_scan_split<LCAP>(tmem_base + ((uint32_t)(warp * 32) << 16), nb, 0, c_mid, ncols, col_begin, rs, rnT,
-                                  row_valid, L, v, ix);
+        epilogue_scan_split<LCAP>(tmem_base + ((uint32_t)(warp * 32) << 16), nb, 0, c_mid, col_begin, rs, rnT, v, ix);
       else {
 #pragma unroll
         for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
@@ -312,8 +293,7 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
       float v[LCAP];
       int ix[LCAP];
       if (acc_ok && grp * 32 < w.nrows)
-        epilogue_scan_split<LCAP>(tmem_base + ((uint32_t)(grp * 32) << 16), nb, c_mid, n_pad, ncols, col_begin, rs, rnT,
-                                  row_valid, L, v, ix);
+        epilogue_scan_split<LCAP>(tmem_base + ((uint32_t)(grp * 32) << 16), nb, c_mid, n_pad, col_begin, rs, rnT, v, ix);
       else {
 #pragma unroll
         for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
