@@ -94,9 +94,10 @@ enum ficoco_flags {
                                     else.  The step's first kernel may then start reading tokens
                                     and attention while that previous step is still finishing,
                                     provided its inputs do not overlap that step's outputs (the
-                                    library checks the address ranges).  Without the flag every
-                                    step starts in plain stream order, which is what a stream
-                                    that also carries other kernels needs. */
+                                    library checks the address ranges).  Without the flag no
+                                    kernel of the step reads or writes anything before the work
+                                    in front of it on the stream is complete, which is what a
+                                    stream that also carries other kernels needs. */
 };
 
 /* Hyper-parameters; defaults are the paper's (Sec. "Implementation Details"):

@@ -87,6 +87,8 @@ __global__ void __launch_bounds__(EQ_THREADS, 2) k_equivalent_token(
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  grid_dep_wait();      // launched under the tail of the kernel before: it may still write the keys or read a_eq
+  grid_dep_launch();
 
   const int ngroups = (nt + EQ_ROWS - 1) / EQ_ROWS;
   if (warp == EQ_WARPS) {
@@ -209,13 +211,15 @@ cudaError_t launch_eq(const void* keys, int batch, int uniform_tokens, const EqO
   cfg.blockDim = dim3(EQ_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = EQ_CLUSTER;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_equivalent_token<T>, (const T*)keys, heads, dk, n_cls, uniform_tokens, offs,
                             a_eq, tpc_max, nstage);
 }

@@ -884,12 +884,12 @@ int get_plan(ficoco_ctx* c, const PlanKey& key, long long attn_rows, cudaStream_
 
 // Launch with programmatic stream serialization: the grid may be staged while the kernel before
 // it in the stream is still running; the kernel itself waits (grid_dep_wait) before it reads
-// anything that kernel wrote.
+// anything that kernel wrote.  Takes a launch's set-up off the stream (about 1.5 us per kernel).
 template <class... KArgs, class... Args>
-cudaError_t launch_dependent(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
+cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st,
                              Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -930,7 +930,7 @@ cudaError_t launch_filter_fused(ficoco_ctx* c, const Plan* p, const T* tok, int 
 template <class T, int VPL>
 void launch_colsum_fused(ficoco_ctx* c, const Plan* p, const T* tok, int D, cudaStream_t st) {
   constexpr int E = VecTraits<T>::E;
-  k_colsum<T, VPL, true><<<dim3(p->n_rows, 1), 256, VPL * 32 * E * sizeof(float), st>>>(
+  launch_dependent(k_colsum<T, VPL, true>, dim3(p->n_rows, 1), 256, VPL * 32 * E * sizeof(float), st,
       tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
 }
 
@@ -958,10 +958,10 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       if (spans_overlap(out_spans[o], in_spans[i])) return FICOCO_ERR_INVALID_ARG;
     if (spans_overlap(out_spans[o], rel_span)) return FICOCO_ERR_INVALID_ARG;
   }
-  // the early start is taken only when the caller vouches for what sits in front of this step
-  // 0: plain stream order; 1: the filter grid may read its inputs under the tail of the step before;
-  // 2: it is fed by that step: launched early all the same, reads only once that step is complete
-  const int overlap_prev = !back_to_back ? 0 : inputs_clear_of_last_outputs(c->device, st, in_spans, 3) ? 1 : 2;
+  // How the filter grid starts.  1: it may read its inputs under the tail of the step before (only when the caller
+  // vouches for what sits in front of this step); 2: launched early, so that its CTAs are in place and set up, but
+  // reads only once whatever is in front of it on the stream is complete.
+  const int overlap_prev = back_to_back && inputs_clear_of_last_outputs(c->device, st, in_spans, 3) ? 1 : 2;
   record_last_outputs(c->device, st, out_spans, N_SPANS);
   if (p->fused) {
     prof_tick(c, st, "filter_fused");
@@ -979,7 +979,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   } else {
   if (rel) {
     prof_tick(c, st, "score_relation");
-    k_score_rel<<<p->n_rows, 256, (size_t)p->max_rc * sizeof(float), st>>>(
+    launch_dependent(k_score_rel, dim3(p->n_rows), 256, (size_t)p->max_rc * sizeof(float), st,
         rel, p->d_desc, p->d_rows, attn, attn_rows, cA, p->key.rel == 2 ? 1 : 0, c->s_raw);
     c->launches += 1;
   } else {
@@ -993,27 +993,31 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     else launch_colsum_fused<T, 8>(c, p, tok, D, st);
     c->launches += 1;
   } else if (wide) {
-    if (nvec <= 512) k_colsum_wide<T, 2, 8><<<p->n_rows, 256, 0, st>>>(tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
-    else k_colsum_wide<T, 4, 4><<<p->n_rows, 256, 0, st>>>(tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
+    if (nvec <= 512) launch_dependent(k_colsum_wide<T, 2, 8>, dim3(p->n_rows), 256, 0, st,
+      tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
+    else launch_dependent(k_colsum_wide<T, 4, 4>, dim3(p->n_rows), 256, 0, st,
+      tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
     c->launches += 1;
   } else {
-    k_rownorm<T><<<p->n_rows, 256, 0, st>>>(tok, D, p->d_desc, p->d_rows, c->rn);
+    launch_dependent(k_rownorm<T>, dim3(p->n_rows), 256, 0, st,
+      tok, D, p->d_desc, p->d_rows, c->rn);
     prof_tick(c, st, "colsum");
     const int slabs = (nvec + 255) / 256;
-    k_colsum<T, 8, false><<<dim3(p->n_rows, slabs), 256, 8 * 32 * E * sizeof(float), st>>>(
+    launch_dependent(k_colsum<T, 8, false>, dim3(p->n_rows, slabs), 256, 8 * 32 * E * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
     c->launches += 2;
   }
   prof_tick(c, st, "score");
-  k_msum<<<dim3(p->key.batch, (D + 255) / 256), 256, 0, st>>>(D, p->d_desc, c->partial, c->msum);
+  launch_dependent(k_msum, dim3(p->key.batch, (D + 255) / 256), 256, 0, st,
+      D, p->d_desc, c->partial, c->msum);
   if (wide && nvec <= 512)
-    k_score_wide<T, 2, 8><<<p->n_rows, 256, (size_t)9 * p->max_rc * sizeof(float), st>>>(
+    launch_dependent(k_score_wide<T, 2, 8>, dim3(p->n_rows), 256, (size_t)9 * p->max_rc * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw);
   else if (wide)
-    k_score_wide<T, 4, 4><<<p->n_rows, 256, (size_t)9 * p->max_rc * sizeof(float), st>>>(
+    launch_dependent(k_score_wide<T, 4, 4>, dim3(p->n_rows), 256, (size_t)9 * p->max_rc * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw);
   else
-    k_score<T><<<p->n_rows, 256, (size_t)(D + 9 * p->max_rc) * sizeof(float), st>>>(
+    launch_dependent(k_score<T>, dim3(p->n_rows), 256, (size_t)(D + 9 * p->max_rc) * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw);
   c->launches += 2;
   }
@@ -1024,7 +1028,8 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   }
   prof_tick(c, st, "select");
   // images of up to 1024 tokens: half the threads (two tokens each), cheaper barriers
-  k_select<<<p->key.batch, p->max_np <= 1024 ? 512 : 1024, sel_smem, st>>>(p->d_desc, c->s_raw, pos, window, coef, penalty,
+  launch_dependent(k_select, dim3(p->key.batch), p->max_np <= 1024 ? 512 : 1024, sel_smem, st,
+      p->d_desc, c->s_raw, pos, window, coef, penalty,
                                                   c->s_pen, scores_out, c->S_idx, c->T_idx, kept_idx,
                                                   pos_out, c->status);
   c->launches += 1;
@@ -1036,7 +1041,8 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       for (const ImgDesc& d : p->h_desc)
         if (d.list_len > 0 && d.cols_per_split > rel_cols) rel_cols = d.cols_per_split;
 #define FICOCO_REL_GO(LC)                                                                              \
-  k_correlate_rel<LC><<<p->n_corr, 256, (size_t)rel_cols * sizeof(int), st>>>(rel, p->d_desc, p->d_corr, c->S_idx, c->T_idx, c->part_val, \
+  launch_dependent(k_correlate_rel<LC>, dim3(p->n_corr), 256, (size_t)rel_cols * sizeof(int), st,       \
+                   rel, p->d_desc, p->d_corr, c->S_idx, c->T_idx, c->part_val,                          \
                                                  c->part_idx, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt,    \
                                                  c->e_w, c->e_c, c->status)
       if (p->max_list <= 2) FICOCO_REL_GO(2);
@@ -1047,7 +1053,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       prof_tick(c, st, "correlate_umma_f32");
       const float* tk = reinterpret_cast<const float*>(tok);
 #define FICOCO_UF32_LAUNCH(LC)                                                                         \
-  launch_dependent(k_correlate_umma_f32<LC>, p->n_corr, UTHREADS, p->um_smem, st, tk, D,               \
+  launch_dependent(k_correlate_umma_f32<LC>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,               \
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
       (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status,                 \
       p->um_a_bytes, p->um_b_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt,        \
@@ -1060,7 +1066,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       prof_tick(c, st, "correlate_umma");
       const __nv_bfloat16* tk = reinterpret_cast<const __nv_bfloat16*>(tok);
 #define FICOCO_UMMA_LAUNCH(NS, LC)                                                                     \
-  launch_dependent(k_correlate_umma<NS, LC>, p->n_corr, UTHREADS, p->um_smem, st, tk, D,               \
+  launch_dependent(k_correlate_umma<NS, LC>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,               \
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
       (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status,                 \
       p->um_stage_bytes, p->um_a_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt,    \
@@ -1079,7 +1085,8 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
 #undef FICOCO_UMMA_LAUNCH
     } else {
       prof_tick(c, st, "correlate_simt");
-      k_correlate_simt<T><<<p->n_corr, 256, 0, st>>>(tok, D, p->d_desc, p->d_corr, c->rn, c->S_idx,
+      launch_dependent(k_correlate_simt<T>, dim3(p->n_corr), 256, 0, st,
+      tok, D, p->d_desc, p->d_corr, c->rn, c->S_idx,
                                                      c->T_idx, tmean, M, gamma, c->part_val, c->part_idx,
                                                      c->tile_cnt, c->corr_cnt, c->tau,
                                                      c->e_tgt, c->e_w, c->e_c, c->status);
@@ -1088,26 +1095,27 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   }
   if (p->max_src > 0 && p->need_finalize) {
     prof_tick(c, st, "finalize");
-    k_finalize_src<<<dim3(p->key.batch, (p->max_src + 255) / 256), 256, 0, st>>>(
+    launch_dependent(k_finalize_src, dim3(p->key.batch, (p->max_src + 255) / 256), 256, 0, st,
         p->d_desc, c->part_val, c->part_idx, c->corr_cnt, c->tau, c->e_tgt, c->e_w, c->e_c);
     c->launches += 1;
   }
   prof_tick(c, st, "merge_compact");
   const int after_correlate = p->n_corr > 0 ? 1 : 0;   // else the grid before may be the filter itself
   if (p->fused)
-    launch_dependent(k_merge_scan<T, 3>, p->n_out, 256, 0, st, tok, D, (const ImgDesc*)p->d_desc,
+    launch_dependent(k_merge_scan<T, 3>, dim3(p->n_out), 256, 0, st, tok, D, (const ImgDesc*)p->d_desc,
                      (const WorkItem*)p->d_out, (const int*)c->S_idx, (const int*)c->T_idx,
                      (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, after_correlate,
                      c->status, c->img_cnt + (size_t)c->last_parity * 3 * c->max_batch, 3 * c->max_batch);
   else
-    launch_dependent(k_merge_scan<T, 4>, p->n_out, 256, 0, st, tok, D, (const ImgDesc*)p->d_desc,
+    launch_dependent(k_merge_scan<T, 4>, dim3(p->n_out), 256, 0, st, tok, D, (const ImgDesc*)p->d_desc,
                      (const WorkItem*)p->d_out, (const int*)c->S_idx, (const int*)c->T_idx,
                      (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, after_correlate,
                      c->status, (int*)nullptr, 0);
   c->launches += 1;
   if (p->key.conv) {
     prof_tick(c, st, "convergent_token");
-    k_convergent_token<T><<<p->key.batch, 256, 0, st>>>(tok, D, p->d_desc, c->S_idx, out_tokens, c->status);
+    launch_dependent(k_convergent_token<T>, dim3(p->key.batch), 256, 0, st,
+      tok, D, p->d_desc, c->S_idx, out_tokens, c->status);
     c->launches += 1;
   }
   prof_tick(c, st, nullptr);
@@ -1298,7 +1306,7 @@ extern "C" int ficoco_v_reduce_schedule(ficoco_ctx* c, const ficoco_v_args* firs
     np = keep[s];
   }
   const int n_out = B * (cls + keep[n_steps - 1]);
-  launch_dependent(k_compose_kept, (n_out + 255) / 256, 256, 0, st, ca, B, first->kept_idx);
+  launch_dependent(k_compose_kept, dim3((n_out + 255) / 256), 256, 0, st, ca, B, first->kept_idx);
   c->launches = total_launches + 1;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { c->last_cuda = (int)e; return FICOCO_ERR_CUDA; }
@@ -1335,7 +1343,8 @@ extern "C" int ficoco_l_reduce(ficoco_ctx* c, const ficoco_l_args* a, const fico
   c->last_plan = p;
   c->launches = 0;
   prof_tick(c, st, "head_mean");
-  k_head_mean<<<a->batch * a->n_text, 256, 0, st>>>(a->attn_t2v, a->heads, a->n_text, a->n_vision, c->tmean);
+  launch_dependent(k_head_mean, dim3(a->batch * a->n_text), 256, 0, st,
+      a->attn_t2v, a->heads, a->n_text, a->n_vision, c->tmean);
   c->launches += 1;
   if (a->dtype == FICOCO_BF16)
     return run_step<__nv_bfloat16>(c, p, (const __nv_bfloat16*)a->tokens, a->dim, c->tmean, a->n_text,

@@ -55,6 +55,8 @@ __global__ void __launch_bounds__(256) k_correlate_simt(
 
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int L = d.list_len;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
 
@@ -289,6 +291,8 @@ __global__ void __launch_bounds__(256) k_finalize_src(
     const int* __restrict__ part_idx, int* __restrict__ corr_cnt, float* __restrict__ tau_out,
     int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c) {
   const ImgDesc d = desc[blockIdx.x];
+  grid_dep_wait();
+  grid_dep_launch();
   const int s = blockIdx.y * 256 + threadIdx.x;
   if (s >= d.n_src) return;
   finalize_source<KCAP>(d, s, part_val, part_idx, corr_cnt, tau_out, e_tgt, e_w, e_c);

@@ -1,4 +1,8 @@
 // Filter stage (Eq. 1, local penalty, top-N^S selection).
+//
+// Every kernel of a step is launched under the tail of the grid before it (programmatic stream serialization): it
+// reads its plan entries, which are constants, then waits for that grid to be complete and only then lets the next
+// one in.  A grid that runs therefore finds everything before its predecessor complete as well.
 #pragma once
 #include "async_ops.cuh"
 #include "common.cuh"
@@ -17,6 +21,8 @@ __global__ void __launch_bounds__(256) k_rownorm(const T* __restrict__ tokens, i
   constexpr int E = VecTraits<T>::E;
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nvec = D / E;
   for (int r = warp; r < w.nrows; r += 8) {
@@ -61,6 +67,8 @@ __global__ void __launch_bounds__(256) k_colsum(const T* __restrict__ tokens, in
   extern __shared__ float sm_acc[];  // VPL*32*E floats
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slab = blockIdx.y;
   const int c0 = slab * (VPL * 32 * E);
@@ -153,6 +161,8 @@ __global__ void __launch_bounds__(256) k_colsum(const T* __restrict__ tokens, in
 __global__ void __launch_bounds__(256) k_msum(int D, const ImgDesc* __restrict__ desc,
                                               const float* __restrict__ partial, float* __restrict__ msum) {
   const ImgDesc d = desc[blockIdx.x];
+  grid_dep_wait();
+  grid_dep_launch();
   const int c = blockIdx.y * 256 + threadIdx.x;
   if (c >= D) return;
   float s = 0.f;
@@ -191,6 +201,8 @@ __global__ void __launch_bounds__(256) k_score(const T* __restrict__ tokens, int
   extern __shared__ float sm[];  // msum[D], v[nrows], attention partial sums [8][nrows]
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   float* msum = sm;
   float* vrow = sm + D;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -274,6 +286,8 @@ __global__ void __launch_bounds__(256, 2) k_colsum_wide(const T* __restrict__ to
   __shared__ __align__(16) float red[2][RB][8];
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nvec = D / E;
   const T* base = tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D;
@@ -343,6 +357,8 @@ __global__ void __launch_bounds__(256) k_score_wide(const T* __restrict__ tokens
   __shared__ __align__(16) float red[2][RB][8];
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nvec = D / E;
   const T* base = tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D;
@@ -399,6 +415,8 @@ __global__ void __launch_bounds__(256) k_score_wide(const T* __restrict__ tokens
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_head_mean(const float* __restrict__ attn, int H, int M,
                                                    int N, float* __restrict__ t) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int b = blockIdx.x / M, k = blockIdx.x % M;
   const float inv_h = 1.0f / (float)H;
   const float* src = attn + ((size_t)b * H * M + k) * N;
@@ -915,6 +933,8 @@ __global__ void __launch_bounds__(1024) k_select(const ImgDesc* __restrict__ des
   __shared__ SelectShared sh;
   __shared__ SelectSmallShared shs;
   const ImgDesc d = desc[blockIdx.x];
+  grid_dep_wait();
+  grid_dep_launch();
   if (d.np <= SEL_SMALL_MAX && blockDim.x == SEL_SMALL_THREADS) {
     select_small_prepare(d, penalty, sm_raw, threadIdx.x);
     __syncthreads();

@@ -360,6 +360,8 @@ __global__ void __launch_bounds__(256) k_convergent_token(
   constexpr int E = VecTraits<T>::E;
   __shared__ float part[8][128 * E];
   const ImgDesc d = desc[blockIdx.x];
+  grid_dep_wait();
+  grid_dep_launch();
   if (!d.n_extra || (*status & STATUS_TIMEOUT)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nvec = D / E;

@@ -31,6 +31,8 @@ __global__ void __launch_bounds__(256) k_score_rel(const float* __restrict__ rel
   __shared__ float4 red4[16][16];
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int np = d.np;
   const float* A = rel + d.rel0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -173,6 +175,8 @@ __global__ void __launch_bounds__(256, LC <= 4 ? 4 : 2) k_correlate_rel(
   __shared__ int is_last;
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
   const int L = d.list_len, np = d.np;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* A = rel + d.rel0;
