@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <mutex>
 #include <vector>
@@ -25,7 +26,7 @@ namespace {
 
 constexpr int N_PLANS = 16;
 constexpr int PART_PER_TOKEN = 64;   // partial top-list entries budgeted per token row
-constexpr int OUT_ROWS_PER_CTA = MROWS_CTA;  // the merge kernel's copy batches are sized for it
+constexpr int OUT_ROWS_PER_CTA = 16;  // the merge kernel's work table is sized for this many
 constexpr int NSPLIT_MAX = 16;
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -59,6 +60,7 @@ struct Plan {
   WorkItem* d_out = nullptr;
   int n_rows = 0, n_corr = 0, n_out = 0;
   int out_rows_cta = 0;         // output rows per merge CTA
+  size_t m_smem = 0;            // and the shared memory for their input rows
   // totals and maxima used to size launches and inspection copies
   int tot_patch = 0, tot_src = 0, tot_tgt = 0, tot_out_rows = 0;
   int max_np = 0, max_tgt = 0, max_src = 0, max_rc = 0, max_nwin_cells = 0, max_list = 0;
@@ -173,8 +175,6 @@ struct ficoco_ctx {
   float* tmean = nullptr;
   unsigned* status = nullptr;
   int* tile_cnt = nullptr;  // per source tile: column splits of the correlate kernel that are done
-  int merge_ctas_per_sm = 1;    // resident CTAs of the merge kernel per SM (register cap for 3)
-  int merge_ctas_per_sm_dense = 1;   // the same with the register cap for 4 (plans without the fused filter)
   int* img_cnt = nullptr;   // two sets of 3 * max_batch per-image counters of the fused filter kernel
   unsigned long long epoch = 0;          // fused filter launches so far (its parity picks the counter set)
   int last_parity = 0;                   // counter set of the latest fused filter launch
@@ -384,7 +384,7 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   c->cap_rows = (int)(MAX_CHUNKS * B);
   if (c->cap_rows < c->num_sms + (int)B + 8) c->cap_rows = c->num_sms + (int)B + 8;
   c->cap_corr = (int)(2 * (T / CBM + B) + 2048);
-  c->cap_out = (int)(T / OUT_ROWS_PER_CTA + B);
+  c->cap_out = (int)(T / OUT_ROWS_PER_CTA + B + 2 * c->num_sms);
   c->cap_part = (long long)T * PART_PER_TOKEN;
   c->off_rows = align_up(B * sizeof(ImgDesc), 256);
   c->off_corr = c->off_rows + align_up((size_t)c->cap_rows * sizeof(WorkItem), 256);
@@ -456,13 +456,8 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
     FICOCO_FUSED_ATTR(__nv_bfloat16, 5); FICOCO_FUSED_ATTR(__nv_bfloat16, 8);
 #undef FICOCO_FUSED_ATTR
   }
-  {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_merge_scan<__nv_bfloat16, 3>, 256, 0) == cudaSuccess && nb > 0)
-      c->merge_ctas_per_sm = nb;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_merge_scan<__nv_bfloat16, 4>, 256, 0) == cudaSuccess && nb > 0)
-      c->merge_ctas_per_sm_dense = nb;
-  }
+  cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
+  cudaFuncSetAttribute(k_merge_rows<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
   cudaFuncSetAttribute(k_score<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   cudaFuncSetAttribute(k_score<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   if (cudaGetLastError() != cudaSuccess) { ficoco_destroy(c); return FICOCO_ERR_CUDA; }
@@ -637,36 +632,22 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     want_split = best.want_split;
   }
 
-  // output rows per merge CTA: fewer than the usual 16 when that would leave most SMs with less
-  // than two CTAs (few or very wide rows), as far as the work table goes
-  int out_rows_cta = OUT_ROWS_PER_CTA;
+  // Output rows per merge CTA: the fewest that make one wave of two CTAs per SM, or else as many as the shared
+  // memory for their input rows takes, evened out over the waves.
+  int out_rows_cta = 1;
   {
+    const size_t row_b = (size_t)key.dim * (key.dtype == FICOCO_BF16 ? 2 : 4);
+    const int most = (int)std::min<size_t>(MROWS, std::max<size_t>(1, MSTAGE_BYTES / row_b));
+    const long long slots = 2LL * c->num_sms;
     auto n_out_ctas = [&](int r) {
       long long n = 0;
       for (int b = 0; b < B; ++b) n += (cls + key.keep[b] + p->h_desc[b].n_extra + tail + r - 1) / r;
       return n;
     };
-    // An output row costs its own input row plus the discarded rows folded into it: with many
-    // discarded tokens per preserved one (keep 1/9: nine rows read per row written) the CTAs are
-    // kept smaller still, up to four per SM slot pair (measured: 16 ragged images keeping 1/9,
-    // 133 -> 125 us per step with 4 instead of 8 rows per CTA; a 1/2 schedule loses 3 us that way).
-    long long rows_out = 0, rows_src = 0;
-    for (int b = 0; b < B; ++b) {
-      rows_out += cls + key.keep[b] + p->h_desc[b].n_extra + tail;
-      rows_src += key.ntok[b] - cls - tail - key.keep[b];
-    }
-    const long long reads_per_row = rows_out > 0 ? (rows_out + rows_src) / rows_out : 1;
-    const long long want_ctas = (reads_per_row >= 4 ? 4LL : 2LL) * c->num_sms;
-    while (out_rows_cta > 2 && n_out_ctas(out_rows_cta) < want_ctas &&
-           n_out_ctas(out_rows_cta / 2) <= c->cap_out)
-      out_rows_cta /= 2;
-    // 24 rows per CTA when the grid then fits the SMs in one go and did not before.  Not ahead of the
-    // persistent filter: the next step's filter grid starts only once every SM has drained, and longer
-    // merge CTAs delay that by more than the saved wave gains (measured: +2.4 us per step with, -4.5 us
-    // per step on a supplied relation map, whose score kernel is an ordinary grid).
-    const long long slots = (long long)c->num_sms * (p->fused ? c->merge_ctas_per_sm : c->merge_ctas_per_sm_dense);
-    if (out_rows_cta == OUT_ROWS_PER_CTA && n_out_ctas(16) > slots && n_out_ctas(24) <= slots && !p->fused) out_rows_cta = 24;
+    const long long waves = (n_out_ctas(most) + slots - 1) / slots;
+    while (out_rows_cta < most && (n_out_ctas(out_rows_cta) > waves * slots || n_out_ctas(out_rows_cta) > c->cap_out)) ++out_rows_cta;
     p->out_rows_cta = out_rows_cta;
+    p->m_smem = out_rows_cta * row_b;
   }
   for (int b = 0; b < B; ++b) {
     ImgDesc& d = p->h_desc[b];
@@ -1101,16 +1082,11 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   }
   prof_tick(c, st, "merge_compact");
   const int after_correlate = p->n_corr > 0 ? 1 : 0;   // else the grid before may be the filter itself
-  if (p->fused)
-    launch_dependent(k_merge_scan<T, 3>, dim3(p->n_out), 256, 0, st, tok, D, (const ImgDesc*)p->d_desc,
-                     (const WorkItem*)p->d_out, (const int*)c->S_idx, (const int*)c->T_idx,
-                     (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, after_correlate,
-                     c->status, c->img_cnt + (size_t)c->last_parity * 3 * c->max_batch, 3 * c->max_batch);
-  else
-    launch_dependent(k_merge_scan<T, 4>, dim3(p->n_out), 256, 0, st, tok, D, (const ImgDesc*)p->d_desc,
-                     (const WorkItem*)p->d_out, (const int*)c->S_idx, (const int*)c->T_idx,
-                     (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, after_correlate,
-                     c->status, (int*)nullptr, 0);
+  launch_dependent(k_merge_rows<T>, dim3(p->n_out), MTHREADS, p->m_smem, st, tok, D, (const ImgDesc*)p->d_desc,
+                   (const WorkItem*)p->d_out, (const int*)c->S_idx, (const int*)c->T_idx,
+                   (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, after_correlate, c->status,
+                   p->fused ? c->img_cnt + (size_t)c->last_parity * 3 * c->max_batch : (int*)nullptr,
+                   p->fused ? 3 * c->max_batch : 0, c->wait_ns);
   c->launches += 1;
   if (p->key.conv) {
     prof_tick(c, st, "convergent_token");

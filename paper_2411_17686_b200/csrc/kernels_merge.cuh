@@ -5,111 +5,100 @@
 
 namespace ficoco {
 
-constexpr int MHUB = 4;        // source rows a lane has in flight for a hub row
-constexpr int MROWS = 32;      // most output rows a CTA can take (sizes of the per-row arrays)
-constexpr int MROWS_CTA = 16;  // output rows per CTA the host plans (two per warp); 24 when that saves a wave
-constexpr int MCOPY = MROWS_CTA / 8;   // rows a warp copies in one batch
-constexpr int MLIST = 1024;    // (source, alpha) entries a CTA can hold in shared memory
-constexpr int MHEAVY = 2;      // rows with more sources than this are split into 32-vector blocks over the warps
-constexpr int MVB = 4;         // 16-byte vectors a lane accumulates at a time
+constexpr int MTHREADS = 512;
+constexpr int MWARPS = MTHREADS / 32;
+constexpr int MROWS = 64;      // most output rows a CTA takes (a lane looks after two in the scan)
+constexpr int MLIST = 1024;    // sources a CTA files in shared memory
+constexpr int MDEPTH = 6;      // source rows a warp has in flight
+constexpr size_t MSTAGE_BYTES = 70 * 1024;   // input rows of a CTA's output rows kept in shared memory (two CTAs per SM)
 
-// acc[b][.] += sum over list entries [k0, k1) of alpha * x, for the MVB vectors v0 + 32 b of
-// each row; source rows are fetched four at a time so that 4 * MVB loads are in flight per lane.
-template <class T>
-__device__ __forceinline__ void merge_accumulate(float (&acc)[MVB][VecTraits<T>::E], const T* pbase, int D,
-                                                 const int* lsrc, const float* lw, int k0, int k1,
-                                                 int v0, int nvec) {
-  constexpr int E = VecTraits<T>::E;
-  #pragma unroll 1
-  for (int k = k0; k < k1; k += 4) {
-    uint4 u[4][MVB];
-    float a[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const bool on = k + j < k1;
-      const T* x = pbase + (size_t)lsrc[on ? k + j : k] * D;
-      a[j] = on ? lw[k + j] : 0.f;
-#pragma unroll
-      for (int b = 0; b < MVB; ++b) {
-        const int v = v0 + 32 * b;
-        u[j][b] = (on && v < nvec) ? ldg16(x + (size_t)v * E) : make_uint4(0, 0, 0, 0);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int b = 0; b < MVB; ++b) {
-        float f[E];
-        unpack(u[j][b], f, (const T*)nullptr);
-#pragma unroll
-        for (int q = 0; q < E; ++q) acc[b][q] = fmaf(a[j], f[q], acc[b][q]);
-      }
-  }
-}
-
-// Compress + compact.  No per-target lists are built in global memory.  A CTA owns up to 32
-// consecutive output rows of one image (warp w: rows w, w + 8, w + 16, w + 24).
-//   1. every warp resolves the input row of its output rows (L1 prefetches of the rows were tried:
-//      they never produced L1 hits and cost 1.7 us per step, so there are none);
-//   2. meanwhile the CTA scans the image's (source -> target) entries twice (count, then fill)
-//      to file those that hit its rows into per-row lists in shared memory (token index,
-//      alpha), and orders every list by token index so that the
-//      fp32 sums have one fixed order and no atomics touch floats;
-//   3. out_j = (x_j + sum_{i in I_j} alpha_ij x_i) / (1 + sum alpha_ij), rounded once:
-//      rows with few sources by their own warp; hub rows are cut into blocks of 32 vectors that
-//      are dealt to the warps, every lane summing the sources of its vector in list order.
+// Compress + compact.  A CTA owns a few consecutive output rows of one image.
+//   rows    the input rows of its output rows are fetched into shared memory by bulk copies (TMA) as soon as the
+//           index lists exist, i.e. under the tail of the correlate grid;
+//   file    the image's (source -> target) entries that hit its rows are filed into per-row lists in shared
+//           memory, ordered by discarded token, so that every fp32 sum has one fixed order and no atomics touch
+//           floats; one pass over the entries, four loads in flight per thread;
+//   copies  a row that nothing is folded into leaves by a bulk store from shared memory: no thread touches it;
+//   merge   out_j = (x_j + sum_{i in I_j} alpha_ij x_i) / (1 + sum alpha_ij), rounded once.  (slices of 32
+//           vectors) x (own rows and sources, in list order) form one sequence of which every warp takes an equal
+//           segment, MDEPTH source rows in flight: rows with one source and hubs with dozens cost what their
+//           elements cost.  A group cut by the end of a segment is left in pieces in shared memory, which are
+//           added in order.
+// What bounds it is the latency of its few dependent trips to L2; the split into 16 warps and the host's choice of
+// one wave of CTAs where possible keep them few: 32 x 577 -> 289 rows of 1024 went from 25 us (a scan per 16 rows,
+// copies and hub rows by warps, two waves of CTAs) to MERGE_US us.
 // If the CTA's rows receive more than MLIST sources in total, a slow in-order rescan is used.
-// MINB (resident CTAs per SM the registers are capped for): 4 fills the SMs better when the merge
-// grid runs between ordinary grids; 3 (no spills, fewer and shorter waves of CTAs draining) is
-// faster when the next step's persistent filter grid is waiting for every SM to drain.
-template <class T, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_merge_scan(
+template <class T>
+__global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
     const T* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
     const WorkItem* __restrict__ work, const int* __restrict__ S_idx, const int* __restrict__ T_idx,
     const int* __restrict__ e_tgt, const float* __restrict__ e_w, T* __restrict__ out,
-    int index_before_wait, unsigned* __restrict__ status, int* __restrict__ filter_cnt, int n_filter_cnt) {
+    int index_before_wait, unsigned* __restrict__ status, int* __restrict__ filter_cnt, int n_filter_cnt,
+    unsigned long long wait_ns) {
   constexpr int E = VecTraits<T>::E;
-  __shared__ int cnt[MROWS], beg[MROWS + 1], cur[MROWS], srow_s[MROWS];
-  __shared__ int lsrc[MLIST];
-  __shared__ float lw[MLIST];
-  __shared__ int tsrc[MLIST];
-  __shared__ float tw[MLIST];
-  __shared__ int heavy_rows[MROWS];
-  __shared__ int n_heavy, dead;
+  constexpr int PW = E + 1;                      // a piece: E sums and the weight of a lane, lanes side by side
+  extern __shared__ __align__(128) unsigned char stage[];     // [rows][row bytes]
+  __shared__ int cnt[MROWS], gbeg[MROWS + 1], beg[MROWS + 1], srow_s[MROWS];
+  __shared__ int m_e[MLIST], bucket[MLIST];
+  __shared__ unsigned short m_rs[MLIST];         // row << 10 | slot inside the row's bucket
+  __shared__ uint2 el[MLIST + MROWS];            // weight, row << 16 | source token (the group's own row: anything)
+  __shared__ float fold[MWARPS * PW * 32];
+  __shared__ uint64_t row_bar;
+  __shared__ int n_match, dead;
   FICOCO_PHASE_BEGIN(2);
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nvec = D / E;
+  const int nvec = D / E, row_bytes = D * (int)sizeof(T);
   const int L = d.list_len;
   const int tp_lo = max(w.r0 - d.n_cls, 0);
   const int tp_hi = min(w.r0 + w.nrows - d.n_cls, d.n_tgt);
-  const int n_ent = d.n_src * L;
+  const int r_tgt = d.n_cls + tp_lo - w.r0;      // row (inside the CTA) of target tp_lo
+  const int n_ent = tp_hi > tp_lo ? d.n_src * L : 0;
   const T* pbase = tokens + (size_t)(d.row0 + d.n_cls) * D;
 
-  if (tid < MROWS) { cnt[tid] = 0; cur[tid] = 0; }
-  if (tid == 0) n_heavy = 0;
+  if (tid < MROWS) cnt[tid] = 0;
+  if (tid == 0) n_match = 0;
   // When the grid before this one is a correlate grid, the filter grid (which wrote T_idx) had
-  // completed before this grid could start, so the row lookup may overlap that
+  // completed before this grid could start, so the rows may be looked up and fetched under that
   // grid's tail; otherwise wait first.
   if (!index_before_wait) grid_dep_wait();
-  // input row of every output row (CLS / preserved token / trailing text row)
-  #pragma unroll 1
-  for (int r = warp; r < w.nrows; r += 8) {
-    const int orow = w.r0 + r;
-    int srow;
-    if (orow < d.n_cls) srow = orow;
-    else if (orow < d.n_cls + d.n_tgt) srow = d.n_cls + checked_index(T_idx[d.tgt0 + orow - d.n_cls], d.np, status);
-    else if (orow < d.n_cls + d.n_tgt + d.n_extra) srow = -1;     // the additional token: written by k_convergent_token
-    else srow = d.n_cls + d.np + (orow - d.n_cls - d.n_tgt - d.n_extra);
-    if (lane == 0) srow_s[r] = srow;
+  if (warp == 0) {
+    // input row of every output row (CLS / preserved token / trailing text row; -1: the additional token, which
+    // k_convergent_token writes)
+    if (lane == 0) {
+      mbar_init(&row_bar, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    int srow[2], n = 0;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int r = lane + 32 * j, orow = w.r0 + r;
+      srow[j] = -1;
+      if (r < w.nrows) {
+        if (orow < d.n_cls) srow[j] = orow;
+        else if (orow < d.n_cls + d.n_tgt) srow[j] = d.n_cls + checked_index(T_idx[d.tgt0 + orow - d.n_cls], d.np, status);
+        else if (orow >= d.n_cls + d.n_tgt + d.n_extra) srow[j] = d.n_cls + d.np + (orow - d.n_cls - d.n_tgt - d.n_extra);
+        srow_s[r] = srow[j];
+        n += srow[j] >= 0 ? 1 : 0;
+      }
+    }
+    n = __reduce_add_sync(0xFFFFFFFFu, n);
+    if (lane == 0) mbar_expect_tx(&row_bar, (uint32_t)n * (uint32_t)row_bytes);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      if (srow[j] >= 0)
+        bulk_load(stage + (size_t)(lane + 32 * j) * row_bytes, tokens + (size_t)(d.row0 + srow[j]) * D, (uint32_t)row_bytes,
+                  &row_bar);
   }
+  __syncthreads();
   if (index_before_wait) grid_dep_wait();
   // The filter grid of this step is complete: its per-image counters are cleared for whichever launch
   // uses that set next (launches replayed from graphs need not alternate between the two sets).  The
   // stores are fenced and the CTA synchronised before it releases the dependent grid.
   if (filter_cnt != nullptr && blockIdx.x == 0) {
-    for (int i = tid; i < n_filter_cnt; i += 256) filter_cnt[i] = 0;
+    for (int i = tid; i < n_filter_cnt; i += MTHREADS) filter_cnt[i] = 0;
     __threadfence();
     __syncthreads();
   }
@@ -117,176 +106,178 @@ __global__ void __launch_bounds__(256, MINB) k_merge_scan(
   FICOCO_PHASE(2, 1);
   // a step whose filter or correlate grid gave up has no valid index lists: write nothing
   if (tid == 0) dead = (*reinterpret_cast<const volatile unsigned*>(status) & STATUS_TIMEOUT) ? 1 : 0;
-  __syncthreads();
-  if (dead) return;
-  // file the entries that hit this CTA's rows.  Up to 1024 entries per image every thread looks
-  // at no more than four, keeps its matches in registers and needs one pass; larger images
-  // take a counting pass and a filling pass.
-  const bool one_pass = n_ent <= 4 * 256;
-  int st_row[4], st_slot[4], st_src[4];
-  float st_w[4];
+  // ---- file the entries that hit this CTA's rows ----------------------------------------------------
+  for (int e0 = tid; e0 < n_ent; e0 += 4 * MTHREADS) {
+    int t[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) st_row[i] = -1;
-  if (tp_hi > tp_lo) {
-    if (one_pass) {
-      int t4[4];
+    for (int i = 0; i < 4; ++i) t[i] = e0 + MTHREADS * i < n_ent ? e_tgt[d.ent0 + e0 + MTHREADS * i] : -1;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        // target, source and weight are fetched together: a source fetched only for the matches
-        // would add a second round trip to L2
-        const int e = tid + 256 * i;
-        const bool on = e < n_ent;
-        t4[i] = on ? e_tgt[d.ent0 + e] : -1;
-        st_src[i] = on ? checked_index(S_idx[d.src0 + e / L], d.np, status) : 0;
-        st_w[i] = on ? e_w[d.ent0 + e] : 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int t = t4[i];
-        if (t >= tp_lo && t < tp_hi) {
-          st_row[i] = t - tp_lo;
-          st_slot[i] = atomicAdd(&cnt[t - tp_lo], 1);
+    for (int i = 0; i < 4; ++i)
+      if (t[i] >= tp_lo && t[i] < tp_hi) {
+        const int r = r_tgt + t[i] - tp_lo, slot = atomicAdd(&cnt[r], 1), k = atomicAdd(&n_match, 1);
+        if (k < MLIST) {
+          m_e[k] = e0 + MTHREADS * i;
+          m_rs[k] = (unsigned short)(r << 10 | (slot & 1023));
         }
       }
-    } else {
-      for (int e = tid; e < n_ent; e += 256) {
-        const int t = e_tgt[d.ent0 + e];
-        if (t >= tp_lo && t < tp_hi) atomicAdd(&cnt[t - tp_lo], 1);
-      }
-    }
   }
   __syncthreads();
+  const int total = n_match;
+  const bool fits = total <= MLIST;
+  bool rows_ok = true;
+  if (dead) {
+    mbar_wait(&row_bar, 0, wait_ns);             // no copy outlives the CTA
+    return;
+  }
   if (warp == 0) {
-    // exclusive scan of the 32 counts
-    const int c = cnt[lane];
-    int inc = c;
+    // starts of the buckets, and of the groups (own row + sources) of the rows that have sources
+    const int c0 = cnt[2 * lane], c1 = cnt[2 * lane + 1];
+    const int g0 = c0 > 0 ? c0 + 1 : 0, g1 = c1 > 0 ? c1 + 1 : 0;
+    int inc = (c0 + c1) << 16 | (g0 + g1);       // (both totals stay below 2^15 where they are used)
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
       if (lane >= o) inc += n;
     }
-    beg[lane] = inc - c;
-    if (lane == 31) beg[MROWS] = inc;
-    if (c > MHEAVY) heavy_rows[atomicAdd(&n_heavy, 1)] = lane;
+    const int exc = inc - ((c0 + c1) << 16 | (g0 + g1));
+    beg[2 * lane] = exc >> 16; beg[2 * lane + 1] = (exc >> 16) + c0;
+    gbeg[2 * lane] = exc & 0xFFFF; gbeg[2 * lane + 1] = (exc & 0xFFFF) + g0;
+    if (lane == 31) { beg[MROWS] = inc >> 16; gbeg[MROWS] = inc & 0xFFFF; }
   }
   __syncthreads();
-  const int total = beg[MROWS];
-  const bool fits = total <= MLIST;
+  int my_src[MLIST / MTHREADS];
+  float my_w[MLIST / MTHREADS];
   if (fits && total > 0) {
-    if (one_pass) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (st_row[i] >= 0) {
-          const int slot = beg[st_row[i]] + st_slot[i];
-          tsrc[slot] = st_src[i];
-          tw[slot] = st_w[i];
-        }
-    } else {
-      for (int e = tid; e < n_ent; e += 256) {
-        const int t = e_tgt[d.ent0 + e];
-        if (t >= tp_lo && t < tp_hi) {
-          const int slot = beg[t - tp_lo] + atomicAdd(&cur[t - tp_lo], 1);
-          const int si = checked_index(S_idx[d.src0 + e / L], d.np, status);
-          tsrc[slot] = si;
-          tw[slot] = e_w[d.ent0 + e];
-        }
+    for (int q = 0; q < MLIST / MTHREADS; ++q) {
+      const int i = tid + MTHREADS * q;
+      if (i < total) {
+        const int e = m_e[i], rs = m_rs[i];
+        my_src[q] = S_idx[d.src0 + e / L];
+        my_w[q] = e_w[d.ent0 + e];
+        bucket[beg[rs >> 10] + (rs & 1023)] = e;
+      }
+    }
+    if (tid < w.nrows && cnt[tid] > 0) el[gbeg[tid]] = make_uint2(__float_as_uint(1.0f), (uint32_t)tid << 16);
+    __syncthreads();
+    // the list of a row is ordered by entry, i.e. by discarded token
+#pragma unroll
+    for (int q = 0; q < MLIST / MTHREADS; ++q) {
+      const int i = tid + MTHREADS * q;
+      if (i < total) {
+        const int e = m_e[i], r = m_rs[i] >> 10, b = beg[r], n = cnt[r];
+        int rank = 0;
+        for (int k = 0; k < n; ++k) rank += bucket[b + k] < e ? 1 : 0;
+        el[gbeg[r] + 1 + rank] = make_uint2(__float_as_uint(my_w[q]), (uint32_t)r << 16 | (uint32_t)checked_index(my_src[q], d.np, status));
       }
     }
     __syncthreads();
-    // order every list by token index (rank of each entry inside its row)
-    for (int i = tid; i < total; i += 256) {
-      int r = 0;
-      while (i >= beg[r + 1]) ++r;
-      const int my = tsrc[i];
-      int rank = 0;
-      for (int k = beg[r]; k < beg[r + 1]; ++k) rank += tsrc[k] < my ? 1 : 0;
-      lsrc[beg[r] + rank] = my;
-      lw[beg[r] + rank] = tw[i];
-    }
   }
-  __syncthreads();
-
   FICOCO_PHASE(2, 2);
-  // ---- rows without sources: plain copies, all of a warp's rows in flight together --------------
-  #pragma unroll 1
-  for (int j0 = 0; 8 * j0 < w.nrows; j0 += MCOPY)
-  #pragma unroll 1
-  for (int v0 = lane; v0 < nvec; v0 += 32 * MVB) {
-    uint4 u[MCOPY][MVB];
+  rows_ok = mbar_wait(&row_bar, 0, wait_ns);
+  if (!rows_ok) { atomicOr(status, STATUS_TIMEOUT); return; }
+  // ---- rows without sources leave shared memory as they came ------------------------------------------
+  if (warp == 0) {
 #pragma unroll
-    for (int j = 0; j < MCOPY; ++j) {
-      const int r = warp + 8 * (j0 + j);
-      const int orow = w.r0 + r;
-      const bool is_tgt = orow >= d.n_cls && orow < d.n_cls + d.n_tgt;
-      const bool copy = r < w.nrows && srow_s[r < w.nrows ? r : 0] >= 0 && (!is_tgt || cnt[orow - d.n_cls - tp_lo] == 0);
-      const T* src = tokens + (size_t)(d.row0 + (copy ? srow_s[r] : 0)) * D;
-#pragma unroll
-      for (int b = 0; b < MVB; ++b) {
-        const int v = v0 + 32 * b;
-        u[j][b] = (copy && v < nvec) ? ldg16(src + (size_t)v * E) : make_uint4(0, 0, 0, 0);
-      }
+    for (int j = 0; j < 2; ++j) {
+      const int r = lane + 32 * j;
+      if (r < w.nrows && cnt[r] == 0 && srow_s[r] >= 0)
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                     ::"l"(out + (size_t)(d.out_row0 + w.r0 + r) * D), "r"(smem_u32(stage + (size_t)r * row_bytes)), "r"(row_bytes)
+                     : "memory");
     }
-#pragma unroll
-    for (int j = 0; j < MCOPY; ++j) {
-      const int r = warp + 8 * (j0 + j);
-      const int orow = w.r0 + r;
-      const bool is_tgt = orow >= d.n_cls && orow < d.n_cls + d.n_tgt;
-      const bool copy = r < w.nrows && srow_s[r < w.nrows ? r : 0] >= 0 && (!is_tgt || cnt[orow - d.n_cls - tp_lo] == 0);
-      T* dst = out + (size_t)(d.out_row0 + orow) * D;
-#pragma unroll
-      for (int b = 0; b < MVB; ++b) {
-        const int v = v0 + 32 * b;
-        if (copy && v < nvec) st_stream16(reinterpret_cast<uint4*>(dst) + v, u[j][b]);
-      }
-    }
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }
-
   FICOCO_PHASE(2, 3);
-  // ---- rows with a few sources: one warp per row --------------------------------------------------
-  #pragma unroll 1
-  for (int r = warp; r < w.nrows; r += 8) {
-    const int orow = w.r0 + r;
-    T* dst = out + (size_t)(d.out_row0 + orow) * D;
-    const bool is_tgt = orow >= d.n_cls && orow < d.n_cls + d.n_tgt;
-    const int li = is_tgt ? orow - d.n_cls - tp_lo : 0;
-    const int n = is_tgt ? cnt[li] : 0;
-    const T* src = tokens + (size_t)(d.row0 + srow_s[r]) * D;
-    if (n == 0) {
-      continue;
-    } else if (fits && n <= MHEAVY) {
-      const int b0 = beg[li];
-      float wsum = 0.f;
-      for (int k = 0; k < n; ++k) wsum += lw[b0 + k];
-      const float inv_den = 1.0f / (1.0f + wsum);   // one division per row, then multiplies
+  // ---- rows with sources ------------------------------------------------------------------------------
+  if (fits && total > 0) {
+    const int n_el = gbeg[MROWS], n_all = n_el * ((nvec + 31) / 32);
+    auto seg = [&](int k) { return (int)((long long)n_all * k / MWARPS); };
+    const int p_hi = seg(warp + 1);
+    float* piece = fold + warp * PW * 32 + lane;
+    float acc[E], den = 0.f;
+    int tail = -1;                               // where a group that goes on behind the segment began
+    #pragma unroll 1
+    for (int p = seg(warp); p < p_hi;) {
+      const int sl = p / n_el, e0 = p - sl * n_el, r = (int)(el[e0].y >> 16);
+      const int start = gbeg[r], end = start + 1 + cnt[r], e_hi = min(end, e0 + (p_hi - p));
+      const int v = 32 * sl + lane;
+      const bool on = v < nvec;
+      const T* col = pbase + (size_t)(on ? v : 0) * E;
+      int e = e0;
+      if (e0 == start) {
+        unpack(*reinterpret_cast<const uint4*>(stage + (size_t)r * row_bytes + (size_t)(on ? v : 0) * 16), acc, (const T*)nullptr);
+        den = 1.0f;
+        ++e;
+      } else {
+        den = 0.f;
+#pragma unroll
+        for (int q = 0; q < E; ++q) acc[q] = 0.f;
+      }
       #pragma unroll 1
-      for (int v0 = lane; v0 < nvec; v0 += 32 * MVB) {
-        float acc[MVB][E];
+      for (; e < e_hi; e += MDEPTH) {
+        uint4 u[MDEPTH];
 #pragma unroll
-        for (int b = 0; b < MVB; ++b) {
-          const int v = v0 + 32 * b;
-          unpack(v < nvec ? ldg16(src + (size_t)v * E) : make_uint4(0, 0, 0, 0), acc[b], (const T*)nullptr);
-        }
-        merge_accumulate<T>(acc, pbase, D, lsrc, lw, b0, b0 + n, v0, nvec);
+        for (int j = 0; j < MDEPTH; ++j)         // (past the end: the last row again, weight 0)
+          u[j] = ldg16(col + (size_t)(el[min(e + j, e_hi - 1)].y & 0xFFFFu) * D);
 #pragma unroll
-        for (int b = 0; b < MVB; ++b) {
-          const int v = v0 + 32 * b;
-          if (v < nvec) {
+        for (int j = 0; j < MDEPTH; ++j) {
+          const float a = e + j < e_hi ? __uint_as_float(el[e + j].x) : 0.f;
+          float x[E];
+          unpack(u[j], x, (const T*)nullptr);
+          den += a;
 #pragma unroll
-            for (int q = 0; q < E; ++q) acc[b][q] = acc[b][q] * inv_den;
-            st_stream16(reinterpret_cast<uint4*>(dst) + v, pack(acc[b], (const T*)nullptr));
-          }
+          for (int q = 0; q < E; ++q) acc[q] = fmaf(a, x[q], acc[q]);
         }
       }
-    } else if (!fits) {
-      // too many sources for shared memory: walk the entries in order (ascending source)
-      const int tp = orow - d.n_cls;
+      if (e0 == start && e_hi < end) {           // stays in registers: it is the last piece of the segment
+        tail = p;
+        break;
+      }
+      if (e0 == start) {
+        const float inv = 1.0f / den;
+#pragma unroll
+        for (int q = 0; q < E; ++q) acc[q] *= inv;
+        if (on) st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r) * D) + v, pack(acc, (const T*)nullptr));
+      } else {
+#pragma unroll
+        for (int q = 0; q < E; ++q) piece[q * 32] = acc[q];
+        piece[E * 32] = den;
+      }
+      p += e_hi - e0;
+    }
+    FICOCO_PHASE(2, 4);
+    __syncthreads();
+    if (tail >= 0) {
+      // add the pieces of the segments that the group reaches
+      const int sl = tail / n_el, r = (int)(el[tail - sl * n_el].y >> 16), end = sl * n_el + gbeg[r] + 1 + cnt[r];
+      const int v = 32 * sl + lane;
+      for (int k = warp + 1; k < MWARPS && seg(k) < end; ++k) {
+        if (seg(k) == seg(k + 1)) continue;
+        const float* x = fold + k * PW * 32 + lane;
+        den += x[E * 32];
+#pragma unroll
+        for (int q = 0; q < E; ++q) acc[q] += x[q * 32];
+      }
+      const float inv = 1.0f / den;
+#pragma unroll
+      for (int q = 0; q < E; ++q) acc[q] *= inv;
+      if (v < nvec)
+        st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r) * D) + v, pack(acc, (const T*)nullptr));
+    }
+  } else if (total > 0) {
+    // too many sources for shared memory: walk the entries in order (ascending source)
+    #pragma unroll 1
+    for (int r = warp; r < w.nrows; r += MWARPS) {
+      if (cnt[r] == 0) continue;
+      const int tp = w.r0 + r - d.n_cls;
       float wsum = 0.f;
       for (int e = 0; e < n_ent; ++e)
         if (e_tgt[d.ent0 + e] == tp) wsum += e_w[d.ent0 + e];
       const float den = 1.0f + wsum;
       for (int v = lane; v < nvec; v += 32) {
         float acc[E];
-        unpack(ldg16(src + (size_t)v * E), acc, (const T*)nullptr);
+        unpack(*reinterpret_cast<const uint4*>(stage + (size_t)r * row_bytes + (size_t)v * 16), acc, (const T*)nullptr);
         for (int e = 0; e < n_ent; ++e) {
           if (e_tgt[d.ent0 + e] != tp) continue;
           const T* x0 = pbase + (size_t)checked_index(S_idx[d.src0 + e / L], d.np, status) * D;
@@ -298,53 +289,11 @@ __global__ void __launch_bounds__(256, MINB) k_merge_scan(
         }
 #pragma unroll
         for (int q = 0; q < E; ++q) acc[q] = acc[q] / den;
-        st_stream16(reinterpret_cast<uint4*>(dst) + v, pack(acc, (const T*)nullptr));
+        st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r) * D) + v, pack(acc, (const T*)nullptr));
       }
     }
   }
-  if (!fits) return;
-
-  FICOCO_PHASE(2, 4);
-  // ---- hub rows: (row, block of 32 vectors) items dealt to the warps; each lane sums all the
-  // sources of its one vector in list order, MHUB source rows in flight ---------------------
-  const int nh = n_heavy;
-  const int nblk = (nvec + 31) / 32;
-  #pragma unroll 1
-  for (int it = warp; it < nh * nblk; it += 8) {
-    const int li = heavy_rows[it / nblk];
-    const int v = (it % nblk) * 32 + lane;
-    if (v >= nvec) continue;
-    const int tp = tp_lo + li;
-    const int b0 = beg[li], n = cnt[li];
-    const T* src = tokens + (size_t)(d.row0 + srow_s[tp + d.n_cls - w.r0]) * D;
-    T* dst = out + (size_t)(d.out_row0 + d.n_cls + tp) * D;
-    float wsum = 0.f;
-    for (int k = 0; k < n; ++k) wsum += lw[b0 + k];
-    const float inv_den = 1.0f / (1.0f + wsum);
-    float acc[E];
-    unpack(ldg16(src + (size_t)v * E), acc, (const T*)nullptr);
-    #pragma unroll 1
-    for (int k = 0; k < n; k += MHUB) {
-      uint4 u[MHUB];
-      float a[MHUB];
-#pragma unroll
-      for (int j = 0; j < MHUB; ++j) {
-        const bool on = k + j < n;
-        a[j] = on ? lw[b0 + k + j] : 0.f;
-        u[j] = on ? ldg16(pbase + (size_t)lsrc[b0 + k + j] * D + (size_t)v * E) : make_uint4(0, 0, 0, 0);
-      }
-#pragma unroll
-      for (int j = 0; j < MHUB; ++j) {
-        float f[E];
-        unpack(u[j], f, (const T*)nullptr);
-#pragma unroll
-        for (int q = 0; q < E; ++q) acc[q] = fmaf(a[j], f[q], acc[q]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < E; ++q) acc[q] = acc[q] * inv_den;
-    st_stream16(reinterpret_cast<uint4*>(dst) + v, pack(acc, (const T*)nullptr));
-  }
+  if (warp == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores have read shared memory
   FICOCO_PHASE(2, 5);
 }
 
