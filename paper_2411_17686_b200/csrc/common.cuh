@@ -44,7 +44,7 @@ struct WorkItem {
   int img;
   int r0;      // first row (patch / source slot / output row) inside the image
   int nrows;
-  int aux;     // row chunks: chunk index inside the image; correlate: column split
+  int aux;     // row chunks: chunk index inside the image; correlate: column split; output rows: distance of a CTA's rows
 };
 
 // ---------------------------------------------------------------------------------------

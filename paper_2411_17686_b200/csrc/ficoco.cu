@@ -705,9 +705,9 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     }
     // output rows
     const int orows = d.n_cls + d.n_tgt + d.n_extra + d.n_tail;
-    for (int r0 = 0; r0 < orows; r0 += out_rows_cta) {
-      WorkItem w; w.img = b; w.r0 = r0; w.nrows = (orows - r0 < out_rows_cta) ? orows - r0 : out_rows_cta;
-      w.aux = r0 / out_rows_cta;
+    const int n_cta = (orows + out_rows_cta - 1) / out_rows_cta;
+    for (int k = 0; k < n_cta; ++k) {            // rows k, k + n_cta, k + 2 n_cta, ...
+      WorkItem w; w.img = b; w.r0 = k; w.nrows = (orows - k + n_cta - 1) / n_cta; w.aux = n_cta;
       outw.push_back(w);
     }
     row0 += key.ntok[b]; patch0 += d.np; out0 += orows; src0 += d.n_src; tgt0 += d.n_tgt;
