@@ -155,6 +155,36 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+def _shape_key(v):
+    """Hashable form of a per-image count or list of counts."""
+    if v is None or isinstance(v, int):
+        return v
+    return tuple(v) if isinstance(v, (list, tuple)) else tuple(np.atleast_1d(np.asarray(v)).tolist())
+
+
+def _current_stream(dev) -> int:
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is not None and dev.index is not None:
+        return raw(dev.index)
+    return torch.cuda.current_stream(dev).cuda_stream
+
+
+@dataclass
+class _Shapes:
+    """The marshalled shapes of a call: the struct with everything but the data pointers filled in, the int32
+    arrays its pointers refer to, and the sizes of the outputs."""
+    args: "object"
+    arrays: "object"
+    out_rows: List[int]
+    n_out: int
+    n_keep: int
+    n_patch: int
+
+
+_SHAPES_KEPT = 64       # marshalled shapes a context remembers
+
+
 @dataclass
 class VResult:
     out_tokens: "object"
@@ -173,6 +203,61 @@ class Context:
         h = C.c_void_p()
         _check(None, self.lib.ficoco_create(C.byref(h), device, max_tokens, max_dim, max_batch, max_text))
         self.h = h
+        # Marshalled shapes of earlier calls (a program meets few; the oldest are dropped).  Rebuilding the arrays
+        # and structs took 20 us of every call, more than the kernels of a small image take.
+        self._shapes = {}
+
+    def _remember(self, key, make) -> _Shapes:
+        s = self._shapes.get(key)
+        if s is None:
+            s = make()
+            while len(self._shapes) >= _SHAPES_KEPT:
+                self._shapes.pop(next(iter(self._shapes)), None)
+            self._shapes[key] = s
+        return s
+
+    def _v_shapes(self, dim, dtype, rows, keep, grid_h, grid_w, heads, n_tokens, seqlens, flags) -> _Shapes:
+        cls = 1 if (flags & FICOCO_HAS_CLS) else 0
+        conv = bool(flags & FICOCO_CONVERGENT)          # one more row per image that discards something
+
+        def make():
+            keep_a, n_keep = _int_array(keep)
+            gh_a, n_gh = _int_array(grid_h)
+            gw_a, n_gw = _int_array(grid_w)
+            assert n_gh == n_gw
+            if seqlens is not None:
+                sl, batch = _int_array(seqlens)
+            else:
+                sl, batch = None, rows // n_tokens if n_tokens else 0
+            keeps = [int(keep_a[0 if n_keep == 1 else b]) for b in range(batch)]
+            ntoks = [int(sl[b]) if sl is not None else n_tokens for b in range(batch)]
+            out_rows = [cls + k + (1 if conv and n - cls - k > 0 else 0) for k, n in zip(keeps, ntoks)]
+            a = ficoco_v_args()
+            a.seqlens = sl.ctypes.data if sl is not None else None
+            a.grid_h, a.grid_w, a.keep = gh_a.ctypes.data, gw_a.ctypes.data, keep_a.ctypes.data
+            a.dtype, a.batch, a.n_tokens, a.dim, a.heads = dtype, batch, n_tokens, dim, heads
+            a.n_grid, a.n_keep = n_gh, n_keep
+            return _Shapes(a, (keep_a, gh_a, gw_a, sl), out_rows, sum(out_rows), sum(keeps), sum(ntoks) - cls * batch)
+
+        key = ("v", dim, dtype, rows, _shape_key(keep), _shape_key(grid_h), _shape_key(grid_w), heads, n_tokens,
+               _shape_key(seqlens), cls, conv)
+        return self._remember(key, make)
+
+    def _l_shapes(self, dim, dtype, rows, keep, n_vision, n_text, heads, flags) -> _Shapes:
+        conv = bool(flags & FICOCO_CONVERGENT)
+
+        def make():
+            keep_a, n_keep = _int_array(keep)
+            batch = rows // (n_vision + n_text)
+            keeps = [int(keep_a[0 if n_keep == 1 else b]) for b in range(batch)]
+            out_rows = [k + n_text + (1 if conv and n_vision - k > 0 else 0) for k in keeps]
+            a = ficoco_l_args()
+            a.keep = keep_a.ctypes.data
+            a.dtype, a.batch, a.n_vision, a.n_text = dtype, batch, n_vision, n_text
+            a.dim, a.heads, a.n_keep = dim, heads, n_keep
+            return _Shapes(a, (keep_a,), out_rows, sum(out_rows), sum(keeps), batch * n_vision)
+
+        return self._remember(("l", dim, dtype, rows, _shape_key(keep), n_vision, n_text, heads, conv), make)
 
     def close(self) -> None:
         if getattr(self, "h", None):
@@ -199,57 +284,34 @@ class Context:
         other; when given the call goes to ficoco_v_reduce_relation."""
         import torch
         p = params or ficoco_default_params()
-        cls = 1 if (p.flags & FICOCO_HAS_CLS) else 0
-        keep_a, n_keep = _int_array(keep)
-        gh_a, n_gh = _int_array(grid_h)
-        gw_a, n_gw = _int_array(grid_w)
-        assert n_gh == n_gw
-        if seqlens is not None:
-            sl, batch = _int_array(seqlens)
-        else:
-            sl = None
-            batch = tokens.shape[0] // n_tokens if n_tokens else 0
-        keeps = [int(keep_a[0 if n_keep == 1 else b]) for b in range(batch)]
-        ntoks = [int(sl[b]) if sl is not None else n_tokens for b in range(batch)]
-        conv = bool(p.flags & FICOCO_CONVERGENT)        # one more row per image that discards something
-        out_rows = [cls + k + (1 if conv and n - cls - k > 0 else 0) for k, n in zip(keeps, ntoks)]
-        dim = tokens.shape[-1]
-        dev = tokens.device
+        dim, dev = tokens.shape[-1], tokens.device
+        sh = self._v_shapes(dim, _dtype_code(tokens), tokens.shape[0], keep, grid_h, grid_w, heads, n_tokens, seqlens,
+                            p.flags)
+        a = ficoco_v_args.from_buffer_copy(sh.args)
+        if stream is None:
+            stream = _current_stream(dev)
         if plan_only:               # ficoco_v_plan: shapes only
-            a = ficoco_v_args()
-            a.seqlens = sl.ctypes.data if sl is not None else None
-            a.grid_h, a.grid_w, a.keep = gh_a.ctypes.data, gw_a.ctypes.data, keep_a.ctypes.data
-            a.dtype, a.batch, a.n_tokens, a.dim, a.heads = _dtype_code(tokens), batch, n_tokens, dim, heads
-            a.n_grid, a.n_keep = n_gh, n_keep
-            if stream is None:
-                stream = torch.cuda.current_stream(dev).cuda_stream
-            _check(self.h, self.lib.ficoco_v_plan(self.h, C.byref(a), C.byref(p), C.c_void_p(stream)))
-            return VResult(None, None, None, None, out_rows)
+            _check(self.h, self.lib.ficoco_v_plan(self.h, C.byref(a), C.byref(p), stream))
+            return VResult(None, None, None, None, list(sh.out_rows))
         if out_tokens is None:
-            out_tokens = torch.empty((sum(out_rows), dim), dtype=tokens.dtype, device=dev)
+            out_tokens = torch.empty((sh.n_out, dim), dtype=tokens.dtype, device=dev)
         if kept_idx is None:
-            kept_idx = torch.empty((sum(out_rows),), dtype=torch.int32, device=dev)
+            kept_idx = torch.empty((sh.n_out,), dtype=torch.int32, device=dev)
         if pos_out is None:
-            pos_out = torch.empty((max(sum(keeps), 1),), dtype=torch.int32, device=dev)
+            pos_out = torch.empty((max(sh.n_keep, 1),), dtype=torch.int32, device=dev)
         if scores_out is None and want_scores:
             scores_out = torch.empty((attn.numel() // heads,), dtype=torch.float32, device=dev)
-        a = ficoco_v_args()
         a.tokens, a.attn, a.pos = _ptr(tokens), _ptr(attn), _ptr(pos)
-        a.seqlens = sl.ctypes.data if sl is not None else None
-        a.grid_h, a.grid_w, a.keep = gh_a.ctypes.data, gw_a.ctypes.data, keep_a.ctypes.data
         a.out_tokens, a.kept_idx = _ptr(out_tokens), _ptr(kept_idx)
         a.pos_out, a.scores_out = _ptr(pos_out), _ptr(scores_out)
-        a.dtype, a.batch, a.n_tokens, a.dim, a.heads = _dtype_code(tokens), batch, n_tokens, dim, heads
-        a.n_grid, a.n_keep = n_gh, n_keep
         a.out_cu_seqlens = _ptr(out_cu_seqlens)
-        if stream is None:
-            stream = torch.cuda.current_stream(dev).cuda_stream
         if relation is not None:
-            _check(self.h, self.lib.ficoco_v_reduce_relation(self.h, C.byref(a), _ptr(relation), int(by_column),
-                                                             C.byref(p), C.c_void_p(stream)))
+            rc = self.lib.ficoco_v_reduce_relation(self.h, C.byref(a), _ptr(relation), int(by_column), C.byref(p), stream)
         else:
-            _check(self.h, self.lib.ficoco_v_reduce(self.h, C.byref(a), C.byref(p), C.c_void_p(stream)))
-        return VResult(out_tokens, kept_idx, pos_out, scores_out, out_rows)
+            rc = self.lib.ficoco_v_reduce(self.h, C.byref(a), C.byref(p), stream)
+        if rc:
+            _check(self.h, rc)
+        return VResult(out_tokens, kept_idx, pos_out, scores_out, list(sh.out_rows))
 
     def ficoco_v_reduce_schedule(self, tokens, attns, keeps, grid_h: int, grid_w: int, heads: int, *, n_tokens: int,
                                  pos=None, params: Optional[ficoco_params] = None, out_tokens=None, kept_idx=None,
@@ -280,9 +342,9 @@ class Context:
         a.n_grid, a.n_keep = 1, 1
         ptrs = (C.c_void_p * n_steps)(*[t.data_ptr() for t in attns])
         if stream is None:
-            stream = torch.cuda.current_stream(dev).cuda_stream
+            stream = _current_stream(dev)
         _check(self.h, self.lib.ficoco_v_reduce_schedule(self.h, C.byref(a), n_steps, keep_a.ctypes.data, ptrs,
-                                                         C.byref(p), C.c_void_p(stream)))
+                                                         C.byref(p), stream))
         return VResult(out_tokens, kept_idx, pos_out, None, [rows] * batch)
 
     def ficoco_l_reduce(self, tokens, attn_t2v, keep, n_vision: int, n_text: int, heads: int, *,
@@ -291,28 +353,23 @@ class Context:
         """tokens: cuda tensor [B*(N+M), D]; attn_t2v: cuda fp32 [B, H, M, N]."""
         import torch
         p = params or ficoco_default_params()
-        keep_a, n_keep = _int_array(keep)
-        batch = tokens.shape[0] // (n_vision + n_text)
-        keeps = [int(keep_a[0 if n_keep == 1 else b]) for b in range(batch)]
-        conv = bool(p.flags & FICOCO_CONVERGENT)
-        out_rows = [k + n_text + (1 if conv and n_vision - k > 0 else 0) for k in keeps]
-        dim = tokens.shape[-1]
-        dev = tokens.device
+        dim, dev = tokens.shape[-1], tokens.device
+        sh = self._l_shapes(dim, _dtype_code(tokens), tokens.shape[0], keep, n_vision, n_text, heads, p.flags)
+        a = ficoco_l_args.from_buffer_copy(sh.args)
         if out_tokens is None:
-            out_tokens = torch.empty((sum(out_rows), dim), dtype=tokens.dtype, device=dev)
+            out_tokens = torch.empty((sh.n_out, dim), dtype=tokens.dtype, device=dev)
         if kept_idx is None:
-            kept_idx = torch.empty((sum(out_rows),), dtype=torch.int32, device=dev)
+            kept_idx = torch.empty((sh.n_out,), dtype=torch.int32, device=dev)
         if scores_out is None and want_scores:
-            scores_out = torch.empty((batch * n_vision,), dtype=torch.float32, device=dev)
-        a = ficoco_l_args()
-        a.tokens, a.attn_t2v, a.keep = _ptr(tokens), _ptr(attn_t2v), keep_a.ctypes.data
+            scores_out = torch.empty((sh.n_patch,), dtype=torch.float32, device=dev)
+        a.tokens, a.attn_t2v = _ptr(tokens), _ptr(attn_t2v)
         a.out_tokens, a.kept_idx, a.scores_out = _ptr(out_tokens), _ptr(kept_idx), _ptr(scores_out)
-        a.dtype, a.batch, a.n_vision, a.n_text = _dtype_code(tokens), batch, n_vision, n_text
-        a.dim, a.heads, a.n_keep = dim, heads, n_keep
         if stream is None:
-            stream = torch.cuda.current_stream(dev).cuda_stream
-        _check(self.h, self.lib.ficoco_l_reduce(self.h, C.byref(a), C.byref(p), C.c_void_p(stream)))
-        return VResult(out_tokens, kept_idx, None, scores_out, out_rows)
+            stream = _current_stream(dev)
+        rc = self.lib.ficoco_l_reduce(self.h, C.byref(a), C.byref(p), stream)
+        if rc:
+            _check(self.h, rc)
+        return VResult(out_tokens, kept_idx, None, scores_out, list(sh.out_rows))
 
     # -- host-buffer entry points (tensors live in host memory, ideally pinned) ------------
     def ficoco_v_reduce_host(self, tokens, attn, keep, grid_h, grid_w, heads: int, *, n_tokens: int = 0,
@@ -454,10 +511,9 @@ def ficoco_equivalent_token(keys, heads: int, head_dim: int, *, n_tokens: int = 
     if a_eq is None:
         a_eq = torch.empty((patches,), dtype=torch.float32, device=keys.device)
     if stream is None:
-        stream = torch.cuda.current_stream(keys.device).cuda_stream
-    rc = lib.ficoco_equivalent_token(C.c_void_p(keys.data_ptr()), _dtype_code(keys), batch, n_tokens,
-                                     C.c_void_p(sl_ptr), heads, head_dim, cls, C.c_void_p(a_eq.data_ptr()),
-                                     C.c_void_p(stream))
+        stream = _current_stream(keys.device)
+    rc = lib.ficoco_equivalent_token(keys.data_ptr(), _dtype_code(keys), batch, n_tokens, sl_ptr, heads, head_dim, cls,
+                                     a_eq.data_ptr(), stream)
     _check(None, rc)
     return a_eq
 
