@@ -997,6 +997,15 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   else if (wide)
     launch_dependent(k_score_wide<T, 4, 4>, dim3(p->n_rows), 256, (size_t)9 * p->max_rc * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw);
+#define FICOCO_SCORE_GO(V) \
+  launch_dependent(k_score_rows<T, V>, dim3(p->n_rows), 256, (size_t)9 * p->max_rc * sizeof(float), st, \
+      tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw)
+  else if (vpl <= 1) FICOCO_SCORE_GO(1);
+  else if (vpl <= 2) FICOCO_SCORE_GO(2);
+  else if (vpl <= 4) FICOCO_SCORE_GO(4);
+  else if (vpl <= 5) FICOCO_SCORE_GO(5);
+  else if (vpl <= 8) FICOCO_SCORE_GO(8);
+#undef FICOCO_SCORE_GO
   else
     launch_dependent(k_score<T>, dim3(p->n_rows), 256, (size_t)(D + 9 * p->max_rc) * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw);

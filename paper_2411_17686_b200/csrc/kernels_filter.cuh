@@ -166,7 +166,14 @@ __global__ void __launch_bounds__(256) k_msum(int D, const ImgDesc* __restrict__
   const int c = blockIdx.y * 256 + threadIdx.x;
   if (c >= D) return;
   float s = 0.f;
-  for (int k = 0; k < d.n_chunks; ++k) s += partial[(size_t)(d.chunk0 + k) * D + c];
+  const float* q0 = partial + (size_t)d.chunk0 * D + c;
+  for (int k0 = 0; k0 < d.n_chunks; k0 += 8) {     // eight chunks' loads in flight
+    float q[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q[k] = k0 + k < d.n_chunks ? q0[(size_t)(k0 + k) * D] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += q[k];
+  }
   msum[(size_t)blockIdx.x * D + c] = s;
 }
 
@@ -186,6 +193,87 @@ __device__ __forceinline__ void attn_mean_rows(const float* __restrict__ a0, int
       for (int j = 0; j < 8; ++j) s += q[j];
     }
     part[warp * nrows + r] = s;
+  }
+}
+
+// Rows of up to 256 vectors.  Bound by the read of the tokens, so a warp keeps two rows in flight while it works on
+// the two before them: the mean direction sits in registers (a lane owns the same columns of every row), and nothing
+// else is fetched inside the loop.  The chunks are taken last to first: a batch larger than the L2 cache leaves its
+// last images there when the column sums are done.  (One row per warp at a time, the direction in shared memory and
+// the norm read behind every dot product: 256 x 577 rows of 1024, 302 MB, took 124 us.)
+template <class T, int VPL>
+__global__ void __launch_bounds__(256, VPL <= 5 ? 2 : 1) k_score_rows(const T* __restrict__ tokens, int D,
+                                                                      const ImgDesc* __restrict__ desc,
+                                                                      const WorkItem* __restrict__ work,
+                                                                      const float* __restrict__ rn,
+                                                                      const float* __restrict__ msum_all,
+                                                                      const float* __restrict__ attn, int H, float cA,
+                                                                      float* __restrict__ s_raw) {
+  constexpr int E = VecTraits<T>::E;
+  extern __shared__ float vrow[];  // v[nrows], attention partial sums [8][nrows]
+  const WorkItem w = work[gridDim.x - 1 - blockIdx.x];
+  const ImgDesc d = desc[w.img];
+  grid_dep_wait();
+  grid_dep_launch();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nvec = D / E;
+  const T* base = tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D;
+  uint4 next[2][VPL];
+  auto fetch = [&](int r) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) {
+        const int v = lane + 32 * k;
+        next[j][k] = (r + 8 * j < w.nrows && v < nvec) ? ldg16(base + (size_t)(r + 8 * j) * D + (size_t)v * E)
+                                                       : make_uint4(0, 0, 0, 0);
+      }
+  };
+  fetch(warp);
+  float m[VPL][E];
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    const int v = lane + 32 * k;
+#pragma unroll
+    for (int e = 0; e < E; e += 4) {
+      const float4 q = v < nvec ? __ldcg(reinterpret_cast<const float4*>(msum_all + (size_t)w.img * D + (size_t)v * E + e))
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+      m[k][e] = q.x; m[k][e + 1] = q.y; m[k][e + 2] = q.z; m[k][e + 3] = q.w;
+    }
+  }
+  float* part = vrow + w.nrows;
+  attn_mean_rows(attn + d.attn0 + w.r0, H, d.np, w.nrows, part, threadIdx.x);
+  #pragma unroll 1
+  for (int r = warp; r < w.nrows; r += 16) {
+    uint4 u[2][VPL];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) u[j][k] = next[j][k];
+    fetch(r + 16);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      float dot = 0.f;
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) {
+        float f[E];
+        unpack(u[j][k], f, (const T*)nullptr);
+#pragma unroll
+        for (int e = 0; e < E; ++e) dot = fmaf(f[e], m[k][e], dot);
+      }
+      dot = warp_sum(dot);
+      if (lane == 0 && r + 8 * j < w.nrows) vrow[r + 8 * j] = dot;
+    }
+  }
+  const float inv_np = 1.0f / (float)d.np, inv_h = 1.0f / (float)H;
+  const float rn_first = threadIdx.x < w.nrows ? __ldcg(rn + d.patch0 + w.r0 + threadIdx.x) : 0.f;
+  __syncthreads();
+  for (int r = threadIdx.x; r < w.nrows; r += 256) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s += part[q * w.nrows + r];
+    const float k = r == threadIdx.x ? rn_first : __ldcg(rn + d.patch0 + w.r0 + r);
+    s_raw[d.patch0 + w.r0 + r] = cA * (vrow[r] * k * inv_np) - (1.0f - cA) * (s * inv_h);
   }
 }
 
@@ -368,7 +456,7 @@ __global__ void __launch_bounds__(256) k_score_wide(const T* __restrict__ tokens
     const int v = tid + 256 * k;
 #pragma unroll
     for (int e = 0; e < E; e += 4) {
-      const float4 q = v < nvec ? __ldg(reinterpret_cast<const float4*>(msum_all + (size_t)w.img * D + (size_t)v * E + e))
+      const float4 q = v < nvec ? __ldcg(reinterpret_cast<const float4*>(msum_all + (size_t)w.img * D + (size_t)v * E + e))
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
       m[k][e] = q.x; m[k][e + 1] = q.y; m[k][e + 2] = q.z; m[k][e + 3] = q.w;
     }
