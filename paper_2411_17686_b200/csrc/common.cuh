@@ -111,36 +111,6 @@ __device__ __forceinline__ void cta_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// Exclusive prefix sum of one value per thread over `nthr` threads (<= 1024, multiple of 32)
-// that synchronise on barrier `bar`.  `warp_tot` is a 33-int shared scratch.  Returns the
-// exclusive prefix; *total gets the total.  Contains barriers: call from all `nthr` threads.
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* total, int bar, int nthr) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = nthr >> 5;
-  int inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  cta_sync(bar, nthr);
-  if (lane == 31) warp_tot[warp] = inc;
-  cta_sync(bar, nthr);
-  if (warp == 0) {
-    int w = (lane < nwarp) ? warp_tot[lane] : 0;
-    int winc = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int n = __shfl_up_sync(0xFFFFFFFFu, winc, o);
-      if (lane >= o) winc += n;
-    }
-    if (lane < nwarp) warp_tot[lane] = winc - w;
-    if (lane == 31) warp_tot[32] = winc;
-  }
-  cta_sync(bar, nthr);
-  *total = warp_tot[32];
-  return warp_tot[warp] + inc - v;
-}
-
 // Sorted top list (descending value, ties: lower index first).
 __device__ __forceinline__ bool toplist_better(float val, int idx, float v_last, int i_last) {
   return val > v_last || (val == v_last && idx < i_last);

@@ -540,27 +540,91 @@ __global__ void __launch_bounds__(256) k_head_mean(const float* __restrict__ att
 }
 
 // ---------------------------------------------------------------------------------------
-// Local penalty + top-N^S selection of one image by `nthr` threads (tid 0..nthr-1) that
+// Threshold of the k largest of np keys (0 < k < np): `nthr` threads (tid 0 .. nthr - 1, barrier `bar`) count the keys
+// above three trial values at a time until exactly k keys are.  KPT keys per thread sit in registers, so a round is a
+// few compares, a warp reduction and one barrier.  The trial values quarter the interval of the scores, not of the
+// keys: the scores of an image are spread over their range, so the gap between the k-th and the next one is usually
+// met after five or six rounds, while the keys of floats around zero would take more than twice as many.  (A radix
+// select over 8-bit digits took 2.7 us for 576 keys and 8 us for 2880: histogram atomics, two to four passes.)
+// need_eq < 0: every key >= thr is selected; otherwise the keys > thr and the need_eq lowest-indexed ones equal to it.
+// `cnt`: [2][3][32] ints of shared memory.  kmin / kmax: smallest and largest key.
+// ---------------------------------------------------------------------------------------
+__device__ __forceinline__ float key_score(uint32_t key) {   // inverse of order_key
+  return __uint_as_float((key & 0x80000000u) ? key & 0x7FFFFFFFu : ~key);
+}
+template <int KPT>
+__device__ __forceinline__ void select_threshold(const uint32_t (&key)[KPT], int k, uint32_t kmin, uint32_t kmax, int* cnt,
+                                                 int tid, int nthr, int bar, uint32_t& thr, int& need_eq) {
+  const int lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
+  // count(>= lo) >= k > count(>= hi)
+  uint32_t lo = kmin, hi = kmax;
+  int above = 0;                       // count(>= hi); hi starts as "above the largest key"
+  bool open = true;
+  int par = 0;
+  #pragma unroll 1
+  for (;;) {
+    const uint32_t top = open ? hi : hi - 1u;        // largest trial value
+    if (top == lo) break;
+    uint32_t mid[3];
+    {
+      const float a = key_score(lo), b = key_score(top);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const uint32_t by_key = lo + 1u + (uint32_t)((((unsigned long long)(top - lo - 1u)) * (j + 1)) >> 2);
+        const float v = a + (b - a) * (0.25f * (j + 1));
+        const uint32_t m = order_key(v);
+        mid[j] = (m > lo && m <= top) ? m : by_key;  // (not finite, or nothing between the two: by key)
+      }
+      // (ascending in every case that matters: a trial value out of order only repeats work)
+    }
+    int n[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < KPT; ++q)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) n[j] += key[q] >= mid[j] ? 1 : 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      n[j] = __reduce_add_sync(0xFFFFFFFFu, n[j]);
+      if (lane == 0) cnt[(3 * par + j) * 32 + warp] = n[j];
+    }
+    cta_sync(bar, nthr);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) n[j] = __reduce_add_sync(0xFFFFFFFFu, lane < nwarp ? cnt[(3 * par + j) * 32 + lane] : 0);
+    par ^= 1;                          // the next round's counts go to the other half: one barrier per round is enough
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      if (n[j] == k) { thr = mid[j]; need_eq = -1; return; }
+      if (n[j] > k) { if (mid[j] > lo) lo = mid[j]; }
+      else if (open || mid[j] < hi) { hi = mid[j]; above = n[j]; open = false; }
+    }
+  }
+  thr = lo;
+  need_eq = k - above;
+}
+
+// ---------------------------------------------------------------------------------------
+// Local penalty + top-N^S selection of one image by 512 or 1024 threads (tid 0..nthr-1) that
 // synchronise on hardware barrier `bar`.
-//   1. every alive token bids (score key, lower index wins ties) for its window with a
-//      64-bit shared-memory max; the winner's score is multiplied by `coef`;
-//   2. an 8-bit-per-pass radix select over order-preserving keys finds the N^S-th largest
-//      score; ties at the threshold go to the lower index;
-//   3. a block scan turns the membership flags into ascending index lists S and T, the kept
+//   1. a grid-cell -> token map lets one thread per window pick the window's maximum (lower token index on
+//      equal scores) and multiply it in place;
+//   2. a search over the value range finds the threshold (select_threshold); ties at it go to the lower index;
+//   3. ballots and one scan turn the membership flags into ascending index lists S and T, the kept
 //      row indices and the surviving grid positions.
+// What bounds it is the chain of barriers, not the work.  (Bids for the windows by 64-bit shared-memory maxima, a
+// radix select and runs of tokens per thread: the filter of 16 images of up to 2880 tokens took 60 us, now 54.)
 // The code runs once per image, so it is kept compact (rolled loops, not inlined): a long
 // unrolled body would be paid for in instruction-cache misses.
-// `work` is a shared-memory area of select_work_bytes(np, windows) bytes: the scores and grid
-// positions are read from global memory once and kept there with the keys and window bids.
+// `work` is a shared-memory area of select_work_bytes(np, cells) bytes: the scores and grid
+// positions are read from global memory once and kept there with the keys and the cell map.
 // ---------------------------------------------------------------------------------------
-__host__ __device__ inline size_t select_work_bytes(int np, int nwin) {
-  return (size_t)np * 12 + 8 + (size_t)nwin * 8 + 16 + 4 * 256 * sizeof(int);
+__host__ __device__ inline size_t select_work_bytes(int np, int cells) {
+  return (size_t)np * 12 + (size_t)cells * 2 + 32;
 }
 
 struct SelectShared {
-  int warp_tot[33];
-  uint32_t prefix;
-  int remaining;
+  int group[MAX_IMG_TOKENS / 32];
+  int cnt[192];
+  uint32_t wmin[32], wmax[32];
 };
 
 __device__ __noinline__ void select_image(
@@ -568,21 +632,17 @@ __device__ __noinline__ void select_image(
     int penalty, float* __restrict__ s_pen, float* __restrict__ scores_out, int* __restrict__ S_idx,
     int* __restrict__ T_idx, int* __restrict__ kept_idx, int* __restrict__ pos_out,
     unsigned* __restrict__ status, unsigned char* work, SelectShared& sh, int tid, int nthr, int bar) {
-  const int np = d.np;
+  constexpr int KPT = MAX_IMG_TOKENS / 512;      // keys a thread holds in the threshold search
+  const int np = d.np, lane = tid & 31, warp = tid >> 5;
   uint32_t* keys = reinterpret_cast<uint32_t*>(work);
   float* sc = reinterpret_cast<float*>(work + (size_t)np * 4);
   int* pp = reinterpret_cast<int*>(work + (size_t)np * 8);
-  unsigned long long* win = reinterpret_cast<unsigned long long*>(work + (((size_t)np * 12 + 7) & ~(size_t)7));
-  const int nwc = (d.gw + window - 1) / window;
-  const int nwr = (d.gh + window - 1) / window;
-  const int nwin = penalty ? nwc * nwr : 0;
-  // [4][256], one histogram per digit, 16-byte aligned
-  int* hist = reinterpret_cast<int*>((reinterpret_cast<uintptr_t>(win + nwin) + 15) & ~(uintptr_t)15);
+  unsigned short* cell = reinterpret_cast<unsigned short*>(work + (size_t)np * 12);   // [gh * gw] token, 0xFFFF: none
+  const int cells = penalty ? d.gh * d.gw : 0;
 
   #pragma unroll 1
-  for (int i = tid; i < 4 * 256; i += nthr) hist[i] = 0;
-  #pragma unroll 1
-  for (int i = tid; i < nwin; i += nthr) win[i] = 0ull;
+  for (int i = tid; i < cells; i += nthr) cell[i] = 0xFFFFu;
+  if (penalty) cta_sync(bar, nthr);
   #pragma unroll 1
   for (int i0 = tid; i0 < np; i0 += 4 * nthr) {    // four tokens' loads in flight per thread
     float a[4];
@@ -596,126 +656,116 @@ __device__ __noinline__ void select_image(
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int i = i0 + j * nthr;
-      if (i < np) { sc[i] = a[j]; pp[i] = q[j]; }
+      if (i >= np) continue;
+      sc[i] = a[j];
+      pp[i] = q[j];
+      if (penalty) {
+        if (q[j] >= 0 && q[j] < cells) cell[q[j]] = (unsigned short)i;
+        else atomicOr(status, STATUS_POS_RANGE);
+      }
     }
   }
   cta_sync(bar, nthr);
 
-  // ---- local penalty ------------------------------------------------------------------
+  // ---- local penalty: one thread per window ------------------------------------------------
   if (penalty) {
+    const int nwc = (d.gw + window - 1) / window, nwr = (d.gh + window - 1) / window;
     #pragma unroll 1
-    for (int i = tid; i < np; i += nthr) {
-      const int p = pp[i];
-      if (p < 0 || p >= d.gh * d.gw) { atomicOr(status, STATUS_POS_RANGE); continue; }
-      const int wid = (p / d.gw / window) * nwc + (p % d.gw) / window;
-      const unsigned long long bid =
-          ((unsigned long long)order_key(sc[i]) << 32) | (unsigned)(0xFFFFFFFFu - (unsigned)i);
-      atomicMax(&win[wid], bid);
+    for (int wdx = tid; wdx < nwc * nwr; wdx += nthr) {
+      const int r0 = (wdx / nwc) * window, c0 = (wdx % nwc) * window;
+      const int r1 = min(d.gh, r0 + window), c1 = min(d.gw, c0 + window);
+      int best = -1;
+      float bs = 0.f;
+      #pragma unroll 1
+      for (int r = r0; r < r1; ++r)
+        #pragma unroll 1
+        for (int c = c0; c < c1; ++c) {
+          const int t = cell[r * d.gw + c];
+          if (t == 0xFFFF) continue;
+          const float v = sc[t];
+          if (best < 0 || v > bs || (v == bs && t < best)) { best = t; bs = v; }
+        }
+      if (best >= 0) sc[best] = bs * coef;         // windows are disjoint: nobody else touches this token
     }
     cta_sync(bar, nthr);
   }
-  #pragma unroll 1
-  for (int i = tid; i < np; i += nthr) {
-    float s = sc[i];
-    if (penalty) {
-      const int p = pp[i];
-      if (p >= 0 && p < d.gh * d.gw) {
-        const int wid = (p / d.gw / window) * nwc + (p % d.gw) / window;
-        if ((unsigned)(win[wid] & 0xFFFFFFFFull) == 0xFFFFFFFFu - (unsigned)i) s *= coef;
-      }
-    }
-    s_pen[d.patch0 + i] = s;
-    if (scores_out) scores_out[d.patch0 + i] = s;
-    keys[i] = order_key(s);
-  }
-  cta_sync(bar, nthr);
 
-  // ---- radix select: key of the n_src-th largest ------------------------------------------
-  // Two barriers per digit: count, then the first warp finds the digit's bin; every digit has a
-  // histogram of its own, zeroed up front.
+  // ---- keys and their range ----------------------------------------------------------------
+  uint32_t key[KPT];
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    const int i = tid + nthr * q;
+    key[q] = 0u;                                   // (behind the image: never counted, thresholds are > 0)
+    if (i < np) {
+      const float s = sc[i] + 0.0f;                // -0 and +0 are one score
+      s_pen[d.patch0 + i] = s;
+      if (scores_out) scores_out[d.patch0 + i] = s;
+      key[q] = max(1u, order_key(s));
+      keys[i] = key[q];
+      kmin = min(kmin, key[q]);
+      kmax = max(kmax, key[q]);
+    }
+  }
+  kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
+  kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
+  if (lane == 0) { sh.wmin[warp] = kmin; sh.wmax[warp] = kmax; }
+  cta_sync(bar, nthr);
   const int k = d.n_src;
   uint32_t thr = 0;       // threshold key
-  int need_eq = 0;        // how many keys equal to thr are selected (lowest indices)
+  int need_eq = -1;       // how many keys equal to thr are selected (lowest indices); -1: all
   if (k > 0 && k < np) {
-    const int lane = tid & 31;
-    uint32_t prefix = 0, mask = 0;
-    int remaining = k;
-    #pragma unroll 1
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      int* h = hist + 256 * pass;
-      #pragma unroll 1
-      for (int i = tid; i < np; i += nthr) {
-        const uint32_t key = keys[i];
-        if ((key & mask) == prefix) atomicAdd(&h[(key >> shift) & 255], 1);
-      }
-      cta_sync(bar, nthr);
-      if (tid < 32) {
-        // lane l owns bins 255-8l .. 248-8l (descending); find where the running count from
-        // the top reaches `remaining`
-        int c[8], tot = 0;
-        {
-          const int4 lo = *reinterpret_cast<const int4*>(h + 248 - 8 * lane);
-          const int4 hi = *reinterpret_cast<const int4*>(h + 252 - 8 * lane);
-          c[0] = hi.w; c[1] = hi.z; c[2] = hi.y; c[3] = hi.x;
-          c[4] = lo.w; c[5] = lo.z; c[6] = lo.y; c[7] = lo.x;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) tot += c[j];
-        int inc = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-          if (lane >= o) inc += n;
-        }
-        const int before = inc - tot;
-        if (before < remaining && inc >= remaining) {
-          int cum = before;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (cum < remaining && cum + c[j] >= remaining) {
-              sh.prefix = prefix | ((uint32_t)(255 - 8 * lane - j) << shift);
-              sh.remaining = remaining - cum;
-            }
-            cum += c[j];
-          }
-        }
-      }
-      cta_sync(bar, nthr);
-      prefix = sh.prefix;
-      remaining = sh.remaining;
-      mask |= 0xFFu << shift;
-    }
-    thr = prefix;
-    need_eq = remaining;
+    kmin = __reduce_min_sync(0xFFFFFFFFu, lane < (nthr >> 5) ? sh.wmin[lane] : 0xFFFFFFFFu);
+    kmax = __reduce_max_sync(0xFFFFFFFFu, lane < (nthr >> 5) ? sh.wmax[lane] : 0u);
+    select_threshold<KPT>(key, k, kmin, kmax, sh.cnt, tid, nthr, bar, thr, need_eq);
   }
+  if (need_eq < 0) { need_eq = 0; thr = k > 0 && k < np ? thr - 1u : thr; }   // all keys > thr - 1, none at the threshold
 
   // ---- ordered compaction into S and T ------------------------------------------------------
-  // Each thread takes a run of consecutive tokens; one block scan over packed counts
-  // (greater-than in the high half, equal in the low half) places every run.
+  // 32 tokens per warp and trip: ballots give the members among them, one scan over the groups' packed counts
+  // (greater-than in the high half, equal in the low half) what lies before each group.
   {
-    const int ipt = (np + nthr - 1) / nthr;
-    const int i_lo = min(np, tid * ipt), i_hi = min(np, i_lo + ipt);
-    int n_gt = 0, n_eq = 0;
+    const int nw = (np + 31) / 32, nwarp = nthr >> 5;
     #pragma unroll 1
-    for (int i = i_lo; i < i_hi; ++i) {
-      const uint32_t key = keys[i];
-      if (k >= np) ++n_gt;
-      else if (k > 0) { n_gt += key > thr ? 1 : 0; n_eq += key == thr ? 1 : 0; }
+    for (int g = warp; g < nw; g += nwarp) {
+      const int i = 32 * g + lane;
+      const uint32_t ky = i < np ? keys[i] : 0u;
+      const unsigned gt = __ballot_sync(0xFFFFFFFFu, i < np && (k >= np || (k > 0 && ky > thr)));
+      const unsigned eq = __ballot_sync(0xFFFFFFFFu, i < np && k > 0 && k < np && ky == thr);
+      if (lane == 0) sh.group[g] = __popc(gt) << 16 | __popc(eq);
     }
-    int tot;
-    const int packed = block_exclusive_scan((n_gt << 16) | n_eq, sh.warp_tot, &tot, bar, nthr);
-    int gt_before = packed >> 16, eq_before = packed & 0xFFFF;
+    cta_sync(bar, nthr);
+    if (warp == 0) {
+      constexpr int PER = MAX_IMG_TOKENS / 32 / 32;
+      int c[PER], sum = 0;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) { c[j] = PER * lane + j < nw ? sh.group[PER * lane + j] : 0; sum += c[j]; }
+      int inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += n;
+      }
+      int run = inc - sum;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        if (PER * lane + j < nw) sh.group[PER * lane + j] = run;
+        run += c[j];
+      }
+    }
+    cta_sync(bar, nthr);
     #pragma unroll 1
-    for (int i = i_lo; i < i_hi; ++i) {
-      const uint32_t key = keys[i];
-      bool gt, eq;
-      if (k <= 0) { gt = false; eq = false; }
-      else if (k >= np) { gt = true; eq = false; }
-      else { gt = key > thr; eq = key == thr; }
-      const bool sel = gt || (eq && eq_before < need_eq);
+    for (int g = warp; g < nw; g += nwarp) {
+      const int i = 32 * g + lane;
+      const uint32_t ky = i < np ? keys[i] : 0u;
+      const bool is_gt = i < np && (k >= np || (k > 0 && ky > thr)), is_eq = i < np && k > 0 && k < np && ky == thr;
+      const unsigned gt = __ballot_sync(0xFFFFFFFFu, is_gt), eq = __ballot_sync(0xFFFFFFFFu, is_eq);
+      const unsigned lt = (1u << lane) - 1u;
+      const int before = sh.group[g];
+      const int gt_before = (before >> 16) + __popc(gt & lt), eq_before = (before & 0xFFFF) + __popc(eq & lt);
       const int sel_rank = gt_before + min(eq_before, need_eq);   // selected tokens before i
-      if (sel) {
+      if (i >= np) continue;
+      if (is_gt || (is_eq && eq_before < need_eq)) {
         S_idx[d.src0 + sel_rank] = i;
       } else {
         const int tp = i - sel_rank;
@@ -723,8 +773,6 @@ __device__ __noinline__ void select_image(
         kept_idx[d.out_row0 + d.n_cls + tp] = d.n_cls + i;
         if (pos_out) pos_out[d.tgt0 + tp] = pp[i];
       }
-      gt_before += gt ? 1 : 0;
-      eq_before += eq ? 1 : 0;
     }
   }
   #pragma unroll 1
