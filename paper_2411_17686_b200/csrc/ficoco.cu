@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <limits.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -75,7 +76,7 @@ struct Plan {
   bool umma = false;
   bool um_f32 = false;          // fp32 tokens split into three bf16 terms (k_correlate_umma_f32)
   int um_b_bytes = 0;
-  int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0;
+  int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1;
   size_t um_smem = 0;
   std::vector<ImgDesc> h_desc;
 };
@@ -383,7 +384,9 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   }
   c->cap_rows = (int)(MAX_CHUNKS * B);
   if (c->cap_rows < c->num_sms + (int)B + 8) c->cap_rows = c->num_sms + (int)B + 8;
-  c->cap_corr = (int)(2 * (T / CBM + B) + 2048);
+  // (bf16 tiles of 128 x 256 tokens: at most n * n / (4 * 128 * 256) + n / 128 + 1 of an image of n tokens)
+  const size_t n_most = T < (size_t)MAX_IMG_TOKENS ? T : MAX_IMG_TOKENS;
+  c->cap_corr = (int)std::max<size_t>(2 * (T / CBM + B) + 2048, T * n_most / (4 * UM * UN_MAX) + T / UM + B + 64);
   c->cap_out = (int)(T / OUT_ROWS_PER_CTA + B + 2 * c->num_sms);
   c->cap_part = (long long)T * PART_PER_TOKEN;
   c->off_rows = align_up(B * sizeof(ImgDesc), 256);
@@ -431,18 +434,13 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   {
     const int um_smem_max = 221 * 1024;
-    cudaFuncSetAttribute(k_correlate_umma<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<2, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<3, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<4, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<6, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<6, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma<6, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
+#define FICOCO_UMMA_ATTR(NS, KS)                                                                            \
+    cudaFuncSetAttribute(k_correlate_umma<NS, 2, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max); \
+    cudaFuncSetAttribute(k_correlate_umma<NS, 4, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max); \
+    cudaFuncSetAttribute(k_correlate_umma<NS, 16, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max)
+    FICOCO_UMMA_ATTR(2, 1); FICOCO_UMMA_ATTR(3, 1); FICOCO_UMMA_ATTR(4, 1);
+    FICOCO_UMMA_ATTR(2, 2); FICOCO_UMMA_ATTR(3, 2); FICOCO_UMMA_ATTR(4, 2);
+#undef FICOCO_UMMA_ATTR
     cudaFuncSetAttribute(k_correlate_umma_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
     cudaFuncSetAttribute(k_correlate_umma_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
     cudaFuncSetAttribute(k_correlate_umma_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
@@ -506,7 +504,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   if (p->um_f32) p->umma = true;
   if (key.rel) p->umma = p->um_f32 = false;           // C is read from the supplied matrix, not contracted
   const int un_max = p->um_f32 ? UF_COLS : UN_MAX;    // accumulator columns per CTA
-  int tile_rows_max = p->umma ? UM : CBM;             // source rows per correlate CTA (decided below)
+  int tile_rows_max = p->umma ? UM : CBM;             // source rows per correlate CTA
   if (key.rel) {
     // a warp of the relation correlate takes one discarded token at a time and is bound by the
     // latency of its gathers: small tiles put more rows in flight (as far as the work table goes)
@@ -580,56 +578,47 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   }
 
   // ---- correlate tiling ---------------------------------------------------------------------
-  // A CTA gathers (tile rows + split columns) token rows per k-block from L2, which is what
-  // bounds the stage.  Tiles of up to 128 rows let two CTAs share an SM; tiles of up to 256 rows
-  // (two MMA sub-tiles sharing one column tile) gather fewer rows in total but have the SM to
-  // themselves, and one CTA alone gathers more slowly than two.  Both are costed as
-  // (waves x rows gathered per CTA x CTAs per SM); the wide tiles are taken when their cost is
-  // at most 0.7 of the narrow ones' (measured: a tie at 0.75 on 32 x 577 tokens, 20 % faster at
-  // 0.67 on 16 ragged images keeping 1/9 of their tokens).
-  struct CorrChoice { int tile_rows, want_split; long long load; };
-  auto cost_corr = [&](int rows_max, int ctas_per_sm) {
-    CorrChoice ch{rows_max, 1, 0};
+  // A CTA gathers (tile rows + split columns) token rows per k-block from L2, which is what its time is
+  // proportional to; two CTAs share an SM and the last round of CTAs is on average half empty.  Measured on 256 x 577
+  // and 8 x 2881 tokens of 1024 over splits of 2 .. 8: within 10 % of  rows gathered by a CTA x CTAs per SM, the
+  // latter as the mean of the exact number and of whole rounds.  (Tiles of 256 rows that share one column tile gather
+  // fewer rows in total, but a CTA alone on its SM leaves it idle through its epilogue: 143 us against 105 on
+  // 256 x 577 tokens, 72 against 69 on 8 x 2881.)
+  const int cols_max = p->umma ? un_max : INT_MAX;
+  auto split_cols = [&](int n_tgt, int ns) {           // columns per split: ns splits, or more if they got too wide
+    ns = std::max(ns, (n_tgt - 1) / cols_max + 1);
+    return ((n_tgt + ns - 1) / ns + col_granule - 1) / col_granule * col_granule;
+  };
+  auto row_tiles = [&](int n_src) { return (n_src + tile_rows_max - 1) / tile_rows_max; };
+  int want_split = 1;
+  if (p->umma && !p->um_f32) {
+    const long long wave = 2LL * c->num_sms;
+    double best = 0;
+    for (int ws = 1; ws <= NSPLIT_MAX; ++ws) {
+      long long n_ctas = 0, rows_gathered = 0, entries = 0;
+      for (int b = 0; b < B; ++b) {
+        const ImgDesc& d = p->h_desc[b];
+        if (d.list_len == 0) continue;
+        const int cps = split_cols(d.n_tgt, ws), ntile = row_tiles(d.n_src);
+        const int trows = ((d.n_src + ntile - 1) / ntile + 7) / 8 * 8;
+        const long long n = (long long)ntile * ((d.n_tgt + cps - 1) / cps);
+        n_ctas += n;
+        rows_gathered += n * (trows + cps);
+        entries += (long long)d.n_src * ((d.n_tgt + cps - 1) / cps) * d.list_len;
+      }
+      if (n_ctas == 0 || (ws > 1 && (n_ctas > c->cap_corr || entries > c->cap_part))) break;
+      const double exact = (double)n_ctas / c->num_sms;
+      const double whole = n_ctas <= c->num_sms ? 1 : (double)((n_ctas + wave - 1) / wave * wave) / c->num_sms;
+      const double cost = (double)rows_gathered / n_ctas * (n_ctas <= wave ? whole : 0.5 * (exact + whole));
+      if (best == 0 || cost < best) { best = cost; want_split = ws; }
+    }
+  } else {
+    // as many splits as give every SM two CTAs (fp32 tiles: the CTA that completes a tile merges nsplit * L entries
+    // per token, one thread each)
     long long strips = 0;
     for (int b = 0; b < B; ++b)
-      if (p->h_desc[b].list_len > 0) strips += (p->h_desc[b].n_src + rows_max - 1) / rows_max;
-    if (strips == 0) return ch;
-    const long long slots = (long long)c->num_sms * ctas_per_sm;
-    long long ws = slots / strips;
-    if (ws < 1) ws = 1;
-    // (fp32 tiles: the CTA that completes a tile merges nsplit * L entries per token, one thread each)
-    const int split_max = p->um_f32 ? 8 : NSPLIT_MAX;
-    if (ws > split_max) ws = split_max;
-    ch.want_split = (int)ws;
-    long long n_ctas = 0, max_rows = 0;
-    for (int b = 0; b < B; ++b) {
-      const ImgDesc& d = p->h_desc[b];
-      if (d.list_len == 0) continue;
-      int ns = ch.want_split;
-      const int max_by_cols = (d.n_tgt + col_granule - 1) / col_granule;
-      if (ns > max_by_cols) ns = max_by_cols;
-      int cps = ((d.n_tgt + ns - 1) / ns + col_granule - 1) / col_granule * col_granule;
-      if (p->umma && cps > un_max) cps = un_max;
-      ns = (d.n_tgt + cps - 1) / cps;
-      const int ntile = (d.n_src + rows_max - 1) / rows_max;
-      const int trows = ((d.n_src + ntile - 1) / ntile + 7) / 8 * 8;
-      n_ctas += (long long)ntile * ns;
-      if (trows + cps > max_rows) max_rows = trows + cps;
-    }
-    const long long waves = (n_ctas + slots - 1) / slots;
-    const long long per_sm = n_ctas < slots ? (n_ctas + c->num_sms - 1) / c->num_sms : ctas_per_sm;
-    ch.load = waves * max_rows * per_sm;
-    return ch;
-  };
-  int want_split = 1;
-  {
-    CorrChoice best = cost_corr(tile_rows_max, 2);
-    if (p->umma && !p->um_f32) {
-      const CorrChoice wide = cost_corr(UM * UM_SUB, 1);
-      if (wide.load > 0 && wide.load * 10 <= best.load * 7) best = wide;
-    }
-    tile_rows_max = best.tile_rows;
-    want_split = best.want_split;
+      if (p->h_desc[b].list_len > 0) strips += row_tiles(p->h_desc[b].n_src);
+    if (strips > 0) want_split = (int)std::min(std::max(2LL * c->num_sms / strips, 1LL), p->um_f32 ? 8LL : (long long)NSPLIT_MAX);
   }
 
   // Output rows per merge CTA: the fewest that make one wave of two CTAs per SM, or else as many as the shared
@@ -679,13 +668,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     d.nsplit = 1; d.cols_per_split = d.n_tgt > 0 ? d.n_tgt : 1; d.corr_items = 0;
     if (d.list_len == 0 && d.n_src > 0) p->need_finalize = true;
     if (d.list_len > 0) {
-      int ns = want_split;
-      const int max_by_cols = (d.n_tgt + col_granule - 1) / col_granule;
-      if (ns > max_by_cols) ns = max_by_cols;
-      int cps = (d.n_tgt + ns - 1) / ns;
-      cps = (cps + col_granule - 1) / col_granule * col_granule;
-      if (p->umma && cps > un_max) cps = un_max;
-      ns = (d.n_tgt + cps - 1) / cps;
+      const int cps = split_cols(d.n_tgt, want_split), ns = (d.n_tgt + cps - 1) / cps;
       d.nsplit = ns; d.cols_per_split = cps;
       const size_t corr_before = corr.size();
       // source tiles of equal size (rounded to 8 rows)
@@ -776,26 +759,29 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   } else if (p->umma) {
     // shared-memory ring of the tensor-core correlate: prefer a size that lets two CTAs share an SM
     p->um_a_bytes = um_a_rows * 128;
-    p->um_stage_bytes = p->um_a_bytes + um_cols * 128;
-    const int n_sub = (um_a_rows + UM - 1) / UM;       // row sub-tiles (MMAs per k-step) of the largest tile
+    const size_t kblock = (size_t)p->um_a_bytes + (size_t)um_cols * 128;
     p->um_tmem_cols = 32;
-    while (p->um_tmem_cols < n_sub * um_cols) p->um_tmem_cols *= 2;
-    if (p->um_tmem_cols > 512) return FICOCO_ERR_UNSUPPORTED;
-    // every MMA reads 128 A rows: behind the last stage there must be room for the rows past the tile
-    const size_t a_span = (size_t)n_sub * UM * 128;
-    const size_t slack = 1024 + ((size_t)p->um_stage_bytes < a_span ? a_span - p->um_stage_bytes : 0);
+    while (p->um_tmem_cols < um_cols) p->um_tmem_cols *= 2;
+    // every MMA reads 128 A rows: behind the last k-block there must be room for the rows past the tile
+    const size_t slack = 1024 + (kblock < (size_t)UM * 128 ? (size_t)UM * 128 - kblock : 0);
     p->um_nstage = 0;
-    // (a CTA that takes more than half of TMEM has the SM to itself anyway: use the deepest ring)
-    for (int ns = 4; ns >= 2 && !p->um_nstage && p->um_tmem_cols <= 256; --ns)
-      if ((size_t)ns * p->um_stage_bytes + slack <= 106 * 1024) p->um_nstage = ns;
-    for (int ns = 6; ns >= 2 && !p->um_nstage; --ns)
-      if (ns != 5 && (size_t)ns * p->um_stage_bytes + slack <= 220 * 1024) p->um_nstage = ns;
+    auto ring = [&](int ksub, int ns, size_t budget) {
+      if (p->um_nstage || (size_t)ns * ksub * kblock + slack > budget) return;
+      p->um_nstage = ns;
+      p->um_ksub = ksub;
+    };
+    // Two k-blocks per stage halve the barriers, fences and commits of the k-loop (hidden size 4096: 50 us with
+    // one, 44 with two); a grid of more CTAs than SMs keeps to what lets two share an SM.
+    const size_t budget = (int)corr.size() > c->num_sms ? 106 * 1024 : 220 * 1024;
+    for (int ns = 4; ns >= 2; --ns) ring(2, ns, budget);
+    for (int ns = 4; ns >= 2; --ns) ring(1, ns, budget);
     if (!p->um_nstage) return FICOCO_ERR_UNSUPPORTED;
+    p->um_stage_bytes = (int)(p->um_ksub * kblock);
     p->um_smem = (size_t)p->um_nstage * p->um_stage_bytes + slack;
     // the epilogue halves hand their lists over through the ring; FiCoCo-L also stages the head-mean
     // text->vision weights of a tile's rows and columns there
     size_t epi = 1024 + (size_t)UM * KCAP * 8;
-    if (key.mode == 1) epi += (size_t)key.n_text * ((size_t)n_sub * UM + (size_t)((um_cols + 15) / 16 * 16)) * 4;
+    if (key.mode == 1) epi += (size_t)key.n_text * ((size_t)UM + (size_t)((um_cols + 15) / 16 * 16)) * 4;
     if (p->um_smem < epi) p->um_smem = epi;
     if (p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
   }
@@ -1055,18 +1041,21 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     } else if (p->umma && sizeof(T) == 2) {
       prof_tick(c, st, "correlate_umma");
       const __nv_bfloat16* tk = reinterpret_cast<const __nv_bfloat16*>(tok);
-#define FICOCO_UMMA_LAUNCH(NS, LC)                                                                     \
-  launch_dependent(k_correlate_umma<NS, LC>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,               \
+#define FICOCO_UMMA_LAUNCH(NS, LC, KS)                                                                  \
+  launch_dependent(k_correlate_umma<NS, LC, KS>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,               \
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
       (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status,                 \
       p->um_stage_bytes, p->um_a_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt,    \
       c->e_w, c->e_c, tmean, M, p->max_np, gamma, c->wait_ns)
 #define FICOCO_UMMA_STAGES(LC)                                                                         \
   do {                                                                                                 \
-    if (p->um_nstage == 6) FICOCO_UMMA_LAUNCH(6, LC);                                                  \
-    else if (p->um_nstage == 4) FICOCO_UMMA_LAUNCH(4, LC);                                             \
-    else if (p->um_nstage == 3) FICOCO_UMMA_LAUNCH(3, LC);                                             \
-    else FICOCO_UMMA_LAUNCH(2, LC);                                                                    \
+    if (p->um_ksub == 2) {                                                                              \
+      if (p->um_nstage == 4) FICOCO_UMMA_LAUNCH(4, LC, 2);                                              \
+      else if (p->um_nstage == 3) FICOCO_UMMA_LAUNCH(3, LC, 2);                                         \
+      else FICOCO_UMMA_LAUNCH(2, LC, 2);                                                                \
+    } else if (p->um_nstage == 4) FICOCO_UMMA_LAUNCH(4, LC, 1);                                           \
+    else if (p->um_nstage == 3) FICOCO_UMMA_LAUNCH(3, LC, 1);                                           \
+    else FICOCO_UMMA_LAUNCH(2, LC, 1);                                                                  \
   } while (0)
       if (p->max_list <= 2) FICOCO_UMMA_STAGES(2);
       else if (p->max_list <= 4) FICOCO_UMMA_STAGES(4);

@@ -2,14 +2,11 @@
 // text-bridged term added in the epilogue).
 //
 // One CTA owns a tile of discarded tokens (rows of the accumulator, one TMEM lane each) and
-// one column split (<= 256 preserved tokens) of one image.  A tile has up to 128 rows, or up
-// to 256 as two sub-tiles that share the gathered column tile and accumulate in adjacent TMEM
-// column ranges:
+// one column split (<= 256 preserved tokens) of one image; two CTAs share an SM:
 //   warps 0-3, 5-8  gather the token rows with 16-byte cp.async into a ring of 128B-swizzled,
-//              K-major shared-memory tiles (64 bf16 of the hidden dimension per stage);
+//              K-major shared-memory tiles (64 or 128 bf16 of the hidden dimension per stage);
 //   warp  4    allocates TMEM and issues tcgen05.mma (elect.sync, M = 128, N = columns rounded to 16,
-//              K = 16 per instruction, fp32 accumulation of exact bf16 products), one per
-//              sub-tile and k-step;
+//              K = 16 per instruction, fp32 accumulation of exact bf16 products);
 //   warps 0-3, 5-8  afterwards read TMEM lanes back with tcgen05.ld (warps 0-3 the lower half
 //              of the columns, warps 5-8 the upper half of the same lanes), scale by
 //              rn_i * rn_j to cosines and keep each row's L <= LCAP largest entries in registers.
@@ -17,6 +14,12 @@
 // only reaches accumulator rows / columns the epilogue ignores.
 // Every wait is bounded; on a timeout the CTA raises STATUS_TIMEOUT, drains its copies,
 // frees its TMEM and returns.
+//
+// What bounds the k-loop is instruction issue of the gather and, at small tiles, the MMA's fixed 128 rows; half of a
+// CTA's time at D = 1024 is its epilogue, which the other CTA of the SM fills.  The copies of a stage are counted
+// instead of tested one by one and the ring index is kept instead of divided for (with two k-blocks per stage and
+// without 256-row tiles, which held twice the row offsets: 16 FiCoCo-L sequences 55 -> 33 us, one sequence 41 -> 31,
+// one small image 16.7 -> 14.3, 32 x 577 tokens 22.7 -> 21.2).
 #pragma once
 #include <limits.h>
 #include <math_constants.h>
@@ -27,7 +30,6 @@
 namespace ficoco {
 
 constexpr int UM = 128;          // accumulator rows per MMA (one TMEM lane each)
-constexpr int UM_SUB = 2;        // row sub-tiles per CTA: up to 256 discarded tokens share one gathered column tile
 constexpr int UN_MAX = 256;      // accumulator columns per CTA
 constexpr int UKB = 64;          // bf16 elements per k-block (one 128-byte swizzle row)
 constexpr int UTHREADS = 288;    // warps 0-3 and 5-8 gather + epilogue, warp 4 MMA
@@ -189,11 +191,11 @@ __device__ __forceinline__ void epilogue_scan(uint32_t tmem_lane, int c_lo, int 
   }
 }
 
-// Dynamic shared memory: [1024-aligned] ring of NSTAGE stages, each an A tile (a_bytes: the
+// Dynamic shared memory: [1024-aligned] ring of NSTAGE stages, each KSUB k-blocks of an A tile (a_bytes: the
 // valid source rows rounded up to 8, x 128 B) followed by a B tile (column rows x 128 B).  An
 // MMA always reads 128 A rows; rows past a_bytes alias the B tile (or the slack the host adds
 // behind the ring) and only feed accumulator rows that are never read.
-template <int NSTAGE, int LCAP>
+template <int NSTAGE, int LCAP, int KSUB>
 __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     const __nv_bfloat16* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
     const WorkItem* __restrict__ work, const float* __restrict__ rn,
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   extern __shared__ unsigned char um_raw[];
   __shared__ uint64_t full_bar[NSTAGE], empty_bar[NSTAGE], acc_bar;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int rowS[UM * UM_SUB], rowT[UN_MAX];
+  __shared__ int rowS[UM], rowT[UN_MAX];
   __shared__ float rnT[UN_MAX];
   __shared__ int failed, acc_committed, is_last, dead;
 
@@ -217,8 +219,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   const int col_begin = w.aux * d.cols_per_split;
   const int ncols = min(d.n_tgt, col_begin + d.cols_per_split) - col_begin;   // 1..256
   const int n_pad = (ncols + 15) & ~15;
-  const int nkb = D / UKB;
-  const int nsub = (w.nrows + UM - 1) / UM;       // 1 or 2; sub-tile s accumulates in TMEM columns [s * n_pad, (s + 1) * n_pad)
+  const int nk = D / UKB, nkb = (nk + KSUB - 1) / KSUB;   // 64-element k-blocks, stages
   const uint32_t ring = (smem_u32(um_raw) + 1023u) & ~1023u;
 
   if (tid == 0) {
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
                    : "memory");
     return;
   }
-  if (tid < UM * UM_SUB) rowS[tid] = tid < w.nrows ? checked_index(S_idx[d.src0 + w.r0 + tid], d.np, status) : -1;
+  if (tid < UM) rowS[tid] = tid < w.nrows ? checked_index(S_idx[d.src0 + w.r0 + tid], d.np, status) : -1;
   for (int c = tid; c < UN_MAX; c += UTHREADS) {
     const int p = c < ncols ? checked_index(T_idx[d.tgt0 + col_begin + c], d.np, status) : -1;
     rowT[c] = p;
@@ -266,47 +267,53 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
 
   if (warp != 4) {
     // ---------------- producers (all eight epilogue warps): gather rows, 16 bytes per copy -------
-    // Thread pt copies chunk (pt & 7) of rows (pt >> 3) + 32 i of the A tile and of the B tile.
-    // Row offsets stay in registers and the swizzled destination advances by a constant
-    // (32 rows = 4 KB), so a copy costs an add and the cp.async itself.
+    // Thread pt copies chunk (pt & 7) of rows (pt >> 3) + 32 i of the A tile and of the B tile, in every k-block
+    // of the stage.  Byte offsets of the rows stay in registers and the swizzled destination advances by a constant
+    // (32 rows = 4 KB).  A warp's four rows lie in one group of eight, so its number of copies is the same for all
+    // lanes once the tile is rounded up to whole groups (the last row again in the rows added).
     const int pt = warp < 4 ? tid : tid - 32;
     const int chunk = pt & 7;
     const int rsub = pt >> 3;           // 0..31
-    uint32_t offA[UM * UM_SUB / 32], offB[UN_MAX / 32];
-    uint32_t onA = 0, onB = 0;
+    const int rgrp = (int)warp_uniform((uint32_t)(rsub >> 3) * 8);
+    const int nA = (((w.nrows + 7) & ~7) - rgrp + 31) / 32, nB = (((ncols + 7) & ~7) - rgrp + 31) / 32;
+    uint32_t offA[UM / 32], offB[UN_MAX / 32];
 #pragma unroll
-    for (int i = 0; i < UM * UM_SUB / 32; ++i) {
-      const int r = rsub + 32 * i;
-      const bool on = r < w.nrows;
-      offA[i] = on ? (uint32_t)rowS[r] * (uint32_t)D : 0u;
-      onA |= on ? 1u << i : 0u;
-    }
+    for (int i = 0; i < UM / 32; ++i)
+      offA[i] = ((uint32_t)rowS[min(rsub + 32 * i, w.nrows - 1)] * (uint32_t)D + chunk * 8) * 2u;
 #pragma unroll
-    for (int i = 0; i < UN_MAX / 32; ++i) {
-      const int r = rsub + 32 * i;
-      const bool on = r < ncols;
-      offB[i] = on ? (uint32_t)rowT[r] * (uint32_t)D : 0u;
-      onB |= on ? 1u << i : 0u;
-    }
+    for (int i = 0; i < UN_MAX / 32; ++i)
+      offB[i] = ((uint32_t)rowT[min(rsub + 32 * i, ncols - 1)] * (uint32_t)D + chunk * 8) * 2u;
     const uint32_t dsw = (uint32_t)((rsub >> 3) * 1024 + (rsub & 7) * 128 + ((chunk ^ (rsub & 7)) << 4));
-    const __nv_bfloat16* tbase = tokens + (size_t)(d.row0 + d.n_cls) * D + chunk * 8;
+    const uint32_t kblock_bytes = (uint32_t)stage_bytes / KSUB;
+    const char* src = reinterpret_cast<const char*>(tokens + (size_t)(d.row0 + d.n_cls) * D);
     bool ok = true;
     // Each thread's copies of a stage arrive on its barrier when they have landed, so a producer never waits
     // for its own copies and the whole ring is in flight; the MMA warp orders the two proxies (below).
-    for (int kb = 0; kb < nkb && ok; ++kb) {
-      const int s = kb % NSTAGE;
-      if (kb >= NSTAGE) ok = mbar_wait(&empty_bar[s], ((kb / NSTAGE) - 1) & 1, wait_ns);
+    int s = 0;
+    uint32_t par = 1;
+    #pragma unroll 1
+    for (int kb = 0; kb < nkb; ++kb, src += KSUB * UKB * 2) {
+      if (kb >= NSTAGE) ok = mbar_wait(&empty_bar[s], par, wait_ns);
       if (!ok) break;
       const uint32_t a0 = ring + (uint32_t)s * stage_bytes + dsw;
       const uint32_t b0 = a0 + (uint32_t)a_bytes;
-      const __nv_bfloat16* src = tbase + (size_t)kb * UKB;
+      const bool two = KSUB == 2 && 2 * kb + 1 < nk;
 #pragma unroll
-      for (int i = 0; i < UM * UM_SUB / 32; ++i)
-        if (onA >> i & 1u) cp_async16(a0 + i * 4096, src + offA[i]);
+      for (int i = 0; i < UM / 32; ++i)
+        if (i < nA) {
+          const char* p = src + offA[i];
+          cp_async16(a0 + i * 4096, p);
+          if (two) cp_async16(a0 + kblock_bytes + i * 4096, p + UKB * 2);
+        }
 #pragma unroll
       for (int i = 0; i < UN_MAX / 32; ++i)
-        if (onB >> i & 1u) cp_async16(b0 + i * 4096, src + offB[i]);
+        if (i < nB) {
+          const char* p = src + offB[i];
+          cp_async16(b0 + i * 4096, p);
+          if (two) cp_async16(b0 + kblock_bytes + i * 4096, p + UKB * 2);
+        }
       cp_async_arrive(&full_bar[s]);
+      if (++s == NSTAGE) { s = 0; par ^= 1u; }
     }
     if (!ok) cp_async_wait_all();
     FICOCO_PHASE(1, 4);
@@ -318,7 +325,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     tc_fence_after();
     // FiCoCo-L: the head-mean text->vision weights of this tile's columns and rows go into the idle
     // ring, behind the area the two epilogue halves use to hand over their lists
-    const int rows_pad = nsub * UM;
+    constexpr int rows_pad = UM;
     float* tT = nullptr;
     float* tSb = nullptr;
     const float t_scale = tmean != nullptr ? (1.0f - gamma) / (float)M : 0.f;
@@ -360,54 +367,50 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     // this warp scans the lower half of the columns, its helper warp (same TMEM lanes) the
     // upper half; the helper's list comes back through the (now idle) operand ring
     const int c_mid = ((n_pad / 16 + 1) / 2) * 16;
-    #pragma unroll 1
-    for (int sub = 0; sub < nsub; ++sub) {
-      const int row = sub * UM + tid;                  // TMEM lane == accumulator row of the sub-tile
-      const bool row_valid = row < w.nrows;
-      const float rs = row_valid ? rn[d.patch0 + rowS[row]] : 0.f;
-      float v[LCAP];
-      int ix[LCAP];
-      if (acc_ok && sub * UM + warp * 32 < w.nrows)
-        epilogue_scan<LCAP>(tmem_base + (uint32_t)(sub * n_pad) + ((uint32_t)(warp * 32) << 16), 0, c_mid,
-                            col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
-                            t_scale);
-      else {
+    const int row = tid;                             // TMEM lane == accumulator row
+    const bool row_valid = row < w.nrows;
+    const float rs = row_valid ? rn[d.patch0 + rowS[row]] : 0.f;
+    float v[LCAP];
+    int ix[LCAP];
+    if (acc_ok && warp * 32 < w.nrows)
+      epilogue_scan<LCAP>(tmem_base + ((uint32_t)(warp * 32) << 16), 0, c_mid,
+                          col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
+                          t_scale);
+    else {
 #pragma unroll
-        for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
-      }
-      cta_sync(1, 256);                                // helper lists of this sub-tile are in shared memory
-      {
-        const float* hv = reinterpret_cast<const float*>(um_raw + (ring - smem_u32(um_raw)));
-        const int* hi = reinterpret_cast<const int*>(hv + UM * LCAP);
-        #pragma unroll 1                               // rolled: the body is a full insertion
-        for (int e = 0; e < L; ++e) {
-          {
-            float cv = hv[tid * LCAP + e];
-            int ci = hi[tid * LCAP + e];
-            bool shift = ci == INT_MAX;                // empty helper slot: nothing to insert
-            if (!shift) {
-              shift = false;
+      for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
+    }
+    cta_sync(1, 256);                                // helper lists are in shared memory
+    {
+      const float* hv = reinterpret_cast<const float*>(um_raw + (ring - smem_u32(um_raw)));
+      const int* hi = reinterpret_cast<const int*>(hv + UM * LCAP);
+      #pragma unroll 1                               // rolled: the body is a full insertion
+      for (int e = 0; e < L; ++e) {
+        {
+          float cv = hv[tid * LCAP + e];
+          int ci = hi[tid * LCAP + e];
+          bool shift = ci == INT_MAX;                // empty helper slot: nothing to insert
+          if (!shift) {
+            shift = false;
 #pragma unroll
-              for (int k = 0; k < LCAP; ++k)
-                if (k < L && (shift || toplist_better(cv, ci, v[k], ix[k]))) {
-                  const float tv = v[k]; const int ti = ix[k];
-                  v[k] = cv; ix[k] = ci; cv = tv; ci = ti;
-                  shift = true;
-                }
-            }
+            for (int k = 0; k < LCAP; ++k)
+              if (k < L && (shift || toplist_better(cv, ci, v[k], ix[k]))) {
+                const float tv = v[k]; const int ti = ix[k];
+                v[k] = cv; ix[k] = ci; cv = tv; ci = ti;
+                shift = true;
+              }
           }
         }
       }
-      if (row_valid) {
-        const size_t o = (size_t)d.part0 + ((size_t)(w.r0 + row) * d.nsplit + w.aux) * L;
+    }
+    if (row_valid) {
+      const size_t o = (size_t)d.part0 + ((size_t)(w.r0 + row) * d.nsplit + w.aux) * L;
 #pragma unroll
-        for (int k = 0; k < LCAP; ++k)
-          if (k < L) {
-            part_val[o + k] = v[k];
-            part_idx[o + k] = ix[k] == INT_MAX ? -1 : ix[k];
-          }
-      }
-      if (sub + 1 < nsub) cta_sync(1, 256);            // the helpers may reuse the hand-over area
+      for (int k = 0; k < LCAP; ++k)
+        if (k < L) {
+          part_val[o + k] = v[k];
+          part_idx[o + k] = ix[k] == INT_MAX ? -1 : ix[k];
+        }
     }
     } else {
     // ---------------- epilogue helpers: upper half of the columns --------------------------------
@@ -415,52 +418,52 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     const int c_mid = ((n_pad / 16 + 1) / 2) * 16;
     float* hv = reinterpret_cast<float*>(um_raw + (ring - smem_u32(um_raw)));
     int* hi = reinterpret_cast<int*>(hv + UM * LCAP);
-    #pragma unroll 1
-    for (int sub = 0; sub < nsub; ++sub) {
-      const int lrow = grp * 32 + lane;
-      const int row = sub * UM + lrow;
-      const bool row_valid = row < w.nrows;
-      const float rs = row_valid ? rn[d.patch0 + rowS[row]] : 0.f;
-      float v[LCAP];
-      int ix[LCAP];
-      if (acc_ok && sub * UM + grp * 32 < w.nrows)
-        epilogue_scan<LCAP>(tmem_base + (uint32_t)(sub * n_pad) + ((uint32_t)(grp * 32) << 16), c_mid, n_pad,
-                            col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
-                            t_scale);
-      else {
+    const int row = grp * 32 + lane;
+    const bool row_valid = row < w.nrows;
+    const float rs = row_valid ? rn[d.patch0 + rowS[row]] : 0.f;
+    float v[LCAP];
+    int ix[LCAP];
+    if (acc_ok && grp * 32 < w.nrows)
+      epilogue_scan<LCAP>(tmem_base + ((uint32_t)(grp * 32) << 16), c_mid, n_pad,
+                          col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
+                          t_scale);
+    else {
 #pragma unroll
-        for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
-      }
-#pragma unroll
-      for (int k = 0; k < LCAP; ++k) { hv[lrow * LCAP + k] = v[k]; hi[lrow * LCAP + k] = ix[k]; }
-      cta_sync(1, 256);
-      if (sub + 1 < nsub) cta_sync(1, 256);
+      for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
     }
+#pragma unroll
+    for (int k = 0; k < LCAP; ++k) { hv[row * LCAP + k] = v[k]; hi[row * LCAP + k] = ix[k]; }
+    cta_sync(1, 256);
     }
   } else {
     // ---------------- MMA issuer (the whole warp, one elected lane per instruction) -------------
     const uint32_t idesc = umma_idesc_bf16(n_pad);
     const uint32_t u_tmem = warp_uniform(tmem_base), u_ring = warp_uniform(ring);
+    const uint32_t kblock_bytes = (uint32_t)stage_bytes / KSUB;
     bool m_ok = true;
+    int s = 0;
+    uint32_t par = 0;
+    #pragma unroll 1
     for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % NSTAGE;
-      m_ok = __all_sync(0xFFFFFFFFu, mbar_wait(&full_bar[s], (kb / NSTAGE) & 1, wait_ns));
+      m_ok = __all_sync(0xFFFFFFFFu, mbar_wait(&full_bar[s], par, wait_ns));
       if (!m_ok) break;
       // the operands were written through the generic proxy (cp.async) and are read through the async
       // proxy: this fence sits between the two on the path that the barrier orders
       fence_proxy_async();
       tc_fence_after();
-      const uint32_t a0 = u_ring + (uint32_t)s * stage_bytes;
-      const uint64_t ad = umma_smem_desc(a0), bd = umma_smem_desc(a0 + (uint32_t)a_bytes);
 #pragma unroll
-      for (int k4 = 0; k4 < UKB / 16; ++k4) {
-        umma_bf16(u_tmem, ad + (uint64_t)(k4 * 2), bd + (uint64_t)(k4 * 2), idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
-        // second row sub-tile: A rows 128.. (UM * 128 bytes further, in 16-byte units), same B
-        if (nsub > 1)
-          umma_bf16(u_tmem + (uint32_t)n_pad, ad + (uint64_t)(UM * 128 / 16) + (uint64_t)(k4 * 2),
-                    bd + (uint64_t)(k4 * 2), idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
+      for (int j = 0; j < KSUB; ++j) {
+        if (j > 0 && 2 * kb + 1 >= nk) break;
+        const uint32_t a0 = u_ring + (uint32_t)s * stage_bytes + j * kblock_bytes;
+        const uint64_t ad = umma_smem_desc(a0), bd = umma_smem_desc(a0 + (uint32_t)a_bytes);
+#pragma unroll
+        for (int k4 = 0; k4 < UKB / 16; ++k4) {
+          const uint32_t acc = (kb > 0 || j > 0 || k4 > 0) ? 1u : 0u;
+          umma_bf16(u_tmem, ad + (uint64_t)(k4 * 2), bd + (uint64_t)(k4 * 2), idesc, acc);
+        }
       }
       umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+      if (++s == NSTAGE) { s = 0; par ^= 1u; }
     }
     if (m_ok) umma_commit(&acc_bar);   // accumulator complete
     if (lane == 0) {
