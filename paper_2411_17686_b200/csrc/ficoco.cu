@@ -29,6 +29,7 @@ constexpr int N_PLANS = 16;
 constexpr int PART_PER_TOKEN = 64;   // partial top-list entries budgeted per token row
 constexpr int OUT_ROWS_PER_CTA = 16;  // the merge kernel's work table is sized for this many
 constexpr int NSPLIT_MAX = 16;
+constexpr int F_PIECE_ROWS = 128;    // rows that a piece of the fused filter costs besides its own
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -559,22 +560,95 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   const int f_nvec = key.dim / (16 / esz);
   p->f_vpl = (f_nvec + 31) / 32;
   p->fused = c->coop_ok && p->f_vpl <= 8 && !key.rel;
-  int f_rc = 0;
+  // Pieces of equal size per image, at most f_rc rows each, are dealt out to the CTAs in order, so that no CTA gets
+  // more than f_cap rows.  The kernel's time follows the fullest CTA, and every piece adds a fold, a hand-over and,
+  // with an image of its own, a selection (F_PIECE_ROWS rows' worth): of the piece sizes that are multiples of 8 the
+  // one with the least of both is taken.
+  int f_rc = 0, f_cap = 0, f_most = 0;
+  auto piece_rows = [](int np, int rc) {
+    const int n = (np + rc - 1) / rc;
+    return ((np + n - 1) / n + 7) / 8 * 8;
+  };
+  // CTAs that a deal with at most `cap` rows and F_MAXWON pieces per CTA takes; *most: pieces of the fullest CTA
+  auto deal = [&](int rc, int cap, int* most) {
+    int n_cta = 1, acc = 0, items = 0;
+    *most = 0;
+    for (int b = 0; b < B; ++b) {
+      const int np = p->h_desc[b].np, step = np > 0 ? piece_rows(np, rc) : 1;
+      for (int r = 0; r < np; r += step) {
+        const int n = std::min(step, np - r);
+        if (items > 0 && (acc + n > cap || items >= F_MAXWON)) { ++n_cta; acc = items = 0; }
+        acc += n;
+        ++items;
+        if (items > *most) *most = items;
+      }
+    }
+    return n_cta;
+  };
   if (p->fused) {
-    long long total = 0;
-    for (int b = 0; b < B; ++b) total += p->h_desc[b].np;
+    long long total = 0, best = -1;
+    int np_max = 0;
+    for (int b = 0; b < B; ++b) { total += p->h_desc[b].np; np_max = std::max(np_max, p->h_desc[b].np); }
+    const int even = (int)((total + c->num_sms - 1) / c->num_sms);
+    const int rc_lo = std::max(32, even / 4 / 8 * 8), rc_hi = std::max(rc_lo, std::min(2 * even + 8, (np_max + 7) / 8 * 8));
+    const int rc_step = std::max(8, (rc_hi - rc_lo) / 24 / 8 * 8);
+    for (int rc = rc_hi; rc >= rc_lo; rc -= rc_step) {
+      long long n_pieces = 0;
+      int biggest = 0, np_last = 0, step = 1, n = 0;
+      for (int b = 0; b < B; ++b) {
+        const int np = p->h_desc[b].np;
+        if (np <= 0) continue;
+        if (np != np_last) { np_last = np; step = piece_rows(np, rc); n = (np + step - 1) / step; }
+        n_pieces += n;
+        biggest = std::max(biggest, std::min(step, np));
+      }
+      int lo = std::max(even, biggest), hi = 2 * lo, most = 0;
+      if (n_pieces > c->cap_rows) break;
+      if (n_pieces <= c->num_sms) { hi = lo = biggest; }          // one piece each
+      else {
+        // (no deal can do better than this: most sizes are ruled out without one)
+        if (best >= 0 && lo + (n_pieces + c->num_sms - 1) / c->num_sms * F_PIECE_ROWS >= best) continue;
+        if (deal(rc, hi, &most) > c->num_sms) continue;
+        while (lo < hi) {
+          const int mid = (lo + hi) / 2;
+          if (deal(rc, mid, &most) <= c->num_sms) hi = mid; else lo = mid + 1;
+        }
+      }
+      deal(rc, hi, &most);
+      const long long cost = hi + (long long)most * F_PIECE_ROWS;
+      if (best < 0 || cost < best) { best = cost; f_rc = rc; f_cap = hi; f_most = most; }
+    }
+    // Several pieces per CTA and tokens that no cache holds between the passes: three plain kernels read them at the
+    // same rate without the waits between pieces (256 x 577 tokens of 1024, 302 MB: 149 us against 160; 200 x 577,
+    // 236 MB: no difference; 170 x 577: 134 against 141).
+    if (best < 0 || (f_most > 1 && total * key.dim * esz > 256LL * 1024 * 1024)) p->fused = false;
+    // shared memory: ring stages of 16 rows (the selection works in them), the fold area, a score per row of a piece
+    const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)f_rc * 4 + 256;
+    const size_t budget = 216 * 1024;
+    int ns = budget > fixed ? (int)((budget - fixed) / stage) : 0;
+    if (ns > F_MAXSTAGE) ns = F_MAXSTAGE;
+    size_t sel_need = 0;
+    for (int b = 0; b < B; ++b) {
+      const int np = p->h_desc[b].np, cells = key.mode == 0 ? p->h_desc[b].gh * p->h_desc[b].gw : 0;
+      sel_need = std::max(sel_need, np <= SEL_SMALL_MAX ? select_small_bytes(np, cells) : select_work_bytes(np, cells));
+    }
+    if (ns < 2 || sel_need > (size_t)ns * stage) p->fused = false;
+    p->f_max_piece = f_rc;
+    p->f_nstage = ns;
+    p->f_smem = (size_t)ns * stage + fixed;
+  }
+  // Unfused filter, rows of up to 256 vectors: the longest chunks that still make one wave of two CTAs per SM (the
+  // fold at the end of a chunk costs as much as reading 50 rows: 256 x 577 tokens in chunks of 64 rows 103 us, of
+  // 576 rows 67).
+  int u_rc = 0;
+  if (!p->fused && p->f_vpl <= 8 && !key.rel) {
     auto count = [&](int rc) {
       long long n = 0;
       for (int b = 0; b < B; ++b) n += (p->h_desc[b].np + rc - 1) / rc;
       return n;
     };
-    int rc0 = (int)((total + c->num_sms - 1) / c->num_sms);
-    if (rc0 < 32) rc0 = 32;
-    rc0 = (rc0 + 7) / 8 * 8;
-    int rc1 = rc0;
-    while (count(rc1) > c->num_sms && rc1 < 2 * rc0) rc1 += 8;
-    // one piece per CTA if that costs at most 60 % more rows per CTA, else several pieces per CTA
-    f_rc = (count(rc1) <= c->num_sms && rc1 * 10 <= rc0 * 16) ? rc1 : rc0;
+    u_rc = 64;
+    while (u_rc < 1024 && count(u_rc) > std::max(2 * c->num_sms, B)) u_rc += 8;
   }
 
   // ---- correlate tiling ---------------------------------------------------------------------
@@ -653,9 +727,9 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     int rc_floor = (int)(262144 / ((size_t)key.dim * (key.dtype == FICOCO_BF16 ? 2 : 4))) / 8 * 8;
     rc_floor = rc_floor < 8 ? 8 : (rc_floor > 64 ? 64 : rc_floor);
     if (rc < rc_floor) rc = rc_floor;
+    if (u_rc > 0 && d.np > 0) rc = std::max(rc, piece_rows(d.np, u_rc));
     if (p->fused) {
-      const int npc = (d.np + f_rc - 1) / f_rc;
-      rc = ((d.np + npc - 1) / npc + 7) / 8 * 8;
+      if (d.np > 0) rc = piece_rows(d.np, f_rc);
     }
     d.n_chunks = (d.np + rc - 1) / rc;
     d.chunk0 = (int)chunk0;
@@ -705,41 +779,18 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   // ---- fused filter kernel: pieces -> CTAs, shared memory -----------------------------------
   std::vector<int> cta_first;
   if (p->fused) {
-    long long total = 0;
-    for (const WorkItem& w : rows) total += w.nrows;
-    const long long target = (total + c->num_sms - 1) / c->num_sms;
     cta_first.push_back(0);
-    long long acc_rows = 0;
-    int items = 0;
+    int acc = 0, items = 0;                            // (the same deal)
     for (size_t i = 0; i < rows.size(); ++i) {
-      if (items > 0 && (acc_rows + rows[i].nrows > target + 8 || items >= F_MAXWON) &&
-          (int)cta_first.size() < c->num_sms) {
+      if (items > 0 && (acc + rows[i].nrows > f_cap || items >= F_MAXWON)) {
         cta_first.push_back((int)i);
-        acc_rows = 0;
-        items = 0;
+        acc = items = 0;
       }
-      acc_rows += rows[i].nrows;
+      acc += rows[i].nrows;
       ++items;
-      if (items > F_MAXWON) p->fused = false;
     }
     cta_first.push_back((int)rows.size());
     p->f_grid = (int)cta_first.size() - 1;
-    p->f_max_piece = p->max_rc;
-    const size_t stage = (size_t)FROWS * key.dim * esz;
-    const size_t fixed = (size_t)FFOLD * key.dim * 4 + (size_t)p->f_max_piece * 4 + 256;
-    const size_t budget = 216 * 1024;
-    int ns = budget > fixed ? (int)((budget - fixed) / stage) : 0;
-    if (ns > F_MAXSTAGE) ns = F_MAXSTAGE;
-    size_t sel_need = 0;
-    for (int b = 0; b < B; ++b) {
-      const ImgDesc& d = p->h_desc[b];
-      const size_t need = d.np <= SEL_SMALL_MAX ? select_small_bytes(d.np, key.mode == 0 ? d.gh * d.gw : 0)
-                                                : select_work_bytes(d.np, key.mode == 0 ? d.gh * d.gw : 0);
-      if (need > sel_need) sel_need = need;
-    }
-    if (ns < 2 || sel_need > (size_t)ns * stage) p->fused = false;
-    p->f_nstage = ns;
-    p->f_smem = (size_t)ns * stage + fixed;
   }
   if (!p->fused && rows.size() > (size_t)MAX_CHUNKS * B) return FICOCO_ERR_UNSUPPORTED;
   if ((int)rows.size() > c->cap_rows || (int)corr.size() > c->cap_corr || (int)outw.size() > c->cap_out ||

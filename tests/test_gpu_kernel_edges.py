@@ -1,0 +1,68 @@
+"""GPU parity at the sizes where a kernel or a rule of its dispatch changes: edges of tiles, remainders, the smallest
+and the largest of a range, against the float64 checker."""
+import pytest
+
+from oracle import ficoco_oracle as fo, gaps
+from paper_2411_17686_b200 import binding, synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = binding.Context(max_tokens=36000, max_dim=4096, max_batch=180, max_text=64, device=0)
+    yield c
+    c.close()
+
+
+def run_v(ctx, seed, batch, gh, gw, dim, keep, dtype="bf16", cls=True, p=fo.Params()):
+    b = synth.make_v_batch(seed, batch, gh, gw, dim, 2, keep, dtype, cls, 1.0)
+    gaps.repair_v(b, p)
+    parity.run_and_compare_v(ctx, b, p, DEV, what=f"{batch} x {gh} x {gw} x {dim} {dtype} keep {keep}")
+
+
+@pytest.mark.parametrize("batch,gh,gw,dim,keep,dtype", [
+    (1, 9, 9, 64, 1, "bf16"),          # one row with every source: a hub cut by all 16 segments
+    (1, 33, 34, 64, 1, "bf16"),        # more sources than a CTA files: the in-order rescan
+    (2, 8, 8, 4096, 9, "fp32"),        # rows of 16 KB: few rows per CTA
+    (1, 6, 7, 72, 41, "bf16"),         # one source; rows that are no multiple of 32 vectors
+    (24, 20, 20, 64, 300, "bf16"),     # many rows per CTA, dealt out with a stride
+], ids=["hub", "rescan", "wide-rows", "one-source", "many-rows"])
+def test_merge_rows(ctx, batch, gh, gw, dim, keep, dtype):
+    run_v(ctx, 91, batch, gh, gw, dim, keep, dtype)
+
+
+@pytest.mark.parametrize("gh,gw,keep", [(31, 33, 900), (32, 32, 1), (25, 41, 1024), (25, 41, 4), (48, 45, 40)])
+def test_selection_sizes(ctx, gh, gw, keep):
+    """1023 and 1024 tokens: two per thread in registers; from 1025 on the search over the score range."""
+    run_v(ctx, 92, 1, gh, gw, 64, keep, cls=False)
+
+
+@pytest.mark.parametrize("dim,n_src,n_tgt", [
+    (64, 1, 16), (64, 128, 17), (128, 129, 256), (192, 127, 257), (320, 8, 255), (448, 40, 300)])
+def test_correlate_tiles(ctx, dim, n_src, n_tgt):
+    """Odd and even numbers of 64-element blocks (one and two per ring stage), tiles and splits around their edges."""
+    n = n_src + n_tgt
+    gw = next(g for g in (16, 11, 9, 7, 5, 4, 3, 2, 1) if n % g == 0)
+    run_v(ctx, 93, 2, n // gw, gw, dim, n_tgt)
+
+
+@pytest.mark.parametrize("batch,gh,gw,dim", [(149, 7, 7, 64), (170, 10, 10, 256), (3, 44, 44, 512)])
+def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
+    """More images than SMs, and images of several pieces."""
+    run_v(ctx, 94, batch, gh, gw, dim, gh * gw // 2)
+
+
+@pytest.mark.parametrize("batch,gh,gw,dim", [(1, 61, 67, 64), (660, 10, 10, 2048)], ids=["large-image", "large-batch"])
+def test_unfused_filter(batch, gh, gw, dim):
+    """The three plain kernels: a selection whose work area outgrows the fused kernel's ring, and several images per
+    SM with more than 256 MB of tokens."""
+    c = binding.Context(max_tokens=batch * (gh * gw + 1), max_dim=dim, max_batch=batch, max_text=0, device=0)
+    try:
+        c.ficoco_profile(True)
+        run_v(c, 95, batch, gh, gw, dim, gh * gw // 2)
+        assert "score" in [name for name, _, _ in c.ficoco_profile_read()]
+    finally:
+        c.close()
