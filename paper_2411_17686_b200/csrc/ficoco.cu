@@ -564,7 +564,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   // more than f_cap rows.  The kernel's time follows the fullest CTA, and every piece adds a fold, a hand-over and,
   // with an image of its own, a selection (F_PIECE_ROWS rows' worth): of the piece sizes that are multiples of 8 the
   // one with the least of both is taken.
-  int f_rc = 0, f_cap = 0, f_most = 0;
+  int f_rc = 0, f_cap = 0;
   auto piece_rows = [](int np, int rc) {
     const int n = (np + rc - 1) / rc;
     return ((np + n - 1) / n + 7) / 8 * 8;
@@ -616,12 +616,13 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
       }
       deal(rc, hi, &most);
       const long long cost = hi + (long long)most * F_PIECE_ROWS;
-      if (best < 0 || cost < best) { best = cost; f_rc = rc; f_cap = hi; f_most = most; }
+      if (best < 0 || cost < best) { best = cost; f_rc = rc; f_cap = hi; }
     }
-    // Several pieces per CTA and tokens that no cache holds between the passes: three plain kernels read them at the
-    // same rate without the waits between pieces (256 x 577 tokens of 1024, 302 MB: 149 us against 160; 200 x 577,
-    // 236 MB: no difference; 170 x 577: 134 against 141).
-    if (best < 0 || (f_most > 1 && total * key.dim * esz > 256LL * 1024 * 1024)) p->fused = false;
+    // A deal that comes out uneven leaves SMs idle through both passes; from about 64 MB of tokens on three plain
+    // kernels then make up for their launches and the second read (85 x 577 tokens of 1024, cost 1.53 of an even
+    // deal: whole step 147 us fused, 135 not; 150 x 577, 1.98: 261 and 231; 110 x 577, 1.26: 182 and 177;
+    // 60 x 2305, 1.2: the same; 30 x 2305, 1.18: 297 and 307; 50 x 577, 1.29 but 56 MB: the same).
+    if (best < 0 || (best * 100 > (even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024)) p->fused = false;
     // shared memory: ring stages of 16 rows (the selection works in them), the fold area, a score per row of a piece
     const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)f_rc * 4 + 256;
     const size_t budget = 216 * 1024;
@@ -637,9 +638,9 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     p->f_nstage = ns;
     p->f_smem = (size_t)ns * stage + fixed;
   }
-  // Unfused filter, rows of up to 256 vectors: the longest chunks that still make one wave of two CTAs per SM (the
-  // fold at the end of a chunk costs as much as reading 50 rows: 256 x 577 tokens in chunks of 64 rows 103 us, of
-  // 576 rows 67).
+  // Unfused filter, rows of up to 256 vectors: chunks of at least 64 rows that make about three and a half waves of
+  // two CTAs per SM, so that the last wave costs little and the folds at their ends do not either (256 x 577 tokens,
+  // whole step: 64 rows 348 us, 144 rows 341, 576 rows in less than one wave 349).
   int u_rc = 0;
   if (!p->fused && p->f_vpl <= 8 && !key.rel) {
     auto count = [&](int rc) {
@@ -648,7 +649,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
       return n;
     };
     u_rc = 64;
-    while (u_rc < 1024 && count(u_rc) > std::max(2 * c->num_sms, B)) u_rc += 8;
+    while (u_rc < 1024 && count(u_rc) > std::max(7 * c->num_sms, B)) u_rc += 8;
   }
 
   // ---- correlate tiling ---------------------------------------------------------------------
@@ -948,7 +949,7 @@ cudaError_t launch_filter_fused(ficoco_ctx* c, const Plan* p, const T* tok, int 
 template <class T, int VPL>
 void launch_colsum_fused(ficoco_ctx* c, const Plan* p, const T* tok, int D, cudaStream_t st) {
   constexpr int E = VecTraits<T>::E;
-  launch_dependent(k_colsum<T, VPL, true>, dim3(p->n_rows, 1), 256, VPL * 32 * E * sizeof(float), st,
+  launch_dependent(k_colsum<T, VPL, true>, dim3(p->n_rows, 1), 256, 4 * VPL * 32 * E * sizeof(float), st,
       tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
 }
 
@@ -1021,7 +1022,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       tok, D, p->d_desc, p->d_rows, c->rn);
     prof_tick(c, st, "colsum");
     const int slabs = (nvec + 255) / 256;
-    launch_dependent(k_colsum<T, 8, false>, dim3(p->n_rows, slabs), 256, 8 * 32 * E * sizeof(float), st,
+    launch_dependent(k_colsum<T, 8, false>, dim3(p->n_rows, slabs), 256, 4 * 8 * 32 * E * sizeof(float), st,
         tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
     c->launches += 2;
   }

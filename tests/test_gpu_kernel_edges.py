@@ -55,10 +55,10 @@ def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
     run_v(ctx, 94, batch, gh, gw, dim, gh * gw // 2)
 
 
-@pytest.mark.parametrize("batch,gh,gw,dim", [(1, 61, 67, 64), (660, 10, 10, 2048)], ids=["large-image", "large-batch"])
+@pytest.mark.parametrize("batch,gh,gw,dim", [(1, 61, 67, 64), (170, 10, 10, 2048)], ids=["large-image", "large-batch"])
 def test_unfused_filter(batch, gh, gw, dim):
-    """The three plain kernels: a selection whose work area outgrows the fused kernel's ring, and several images per
-    SM with more than 256 MB of tokens."""
+    """The three plain kernels: a selection whose work area outgrows the fused kernel's ring, and more images than
+    SMs with more than 64 MB of tokens."""
     c = binding.Context(max_tokens=batch * (gh * gw + 1), max_dim=dim, max_batch=batch, max_text=0, device=0)
     try:
         c.ficoco_profile(True)
