@@ -13,6 +13,7 @@
 
 #include "../../include/ficoco.h"
 #include "common.cuh"
+#include "filter_plan.h"
 #include "kernels_correlate.cuh"
 #include "kernels_correlate_umma.cuh"
 #include "kernels_correlate_umma_f32.cuh"
@@ -29,7 +30,6 @@ constexpr int N_PLANS = 16;
 constexpr int PART_PER_TOKEN = 64;   // partial top-list entries budgeted per token row
 constexpr int OUT_ROWS_PER_CTA = 16;  // the merge kernel's work table is sized for this many
 constexpr int NSPLIT_MAX = 16;
-constexpr int F_PIECE_ROWS = 128;    // rows that a piece of the fused filter costs besides its own
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -70,7 +70,7 @@ struct Plan {
   bool fused = false;
   int* d_ctafirst = nullptr;
   int* d_out_cu = nullptr;      // device int32[batch + 1]: first output row of every image, then the total
-  int f_grid = 0, f_nstage = 0, f_max_piece = 0, f_vpl = 0;
+  int f_grid = 0, f_nstage = 0, f_vpl = 0;
   size_t f_smem = 0;
   // tensor-core correlate (bf16, hidden size a multiple of 64, FiCoCo-V)
   bool need_finalize = false;   // some image merges nothing: its per-token counts are zeroed by a kernel
@@ -560,71 +560,21 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   const int f_nvec = key.dim / (16 / esz);
   p->f_vpl = (f_nvec + 31) / 32;
   p->fused = c->coop_ok && p->f_vpl <= 8 && !key.rel;
-  // Pieces of equal size per image, at most f_rc rows each, are dealt out to the CTAs in order, so that no CTA gets
-  // more than f_cap rows.  The kernel's time follows the fullest CTA, and every piece adds a fold, a hand-over and,
-  // with an image of its own, a selection (F_PIECE_ROWS rows' worth): of the piece sizes that are multiples of 8 the
-  // one with the least of both is taken.
   int f_rc = 0, f_cap = 0;
-  auto piece_rows = [](int np, int rc) {
-    const int n = (np + rc - 1) / rc;
-    return ((np + n - 1) / n + 7) / 8 * 8;
-  };
-  // CTAs that a deal with at most `cap` rows and F_MAXWON pieces per CTA takes; *most: pieces of the fullest CTA
-  auto deal = [&](int rc, int cap, int* most) {
-    int n_cta = 1, acc = 0, items = 0;
-    *most = 0;
-    for (int b = 0; b < B; ++b) {
-      const int np = p->h_desc[b].np, step = np > 0 ? piece_rows(np, rc) : 1;
-      for (int r = 0; r < np; r += step) {
-        const int n = std::min(step, np - r);
-        if (items > 0 && (acc + n > cap || items >= F_MAXWON)) { ++n_cta; acc = items = 0; }
-        acc += n;
-        ++items;
-        if (items > *most) *most = items;
-      }
-    }
-    return n_cta;
-  };
   if (p->fused) {
-    long long total = 0, best = -1;
-    int np_max = 0;
-    for (int b = 0; b < B; ++b) { total += p->h_desc[b].np; np_max = std::max(np_max, p->h_desc[b].np); }
-    const int even = (int)((total + c->num_sms - 1) / c->num_sms);
-    const int rc_lo = std::max(32, even / 4 / 8 * 8), rc_hi = std::max(rc_lo, std::min(2 * even + 8, (np_max + 7) / 8 * 8));
-    const int rc_step = std::max(8, (rc_hi - rc_lo) / 24 / 8 * 8);
-    for (int rc = rc_hi; rc >= rc_lo; rc -= rc_step) {
-      long long n_pieces = 0;
-      int biggest = 0, np_last = 0, step = 1, n = 0;
-      for (int b = 0; b < B; ++b) {
-        const int np = p->h_desc[b].np;
-        if (np <= 0) continue;
-        if (np != np_last) { np_last = np; step = piece_rows(np, rc); n = (np + step - 1) / step; }
-        n_pieces += n;
-        biggest = std::max(biggest, std::min(step, np));
-      }
-      int lo = std::max(even, biggest), hi = 2 * lo, most = 0;
-      if (n_pieces > c->cap_rows) break;
-      if (n_pieces <= c->num_sms) { hi = lo = biggest; }          // one piece each
-      else {
-        // (no deal can do better than this: most sizes are ruled out without one)
-        if (best >= 0 && lo + (n_pieces + c->num_sms - 1) / c->num_sms * F_PIECE_ROWS >= best) continue;
-        if (deal(rc, hi, &most) > c->num_sms) continue;
-        while (lo < hi) {
-          const int mid = (lo + hi) / 2;
-          if (deal(rc, mid, &most) <= c->num_sms) hi = mid; else lo = mid + 1;
-        }
-      }
-      deal(rc, hi, &most);
-      const long long cost = hi + (long long)most * F_PIECE_ROWS;
-      if (best < 0 || cost < best) { best = cost; f_rc = rc; f_cap = hi; }
-    }
+    std::vector<int> nps(B);
+    long long total = 0;
+    for (int b = 0; b < B; ++b) total += nps[b] = p->h_desc[b].np;
+    const PieceDeal best = best_deal(nps.data(), B, c->num_sms, c->cap_rows, F_MAXWON);
+    f_rc = best.rc;
+    f_cap = best.cap;
     // A deal that comes out uneven leaves SMs idle through both passes; from about 64 MB of tokens on three plain
     // kernels then make up for their launches and the second read (85 x 577 tokens of 1024, cost 1.53 of an even
     // deal: whole step 147 us fused, 135 not; 150 x 577, 1.98: 261 and 231; 110 x 577, 1.26: 182 and 177;
     // 60 x 2305, 1.2: the same; 30 x 2305, 1.18: 297 and 307; 50 x 577, 1.29 but 56 MB: the same).
-    if (best < 0 || (best * 100 > (even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024)) p->fused = false;
+    if (best.cost < 0 || (best.cost * 100 > (best.even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024)) p->fused = false;
     // shared memory: ring stages of 16 rows (the selection works in them), the fold area, a score per row of a piece
-    const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)f_rc * 4 + 256;
+    const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)best.max_piece * 4 + 256;
     const size_t budget = 216 * 1024;
     int ns = budget > fixed ? (int)((budget - fixed) / stage) : 0;
     if (ns > F_MAXSTAGE) ns = F_MAXSTAGE;
@@ -634,7 +584,6 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
       sel_need = std::max(sel_need, np <= SEL_SMALL_MAX ? select_small_bytes(np, cells) : select_work_bytes(np, cells));
     }
     if (ns < 2 || sel_need > (size_t)ns * stage) p->fused = false;
-    p->f_max_piece = f_rc;
     p->f_nstage = ns;
     p->f_smem = (size_t)ns * stage + fixed;
   }
@@ -942,7 +891,7 @@ cudaError_t launch_filter_fused(ficoco_ctx* c, const Plan* p, const T* tok, int 
                             (const WorkItem*)p->d_rows, (const int*)p->d_ctafirst, c->rn, c->partial, attn,
                             attn_rows, cA, c->s_raw, c->img_cnt, p->key.batch, pos, window, coef, penalty,
                             c->s_pen, scores_out, c->S_idx, c->T_idx, kept_idx, pos_out, c->status,
-                            p->f_nstage, p->f_max_piece, c->last_parity, 3 * c->max_batch, c->wait_ns,
+                            p->f_nstage, c->last_parity, 3 * c->max_batch, c->wait_ns,
                             c->dbg_extra_arrivals, (c->coop_pdl_ok && overlap_prev == 2) ? 1 : 0);
 }
 

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
     const int* __restrict__ pos, int window, float coef, int penalty, float* __restrict__ s_pen,
     float* __restrict__ scores_out, int* __restrict__ S_idx, int* __restrict__ T_idx,
     int* __restrict__ kept_idx, int* __restrict__ pos_out, unsigned* __restrict__ status,
-    int nstage, int max_piece, int parity, int set_stride, unsigned long long wait_ns, int dbg_extra_arrivals,
+    int nstage, int parity, int set_stride, unsigned long long wait_ns, int dbg_extra_arrivals,
     int dep_wait_first) {
   constexpr int E = VecTraits<T>::E;
   constexpr int F_P2B = VPL <= 4 ? 2 : 1;   // rows a warp scores together in pass 2 (and has in flight from L2)
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
   const int nvec = D / E;
   unsigned char* ring = fs_raw;
   float* fold = reinterpret_cast<float*>(fs_raw + (size_t)nstage * stage_bytes);   // [FFOLD][D], msum aliases fold[0]
-  float* a_s = fold + (size_t)FFOLD * D;                                            // [max_piece]
+  float* a_s = fold + (size_t)FFOLD * D;                                            // a float per row of the largest piece
   const int p_begin = cta_first[blockIdx.x], p_end = cta_first[blockIdx.x + 1];
   // counters of this launch: [0, B) pieces through pass 1, [B, 2B) pieces scored ([2B, 3B) unused).
   // The other set belongs to the launch before and the one after: it is zeroed here for the latter
