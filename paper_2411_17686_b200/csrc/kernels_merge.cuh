@@ -9,8 +9,42 @@ constexpr int MTHREADS = 512;
 constexpr int MWARPS = MTHREADS / 32;
 constexpr int MROWS = 64;      // most output rows a CTA takes (a lane looks after two in the scan)
 constexpr int MLIST = 1024;    // sources a CTA files in shared memory
-constexpr int MDEPTH = 6;      // source rows a warp has in flight
+constexpr int MDEPTH = 6;      // source rows a warp has in flight; rows with more sources than that go first
+constexpr int MUNITS = 256;    // (row with sources, 512 bytes of it) units of a CTA
 constexpr size_t MSTAGE_BYTES = 70 * 1024;   // input rows of a CTA's output rows kept in shared memory (two CTAs per SM)
+static_assert(MSTAGE_BYTES / 512 + MROWS <= MUNITS, "every unit of a CTA needs an entry");
+
+// 16 bytes of row `own` (shared memory) plus its sources, at byte `off` of their rows; lanes past the row's end idle.
+template <class T>
+__device__ __forceinline__ void merge_unit(const unsigned char* own, const uint2* list, int n, const unsigned char* image,
+                                           unsigned char* dst, int off, int row_bytes) {
+  constexpr int E = VecTraits<T>::E;
+  const bool on = off < row_bytes;
+  if (!on) off = 0;
+  float acc[E], den = 1.0f;
+  unpack(*reinterpret_cast<const uint4*>(own + off), acc, (const T*)nullptr);
+  image += off;
+  #pragma unroll 1
+  for (int e = 0; e < n; e += MDEPTH) {
+    uint4 u[MDEPTH];
+#pragma unroll
+    for (int j = 0; j < MDEPTH; ++j) u[j] = ldg16(image + list[min(e + j, n - 1)].y);   // (past the end: the last row again)
+#pragma unroll
+    for (int j = 0; j < MDEPTH; ++j)
+      if (e + j < n) {
+        const float a = __uint_as_float(list[e + j].x);
+        float x[E];
+        unpack(u[j], x, (const T*)nullptr);
+        den += a;
+#pragma unroll
+        for (int q = 0; q < E; ++q) acc[q] = fmaf(a, x[q], acc[q]);
+      }
+  }
+  const float inv = 1.0f / den;
+#pragma unroll
+  for (int q = 0; q < E; ++q) acc[q] *= inv;
+  if (on) st_stream16(reinterpret_cast<uint4*>(dst + off), pack(acc, (const T*)nullptr));
+}
 
 // Compress + compact.  A CTA owns a few output rows of one image, the ones `stride` apart from its first: targets
 // with many sources lie close together (neighbouring patches look alike), and dealt out like cards they load the
@@ -19,17 +53,23 @@ constexpr size_t MSTAGE_BYTES = 70 * 1024;   // input rows of a CTA's output row
 //   rows    the input rows of its output rows are fetched into shared memory by bulk copies (TMA) as soon as the
 //           index lists exist, i.e. under the tail of the correlate grid;
 //   file    the image's (source -> target) entries that hit its rows are filed into per-row lists in shared
-//           memory, ordered by discarded token, so that every fp32 sum has one fixed order and no atomics touch
-//           floats; one pass over the entries, four loads in flight per thread;
+//           memory, ordered by discarded token; no atomics touch floats; one pass over the entries, four loads in
+//           flight per thread;
 //   copies  a row that nothing is folded into leaves by a bulk store from shared memory: no thread touches it;
-//   merge   out_j = (x_j + sum_{i in I_j} alpha_ij x_i) / (1 + sum alpha_ij), rounded once.  (slices of 32
-//           vectors) x (own rows and sources, in list order) form one sequence of which every warp takes an equal
-//           segment, MDEPTH source rows in flight: rows with one source and hubs with dozens cost what their
-//           elements cost.  A group cut by the end of a segment is left in pieces in shared memory, which are
-//           added in order.
+//   merge   out_j = (x_j + sum_{i in I_j} alpha_ij x_i) / (1 + sum alpha_ij), rounded once.  A unit is one row and
+//           512 bytes of it; a warp adds the row's sources in list order, several of them in flight, and draws its
+//           next unit from a counter.  Rows with many sources go first.
+// Every fp32 sum runs over its row's whole list, in order, in one thread, whatever else the CTA owns: an output row
+// is the same bits alone, in a batch of any size and in a group of a batch.
 // What bounds it is the latency of its few dependent trips to L2; the split into 16 warps and the host's choice of
 // one wave of CTAs where possible keep them few: 32 x 577 -> 289 rows of 1024 went from 25 us (a scan per 16 rows,
-// copies and hub rows by warps, two waves of CTAs) to 20 us, 16 ragged images keeping 1/9 from 48 to 28 us.
+// copies and hub rows by warps, two waves of CTAs) to 20 us, 16 ragged images keeping 1/9 from 48 to 28 us.  (Equal
+// segments of the sequence slices x sources per warp, with a list cut wherever a segment ended, are balanced better
+// where a CTA has one long list, but the order of a sum then follows the rows per CTA and with them the batch: whole
+// step 53.4 us instead of 54.7 for one fp32 image, 102 and 104 for 16 ragged images, but 61.3 and 59.8 for 32 x 577,
+// 139 and 135 for 8 x 2881, 112 and 104 for 16 FiCoCo-L sequences, 53.4 and 44.4 with a relation map, as the pieces
+// took a barrier, 18 KB of shared memory and another pass.  Parts of 256 bytes with twice as many sources in flight
+// for the longer lists: 8 x 2881 tokens 139 us, the others the same.  8 or 10 sources in flight: the same.)
 // If the CTA's rows receive more than MLIST sources in total, a slow in-order rescan is used.
 template <class T>
 __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
@@ -39,15 +79,14 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
     int index_before_wait, unsigned* __restrict__ status, int* __restrict__ filter_cnt, int n_filter_cnt,
     unsigned long long wait_ns) {
   constexpr int E = VecTraits<T>::E;
-  constexpr int PW = E + 1;                      // a piece: E sums and the weight of a lane, lanes side by side
   extern __shared__ __align__(128) unsigned char stage[];     // [rows][row bytes]
-  __shared__ int cnt[MROWS], gbeg[MROWS + 1], beg[MROWS + 1], srow_s[MROWS];
+  __shared__ int cnt[MROWS], beg[MROWS], ubeg[MROWS], srow_s[MROWS];
   __shared__ int m_e[MLIST], bucket[MLIST];
   __shared__ unsigned short m_rs[MLIST];         // row << 10 | slot inside the row's bucket
-  __shared__ uint2 el[MLIST + MROWS];            // weight, row << 16 | source token (the group's own row: anything)
-  __shared__ float fold[MWARPS * PW * 32];
+  __shared__ uint2 el[MLIST];                    // weight, byte offset of the source row in its image
+  __shared__ unsigned short unit[MUNITS];        // row << 8 | part
   __shared__ uint64_t row_bar;
-  __shared__ int n_match, dead;
+  __shared__ int n_match, n_unit, next_unit, dead;
   FICOCO_PHASE_BEGIN(2);
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
@@ -60,7 +99,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
   const T* pbase = tokens + (size_t)(d.row0 + d.n_cls) * D;
 
   if (tid < MROWS) cnt[tid] = 0;
-  if (tid == 0) n_match = 0;
+  if (tid == 0) { n_match = 0; next_unit = MWARPS; }
   // When the grid before this one is a correlate grid, the filter grid (which wrote T_idx) had
   // completed before this grid could start, so the rows may be looked up and fetched under that
   // grid's tail; otherwise wait first.
@@ -134,20 +173,24 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
     mbar_wait(&row_bar, 0, wait_ns);             // no copy outlives the CTA
     return;
   }
+  const int n_parts = (row_bytes + 511) / 512;
   if (warp == 0) {
-    // starts of the buckets, and of the groups (own row + sources) of the rows that have sources
+    // starts of the lists, and of the units of the rows that have sources: those with many first
     const int c0 = cnt[2 * lane], c1 = cnt[2 * lane + 1];
-    const int g0 = c0 > 0 ? c0 + 1 : 0, g1 = c1 > 0 ? c1 + 1 : 0;
-    int inc = (c0 + c1) << 16 | (g0 + g1);       // (both totals stay below 2^15 where they are used)
+    const int u0 = c0 > MDEPTH ? n_parts << 16 : c0 > 0 ? n_parts : 0;
+    const int u1 = c1 > MDEPTH ? n_parts << 16 : c1 > 0 ? n_parts : 0;
+    int ci = c0 + c1, ui = u0 + u1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-      if (lane >= o) inc += n;
+      const int nc = __shfl_up_sync(0xFFFFFFFFu, ci, o), nu = __shfl_up_sync(0xFFFFFFFFu, ui, o);
+      if (lane >= o) { ci += nc; ui += nu; }
     }
-    const int exc = inc - ((c0 + c1) << 16 | (g0 + g1));
-    beg[2 * lane] = exc >> 16; beg[2 * lane + 1] = (exc >> 16) + c0;
-    gbeg[2 * lane] = exc & 0xFFFF; gbeg[2 * lane + 1] = (exc & 0xFFFF) + g0;
-    if (lane == 31) { beg[MROWS] = inc >> 16; gbeg[MROWS] = inc & 0xFFFF; }
+    const int all = __shfl_sync(0xFFFFFFFFu, ui, 31), many = all >> 16;
+    const int ux = ui - u0 - u1, uy = ui - u1;
+    beg[2 * lane] = ci - c0 - c1; beg[2 * lane + 1] = ci - c1;
+    ubeg[2 * lane] = c0 > MDEPTH ? ux >> 16 : many + (ux & 0xFFFF);
+    ubeg[2 * lane + 1] = c1 > MDEPTH ? uy >> 16 : many + (uy & 0xFFFF);
+    if (lane == 0) n_unit = many + (all & 0xFFFF);
   }
   __syncthreads();
   int my_src[MLIST / MTHREADS];
@@ -163,7 +206,8 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
         bucket[beg[rs >> 10] + (rs & 1023)] = e;
       }
     }
-    if (tid < w.nrows && cnt[tid] > 0) el[gbeg[tid]] = make_uint2(__float_as_uint(1.0f), (uint32_t)tid << 16);
+    for (int r = warp; r < w.nrows; r += MWARPS)
+      for (int k = lane; cnt[r] > 0 && k < n_parts; k += 32) unit[ubeg[r] + k] = (unsigned short)(r << 8 | k);
     __syncthreads();
     // the list of a row is ordered by entry, i.e. by discarded token
 #pragma unroll
@@ -173,7 +217,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
         const int e = m_e[i], r = m_rs[i] >> 10, b = beg[r], n = cnt[r];
         int rank = 0;
         for (int k = 0; k < n; ++k) rank += bucket[b + k] < e ? 1 : 0;
-        el[gbeg[r] + 1 + rank] = make_uint2(__float_as_uint(my_w[q]), (uint32_t)r << 16 | (uint32_t)checked_index(my_src[q], d.np, status));
+        el[b + rank] = make_uint2(__float_as_uint(my_w[q]), (uint32_t)checked_index(my_src[q], d.np, status) * (uint32_t)row_bytes);
       }
     }
     __syncthreads();
@@ -196,90 +240,26 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
   FICOCO_PHASE(2, 3);
   // ---- rows with sources ------------------------------------------------------------------------------
   if (fits && total > 0) {
-    const int n_el = gbeg[MROWS], n_all = n_el * ((nvec + 31) / 32);
-    auto seg = [&](int k) { return (int)((long long)n_all * k / MWARPS); };
-    const int p_hi = seg(warp + 1);
-    float* piece = fold + warp * PW * 32 + lane;
-    float acc[E], den = 0.f;
-    int tail = -1;                               // where a group that goes on behind the segment began
     #pragma unroll 1
-    for (int p = seg(warp); p < p_hi;) {
-      const int sl = p / n_el, e0 = p - sl * n_el, r = (int)(el[e0].y >> 16);
-      const int start = gbeg[r], end = start + 1 + cnt[r], e_hi = min(end, e0 + (p_hi - p));
-      const int v = 32 * sl + lane;
-      const bool on = v < nvec;
-      const T* col = pbase + (size_t)(on ? v : 0) * E;
-      int e = e0;
-      if (e0 == start) {
-        unpack(*reinterpret_cast<const uint4*>(stage + (size_t)r * row_bytes + (size_t)(on ? v : 0) * 16), acc, (const T*)nullptr);
-        den = 1.0f;
-        ++e;
-      } else {
-        den = 0.f;
-#pragma unroll
-        for (int q = 0; q < E; ++q) acc[q] = 0.f;
-      }
-      #pragma unroll 1
-      for (; e < e_hi; e += MDEPTH) {
-        uint4 u[MDEPTH];
-#pragma unroll
-        for (int j = 0; j < MDEPTH; ++j)         // (past the end: the last row again, weight 0)
-          u[j] = ldg16(col + (size_t)(el[min(e + j, e_hi - 1)].y & 0xFFFFu) * D);
-#pragma unroll
-        for (int j = 0; j < MDEPTH; ++j) {
-          const float a = e + j < e_hi ? __uint_as_float(el[e + j].x) : 0.f;
-          float x[E];
-          unpack(u[j], x, (const T*)nullptr);
-          den += a;
-#pragma unroll
-          for (int q = 0; q < E; ++q) acc[q] = fmaf(a, x[q], acc[q]);
-        }
-      }
-      if (e0 == start && e_hi < end) {           // stays in registers: it is the last piece of the segment
-        tail = p;
-        break;
-      }
-      if (e0 == start) {
-        const float inv = 1.0f / den;
-#pragma unroll
-        for (int q = 0; q < E; ++q) acc[q] *= inv;
-        if (on) st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D) + v, pack(acc, (const T*)nullptr));
-      } else {
-#pragma unroll
-        for (int q = 0; q < E; ++q) piece[q * 32] = acc[q];
-        piece[E * 32] = den;
-      }
-      p += e_hi - e0;
+    for (int u = warp; u < n_unit;) {
+      const int r = unit[u] >> 8, part = unit[u] & 255;
+      merge_unit<T>(stage + (size_t)r * row_bytes, el + beg[r], cnt[r], reinterpret_cast<const unsigned char*>(pbase),
+                    reinterpret_cast<unsigned char*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D),
+                    (32 * part + lane) * 16, row_bytes);
+      if (lane == 0) u = atomicAdd(&next_unit, 1);
+      u = __shfl_sync(0xFFFFFFFFu, u, 0);
     }
     FICOCO_PHASE(2, 4);
-    __syncthreads();
-    if (tail >= 0) {
-      // add the pieces of the segments that the group reaches
-      const int sl = tail / n_el, r = (int)(el[tail - sl * n_el].y >> 16), end = sl * n_el + gbeg[r] + 1 + cnt[r];
-      const int v = 32 * sl + lane;
-      for (int k = warp + 1; k < MWARPS && seg(k) < end; ++k) {
-        if (seg(k) == seg(k + 1)) continue;
-        const float* x = fold + k * PW * 32 + lane;
-        den += x[E * 32];
-#pragma unroll
-        for (int q = 0; q < E; ++q) acc[q] += x[q * 32];
-      }
-      const float inv = 1.0f / den;
-#pragma unroll
-      for (int q = 0; q < E; ++q) acc[q] *= inv;
-      if (v < nvec)
-        st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D) + v, pack(acc, (const T*)nullptr));
-    }
   } else if (total > 0) {
     // too many sources for shared memory: walk the entries in order (ascending source)
     #pragma unroll 1
     for (int r = warp; r < w.nrows; r += MWARPS) {
       if (cnt[r] == 0) continue;
       const int tp = w.r0 + r * stride - d.n_cls;
-      float wsum = 0.f;
-      for (int e = 0; e < n_ent; ++e)
-        if (e_tgt[d.ent0 + e] == tp) wsum += e_w[d.ent0 + e];
-      const float den = 1.0f + wsum;
+      float den = 1.0f;                          // (sums and quotient as in merge_unit: which path a row takes follows
+      for (int e = 0; e < n_ent; ++e)            // the rows of its CTA)
+        if (e_tgt[d.ent0 + e] == tp) den += e_w[d.ent0 + e];
+      const float inv = 1.0f / den;
       for (int v = lane; v < nvec; v += 32) {
         float acc[E];
         unpack(*reinterpret_cast<const uint4*>(stage + (size_t)r * row_bytes + (size_t)v * 16), acc, (const T*)nullptr);
@@ -293,7 +273,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
           for (int q = 0; q < E; ++q) acc[q] = fmaf(a0, f[q], acc[q]);
         }
 #pragma unroll
-        for (int q = 0; q < E; ++q) acc[q] = acc[q] / den;
+        for (int q = 0; q < E; ++q) acc[q] *= inv;
         st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D) + v, pack(acc, (const T*)nullptr));
       }
     }
