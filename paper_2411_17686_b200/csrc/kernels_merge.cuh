@@ -227,13 +227,13 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
   if (!rows_ok) { atomicOr(status, STATUS_TIMEOUT); return; }
   // ---- rows without sources leave shared memory as they came ------------------------------------------
   if (warp == 0) {
+    const uint64_t policy = l2_evict_first();
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int r = lane + 32 * j;
       if (r < w.nrows && cnt[r] == 0 && srow_s[r] >= 0)
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                     ::"l"(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D), "r"(smem_u32(stage + (size_t)r * row_bytes)), "r"(row_bytes)
-                     : "memory");
+        bulk_store_streaming(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D, stage + (size_t)r * row_bytes,
+                             (uint32_t)row_bytes, policy);
     }
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }
