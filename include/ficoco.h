@@ -281,6 +281,11 @@ int ficoco_status(ficoco_ctx* ctx, void* cuda_stream, int* device_status);
  * spins past the bound, nothing faults); 0 restores normal operation.  Affects later calls. */
 int ficoco_debug_waits(ficoco_ctx* ctx, long long wait_ns, int extra_arrivals);
 
+/* Testing hook: waits on a shared-memory barrier that nothing completes with the context's bound
+ * (ficoco_debug_waits) and gives in *cycles the SM clock cycles until the wait gave up.
+ * Synchronises the device. */
+int ficoco_debug_barrier_wait(ficoco_ctx* ctx, long long* cycles);
+
 /*
  * Inspection of the intermediate results of the most recent reduce call on this context
  * (for tests and debugging).  Synchronises the device, then copies up to `bytes` bytes of

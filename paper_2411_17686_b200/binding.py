@@ -33,7 +33,7 @@ EXPORTS = [
     "ficoco_l_reduce_host", "ficoco_status", "ficoco_inspect", "ficoco_last_launch_count",
     "ficoco_profile", "ficoco_profile_read", "ficoco_vision_redundancy_noalloc",
     "ficoco_equivalent_token", "ficoco_v_reduce_relation", "ficoco_debug_waits", "ficoco_v_reduce_schedule",
-    "ficoco_v_plan",
+    "ficoco_v_plan", "ficoco_debug_barrier_wait",
 ]
 
 
@@ -96,6 +96,7 @@ def load_library() -> C.CDLL:
     lib.ficoco_l_reduce_host.argtypes = [C.c_void_p, C.POINTER(ficoco_l_args), C.POINTER(ficoco_params)]
     lib.ficoco_status.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(C.c_int)]
     lib.ficoco_debug_waits.argtypes = [C.c_void_p, C.c_longlong, C.c_int]
+    lib.ficoco_debug_barrier_wait.argtypes = [C.c_void_p, C.POINTER(C.c_longlong)]
     lib.ficoco_v_plan.argtypes = [C.c_void_p, C.POINTER(ficoco_v_args), C.POINTER(ficoco_params), C.c_void_p]
     lib.ficoco_v_reduce_schedule.argtypes = [C.c_void_p, C.POINTER(ficoco_v_args), C.c_int, C.c_void_p, C.c_void_p,
                                              C.POINTER(ficoco_params), C.c_void_p]
@@ -448,6 +449,11 @@ class Context:
 
     def ficoco_debug_waits(self, wait_ns: int = 0, extra_arrivals: int = 0) -> None:
         _check(self.h, self.lib.ficoco_debug_waits(self.h, wait_ns, extra_arrivals))
+
+    def ficoco_debug_barrier_wait(self) -> int:
+        v = C.c_longlong(0)
+        _check(self.h, self.lib.ficoco_debug_barrier_wait(self.h, C.byref(v)))
+        return v.value
 
     def ficoco_last_launch_count(self) -> int:
         return int(self.lib.ficoco_last_launch_count(self.h))

@@ -1,6 +1,7 @@
 // mbarrier, cp.async and bulk-copy (TMA) primitives shared by the kernels.  Every wait is
-// bounded by elapsed time on the SM's clock: it gives up after `limit_ns` nanoseconds (WAIT_NS_DEFAULT
-// unless the kernel is given another limit) and the caller raises STATUS_TIMEOUT.
+// bounded by elapsed time on the SM's clock: it gives up after `limit_ns` nanoseconds, counted as cycles of a 2 GHz
+// clock (WAIT_NS_DEFAULT unless the kernel is given another limit), and the caller raises STATUS_TIMEOUT, waits, as
+// long again at most, for its own copies in flight and returns.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -59,13 +60,14 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// Bounded wait on a phase parity; false = gave up after limit_ns (counted as cycles of a 2 GHz clock).  A wait
-// that succeeds at once costs one instruction, and only every 32nd failed try looks at the clock.
+// Bounded wait on a phase parity; false = gave up.  A wait that succeeds at once costs one instruction.  A try that
+// fails has suspended the thread for a while, 7800 cycles = 4 us on B200 (a time hint changes nothing), so every one
+// looks at the clock: the wait ends at most two tries, 8 us, after its limit.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
                                           unsigned long long limit_ns = WAIT_NS_DEFAULT) {
   const uint32_t a = smem_u32(bar);
   unsigned long long t0 = 0;
-  for (unsigned n = 1;; ++n) {
+  for (;;) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -73,7 +75,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
         "selp.b32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(a), "r"(parity) : "memory");
     if (ok) return true;
-    if ((n & 31u) != 0) continue;
     const unsigned long long t = sm_cycles();
     if (t0 == 0) t0 = t;
     else if (t - t0 > 2 * limit_ns) return false;

@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(EQ_THREADS, 2) k_equivalent_token(
       const unsigned char* base =
           reinterpret_cast<const unsigned char*>(keys + (size_t)(row0 + n_cls + t_lo) * row_elems);
       bool ok = true;
-      for (int g = 0; g < ngroups && ok; ++g) {
+      int g = 0;
+      for (; g < ngroups; ++g) {
         const int s = g % nstage;
         if (g >= nstage) ok = mbar_wait(&empty_bar[s], ((g / nstage) - 1) & 1);
         if (!ok) break;
@@ -107,6 +108,8 @@ __global__ void __launch_bounds__(EQ_THREADS, 2) k_equivalent_token(
                   &full_bar[s]);
       }
       if (!ok) failed = 1;
+      // no copy outlives the CTA, also where the consumers have given up (nobody re-arms these barriers)
+      for (int q = max(0, g - nstage); q < g; ++q) mbar_wait(&full_bar[q % nstage], (q / nstage) & 1);
     }
   } else {
     // ---------------- consumers: head mean, squared norm, column sums --------------------------

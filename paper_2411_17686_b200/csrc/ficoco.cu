@@ -339,6 +339,21 @@ extern "C" int ficoco_debug_waits(ficoco_ctx* c, long long wait_ns, int extra_ar
   c->dbg_extra_arrivals = extra_arrivals;
   return FICOCO_OK;
 }
+__global__ void k_barrier_wait(unsigned long long wait_ns, unsigned long long* cycles) {
+  __shared__ uint64_t bar;
+  mbar_init(&bar, 1);
+  const unsigned long long t0 = sm_cycles();
+  mbar_wait(&bar, 0, wait_ns);
+  *cycles = sm_cycles() - t0;
+}
+extern "C" int ficoco_debug_barrier_wait(ficoco_ctx* c, long long* cycles) {
+  if (!c || !cycles) return FICOCO_ERR_INVALID_ARG;
+  CUDA_TRY(c, cudaSetDevice(c->device));
+  unsigned long long* d = reinterpret_cast<unsigned long long*>(c->status + 2);   // spare bytes behind the status word
+  k_barrier_wait<<<1, 1>>>(c->wait_ns, d);
+  CUDA_TRY(c, cudaMemcpy(cycles, d, sizeof(*d), cudaMemcpyDeviceToHost));
+  return FICOCO_OK;
+}
 extern "C" int ficoco_last_launch_count(const ficoco_ctx* ctx) { return ctx ? ctx->launches : 0; }
 
 extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens, int max_dim,

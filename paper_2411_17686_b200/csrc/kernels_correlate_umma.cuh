@@ -315,12 +315,11 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
       cp_async_arrive(&full_bar[s]);
       if (++s == NSTAGE) { s = 0; par ^= 1u; }
     }
-    if (!ok) cp_async_wait_all();
     FICOCO_PHASE(1, 4);
     if (!ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
     bool acc_ok = ok && mbar_wait(&acc_bar, 0, wait_ns);
     FICOCO_PHASE(1, 5);
-    if (!acc_ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
+    if (!acc_ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; cp_async_wait_all(); }
     acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);          // tcgen05.ld below is warp-collective
     tc_fence_after();
     // FiCoCo-L: the head-mean text->vision weights of this tile's columns and rows go into the idle

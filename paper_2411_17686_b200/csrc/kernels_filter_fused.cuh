@@ -175,6 +175,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
         }
       }
       if (!ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
+      // no copy outlives the CTA, also where the consumers have given up (nobody re-arms these barriers)
+      for (int q = max(0, seq - nstage); q < seq; ++q) mbar_wait(&full_bar[q % nstage], (q / nstage) & 1, wait_ns);
     }
     return;
   }

@@ -224,7 +224,11 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
   }
   FICOCO_PHASE(2, 2);
   rows_ok = mbar_wait(&row_bar, 0, wait_ns);
-  if (!rows_ok) { atomicOr(status, STATUS_TIMEOUT); return; }
+  if (!rows_ok) {
+    atomicOr(status, STATUS_TIMEOUT);
+    mbar_wait(&row_bar, 0, wait_ns);             // (as above)
+    return;
+  }
   // ---- rows without sources leave shared memory as they came ------------------------------------------
   if (warp == 0) {
     const uint64_t policy = l2_evict_first();

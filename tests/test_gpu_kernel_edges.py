@@ -55,6 +55,18 @@ def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
     run_v(ctx, 94, batch, gh, gw, dim, gh * gw // 2)
 
 
+@pytest.mark.parametrize("wait_ns", [20_000, 200_000, 2_000_000])
+def test_barrier_wait_ends_soon_after_its_limit(ctx, wait_ns):
+    """The limit counts cycles of a 2 GHz clock; a failed try suspends the thread for about 8000 cycles, and the one
+    before the clock is first read and the one that outlasts the limit come on top."""
+    ctx.ficoco_debug_waits(wait_ns, 0)
+    try:
+        cycles = ctx.ficoco_debug_barrier_wait()
+    finally:
+        ctx.ficoco_debug_waits(0, 0)
+    assert 2 * wait_ns < cycles < 2 * wait_ns + 3 * 8000
+
+
 @pytest.mark.parametrize("batch,gh,gw,dim", [(1, 61, 67, 64), (170, 10, 10, 2048)], ids=["large-image", "large-batch"])
 def test_unfused_filter(batch, gh, gw, dim):
     """The three plain kernels: a selection whose work area outgrows the fused kernel's ring, and more images than
