@@ -152,7 +152,8 @@ typedef struct ficoco_v_args {
   const int* grid_w;       /* host int32[n_grid]: columns of the original patch grid */
   const int* pos;          /* device int32 per patch: linear index r * grid_w + c on the
                               original grid (used by the local penalty); NULL means
-                              pos = 0..Np-1 (nothing discarded yet) */
+                              pos = 0..Np-1 (nothing discarded yet).  Tokens may share a
+                              position: the best of a window gets the penalty */
   const int* keep;         /* host int32[n_keep]: N^T, patch tokens preserved per image */
   void* out_tokens;        /* device, dtype, packed [sum_b (c + keep_b), dim] */
   int* kept_idx;           /* device int32, packed like out_tokens rows: for every output

@@ -111,6 +111,18 @@ __device__ __forceinline__ void cta_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+// The same barrier; true for all threads when `pred` is true for any.
+__device__ __forceinline__ bool cta_sync_or(int id, int n, bool pred) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "barrier.cta.red.or.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any) : "r"(id), "r"(n), "r"((uint32_t)pred) : "memory");
+  return any != 0;
+}
+
 // Sorted top list (descending value, ties: lower index first).
 __device__ __forceinline__ bool toplist_better(float val, int idx, float v_last, int i_last) {
   return val > v_last || (val == v_last && idx < i_last);

@@ -610,6 +610,30 @@ __device__ __forceinline__ void select_threshold(const uint32_t (&key)[KPT], int
   need_eq = k - above;
 }
 
+// Positions that occur more than once: the map keeps whichever token was written last, so until nothing changes any
+// more a token that beats the one its cell holds (higher score, lower index on equal scores) takes its place.  Every
+// round leaves each contested cell with a better token, so the rounds end, with the best one, whatever the order of
+// the writes; where all positions differ there is one round, a read per token and a barrier.  pos_of(i, k): position of
+// token i, the thread's k-th.
+template <class Cell, class PosOf>
+__device__ __forceinline__ void settle_cells(Cell* cell, int cells, const float* sc, PosOf pos_of, int np, int tid, int nthr,
+                                             int bar) {
+  volatile Cell* map = cell;
+  bool again;
+  do {
+    again = false;
+    #pragma unroll 1
+    for (int i = tid, k = 0; i < np; i += nthr, ++k) {
+      const int p = pos_of(i, k);
+      if (p < 0 || p >= cells) continue;
+      const int holder = map[p];
+      if (holder == i) continue;
+      const uint32_t mine = order_key(sc[i] + 0.0f), theirs = order_key(sc[holder] + 0.0f);
+      if (mine > theirs || (mine == theirs && i < holder)) { map[p] = (Cell)i; again = true; }
+    }
+  } while (cta_sync_or(bar, nthr, again));
+}
+
 // ---------------------------------------------------------------------------------------
 // Local penalty + top-N^S selection of one image by 512 or 1024 threads (tid 0..nthr-1) that
 // synchronise on hardware barrier `bar`.
@@ -677,6 +701,7 @@ __device__ __noinline__ void select_image(
 
   // ---- local penalty: one thread per window ------------------------------------------------
   if (penalty) {
+    if (pos) settle_cells(cell, cells, sc, [&](int i, int) { return pp[i]; }, np, tid, nthr, bar);
     const int nwc = (d.gw + window - 1) / window, nwr = (d.gh + window - 1) / window;
     #pragma unroll 1
     for (int wdx = tid; wdx < nwc * nwr; wdx += nthr) {
@@ -882,6 +907,7 @@ __device__ __noinline__ void select_small(
 
   // ---- local penalty: one thread per window ------------------------------------------------
   if (penalty) {
+    if (pos) settle_cells(wk.cell, cells, wk.sc, [&](int, int k) { return k == 0 ? pp[0] : pp[1]; }, np, tid, NT, bar);
     const int nwc = (d.gw + window - 1) / window, nwr = (d.gh + window - 1) / window;
     #pragma unroll 1
     for (int wdx = tid; wdx < nwc * nwr; wdx += NT) {

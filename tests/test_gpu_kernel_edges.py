@@ -78,3 +78,26 @@ def test_unfused_filter(batch, gh, gw, dim):
         assert "score" in [name for name, _, _ in c.ficoco_profile_read()]
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("fused", [True, False], ids=["fused", "unfused"])
+@pytest.mark.parametrize("n,gh,gw,same", [(600, 20, 40, False), (1000, 32, 32, True), (1100, 30, 40, False), (2000, 40, 50, True)])
+def test_positions_that_occur_twice(n, gh, gw, same, fused):
+    """The best token of a window gets the penalty wherever several tokens share a cell, in every repetition: positions
+    drawn with replacement, and half of the tokens in one cell."""
+    dim = 64 if fused else 4096
+    b = synth.make_v_batch(97, 2, n // 50, 50, dim, 2, n // 2, "bf16", False, 1.0)
+    for i in range(2):
+        r = synth.rng_for(97, i, 8)
+        b.pos[i] = r.integers(0, gh * gw, n).astype("int32")
+        if same:
+            b.pos[i][r.permutation(n)[:n // 2]] = 7
+        b.grid[i] = (gh, gw)
+    prune = fo.Params(max_targets=0)
+    gaps.repair_v(b, prune)
+    c = binding.Context(max_tokens=2 * n, max_dim=dim, max_batch=2, device=0)
+    try:
+        for _ in range(3):
+            parity.run_and_compare_v(c, b, prune, DEV, what=f"{n} tokens, repeated positions")
+    finally:
+        c.close()
