@@ -28,7 +28,7 @@ namespace {
 
 constexpr int N_PLANS = 16;
 constexpr int PART_PER_TOKEN = 64;   // partial top-list entries budgeted per token row
-constexpr int OUT_ROWS_PER_CTA = 16;  // the merge kernel's work table is sized for this many
+constexpr int OUT_ROWS_PER_CTA = 16;  // the merge kernel's work table is sized for this many (wide rows: fewer)
 constexpr int NSPLIT_MAX = 16;
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -403,7 +403,9 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   // (bf16 tiles of 128 x 256 tokens: at most n * n / (4 * 128 * 256) + n / 128 + 1 of an image of n tokens)
   const size_t n_most = T < (size_t)MAX_IMG_TOKENS ? T : MAX_IMG_TOKENS;
   c->cap_corr = (int)std::max<size_t>(2 * (T / CBM + B) + 2048, T * n_most / (4 * UM * UN_MAX) + T / UM + B + 64);
-  c->cap_out = (int)(T / OUT_ROWS_PER_CTA + B + 2 * c->num_sms);
+  // (wide rows: no more of them per merge CTA than its shared memory takes, fp32 being the widest)
+  const size_t out_rows = std::min<size_t>(OUT_ROWS_PER_CTA, std::max<size_t>(1, MSTAGE_BYTES / ((size_t)max_dim * 4)));
+  c->cap_out = (int)(T / out_rows + B + 2 * c->num_sms);
   c->cap_part = (long long)T * PART_PER_TOKEN;
   c->off_rows = align_up(B * sizeof(ImgDesc), 256);
   c->off_corr = c->off_rows + align_up((size_t)c->cap_rows * sizeof(WorkItem), 256);

@@ -1,6 +1,7 @@
 """GPU parity at the sizes where a kernel or a rule of its dispatch changes: edges of tiles, remainders, the smallest
 and the largest of a range, against the float64 checker."""
 import pytest
+import torch
 
 from oracle import ficoco_oracle as fo, gaps
 from paper_2411_17686_b200 import binding, synth
@@ -32,6 +33,31 @@ def run_v(ctx, seed, batch, gh, gw, dim, keep, dtype="bf16", cls=True, p=fo.Para
 ], ids=["hub", "rescan", "wide-rows", "one-source", "many-rows"])
 def test_merge_rows(ctx, batch, gh, gw, dim, keep, dtype):
     run_v(ctx, 91, batch, gh, gw, dim, keep, dtype)
+
+
+@pytest.mark.parametrize("kind,batch,dim,dtype", [("l", 16, 4096, "bf16"), ("v", 40, 1664, "fp32"), ("v", 24, 4096, "fp32")])
+def test_most_rows_kept_of_wide_rows(kind, batch, dim, dtype):
+    """Many output rows of which a merge CTA's shared memory takes few: the work table has to hold them all."""
+    n, keep, heads, text = 576, 560, 2, 64
+    rows = n + (text if kind == "l" else 0)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((batch * rows, dim), generator=g, device="cuda").to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    c = binding.Context(max_tokens=batch * rows, max_dim=dim, max_batch=batch, max_text=text, device=0)
+    try:
+        if kind == "l":
+            attn = torch.softmax(torch.randn((batch, heads, text, n), generator=g, device="cuda"), dim=3)
+            r = c.ficoco_l_reduce(x, attn, keep, n, text, heads, params=binding.make_params(max_targets=0))
+            kept = keep + text
+        else:
+            attn = torch.softmax(torch.randn((batch, heads, n), generator=g, device="cuda"), dim=2)
+            r = c.ficoco_v_reduce(x, attn, keep, 24, 24, heads, n_tokens=n,
+                                  params=binding.make_params(has_cls=False, max_targets=0))
+            kept = keep
+        first = torch.arange(batch, device="cuda").repeat_interleave(kept) * rows
+        assert torch.equal(r.out_tokens, x[first + r.kept_idx])          # pruning: rows pass through
+        assert c.ficoco_status() == 0
+    finally:
+        c.close()
 
 
 @pytest.mark.parametrize("gh,gw,keep", [(31, 33, 900), (32, 32, 1), (25, 41, 1024), (25, 41, 4), (48, 45, 40)])
