@@ -61,8 +61,7 @@ struct Plan {
   WorkItem* d_corr = nullptr;
   WorkItem* d_out = nullptr;
   int n_rows = 0, n_corr = 0, n_out = 0;
-  int out_rows_cta = 0;         // output rows per merge CTA
-  size_t m_smem = 0;            // and the shared memory for their input rows
+  size_t m_smem = 0;            // shared memory of a merge CTA: the input rows of its output rows
   // totals and maxima used to size launches and inspection copies
   int tot_patch = 0, tot_src = 0, tot_tgt = 0, tot_out_rows = 0;
   int max_np = 0, max_tgt = 0, max_src = 0, max_rc = 0, max_nwin_cells = 0, max_list = 0;
@@ -676,7 +675,6 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     };
     const long long waves = (n_out_ctas(most) + slots - 1) / slots;
     while (out_rows_cta < most && (n_out_ctas(out_rows_cta) > waves * slots || n_out_ctas(out_rows_cta) > c->cap_out)) ++out_rows_cta;
-    p->out_rows_cta = out_rows_cta;
     p->m_smem = out_rows_cta * row_b;
   }
   for (int b = 0; b < B; ++b) {
@@ -706,12 +704,11 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     }
     if (rc > p->max_rc) p->max_rc = rc;
     // correlate
-    d.nsplit = 1; d.cols_per_split = d.n_tgt > 0 ? d.n_tgt : 1; d.corr_items = 0;
+    d.nsplit = 1; d.cols_per_split = d.n_tgt > 0 ? d.n_tgt : 1;
     if (d.list_len == 0 && d.n_src > 0) p->need_finalize = true;
     if (d.list_len > 0) {
       const int cps = split_cols(d.n_tgt, want_split), ns = (d.n_tgt + cps - 1) / cps;
       d.nsplit = ns; d.cols_per_split = cps;
-      const size_t corr_before = corr.size();
       // source tiles of equal size (rounded to 8 rows)
       const int ntile = (d.n_src + tile_rows_max - 1) / tile_rows_max;
       int trows = (d.n_src + ntile - 1) / ntile;
@@ -723,7 +720,6 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
           WorkItem w; w.img = b; w.r0 = s0; w.nrows = (d.n_src - s0 < trows) ? d.n_src - s0 : trows; w.aux = sp;
           corr.push_back(w);
         }
-      d.corr_items = (int)(corr.size() - corr_before);
       part0 += (long long)d.n_src * ns * d.list_len;
       ent0 += (long long)d.n_src * d.list_len;
     }
