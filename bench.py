@@ -515,7 +515,7 @@ def kernel_roofline(name: str, avg_us: float, pk: dict, ab: dict) -> dict:
 
 
 def cpu_baseline(batch, budget_s: float = 12.0) -> dict:
-    """The float64 checker as it stands, on the host cores, over whole batches of the same
+    """The float64 oracle as it stands, on the host cores, over whole batches of the same
     workload until the time budget is used."""
     from oracle import ficoco_oracle as fo
     cores = os.cpu_count() or 1
@@ -539,7 +539,7 @@ def cpu_baseline(batch, budget_s: float = 12.0) -> dict:
 
 
 def run_reference(args, rank: int):
-    """Reference arm: the float64 checker on the host cores, each step one whole batch of the
+    """Reference arm: the float64 oracle on the host cores, each step one whole batch of the
     workload (all 32 images, about a quarter of a second)."""
     if rank != 0:
         return None

@@ -1,4 +1,4 @@
-"""CPU checker for the FiCoCo reduce step (filter -> correlate -> compress -> compact).
+"""CPU oracle for the FiCoCo reduce step (filter -> correlate -> compress -> compact).
 
 TEST INFRASTRUCTURE ONLY.  This is a plain, slow, float64 restatement of what the
 paper defines, used to judge the CUDA library.  It shares no code with the CUDA path,
@@ -86,7 +86,7 @@ def round_to_bf16_bits(x: np.ndarray) -> np.ndarray:
 
     bf16 keeps 8 significand bits (7 stored); a float64 stores 52, so the low 45 stored
     bits are rounded away on the integer representation.  Valid for finite values in the
-    normal range of bf16 (|x| >= 2^-126 or x == 0), which is all this checker produces."""
+    normal range of bf16 (|x| >= 2^-126 or x == 0), which is all this oracle produces."""
     b = np.ascontiguousarray(x, dtype=np.float64).view(np.int64)
     drop = np.int64(45)
     lsb = (b >> drop) & np.int64(1)

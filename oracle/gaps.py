@@ -1,11 +1,11 @@
 """Decision margins of a reduce step, and deterministic input repair.
 
-TEST INFRASTRUCTURE ONLY (uses the float64 checker; never imported by the product).
+TEST INFRASTRUCTURE ONLY (uses the float64 oracle; never imported by the product).
 
 The reduce step takes three kinds of discontinuous decisions: which score wins a
 local-penalty window, where the top-N^S selection boundary falls, and which preserved
 tokens pass the quantile threshold tau_i of a discarded token.  An fp32 GPU path and a
-float64 checker can only agree bit-exactly on those decisions when the competing values
+float64 oracle can only agree bit-exactly on those decisions when the competing values
 are further apart than fp32 rounding noise.  ``margins`` measures the distances;
 ``repair_v`` / ``repair_l`` perturb the *inputs* (never the expected outputs) until
 every distance exceeds its floor, so that both implementations are then given the same,

@@ -585,9 +585,14 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     f_rc = best.rc;
     f_cap = best.cap;
     // A deal that comes out uneven leaves SMs idle through both passes; from about 64 MB of tokens on three plain
-    // kernels then make up for their launches and the second read (85 x 577 tokens of 1024, cost 1.53 of an even
-    // deal: whole step 147 us fused, 135 not; 150 x 577, 1.98: 261 and 231; 110 x 577, 1.26: 182 and 177;
-    // 60 x 2305, 1.2: the same; 30 x 2305, 1.18: 297 and 307; 50 x 577, 1.29 but 56 MB: the same).
+    // kernels then make up for their launches and the second read.  Both paths forced on 192 uniform batches (257,
+    // 577, 1025 and 2305 tokens, 15 to 340 MB; 768, 1024, 1664, 2048 values in bf16, 768, 1024 in fp32), time of the
+    // whole step fused / unfused:
+    //   rows of up to 256 vectors but no more than 1024 values: uneven and large 1.00 to 1.21 (mean 1.065 of 30),
+    //   uneven but below 64 MB 0.97 to 1.27 (four), even 0.94 to 1.08 (mean 1.003 of 94; the fused path is ahead above
+    //   64 MB, the plain kernels below about 25);
+    //   1664 and 2048 values in bf16, where a warp of the fused kernel holds one row at a time: 1.06 to 1.54, so the
+    //   plain kernels are ahead in all 64 and the rule leaves 6 to 31 % there where the deal is even.
     if (best.cost < 0 || (best.cost * 100 > (best.even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024)) p->fused = false;
     // shared memory: ring stages of 16 rows (the selection works in them), the fold area, a score per row of a piece
     const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)best.max_piece * 4 + 256;

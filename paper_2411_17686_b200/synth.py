@@ -2,7 +2,7 @@
 
 This module only draws random numbers and arranges them (fields on a patch grid,
 softmax-normalised attention logits, ragged packing).  It contains none of the
-token-reduction arithmetic, so both the CUDA path and the CPU checker can be fed
+token-reduction arithmetic, so both the CUDA path and the CPU oracle can be fed
 from it without sharing any of the method's code.
 
 Shapes follow the models the paper evaluates (Sec. "Implementation Details",

@@ -3,7 +3,7 @@
 Written with scalar loops, sets and dicts straight from the paper's element-wise
 definitions (Eq. 1, the local-penalty paragraph, the quantile threshold, Eq. 2 and the
 FiCoCo-L score / correlation).  It deliberately avoids every helper of ``oracle/`` and
-every numpy matrix routine so that a mistake in the checker's vectorised code (a dropped
+every numpy matrix routine so that a mistake in the oracle's vectorised code (a dropped
 term, a transposed operand, a wrong index set) shows up as a disagreement.
 """
 import math

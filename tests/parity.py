@@ -1,5 +1,5 @@
 """Shared comparison logic for the GPU parity tests: run one reduce step through the C ABI
-and compare every stage with the float64 checker on the same (margin-repaired) inputs."""
+and compare every stage with the float64 oracle on the same (margin-repaired) inputs."""
 from __future__ import annotations
 
 from typing import List
@@ -60,7 +60,7 @@ def compare_tokens(got: np.ndarray, exp: np.ndarray, wsum: np.ndarray, c: int, t
 
 def compare_stages(ctx: binding.Context, results: List[fo.StepResult], n_cls: int, what: str,
                    check_rn: bool = True):
-    """Intermediate arrays of the last call vs the checker, image by image."""
+    """Intermediate arrays of the last call vs the oracle, image by image."""
     rn = ctx.ficoco_inspect("rnorm")
     s_raw = ctx.ficoco_inspect("score_raw")
     s_pen = ctx.ficoco_inspect("score")
@@ -140,7 +140,7 @@ def run_and_compare_v(ctx: binding.Context, batch, p: fo.Params, device, stages:
 
 def run_and_compare_v_relation(ctx: binding.Context, batch, rels, by_column: bool, p: fo.Params, device,
                                what: str = ""):
-    """ficoco_v_reduce_relation against the checker given the same relation blocks."""
+    """ficoco_v_reduce_relation against the oracle given the same relation blocks."""
     import torch
     pk = packing.pack_v(batch, device)
     prm = params_to_abi(p, batch.has_cls)

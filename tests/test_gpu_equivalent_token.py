@@ -1,4 +1,4 @@
-"""GPU parity of the equivalent token (no-CLS variant) against the float64 checker."""
+"""GPU parity of the equivalent token (no-CLS variant) against the float64 oracle."""
 import numpy as np
 import pytest
 import torch

@@ -1,5 +1,5 @@
 """GPU parity at the sizes where a kernel or a rule of its dispatch changes: edges of tiles, remainders, the smallest
-and the largest of a range, against the float64 checker."""
+and the largest of a range, against the float64 oracle."""
 import pytest
 import torch
 

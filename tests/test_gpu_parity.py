@@ -1,4 +1,4 @@
-"""GPU parity: the CUDA library (through its C ABI) against the float64 checker, element by
+"""GPU parity: the CUDA library (through its C ABI) against the float64 oracle, element by
 element, on seeded inputs whose discrete decisions were made unambiguous beforehand."""
 import collections
 import copy
@@ -43,7 +43,7 @@ def test_small_workload_l(ctx):
 
 @pytest.mark.parametrize("idx", [2, 3])
 def test_small_progressive_schedule(ctx, idx):
-    """Every step of the schedule is checked on the checker's previous output (so both
+    """Every step of the schedule is checked on the oracle's previous output (so both
     sides always see identical inputs), with attention regenerated and pos chained."""
     batch = synth.workload(idx, small=True)
     sched = synth.SCHEDULES_SMALL[idx]
@@ -146,7 +146,7 @@ def _relations(batch, seed, stochastic=True, times_n=False):
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 def test_relation_mode(ctx, by_column, dtype):
     """Caller-supplied relation map in place of the cosine similarity: scores, S / T, target
-    sets, weights and merged rows against the checker given the same map."""
+    sets, weights and merged rows against the oracle given the same map."""
     batch = synth.make_v_batch(90, 3, 13, 11, 192, 5, 60, dtype, True, 1.2)
     rels = _relations(batch, 90, stochastic=by_column)
     for p in (fo.Params(), fo.Params(eps=0.97, local_penalty=False)):
@@ -297,7 +297,7 @@ def test_pairwise_correlation_gap_from_inspection(ctx):
     """The paper's diagnostic for choosing K (Sec. "Correlation-based Information Recycling"):
     top-1 minus top-2 correlation of every discarded token.  With the adaptive threshold the
     library keeps each row's two (or more) largest correlations, so the gap can be read from
-    the inspection arrays; it must match the checker's full correlation rows."""
+    the inspection arrays; it must match the oracle's full correlation rows."""
     batch = synth.workload(2, small=True)
     gaps.repair_v(batch)
     p = fo.Params()
@@ -335,7 +335,7 @@ def test_canaries_around_outputs(ctx):
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 def test_convergent_correlation_variant(ctx, dtype):
     """Ablation 'convergent correlation': preserved rows bit for bit, one additional row per image
-    (the mean of the discarded rows) with kept index -1, against the checker; uniform and ragged
+    (the mean of the discarded rows) with kept index -1, against the oracle; uniform and ragged
     batches, nothing appended where nothing is discarded, and the FiCoCo-L layout."""
     p = fo.Params(convergent=True)
     batch = synth.make_v_batch(98, 3, 13, 11, 192, 5, 80, dtype, True, 1.2)
@@ -360,7 +360,7 @@ def test_convergent_correlation_variant(ctx, dtype):
 def test_hand_built_ties_follow_the_lower_index(ctx):
     """The two hand-built tie inputs of tests/golden (bit-identical scores across the selection
     boundary, and inside one local-penalty window), with no margin repair: the library takes the
-    same decisions as the checker, which the golden file pins by hand."""
+    same decisions as the oracle, which the golden file pins by hand."""
     g = json.load(open(os.path.join(os.path.dirname(__file__), "golden", "hand_example.json")))["tie_cases"]
     P = np.array(g["patches"], dtype=np.float32)
     attn = np.array(g["cls_attention"], dtype=np.float32)
@@ -389,7 +389,7 @@ def test_hand_built_ties_follow_the_lower_index(ctx):
         res, results = parity.run_and_compare_v(ctx, batch, fo.Params(local_penalty=penalty, max_targets=0), DEV,
                                                 what="ties-wide")
         # groups straddling the boundary exist (160 - keep is not a multiple of four), and the
-        # checker's scores really tie bit for bit inside a group
+        # oracle's scores really tie bit for bit inside a group
         sraw = results[0].score_raw.reshape(40, 4)
         assert np.all(sraw == sraw[:, :1]) and (160 - keep) % 4 != 0
 
@@ -644,7 +644,7 @@ def test_full_c2_shape_relation_mode(ctx, by_column):
 
 
 def test_full_c3_schedule(ctx):
-    """2880 -> 1440 -> 720 -> 320 at full size (8 images x 2881 tokens), every step on the checker's
+    """2880 -> 1440 -> 720 -> 320 at full size (8 images x 2881 tokens), every step on the oracle's
     previous output; the later steps reach top lists of three and two entries."""
     batch = synth.workload(3)
     p = fo.Params()
@@ -659,8 +659,8 @@ def test_full_c3_schedule(ctx):
     _report_plain_score_error("c3 schedule")
 
 
-def _checker_chain(batch, sched, seed, sigma):
-    """The checker's chained run of a schedule: per step the (margin-repaired) attention it used,
+def _oracle_chain(batch, sched, seed, sigma):
+    """The oracle's chained run of a schedule: per step the (margin-repaired) attention it used,
     and at the end the tokens, the composed kept indices and the positions."""
     p = fo.Params()
     attns, chain = [], None
@@ -680,10 +680,10 @@ def _checker_chain(batch, sched, seed, sigma):
 @pytest.mark.parametrize("idx,small", [(2, True), (3, True), (2, False)], ids=["c2-small", "c3-small", "c2-full"])
 def test_schedule_entry_point_chains_its_own_outputs(ctx, idx, small):
     """ficoco_v_reduce_schedule runs all steps on the GPU's own intermediate outputs; the result is
-    compared with the checker's chained run of the same schedule: the composed kept indices and
+    compared with the oracle's chained run of the same schedule: the composed kept indices and
     the final positions exactly, the final tokens within the bf16 tolerance once per step (a
     merged row may be rounded differently by one ulp in one step and feed the next).  The margins
-    that make a step's decisions unambiguous were established on the checker's intermediates; on
+    that make a step's decisions unambiguous were established on the oracle's intermediates; on
     intermediates that differ by an ulp here and there a discarded token whose two best targets are
     nearly tied can go to the other one, which moves two output rows: at most 1 % of the rows may
     be off for that reason (what is kept, and where, must still agree exactly)."""
@@ -691,7 +691,7 @@ def test_schedule_entry_point_chains_its_own_outputs(ctx, idx, small):
     sched = (synth.SCHEDULES_SMALL if small else synth.SCHEDULES)[idx]
     pk = packing.pack_v(batch, DEV)
     gh, gw = batch.grid[0]
-    attns, results, chain = _checker_chain(batch, sched, 1000 * idx, 1.5 if idx == 2 else 1.0)
+    attns, results, chain = _oracle_chain(batch, sched, 1000 * idx, 1.5 if idx == 2 else 1.0)
     attn_d = [torch.from_numpy(a.reshape(-1)).to(DEV) for a in attns]
     pk.attn = attn_d[0]
     prm = parity.params_to_abi(fo.Params(), True)

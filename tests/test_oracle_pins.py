@@ -1,5 +1,5 @@
-"""Pins for the float64 checker: everything here is fixed by the paper's equations or by
-mathematics, not by the checker itself (hand-worked values, an independent scalar-loop
+"""Pins for the float64 oracle: everything here is fixed by the paper's equations or by
+mathematics, not by the oracle itself (hand-worked values, an independent scalar-loop
 transcription, closed forms, invariants, library routines for special cases)."""
 import json
 import os
@@ -192,7 +192,7 @@ def test_fixed_k_ties_go_to_the_lower_column():
 
 
 def test_planted_mistakes_in_fixed_k_and_tie_rules_are_caught(monkeypatch):
-    """The fixed-K branch and the two tie rules, each flipped in the checker, must break a pin."""
+    """The fixed-K branch and the two tie rules, each flipped in the oracle, must break a pin."""
     real_tw, real_topk, real_pen = fo.targets_and_weights, fo.filter_topk, fo.local_penalty
 
     def fails(check):
@@ -262,7 +262,7 @@ def test_planted_mistakes_in_fixed_k_and_tie_rules_are_caught(monkeypatch):
 
 
 def test_planted_mistakes_are_caught(monkeypatch):
-    """Each plausible slip in the checker must break agreement with the scalar transcription."""
+    """Each plausible slip in the oracle must break agreement with the scalar transcription."""
     batch = tiny_v(5)
     tok, attn = batch.tokens[0], batch.attn[0]
     P = tok[1:].astype(np.float64)
@@ -591,7 +591,7 @@ def test_edge_counts():
 # ---------------------------------------------------------------------------
 
 def _eq_token_loops(keys, n_cls):
-    """Scalar-loop transcription of the appendix equations (independent of the checker)."""
+    """Scalar-loop transcription of the appendix equations (independent of the oracle)."""
     T, H, d = keys.shape
     M = [[sum(float(keys[t, h, o]) for h in range(H)) / H for o in range(d)] for t in range(T)]
     P = M[n_cls:]

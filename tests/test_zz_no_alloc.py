@@ -40,7 +40,7 @@ def test_noalloc_matches_context_entry_point_twice():
         got = got.cpu().numpy().astype(np.float64)
         scale = float(np.mean(np.abs(want)))
         assert np.all(np.abs(got - want) <= 1e-5 * np.maximum(np.abs(want), scale))
-        # and against the float64 checker: the first term of Eq. 1 from the literal N x N relation
+        # and against the float64 oracle: the first term of Eq. 1 from the literal N x N relation
         np_ = n_tokens - 1
         for b in range(batch.batch):
             P = fo.widen(batch.tokens[b])[1:]
