@@ -13,7 +13,7 @@ constexpr unsigned STATUS_POS_RANGE = 1u;
 
 // One image (FiCoCo-V) or sequence (FiCoCo-L) of the batch.  All offsets are in elements of
 // the array they index, counted over the whole packed batch.
-struct ImgDesc {
+struct alignas(16) ImgDesc {
   int row0;        // first token row in `tokens`
   int n_cls;       // leading pass-through rows (CLS)
   int np;          // alive vision tokens
