@@ -9,30 +9,56 @@ constexpr int MTHREADS = 512;
 constexpr int MWARPS = MTHREADS / 32;
 constexpr int MROWS = 64;      // most output rows a CTA takes (a lane looks after two in the scan)
 constexpr int MLIST = 1024;    // sources a CTA files in shared memory
-constexpr int MDEPTH = 6;      // source rows a warp has in flight; rows with more sources than that go first
-constexpr int MUNITS = 256;    // (row with sources, 512 bytes of it) units of a CTA
+constexpr int MDEPTH = 6;      // loads a lane has in flight; rows with more sources than that go first
+constexpr int MUNITS = 640;    // (row with sources, part of it) units of a CTA
 constexpr size_t MSTAGE_BYTES = 70 * 1024;   // input rows of a CTA's output rows kept in shared memory (two CTAs per SM)
-static_assert(MSTAGE_BYTES / 512 + MROWS <= MUNITS, "every unit of a CTA needs an entry");
+static_assert(MSTAGE_BYTES / 128 + MROWS <= MUNITS, "every unit of a CTA needs an entry");
 
-// 16 bytes of row `own` (shared memory) plus its sources, at byte `off` of their rows; lanes past the row's end idle.
-template <class T>
-__device__ __forceinline__ void merge_unit(const unsigned char* own, const uint2* list, int n, const unsigned char* image,
-                                           unsigned char* dst, int off, int row_bytes) {
-  constexpr int E = VecTraits<T>::E;
+// A warp walks a row's list over 512 bytes of the row, a long list over 128: its lanes then form MGROUPS groups of
+// eight, group k takes the sources k, k + MGROUPS, ... and the groups' sums are added at the end, which puts four times
+// as many sources in flight.  Which of the two it is, and with it the order of the sum, follows the list and the
+// hidden size alone (rows of 16 parts and more give every warp one as they are).
+constexpr int MLONG = 12 * MDEPTH, MGROUPS = 4;
+__device__ __forceinline__ bool list_long(int n, int row_bytes) { return n > MLONG && row_bytes <= 512 * (MWARPS - 1); }
+__device__ __forceinline__ int list_parts(int n, int row_bytes) {
+  return n == 0 ? 0 : list_long(n, row_bytes) ? (row_bytes + 127) / 128 : (row_bytes + 511) / 512;
+}
+// The groups' sums: (0 + 1) + (2 + 3), in every lane.
+template <int E>
+__device__ __forceinline__ void add_groups(float (&acc)[E], float& den) {
+#pragma unroll
+  for (int o = 32 / MGROUPS; o < 32; o <<= 1) {
+    den += __shfl_xor_sync(0xFFFFFFFFu, den, o);
+#pragma unroll
+    for (int q = 0; q < E; ++q) acc[q] += __shfl_xor_sync(0xFFFFFFFFu, acc[q], o);
+  }
+}
+
+// Byte `off` of row `own` (shared memory) plus its sources, 16 bytes per lane; lanes past the row's end idle.  LONG: as
+// one of MGROUPS groups of lanes, the `first`-th; a function of its own, so that the usual lists keep their registers
+// and instructions.
+template <class T, bool LONG>
+__device__ __forceinline__ void merge_list(const unsigned char* own, const uint2* list, int n, const unsigned char* image,
+                                           unsigned char* dst, int off, int first, int row_bytes) {
+  constexpr int E = VecTraits<T>::E, STEP = LONG ? MGROUPS : 1;
   const bool on = off < row_bytes;
   if (!on) off = 0;
-  float acc[E], den = 1.0f;
+  float acc[E], den = first == 0 ? 1.0f : 0.0f;
   unpack(*reinterpret_cast<const uint4*>(own + off), acc, (const T*)nullptr);
+  if (LONG && first != 0) {
+#pragma unroll
+    for (int q = 0; q < E; ++q) acc[q] = 0.f;
+  }
   image += off;
   #pragma unroll 1
-  for (int e = 0; e < n; e += MDEPTH) {
+  for (int e = first; e < n; e += MDEPTH * STEP) {
     uint4 u[MDEPTH];
 #pragma unroll
-    for (int j = 0; j < MDEPTH; ++j) u[j] = ldg16(image + list[min(e + j, n - 1)].y);   // (past the end: the last row again)
+    for (int j = 0; j < MDEPTH; ++j) u[j] = ldg16(image + list[min(e + j * STEP, n - 1)].y);   // (past the end: the last row)
 #pragma unroll
     for (int j = 0; j < MDEPTH; ++j)
-      if (e + j < n) {
-        const float a = __uint_as_float(list[e + j].x);
+      if (e + j * STEP < n) {
+        const float a = __uint_as_float(list[e + j * STEP].x);
         float x[E];
         unpack(u[j], x, (const T*)nullptr);
         den += a;
@@ -40,10 +66,19 @@ __device__ __forceinline__ void merge_unit(const unsigned char* own, const uint2
         for (int q = 0; q < E; ++q) acc[q] = fmaf(a, x[q], acc[q]);
       }
   }
+  if (LONG) {
+    __syncwarp();
+    add_groups(acc, den);
+  }
   const float inv = 1.0f / den;
 #pragma unroll
   for (int q = 0; q < E; ++q) acc[q] *= inv;
-  if (on) st_stream16(reinterpret_cast<uint4*>(dst + off), pack(acc, (const T*)nullptr));
+  if (on && first == 0) st_stream16(reinterpret_cast<uint4*>(dst + off), pack(acc, (const T*)nullptr));
+}
+template <class T>
+__device__ __noinline__ void merge_long_list(const unsigned char* own, const uint2* list, int n, const unsigned char* image,
+                                             unsigned char* dst, int part, int lane, int row_bytes) {
+  merge_list<T, true>(own, list, n, image, dst, (8 * part + (lane & 7)) * 16, lane >> 3, row_bytes);
 }
 
 // Compress + compact.  A CTA owns a few output rows of one image, the ones `stride` apart from its first: targets
@@ -57,19 +92,20 @@ __device__ __forceinline__ void merge_unit(const unsigned char* own, const uint2
 //           flight per thread;
 //   copies  a row that nothing is folded into leaves by a bulk store from shared memory: no thread touches it;
 //   merge   out_j = (x_j + sum_{i in I_j} alpha_ij x_i) / (1 + sum alpha_ij), rounded once.  A unit is one row and
-//           512 bytes of it; a warp adds the row's sources in list order, several of them in flight, and draws its
-//           next unit from a counter.  Rows with many sources go first.
-// Every fp32 sum runs over its row's whole list, in order, in one thread, whatever else the CTA owns: an output row
-// is the same bits alone, in a batch of any size and in a group of a batch.
+//           512 bytes of it, or 128 where its list is long; a warp adds the row's sources, several of them in flight,
+//           and draws its next unit from a counter.  Rows with many sources go first.
+// The order of every fp32 sum follows its row's list alone, whatever else the CTA owns: an output row is the same bits
+// alone, in a batch of any size and in a group of a batch.
 // What bounds it is the latency of its few dependent trips to L2; the split into 16 warps and the host's choice of
 // one wave of CTAs where possible keep them few: 32 x 577 -> 289 rows of 1024 went from 25 us (a scan per 16 rows,
-// copies and hub rows by warps, two waves of CTAs) to 20 us, 16 ragged images keeping 1/9 from 48 to 28 us.  (Equal
+// copies and hub rows by warps, two waves of CTAs) to 18 us, 16 ragged images keeping 1/9 from 48 to 30 us.  (Equal
 // segments of the sequence slices x sources per warp, with a list cut wherever a segment ended, are balanced better
 // where a CTA has one long list, but the order of a sum then follows the rows per CTA and with them the batch: whole
-// step 53.4 us instead of 54.7 for one fp32 image, 102 and 104 for 16 ragged images, but 61.3 and 59.8 for 32 x 577,
-// 139 and 135 for 8 x 2881, 112 and 104 for 16 FiCoCo-L sequences, 53.4 and 44.4 with a relation map, as the pieces
-// took a barrier, 18 KB of shared memory and another pass.  Parts of 256 bytes with twice as many sources in flight
-// for the longer lists: 8 x 2881 tokens 139 us, the others the same.  8 or 10 sources in flight: the same.)
+// step 100.6 us instead of 102.9 for 16 ragged images, but 61.2 and 59.7 for 32 x 577, 138 and 135 for 8 x 2881, 112.7
+// and 105.5 for 16 FiCoCo-L sequences, 53.4 and 44.5 with a relation map, as the pieces took a barrier, 18 KB of shared
+// memory and another pass.  Long lists like the others: 16 ragged images of up to 4096 tokens 105.5 us instead of 99.6;
+// long from 36 sources on: 100.4.  One function for both kinds, the number of groups a variable: 8 x 2881 tokens 138 us
+// instead of 135.  8 or 10 sources in flight: the same.)
 // If the CTA's rows receive more than MLIST sources in total, a slow in-order rescan is used.
 template <class T>
 __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
@@ -91,7 +127,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
   const WorkItem w = work[blockIdx.x];
   const ImgDesc d = desc[w.img];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nvec = D / E, row_bytes = D * (int)sizeof(T);
+  const int row_bytes = D * (int)sizeof(T);
   const int L = d.list_len;
   const int stride = w.aux;                      // row r of the CTA is output row w.r0 + r * stride of the image
   const float inv_stride = 1.0f / (float)stride;
@@ -173,12 +209,11 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
     mbar_wait(&row_bar, 0, wait_ns);             // no copy outlives the CTA
     return;
   }
-  const int n_parts = (row_bytes + 511) / 512;
   if (warp == 0) {
     // starts of the lists, and of the units of the rows that have sources: those with many first
     const int c0 = cnt[2 * lane], c1 = cnt[2 * lane + 1];
-    const int u0 = c0 > MDEPTH ? n_parts << 16 : c0 > 0 ? n_parts : 0;
-    const int u1 = c1 > MDEPTH ? n_parts << 16 : c1 > 0 ? n_parts : 0;
+    const int u0 = list_parts(c0, row_bytes) << (c0 > MDEPTH ? 16 : 0);
+    const int u1 = list_parts(c1, row_bytes) << (c1 > MDEPTH ? 16 : 0);
     int ci = c0 + c1, ui = u0 + u1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -207,7 +242,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
       }
     }
     for (int r = warp; r < w.nrows; r += MWARPS)
-      for (int k = lane; cnt[r] > 0 && k < n_parts; k += 32) unit[ubeg[r] + k] = (unsigned short)(r << 8 | k);
+      for (int k = lane; k < list_parts(cnt[r], row_bytes); k += 32) unit[ubeg[r] + k] = (unsigned short)(r << 8 | k);
     __syncthreads();
     // the list of a row is ordered by entry, i.e. by discarded token
 #pragma unroll
@@ -247,38 +282,54 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
     #pragma unroll 1
     for (int u = warp; u < n_unit;) {
       const int r = unit[u] >> 8, part = unit[u] & 255;
-      merge_unit<T>(stage + (size_t)r * row_bytes, el + beg[r], cnt[r], reinterpret_cast<const unsigned char*>(pbase),
-                    reinterpret_cast<unsigned char*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D),
-                    (32 * part + lane) * 16, row_bytes);
+      const unsigned char* own = stage + (size_t)r * row_bytes;
+      const unsigned char* image = reinterpret_cast<const unsigned char*>(pbase);
+      unsigned char* dst = reinterpret_cast<unsigned char*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D);
+      if (list_long(cnt[r], row_bytes)) merge_long_list<T>(own, el + beg[r], cnt[r], image, dst, part, lane, row_bytes);
+      else merge_list<T, false>(own, el + beg[r], cnt[r], image, dst, (32 * part + lane) * 16, 0, row_bytes);
       if (lane == 0) u = atomicAdd(&next_unit, 1);
       u = __shfl_sync(0xFFFFFFFFu, u, 0);
     }
     FICOCO_PHASE(2, 4);
   } else if (total > 0) {
-    // too many sources for shared memory: walk the entries in order (ascending source)
+    // too many sources for shared memory: walk the entries in order (ascending source).  Sums and quotient as in
+    // merge_list, because whether a CTA comes here follows its other rows.
     #pragma unroll 1
     for (int r = warp; r < w.nrows; r += MWARPS) {
-      if (cnt[r] == 0) continue;
-      const int tp = w.r0 + r * stride - d.n_cls;
-      float den = 1.0f;                          // (sums and quotient as in merge_unit: which path a row takes follows
-      for (int e = 0; e < n_ent; ++e)            // the rows of its CTA)
-        if (e_tgt[d.ent0 + e] == tp) den += e_w[d.ent0 + e];
-      const float inv = 1.0f / den;
-      for (int v = lane; v < nvec; v += 32) {
-        float acc[E];
-        unpack(*reinterpret_cast<const uint4*>(stage + (size_t)r * row_bytes + (size_t)v * 16), acc, (const T*)nullptr);
+      const int n = cnt[r], tp = w.r0 + r * stride - d.n_cls;
+      const bool is_long = list_long(n, row_bytes);
+      const int width = is_long ? 32 / MGROUPS : 32, first = lane / width;
+      #pragma unroll 1
+      for (int part = 0; part < list_parts(n, row_bytes); ++part) {
+        int off = (part * width + (lane & (width - 1))) * 16;
+        const bool on = off < row_bytes;
+        if (!on) off = 0;
+        float acc[E], den = first == 0 ? 1.0f : 0.0f;
+        unpack(*reinterpret_cast<const uint4*>(stage + (size_t)r * row_bytes + off), acc, (const T*)nullptr);
+        if (first != 0) {
+#pragma unroll
+          for (int q = 0; q < E; ++q) acc[q] = 0.f;
+        }
+        int k = 0;
         for (int e = 0; e < n_ent; ++e) {
           if (e_tgt[d.ent0 + e] != tp) continue;
+          if (is_long && k++ % MGROUPS != first) continue;
           const T* x0 = pbase + (size_t)checked_index(S_idx[d.src0 + e / L], d.np, status) * D;
           float f[E];
-          unpack(ldg16(x0 + (size_t)v * E), f, (const T*)nullptr);
+          unpack(ldg16(reinterpret_cast<const unsigned char*>(x0) + off), f, (const T*)nullptr);
           const float a0 = e_w[d.ent0 + e];
+          den += a0;
 #pragma unroll
           for (int q = 0; q < E; ++q) acc[q] = fmaf(a0, f[q], acc[q]);
         }
+        __syncwarp();
+        if (is_long) add_groups(acc, den);
+        const float inv = 1.0f / den;
 #pragma unroll
         for (int q = 0; q < E; ++q) acc[q] *= inv;
-        st_stream16(reinterpret_cast<uint4*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D) + v, pack(acc, (const T*)nullptr));
+        if (on && first == 0)
+          st_stream16(reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(out + (size_t)(d.out_row0 + w.r0 + r * stride) * D) + off),
+                      pack(acc, (const T*)nullptr));
       }
     }
   }

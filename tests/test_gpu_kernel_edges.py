@@ -25,12 +25,15 @@ def run_v(ctx, seed, batch, gh, gw, dim, keep, dtype="bf16", cls=True, p=fo.Para
 
 
 @pytest.mark.parametrize("batch,gh,gw,dim,keep,dtype", [
-    (1, 9, 9, 64, 1, "bf16"),          # one row with every source: a hub cut by all 16 segments
+    (1, 9, 9, 64, 1, "bf16"),          # one row with every source
     (1, 33, 34, 64, 1, "bf16"),        # more sources than a CTA files: the in-order rescan
     (2, 8, 8, 4096, 9, "fp32"),        # rows of 16 KB: few rows per CTA
     (1, 6, 7, 72, 41, "bf16"),         # one source; rows that are no multiple of 32 vectors
     (24, 20, 20, 64, 300, "bf16"),     # many rows per CTA, dealt out with a stride
-], ids=["hub", "rescan", "wide-rows", "one-source", "many-rows"])
+    (1, 1, 73, 72, 1, "bf16"),         # 72 sources: the longest list that is not split over groups of lanes
+    (1, 2, 37, 72, 1, "bf16"),         # 73: the shortest that is, in a row that ends inside its second part
+    (1, 7, 14, 1280, 1, "fp32"),       # 97: the groups' lists differ in length by a batch
+], ids=["hub", "rescan", "wide-rows", "one-source", "many-rows", "72", "73", "97"])
 def test_merge_rows(ctx, batch, gh, gw, dim, keep, dtype):
     run_v(ctx, 91, batch, gh, gw, dim, keep, dtype)
 
