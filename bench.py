@@ -33,7 +33,7 @@ MIN_TIMED_MS = 50.0   # device time the timed repetitions add up to, at least
 NOMINAL = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}   # vendor figures, reported beside the measured peaks
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised under
 # profiles/ (bytes); an entry is removed when its kernel changes after the capture.
-NCU_TRAFFIC = {"filter_fused": 39019520 + 25344, "correlate_umma": 37962752, "merge_compact": 38096640}
+NCU_TRAFFIC = {"filter_fused": 39087616 + 40960, "correlate_umma": 37961472, "merge_compact": 37873152 + 9728}
 
 
 def algorithmic_bytes() -> dict:

@@ -76,9 +76,9 @@ __device__ __forceinline__ uint4 pack(const float (&f)[8], const __nv_bfloat16*)
 }
 
 __device__ __forceinline__ uint4 ldg16(const void* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
-// Streaming store (st.global.cs) for the output rows.  A step's token rows, read by all three of
-// its kernels, plus its output rows are about as much as L2 keeps; written as ordinary stores the
-// output pushes the token rows out before the next kernel reads them again.
+// Streaming store (st.global.cs) for the output rows.  A step's token rows, read by all three of its kernels, plus its
+// output rows are about as much as L2 keeps.  32 x 577 tokens of 1024, DRAM reads of correlate and merge in the running
+// step: 0.64 and 0.18 MB where inputs are used again, 1.50 and 0.47 with ordinary stores; on cycled inputs 0.3 MB both ways.
 __device__ __forceinline__ void st_stream16(uint4* p, const uint4& v) { __stcs(p, v); }
 
 // A token index read from an index list of the step, as a row offset inside its image: anything

@@ -208,7 +208,7 @@ __device__ __forceinline__ void attn_mean_rows(const float* __restrict__ a0, int
 // the two before them: the mean direction sits in registers (a lane owns the same columns of every row), and nothing
 // else is fetched inside the loop.  The chunks are taken last to first: a batch larger than the L2 cache leaves its
 // last images there when the column sums are done.  (One row per warp at a time, the direction in shared memory and
-// the norm read behind every dot product: 256 x 577 rows of 1024, 302 MB, took 124 us.)
+// the norm read behind every dot product: 256 x 577 rows of 1024, 302 MB, took 139 us, now 63.)
 template <class T, int VPL>
 __global__ void __launch_bounds__(256, VPL <= 5 ? 2 : 1) k_score_rows(const T* __restrict__ tokens, int D,
                                                                       const ImgDesc* __restrict__ desc,
@@ -643,7 +643,7 @@ __device__ __forceinline__ void settle_cells(Cell* cell, int cells, const float*
 //   3. ballots and one scan turn the membership flags into ascending index lists S and T, the kept
 //      row indices and the surviving grid positions.
 // What bounds it is the chain of barriers, not the work.  (Bids for the windows by 64-bit shared-memory maxima, a
-// radix select and runs of tokens per thread: the filter of 16 images of up to 2880 tokens took 60 us, now 54.)
+// radix select and runs of tokens per thread: the filter of 16 ragged images of up to 4096 tokens took 60 us, now 56.)
 // The code runs once per image, so it is kept compact (rolled loops, not inlined): a long
 // unrolled body would be paid for in instruction-cache misses.
 // `work` is a shared-memory area of select_work_bytes(np, cells) bytes: the scores and grid

@@ -30,7 +30,7 @@ NAMES = {
                            "merge grid before complete", "scores seen", "end"]),
     1: ("k_correlate_umma", ["start", "setup", "filter grid complete", "lists loaded", "k-loop done", "accumulator ready",
                              "top lists written", "synced", "end"]),
-    2: ("k_merge_rows", ["start", "correlate grid complete", "entries filed", "copies issued", "units done", "end"]),
+    2: ("k_merge_rows", ["start", "correlate grid complete", "entries filed", "copies issued", "warp 0: no unit left", "warp 0: end"]),
     3: ("k_correlate_umma_f32", ["start", "setup", "filter grid complete", "lists loaded", "k-loop done",
                                  "accumulator ready", "top lists written", "end"]),
 }
