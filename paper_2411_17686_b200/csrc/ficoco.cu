@@ -76,9 +76,16 @@ struct Plan {
   bool umma = false;
   bool um_f32 = false;          // fp32 tokens split into three bf16 terms (k_correlate_umma_f32)
   int um_b_bytes = 0;
-  int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1;
+  int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1, um_text_off = 0;
   size_t um_smem = 0;
   std::vector<ImgDesc> h_desc;
+};
+
+// Shared memory of a CTA of the bf16 tensor-core correlate.
+struct UmRing {
+  int nstage = 0, ksub = 1, stage_bytes = 0;
+  int text_off = 0;             // where FiCoCo-L's text weights lie, behind the ring's start
+  size_t smem = 0;
 };
 
 // ---- what the last step on a stream wrote ------------------------------------------------------
@@ -399,9 +406,10 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   }
   c->cap_rows = (int)(MAX_CHUNKS * B);
   if (c->cap_rows < c->num_sms + (int)B + 8) c->cap_rows = c->num_sms + (int)B + 8;
-  // (bf16 tiles of 128 x 256 tokens: at most n * n / (4 * 128 * 256) + n / 128 + 1 of an image of n tokens)
+  // (bf16 tiles of 64 x 256 tokens, the largest that leave room for 101 text tokens: at most n * n / (4 * 64 * 256) +
+  // n / 64 + n / 256 + 1 of an image of n tokens)
   const size_t n_most = T < (size_t)MAX_IMG_TOKENS ? T : MAX_IMG_TOKENS;
-  c->cap_corr = (int)std::max<size_t>(2 * (T / CBM + B) + 2048, T * n_most / (4 * UM * UN_MAX) + T / UM + B + 64);
+  c->cap_corr = (int)std::max<size_t>(2 * (T / CBM + B) + 2048, T * n_most / (2 * UM * UN_MAX) + T / 32 + B + 64);
   // (wide rows: no more of them per merge CTA than its shared memory takes, fp32 being the widest)
   const size_t out_rows = std::min<size_t>(OUT_ROWS_PER_CTA, std::max<size_t>(1, MSTAGE_BYTES / ((size_t)max_dim * 4)));
   c->cap_out = (int)(T / out_rows + B + 2 * c->num_sms);
@@ -451,12 +459,11 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   {
     const int um_smem_max = 221 * 1024;
-#define FICOCO_UMMA_ATTR(NS, KS)                                                                            \
-    cudaFuncSetAttribute(k_correlate_umma<NS, 2, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max); \
-    cudaFuncSetAttribute(k_correlate_umma<NS, 4, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max); \
-    cudaFuncSetAttribute(k_correlate_umma<NS, 16, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max)
-    FICOCO_UMMA_ATTR(2, 1); FICOCO_UMMA_ATTR(3, 1); FICOCO_UMMA_ATTR(4, 1);
-    FICOCO_UMMA_ATTR(2, 2); FICOCO_UMMA_ATTR(3, 2); FICOCO_UMMA_ATTR(4, 2);
+#define FICOCO_UMMA_ATTR(LC)                                                                                  \
+    cudaFuncSetAttribute(k_correlate_umma<LC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);     \
+    cudaFuncSetAttribute(k_correlate_umma<LC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);     \
+    cudaFuncSetAttribute(k_correlate_umma<LC, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max)
+    FICOCO_UMMA_ATTR(2); FICOCO_UMMA_ATTR(4); FICOCO_UMMA_ATTR(16);
 #undef FICOCO_UMMA_ATTR
     cudaFuncSetAttribute(k_correlate_umma_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
     cudaFuncSetAttribute(k_correlate_umma_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
@@ -473,6 +480,12 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   }
   cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
   cudaFuncSetAttribute(k_merge_rows<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
+  // Two merge CTAs need 184 KB of shared memory.  Left to itself the SM stays at the largest carve-out when the correlate
+  // kernel has set it, and the 28 KB of L1 that leaves slow the streaming kernels of the next step, which start beside
+  // the merge (16 FiCoCo-L sequences, correlate CTAs of 205 KB: head mean 15.5 -> 17.4 us, column sums 18.9 -> 20.9,
+  // step 108 us instead of 102).  76 % is the 196 KB setting.
+  cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributePreferredSharedMemoryCarveout, 76);
+  cudaFuncSetAttribute(k_merge_rows<__nv_bfloat16>, cudaFuncAttributePreferredSharedMemoryCarveout, 76);
   cudaFuncSetAttribute(k_score<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   cudaFuncSetAttribute(k_score<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   if (cudaGetLastError() != cudaSuccess) { ficoco_destroy(c); return FICOCO_ERR_CUDA; }
@@ -623,40 +636,91 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   }
 
   // ---- correlate tiling ---------------------------------------------------------------------
-  // A CTA gathers (tile rows + split columns) token rows per k-block from L2, which is what its time is
-  // proportional to; two CTAs share an SM and the last round of CTAs is on average half empty.  Measured on 256 x 577
-  // and 8 x 2881 tokens of 1024 over splits of 2 .. 8: within 10 % of  rows gathered by a CTA x CTAs per SM, the
-  // latter as the mean of the exact number and of whole rounds.  (Tiles of 256 rows that share one column tile gather
-  // fewer rows in total, but a CTA alone on its SM leaves it idle through its epilogue: 143 us against 105 on
-  // 256 x 577 tokens, 72 against 69 on 8 x 2881.)
   const int cols_max = p->umma ? un_max : INT_MAX;
   auto split_cols = [&](int n_tgt, int ns) {           // columns per split: ns splits, or more if they got too wide
     ns = std::max(ns, (n_tgt - 1) / cols_max + 1);
     return ((n_tgt + ns - 1) / ns + col_granule - 1) / col_granule * col_granule;
   };
   auto row_tiles = [&](int n_src) { return (n_src + tile_rows_max - 1) / tile_rows_max; };
+  // Shared memory of the bf16 tensor-core correlate: as many stages as fit, with four k-blocks per stage where that
+  // leaves four stages, else two (a stage costs about 400 cycles besides its copies and MMAs: one FiCoCo-L sequence,
+  // 80 rows per CTA: k-loop 15 us with one, 11 with two, 9 with four); a grid of more CTAs than SMs keeps to what lets
+  // two share an SM.
+  auto um_ring = [&](int a_rows, int cols, long long n_ctas) {
+    UmRing r;
+    cols = (cols + 15) / 16 * 16;
+    const size_t kblock = (size_t)(a_rows + cols) * 128;
+    const size_t text = key.mode == 1 ? (size_t)key.n_text * (a_rows + cols) * 4 : 0;
+    // every MMA reads 128 A rows: behind the last k-block there must be room for the rows past the tile
+    const size_t slack = 1024 + (kblock < (size_t)UM * 128 ? (size_t)UM * 128 - kblock : 0);
+    const size_t most = 220 * 1024, budget = n_ctas > c->num_sms ? 106 * 1024 : most;
+    auto fit = [&](int ksub, int ns, size_t limit) {
+      if (r.nstage || (size_t)ns * ksub * kblock + slack + text > limit) return;
+      r.nstage = ns;
+      r.ksub = ksub;
+      r.stage_bytes = (int)(ksub * kblock);
+      r.text_off = (int)((size_t)ns * ksub * kblock + slack - 1024);
+      r.smem = (size_t)ns * ksub * kblock + slack + text;
+    };
+    const int nk = key.dim / UKB;
+    for (const size_t limit : {budget, most}) {        // (FiCoCo-L with much text: rather one CTA per SM)
+      for (int ns = std::min(UM_STAGES, (nk + 3) / 4); ns >= 4; --ns) fit(4, ns, limit);
+      for (int ksub = 2; ksub >= 1; --ksub)
+        for (int ns = std::max(2, std::min(UM_STAGES, (nk + ksub - 1) / ksub)); ns >= 2; --ns) fit(ksub, ns, limit);
+    }
+    // the epilogue halves hand their lists over through the ring
+    r.smem = std::max(r.smem, 1024 + (size_t)UM * KCAP * 8);
+    if (r.smem > most) r.nstage = 0;
+    return r;
+  };
+  // Tile of the bf16 tensor-core correlate: rows, and column splits, by the least estimated time (ns), fitted to the
+  // kernel's time on eleven batches (one to 32 images of 144 to 2880 tokens of 1024, one to 16 FiCoCo-L sequences of 4096)
+  // under twenty tilings each: a chain of phases and k-blocks that no tiling shortens, the rows that a CTA gathers, the
+  // columns that its epilogue reads (with a text term per text token), a trip through L2 where a tile is split and one for
+  // every four entries per lane when its lists are merged.  A second CTA on the SM costs its rows again, and a grid that
+  // needs more than one round of two is on average half empty in the last.  Tiles below 128 rows serve small grids:
+  // one sequence of 576 + 64 tokens of 4096, 512 x 64 entries: 22.5 us in 16 CTAs of 128 x 16, 15 in 128 of 16 x 16;
+  // 32 x 288 tokens, 144 x 144 entries: 9.25 us in tiles of 72 x 80, 8.75 in 48 x 144 (no split, no counters); 32 x 576
+  // tokens take 13.5 us in tiles of 96 x 96 and 22 to 82 in any that make a second round.
   int want_split = 1;
   if (p->umma && !p->um_f32) {
-    const long long wave = 2LL * c->num_sms;
     double best = 0;
-    for (int ws = 1; ws <= NSPLIT_MAX; ++ws) {
-      long long n_ctas = 0, rows_gathered = 0, entries = 0;
-      for (int b = 0; b < B; ++b) {
-        const ImgDesc& d = p->h_desc[b];
-        if (d.list_len == 0) continue;
-        const int cps = split_cols(d.n_tgt, ws), ntile = row_tiles(d.n_src);
-        const int trows = ((d.n_src + ntile - 1) / ntile + 7) / 8 * 8;
-        const long long n = (long long)ntile * ((d.n_tgt + cps - 1) / cps);
-        n_ctas += n;
-        rows_gathered += n * (trows + cps);
-        entries += (long long)d.n_src * ((d.n_tgt + cps - 1) / cps) * d.list_len;
+    int best_rows = tile_rows_max;
+    const double k_scale = key.dim / 1024.0, text_scale = key.mode == 1 ? 1.0 + key.n_text / 9.5 : 1.0;
+    const long long wave = 2LL * c->num_sms;
+    for (int t : {128, 64, 32, 16}) {
+      tile_rows_max = t;
+      for (int ws = 1; ws <= NSPLIT_MAX; ++ws) {
+        long long n_ctas = 0, rows_gathered = 0, cols = 0, entries = 0;
+        int rows_most = 8, cols_most = 16, list_most = 0;
+        for (int b = 0; b < B; ++b) {
+          const ImgDesc& d = p->h_desc[b];
+          if (d.list_len == 0) continue;
+          const int cps = split_cols(d.n_tgt, ws), ntile = row_tiles(d.n_src), ns = (d.n_tgt + cps - 1) / cps;
+          const int trows = ((d.n_src + ntile - 1) / ntile + 7) / 8 * 8;
+          const long long n = (long long)ntile * ns;
+          n_ctas += n;
+          rows_gathered += n * (trows + cps);
+          cols += n * cps;
+          entries += (long long)d.n_src * ns * d.list_len;
+          rows_most = std::max(rows_most, trows);
+          cols_most = std::max(cols_most, cps);
+          list_most = std::max(list_most, ns * d.list_len);
+        }
+        if (n_ctas == 0) break;
+        if ((ws > 1 || t < UM) && (n_ctas > c->cap_corr || entries > c->cap_part)) break;
+        if (um_ring(rows_most, cols_most, n_ctas).nstage == 0) continue;
+        int lanes = 1;                                 // lanes that share a token when the lists are merged
+        while (lanes < 8 && rows_most * 2 * lanes <= 256) lanes *= 2;
+        const double rows = k_scale * rows_gathered / n_ctas;
+        double cost = 2900.0 + 2270.0 * k_scale + 9.0 * rows + 10.0 * cols / n_ctas * text_scale +
+                      600.0 * ((list_most + 4 * lanes - 1) / (4 * lanes)) + (list_most > p->max_list ? 700.0 : 0.0);
+        if (n_ctas > c->num_sms) cost += 26.0 * rows;
+        if (n_ctas > wave) cost *= 0.5 * ((double)n_ctas / wave + (double)((n_ctas + wave - 1) / wave));
+        if (best == 0 || cost < best) { best = cost; want_split = ws; best_rows = t; }
       }
-      if (n_ctas == 0 || (ws > 1 && (n_ctas > c->cap_corr || entries > c->cap_part))) break;
-      const double exact = (double)n_ctas / c->num_sms;
-      const double whole = n_ctas <= c->num_sms ? 1 : (double)((n_ctas + wave - 1) / wave * wave) / c->num_sms;
-      const double cost = (double)rows_gathered / n_ctas * (n_ctas <= wave ? whole : 0.5 * (exact + whole));
-      if (best == 0 || cost < best) { best = cost; want_split = ws; }
     }
+    tile_rows_max = best_rows;
   } else {
     // as many splits as give every SM two CTAs (fp32 tiles: the CTA that completes a tile merges nsplit * L entries
     // per token, one thread each)
@@ -776,33 +840,16 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     p->um_smem = (size_t)UF_STAGES * 3 * (p->um_a_bytes + p->um_b_bytes) + (size_t)UM * 128 + 2048;
     if (um_a_rows > UM || um_cols > UF_COLS || p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
   } else if (p->umma) {
-    // shared-memory ring of the tensor-core correlate: prefer a size that lets two CTAs share an SM
+    const UmRing r = um_ring(um_a_rows, um_cols, (long long)corr.size());
+    if (r.nstage == 0) return FICOCO_ERR_UNSUPPORTED;
     p->um_a_bytes = um_a_rows * 128;
-    const size_t kblock = (size_t)p->um_a_bytes + (size_t)um_cols * 128;
     p->um_tmem_cols = 32;
     while (p->um_tmem_cols < um_cols) p->um_tmem_cols *= 2;
-    // every MMA reads 128 A rows: behind the last k-block there must be room for the rows past the tile
-    const size_t slack = 1024 + (kblock < (size_t)UM * 128 ? (size_t)UM * 128 - kblock : 0);
-    p->um_nstage = 0;
-    auto ring = [&](int ksub, int ns, size_t budget) {
-      if (p->um_nstage || (size_t)ns * ksub * kblock + slack > budget) return;
-      p->um_nstage = ns;
-      p->um_ksub = ksub;
-    };
-    // Two k-blocks per stage halve the barriers, fences and commits of the k-loop (hidden size 4096: 50 us with
-    // one, 44 with two); a grid of more CTAs than SMs keeps to what lets two share an SM.
-    const size_t budget = (int)corr.size() > c->num_sms ? 106 * 1024 : 220 * 1024;
-    for (int ns = 4; ns >= 2; --ns) ring(2, ns, budget);
-    for (int ns = 4; ns >= 2; --ns) ring(1, ns, budget);
-    if (!p->um_nstage) return FICOCO_ERR_UNSUPPORTED;
-    p->um_stage_bytes = (int)(p->um_ksub * kblock);
-    p->um_smem = (size_t)p->um_nstage * p->um_stage_bytes + slack;
-    // the epilogue halves hand their lists over through the ring; FiCoCo-L also stages the head-mean
-    // text->vision weights of a tile's rows and columns there
-    size_t epi = 1024 + (size_t)UM * KCAP * 8;
-    if (key.mode == 1) epi += (size_t)key.n_text * ((size_t)UM + (size_t)((um_cols + 15) / 16 * 16)) * 4;
-    if (p->um_smem < epi) p->um_smem = epi;
-    if (p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
+    p->um_nstage = r.nstage;
+    p->um_ksub = r.ksub;
+    p->um_stage_bytes = r.stage_bytes;
+    p->um_text_off = r.text_off;
+    p->um_smem = r.smem;
   }
 
   char* slot_dev = c->plan_slots + (size_t)slot * c->slot_bytes;
@@ -1060,21 +1107,17 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     } else if (p->umma && sizeof(T) == 2) {
       prof_tick(c, st, "correlate_umma");
       const __nv_bfloat16* tk = reinterpret_cast<const __nv_bfloat16*>(tok);
-#define FICOCO_UMMA_LAUNCH(NS, LC, KS)                                                                  \
-  launch_dependent(k_correlate_umma<NS, LC, KS>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,               \
+#define FICOCO_UMMA_LAUNCH(LC, KS)                                                                      \
+  launch_dependent(k_correlate_umma<LC, KS>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,                   \
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
-      (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status,                 \
-      p->um_stage_bytes, p->um_a_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt,    \
-      c->e_w, c->e_c, tmean, M, p->max_np, gamma, c->wait_ns)
+      (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status, p->um_nstage,    \
+      p->um_stage_bytes, p->um_a_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt, \
+      c->e_w, c->e_c, tmean, M, p->max_np, gamma, p->um_text_off, c->wait_ns)
 #define FICOCO_UMMA_STAGES(LC)                                                                         \
   do {                                                                                                 \
-    if (p->um_ksub == 2) {                                                                              \
-      if (p->um_nstage == 4) FICOCO_UMMA_LAUNCH(4, LC, 2);                                              \
-      else if (p->um_nstage == 3) FICOCO_UMMA_LAUNCH(3, LC, 2);                                         \
-      else FICOCO_UMMA_LAUNCH(2, LC, 2);                                                                \
-    } else if (p->um_nstage == 4) FICOCO_UMMA_LAUNCH(4, LC, 1);                                           \
-    else if (p->um_nstage == 3) FICOCO_UMMA_LAUNCH(3, LC, 1);                                           \
-    else FICOCO_UMMA_LAUNCH(2, LC, 1);                                                                  \
+    if (p->um_ksub == 4) FICOCO_UMMA_LAUNCH(LC, 4);                                                     \
+    else if (p->um_ksub == 2) FICOCO_UMMA_LAUNCH(LC, 2);                                                     \
+    else FICOCO_UMMA_LAUNCH(LC, 1);                                                                     \
   } while (0)
       if (p->max_list <= 2) FICOCO_UMMA_STAGES(2);
       else if (p->max_list <= 4) FICOCO_UMMA_STAGES(4);
@@ -1094,7 +1137,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   if (p->max_src > 0 && p->need_finalize) {
     prof_tick(c, st, "finalize");
     launch_dependent(k_finalize_src, dim3(p->key.batch, (p->max_src + 255) / 256), 256, 0, st,
-        p->d_desc, c->part_val, c->part_idx, c->corr_cnt, c->tau, c->e_tgt, c->e_w, c->e_c);
+        p->d_desc, c->corr_cnt, c->tau);
     c->launches += 1;
   }
   prof_tick(c, st, "merge_compact");

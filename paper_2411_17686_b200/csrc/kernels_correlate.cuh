@@ -207,55 +207,21 @@ __global__ void __launch_bounds__(256) k_correlate_simt(
 namespace ficoco {
 
 // ---------------------------------------------------------------------------------------
-// One thread per discarded token: merge the column splits' partial top lists, then
-//   tau_i = v[L-1] + frac * (v[L-2] - v[L-1])  (v descending: the two order statistics around
-//   eps*(n-1)), J_i = { entries >= tau_i }, alpha_ij = C+_ij / sum_{J_i} C+  (Eq. 2).
+// tau_i, J_i and alpha_ij of one discarded token from its list of the L largest C_ij (v descending, ix their positions
+// in T, INT_MAX in empty slots):
+//   tau_i = v[L-1] + frac * (v[L-2] - v[L-1])  (the two order statistics around eps*(n-1)),
+//   J_i = { entries >= tau_i },  alpha_ij = C+_ij / sum_{J_i} C+  (Eq. 2).
 // Results go to compact per-image arrays with L slots per token: e_tgt (position in T, or -1),
 // e_w (alpha), e_c (the L largest C, descending).
-// grid = (images, ceil(max N^S / 256)).
 // ---------------------------------------------------------------------------------------
 // LC: compile-time bound on the list length L of the image (lists live in registers).
 template <int LC>
-__device__ __forceinline__ void finalize_source(
-    const ImgDesc& d, int s, const float* __restrict__ part_val, const int* __restrict__ part_idx,
+__device__ __forceinline__ void finish_source(
+    const ImgDesc& d, int s, const float (&v)[LC], const int (&ix)[LC],
     int* __restrict__ corr_cnt, float* __restrict__ tau_out, int* __restrict__ e_tgt,
     float* __restrict__ e_w, float* __restrict__ e_c) {
   const int L = d.list_len;
   const size_t o = (size_t)(d.src0 + s);
-  if (L == 0) { corr_cnt[o] = 0; tau_out[o] = 0.f; return; }
-  float v[LC];
-  int ix[LC];
-#pragma unroll
-  for (int k = 0; k < LC; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
-  const size_t pbase = (size_t)d.part0 + (size_t)s * d.nsplit * L;
-  const int ne = d.nsplit * L;
-#pragma unroll 1
-  for (int e0 = 0; e0 < ne; e0 += 4) {
-    // four entries of the partial lists in flight at a time: the insertion below is unrolled per entry,
-    // and a longer body costs more in instruction fetch than the extra round trips (eight at a time:
-    // +0.25 us per step on 32 x 577 tokens, +7 us on 8 x 2881; sixteen: +0.9 and +25 us)
-    float pv[4];
-    int pi[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const bool on = e0 + j < ne;
-      pv[j] = on ? __ldcg(part_val + pbase + e0 + j) : 0.f;
-      pi[j] = on ? __ldcg(part_idx + pbase + e0 + j) : -1;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float cv = pv[j];
-      int ci = pi[j];
-      if (ci < 0) continue;
-#pragma unroll
-      for (int k = 0; k < LC; ++k) {
-        if (k < L && toplist_better(cv, ci, v[k], ix[k])) {
-          const float tv = v[k]; const int ti = ix[k];
-          v[k] = cv; ix[k] = ci; cv = tv; ci = ti;
-        }
-      }
-    }
-  }
   float vl1 = 0.f, vl2 = 0.f;
 #pragma unroll
   for (int k = 0; k < LC; ++k) {
@@ -286,23 +252,102 @@ __device__ __forceinline__ void finalize_source(
   }
 }
 
+// The tokens of an image that merges nothing (the other images are finished by the correlate grid's tails).
 __global__ void __launch_bounds__(256) k_finalize_src(
-    const ImgDesc* __restrict__ desc, const float* __restrict__ part_val,
-    const int* __restrict__ part_idx, int* __restrict__ corr_cnt, float* __restrict__ tau_out,
-    int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c) {
+    const ImgDesc* __restrict__ desc, int* __restrict__ corr_cnt, float* __restrict__ tau_out) {
   const ImgDesc d = desc[blockIdx.x];
   grid_dep_wait();
   grid_dep_launch();
   const int s = blockIdx.y * 256 + threadIdx.x;
-  if (s >= d.n_src) return;
-  finalize_source<KCAP>(d, s, part_val, part_idx, corr_cnt, tau_out, e_tgt, e_w, e_c);
+  if (s >= d.n_src || d.list_len > 0) return;
+  corr_cnt[d.src0 + s] = 0;
+  tau_out[d.src0 + s] = 0.f;
+}
+
+// Merges the column splits' partial top lists of the discarded tokens [r0, r0 + nrows) and finishes the tokens.  All
+// threads of the CTA.  Up to eight lanes share a token: each takes every G-th of its nsplit * L entries (four in flight)
+// into a list of its own, then the group draws the L best heads one by one.  What bounds it is round trips to L2 (a
+// thread per token read 24 entries of eight splits in six of them: 7 us; one image of 576 fp32 tokens); the insertion
+// stays rolled over groups of four, since a longer body costs more in instruction fetch than the trips it saves.
+template <int LC>
+__device__ __forceinline__ void finalize_tile(
+    const ImgDesc& d, int r0, int nrows, const float* __restrict__ part_val, const int* __restrict__ part_idx,
+    int* __restrict__ corr_cnt, float* __restrict__ tau_out, int* __restrict__ e_tgt, float* __restrict__ e_w,
+    float* __restrict__ e_c) {
+  const int L = d.list_len, ne = d.nsplit * L, nthr = (int)blockDim.x;
+  int lg = 0;
+  while (lg < 3 && (nrows << (lg + 1)) <= nthr && (4 << lg) < ne) ++lg;
+  const int G = 1 << lg, sub = (int)threadIdx.x & (G - 1);
+  #pragma unroll 1
+  for (int base = 0; base < nrows << lg; base += nthr) {
+    const int r = (base + (int)threadIdx.x) >> lg;
+    const bool on = r < nrows;
+    float v[LC];
+    int ix[LC];
+#pragma unroll
+    for (int k = 0; k < LC; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
+    const size_t pbase = (size_t)d.part0 + (size_t)(r0 + r) * ne;
+#pragma unroll 1
+    for (int e0 = sub; on && e0 < ne; e0 += 4 * G) {
+      float pv[4];
+      int pi[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool in = e0 + j * G < ne;
+        pv[j] = in ? __ldcg(part_val + pbase + e0 + j * G) : 0.f;
+        pi[j] = in ? __ldcg(part_idx + pbase + e0 + j * G) : -1;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float cv = pv[j];
+        int ci = pi[j];
+        if (ci < 0) continue;
+#pragma unroll
+        for (int k = 0; k < LC; ++k) {
+          if (k < L && toplist_better(cv, ci, v[k], ix[k])) {
+            const float tv = v[k]; const int ti = ix[k];
+            v[k] = cv; ix[k] = ci; cv = tv; ci = ti;
+          }
+        }
+      }
+    }
+    __syncwarp();
+    if (lg > 0) {
+      float bv[LC];
+      int bi[LC];
+#pragma unroll
+      for (int k = 0; k < LC; ++k) { bv[k] = -CUDART_INF_F; bi[k] = INT_MAX; }
+#pragma unroll (LC <= 4 ? LC : 1)
+      for (int k = 0; k < LC; ++k) {
+        if (k >= L) break;
+        float hv = v[0];
+        int hi = ix[0];
+        #pragma unroll 1
+        for (int m = 1; m < G; m <<= 1) {
+          const float ov = __shfl_xor_sync(0xFFFFFFFFu, hv, m);
+          const int oi = __shfl_xor_sync(0xFFFFFFFFu, hi, m);
+          if (toplist_better(ov, oi, hv, hi)) { hv = ov; hi = oi; }
+        }
+        bv[k] = hv;
+        bi[k] = hi;
+        if (hi != INT_MAX && hi == ix[0]) {          // the lane whose head was drawn
+#pragma unroll
+          for (int q = 0; q + 1 < LC; ++q) { v[q] = v[q + 1]; ix[q] = ix[q + 1]; }
+          v[LC - 1] = -CUDART_INF_F; ix[LC - 1] = INT_MAX;
+        }
+      }
+      if (on && sub == 0) finish_source<LC>(d, r0 + r, bv, bi, corr_cnt, tau_out, e_tgt, e_w, e_c);
+    } else if (on) {
+      finish_source<LC>(d, r0 + r, v, ix, corr_cnt, tau_out, e_tgt, e_w, e_c);
+    }
+  }
 }
 
 // Tail of a correlate CTA: once its partial lists are written it bumps the counter of its
 // source tile (`tile` = index of the tile's first work item); the CTA that completes the tile
 // (the last of its d.nsplit column splits) turns the partial lists of the tile's discarded
 // tokens into tau_i, J_i and alpha_ij, and resets the counter.  Nobody waits: there is no
-// spinning.  Call from all threads of the CTA.
+// spinning.  A tile that was not split is complete as it is.  Call from all threads of the CTA.
 template <int LC>
 __device__ __forceinline__ void correlate_tail(
     const ImgDesc& d, const WorkItem& w, int tile, int* __restrict__ tile_done,
@@ -310,17 +355,18 @@ __device__ __forceinline__ void correlate_tail(
     const int* __restrict__ part_idx, int* __restrict__ corr_cnt, float* __restrict__ tau_out,
     int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c, int* is_last_smem) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // publishes this CTA's partial lists and, for the split that arrives last, observes the others'
-    const int old = atom_acq_rel_add(&tile_done[tile], 1);
-    const int last = old == d.nsplit - 1;
-    if (last) tile_done[tile] = 0;
-    *is_last_smem = last;
+  if (d.nsplit > 1) {
+    if (threadIdx.x == 0) {
+      // publishes this CTA's partial lists and, for the split that arrives last, observes the others'
+      const int old = atom_acq_rel_add(&tile_done[tile], 1);
+      const int last = old == d.nsplit - 1;
+      if (last) tile_done[tile] = 0;
+      *is_last_smem = last;
+    }
+    __syncthreads();
+    if (!*is_last_smem) return;
   }
-  __syncthreads();
-  if (*is_last_smem)
-    for (int s = w.r0 + (int)threadIdx.x; s < w.r0 + w.nrows; s += blockDim.x)
-      finalize_source<LC>(d, s, part_val, part_idx, corr_cnt, tau_out, e_tgt, e_w, e_c);
+  finalize_tile<LC>(d, w.r0, w.nrows, part_val, part_idx, corr_cnt, tau_out, e_tgt, e_w, e_c);
 }
 
 }  // namespace ficoco

@@ -4,7 +4,7 @@
 // One CTA owns a tile of discarded tokens (rows of the accumulator, one TMEM lane each) and
 // one column split (<= 256 preserved tokens) of one image; two CTAs share an SM:
 //   warps 0-3, 5-8  gather the token rows with 16-byte cp.async into a ring of 128B-swizzled,
-//              K-major shared-memory tiles (64 or 128 bf16 of the hidden dimension per stage);
+//              K-major shared-memory tiles (64, 128 or 256 bf16 of the hidden dimension per stage);
 //   warp  4    allocates TMEM and issues tcgen05.mma (elect.sync, M = 128, N = columns rounded to 16,
 //              K = 16 per instruction, fp32 accumulation of exact bf16 products);
 //   warps 0-3, 5-8  afterwards read TMEM lanes back with tcgen05.ld (warps 0-3 the lower half
@@ -15,11 +15,16 @@
 // Every wait is bounded; on a timeout the CTA raises STATUS_TIMEOUT, drains its copies,
 // frees its TMEM and returns.
 //
-// What bounds the k-loop is instruction issue of the gather and, at small tiles, the MMA's fixed 128 rows; half of a
-// CTA's time at D = 1024 is its epilogue, which the other CTA of the SM fills.  The copies of a stage are counted
-// instead of tested one by one and the ring index is kept instead of divided for (with two k-blocks per stage and
-// without 256-row tiles, which held twice the row offsets: 16 FiCoCo-L sequences 55 -> 33 us, one sequence 41 -> 31,
-// one small image 16.7 -> 14.3, 32 x 577 tokens 22.7 -> 21.2).
+// What bounds the k-loop: large tiles, the rate at which copies fill shared memory (66 to 79 bytes per cycle and SM at
+// 360 and 192 rows per CTA); small ones, the instructions of a stage (waits, addresses, arrivals: about 400 cycles a
+// warp), as a stage costs the same with its copies or its MMAs left out.  So a copy is predicated instead of branched
+// around, a stage takes up to four k-blocks, the descriptors are made from the ring's address as it is (a shuffle
+// "to make it uniform" put 47 cycles on every MMA, 31 without), and row indices and norms are asked for as soon as the
+// lists exist.  k-loop of one FiCoCo-L sequence (80 rows per CTA, 64 k-blocks) 15.4 -> 10 us, of one image of 144 tokens
+// 3.5 -> 2.2, of 32 x 577 tokens 5.6 -> 5.8, of 16 sequences 16.6 -> 13.
+// Taken back: one arrival per warp after waiting for its copies (one sequence 17 to 28 us: the loop then runs at the
+// latency of a copy), groups of warps that fill different stages with the row offsets in shared memory (10 us there, but
+// 8 x 2881 tokens 12 -> 15), up to four accumulators in turn (the same).
 #pragma once
 #include <limits.h>
 #include <math_constants.h>
@@ -33,6 +38,7 @@ constexpr int UM = 128;          // accumulator rows per MMA (one TMEM lane each
 constexpr int UN_MAX = 256;      // accumulator columns per CTA
 constexpr int UKB = 64;          // bf16 elements per k-block (one 128-byte swizzle row)
 constexpr int UTHREADS = 288;    // warps 0-3 and 5-8 gather + epilogue, warp 4 MMA
+constexpr int UM_STAGES = 8;     // most stages of the operand ring
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -159,7 +165,7 @@ __device__ __forceinline__ void epilogue_scan(uint32_t tmem_lane, int c_lo, int 
     float tx[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) tx[j] = 0.f;
-    #pragma unroll 1
+    #pragma unroll 4
     for (int k = 0; k < M; ++k) {
       const float a = tS[(size_t)k * s_stride];
       const float4* q = reinterpret_cast<const float4*>(tT + (size_t)k * t_stride + c0);
@@ -179,23 +185,23 @@ __device__ __forceinline__ void epilogue_scan(uint32_t tmem_lane, int c_lo, int 
   }
 }
 
-// Dynamic shared memory: [1024-aligned] ring of NSTAGE stages, each KSUB k-blocks of an A tile (a_bytes: the
+// Dynamic shared memory: [1024-aligned] ring of nstage stages, each KSUB k-blocks of an A tile (a_bytes: the
 // valid source rows rounded up to 8, x 128 B) followed by a B tile (column rows x 128 B).  An
 // MMA always reads 128 A rows; rows past a_bytes alias the B tile (or the slack the host adds
-// behind the ring) and only feed accumulator rows that are never read.
-template <int NSTAGE, int LCAP, int KSUB>
+// behind the ring) and only feed accumulator rows that are never read.  FiCoCo-L's text weights lie text_off bytes behind
+// the ring's start and are gathered ahead of the operands.
+template <int LCAP, int KSUB>
 __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     const __nv_bfloat16* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
     const WorkItem* __restrict__ work, const float* __restrict__ rn,
     const int* __restrict__ S_idx, const int* __restrict__ T_idx,
     float* __restrict__ part_val, int* __restrict__ part_idx, unsigned* __restrict__ status,
-    int stage_bytes, int a_bytes, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
+    int nstage, int stage_bytes, int a_bytes, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
     float* __restrict__ tau_out, int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c,
-    const float* __restrict__ tmean, int M, int NV, float gamma, unsigned long long wait_ns) {
+    const float* __restrict__ tmean, int M, int NV, float gamma, int text_off, unsigned long long wait_ns) {
   extern __shared__ unsigned char um_raw[];
-  __shared__ uint64_t full_bar[NSTAGE], empty_bar[NSTAGE], acc_bar;
+  __shared__ uint64_t full_bar[UM_STAGES], empty_bar[UM_STAGES], acc_bar;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int rowS[UM], rowT[UN_MAX];
   __shared__ float rnT[UN_MAX];
   __shared__ int failed, acc_committed, is_last, dead;
 
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   const uint32_t ring = (smem_u32(um_raw) + 1023u) & ~1023u;
 
   if (tid == 0) {
-    for (int s = 0; s < NSTAGE; ++s) { mbar_init(&full_bar[s], 256); mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < nstage; ++s) { mbar_init(&full_bar[s], 256); mbar_init(&empty_bar[s], 1); }
     mbar_init(&acc_bar, 1);
     failed = 0;
     acc_committed = 0;
@@ -230,50 +236,79 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   grid_dep_wait();
   grid_dep_launch();
   FICOCO_PHASE(1, 2);
+  // Producer pt copies chunk (pt & 7) of rows (pt >> 3) + 32 i of the A tile and of the B tile, in every k-block
+  // of the stage.  Byte offsets of the rows stay in registers and the swizzled destination advances by a constant
+  // (32 rows = 4 KB).  A warp's four rows lie in one group of eight, so its number of copies is the same for all
+  // lanes once the tile is rounded up to whole groups (the last row again in the rows added).  A thread looks its rows
+  // up by itself, all of them at once; list entries are range-checked, so those of a step that gave up do no harm.
+  const int pt = warp < 4 ? tid : tid - 32;
+  const int chunk = pt & 7;
+  const int rsub = pt >> 3;           // 0..31
+  const int rgrp = (int)warp_uniform((uint32_t)(rsub >> 3) * 8);
+  const int nA = (((w.nrows + 7) & ~7) - rgrp + 31) / 32, nB = (((ncols + 7) & ~7) - rgrp + 31) / 32;
+  const int* Sl = S_idx + d.src0 + w.r0;
+  const int* Tl = T_idx + d.tgt0 + col_begin;
+  uint32_t offA[UM / 32], offB[UN_MAX / 32];
+  const int row = ((warp & 3) << 5) + lane;       // accumulator row (TMEM lane) of this thread's epilogue
+  const bool row_valid = row < w.nrows;
+  int my_row = 0, my_col = -1;
+  if (warp != 4) {
+#pragma unroll
+    for (int i = 0; i < UM / 32; ++i) offA[i] = i < nA ? (uint32_t)Sl[min(rsub + 32 * i, w.nrows - 1)] : 0u;
+#pragma unroll
+    for (int i = 0; i < UN_MAX / 32; ++i) offB[i] = i < nB ? (uint32_t)Tl[min(rsub + 32 * i, ncols - 1)] : 0u;
+    if (row_valid) my_row = Sl[row];
+    if (pt < ncols) my_col = Tl[pt];
+  }
   // A filter grid that gave up left no valid index lists: do nothing but give the TMEM back.
   if (tid == 0) dead = (*reinterpret_cast<const volatile unsigned*>(status) & STATUS_TIMEOUT) ? 1 : 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  const uint32_t tmem_base = tmem_base_s;
   if (dead) {
     if (warp == 4)
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"((uint32_t)tmem_cols)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)tmem_cols)
                    : "memory");
     return;
   }
-  if (tid < UM) rowS[tid] = tid < w.nrows ? checked_index(S_idx[d.src0 + w.r0 + tid], d.np, status) : -1;
-  for (int c = tid; c < UN_MAX; c += UTHREADS) {
-    const int p = c < ncols ? checked_index(T_idx[d.tgt0 + col_begin + c], d.np, status) : -1;
-    rowT[c] = p;
-    rnT[c] = p >= 0 ? rn[d.patch0 + p] : CUDART_NAN_F;       // a padding column: no list takes its products
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = tmem_base_s;
   FICOCO_PHASE(1, 3);
 
   if (warp != 4) {
     // ---------------- producers (all eight epilogue warps): gather rows, 16 bytes per copy -------
-    // Thread pt copies chunk (pt & 7) of rows (pt >> 3) + 32 i of the A tile and of the B tile, in every k-block
-    // of the stage.  Byte offsets of the rows stay in registers and the swizzled destination advances by a constant
-    // (32 rows = 4 KB).  A warp's four rows lie in one group of eight, so its number of copies is the same for all
-    // lanes once the tile is rounded up to whole groups (the last row again in the rows added).
-    const int pt = warp < 4 ? tid : tid - 32;
-    const int chunk = pt & 7;
-    const int rsub = pt >> 3;           // 0..31
-    const int rgrp = (int)warp_uniform((uint32_t)(rsub >> 3) * 8);
-    const int nA = (((w.nrows + 7) & ~7) - rgrp + 31) / 32, nB = (((ncols + 7) & ~7) - rgrp + 31) / 32;
-    uint32_t offA[UM / 32], offB[UN_MAX / 32];
 #pragma unroll
     for (int i = 0; i < UM / 32; ++i)
-      offA[i] = ((uint32_t)rowS[min(rsub + 32 * i, w.nrows - 1)] * (uint32_t)D + chunk * 8) * 2u;
+      offA[i] = ((uint32_t)checked_index((int)offA[i], d.np, status) * (uint32_t)D + chunk * 8) * 2u;
 #pragma unroll
     for (int i = 0; i < UN_MAX / 32; ++i)
-      offB[i] = ((uint32_t)rowT[min(rsub + 32 * i, ncols - 1)] * (uint32_t)D + chunk * 8) * 2u;
+      offB[i] = ((uint32_t)checked_index((int)offB[i], d.np, status) * (uint32_t)D + chunk * 8) * 2u;
     const uint32_t dsw = (uint32_t)((rsub >> 3) * 1024 + (rsub & 7) * 128 + ((chunk ^ (rsub & 7)) << 4));
     const uint32_t kblock_bytes = (uint32_t)stage_bytes / KSUB;
     const char* src = reinterpret_cast<const char*>(tokens + (size_t)(d.row0 + d.n_cls) * D);
+    // norms of this thread's column and of its accumulator row: asked for here, used in the epilogue
+    const float rn_col = my_col >= 0 ? rn[d.patch0 + checked_index(my_col, d.np, status)] : CUDART_NAN_F;
+    const float rs = row_valid ? rn[d.patch0 + checked_index(my_row, d.np, status)] : 0.f;
+    // FiCoCo-L: the head-mean text->vision weights of the tile's columns and rows, a warp per eighth of the text.  (Gathered
+    // behind the k-loop, eight at a time through registers, and for 128 rows whatever the tile, they took 4 of the 7 us
+    // between accumulator and lists: one sequence of 576 + 64 tokens.)
+    const int s_stride = (w.nrows + 7) & ~7;
+    float* tT = nullptr;
+    float* tSb = nullptr;
+    if (tmean != nullptr) {
+      tT = reinterpret_cast<float*>(um_raw + (ring - smem_u32(um_raw)) + text_off);
+      tSb = tT + (size_t)M * n_pad;
+      const float* tb = tmean + (size_t)w.img * M * NV;
+      #pragma unroll 1
+      for (int j = lane; j < n_pad + s_stride; j += 32) {       // a column or a row of the tile
+        const bool col = j < n_pad;
+        const int at = col ? j : j - n_pad;
+        if (at >= (col ? ncols : w.nrows)) continue;
+        const float* from = tb + checked_index(col ? Tl[at] : Sl[at], d.np, status);
+        const uint32_t to = smem_u32((col ? tT : tSb) + at), step = (uint32_t)(col ? n_pad : s_stride) * 4u;
+        #pragma unroll 4
+        for (int k = pt >> 5; k < M; k += 8) cp_async4(to + (uint32_t)k * step, from + (size_t)k * NV);
+      }
+    }
     bool ok = true;
     // Each thread's copies of a stage arrive on its barrier when they have landed, so a producer never waits
     // for its own copies and the whole ring is in flight; the MMA warp orders the two proxies (below).
@@ -281,151 +316,88 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     uint32_t par = 1;
     #pragma unroll 1
     for (int kb = 0; kb < nkb; ++kb, src += KSUB * UKB * 2) {
-      if (kb >= NSTAGE) ok = mbar_wait(&empty_bar[s], par, wait_ns);
+      if (kb >= nstage) ok = mbar_wait(&empty_bar[s], par, wait_ns);
       if (!ok) break;
       const uint32_t a0 = ring + (uint32_t)s * stage_bytes + dsw;
       const uint32_t b0 = a0 + (uint32_t)a_bytes;
-      const bool two = KSUB == 2 && 2 * kb + 1 < nk;
+      const int nsub = KSUB == 1 ? 1 : min(KSUB, nk - KSUB * kb);    // k-blocks of this stage
 #pragma unroll
-      for (int i = 0; i < UM / 32; ++i)
-        if (i < nA) {
-          const char* p = src + offA[i];
-          cp_async16(a0 + i * 4096, p);
-          if (two) cp_async16(a0 + kblock_bytes + i * 4096, p + UKB * 2);
-        }
+      for (int i = 0; i < UM / 32; ++i) {
+        const char* p = src + offA[i];
 #pragma unroll
-      for (int i = 0; i < UN_MAX / 32; ++i)
-        if (i < nB) {
-          const char* p = src + offB[i];
-          cp_async16(b0 + i * 4096, p);
-          if (two) cp_async16(b0 + kblock_bytes + i * 4096, p + UKB * 2);
-        }
+        for (int j = 0; j < KSUB; ++j) cp_async16_if(i < nA && (KSUB == 1 || j < nsub), a0 + j * kblock_bytes + i * 4096, p + j * (UKB * 2));
+      }
+#pragma unroll
+      for (int i = 0; i < UN_MAX / 32; ++i) {
+        const char* p = src + offB[i];
+#pragma unroll
+        for (int j = 0; j < KSUB; ++j) cp_async16_if(i < nB && (KSUB == 1 || j < nsub), b0 + j * kblock_bytes + i * 4096, p + j * (UKB * 2));
+      }
       cp_async_arrive(&full_bar[s]);
-      if (++s == NSTAGE) { s = 0; par ^= 1u; }
+      if (++s == nstage) { s = 0; par ^= 1u; }
     }
     FICOCO_PHASE(1, 4);
+    rnT[pt] = rn_col;                                  // NaN in a padding column: no list takes its products
     if (!ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
     bool acc_ok = ok && mbar_wait(&acc_bar, 0, wait_ns);
     FICOCO_PHASE(1, 5);
     if (!acc_ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; cp_async_wait_all(); }
     acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);          // tcgen05.ld below is warp-collective
     tc_fence_after();
-    // FiCoCo-L: the head-mean text->vision weights of this tile's columns and rows go into the idle
-    // ring, behind the area the two epilogue halves use to hand over their lists
-    constexpr int rows_pad = UM;
-    float* tT = nullptr;
-    float* tSb = nullptr;
     const float t_scale = tmean != nullptr ? (1.0f - gamma) / (float)M : 0.f;
-    if (tmean != nullptr) {
-      tT = reinterpret_cast<float*>(um_raw + (ring - smem_u32(um_raw)) + (size_t)UM * LCAP * 8);
-      tSb = tT + (size_t)M * n_pad;
-      const float* tb = tmean + (size_t)w.img * M * NV;
-      // eight gathers in flight per thread (one at a time cost a round trip each: 13 us per CTA)
-      #pragma unroll 1
-      for (int i0 = pt; i0 < M * n_pad; i0 += 8 * 256) {
-        float q[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int i = i0 + 256 * j;
-          const int k = i / n_pad, cc = i - k * n_pad;
-          q[j] = (i < M * n_pad && cc < ncols) ? __ldg(tb + (size_t)k * NV + rowT[cc]) : 0.f;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (i0 + 256 * j < M * n_pad) tT[i0 + 256 * j] = q[j];
-      }
-      #pragma unroll 1
-      for (int i0 = pt; i0 < M * rows_pad; i0 += 8 * 256) {
-        float q[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int i = i0 + 256 * j;
-          const int k = i / rows_pad, rr = i - k * rows_pad;
-          q[j] = (i < M * rows_pad && rr < w.nrows) ? __ldg(tb + (size_t)k * NV + rowS[rr]) : 0.f;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (i0 + 256 * j < M * rows_pad) tSb[i0 + 256 * j] = q[j];
-      }
-      cta_sync(1, 256);
-    }
-    if (warp < 4) {
+    if (tmean != nullptr) cp_async_wait_all();
+    cta_sync(1, 256);                                  // norms and text weights are in shared memory
     // ---------------- epilogue: lane = accumulator row ---------------------------------------
-    // this warp scans the lower half of the columns, its helper warp (same TMEM lanes) the
-    // upper half; the helper's list comes back through the (now idle) operand ring
+    // Warps 0-3 scan the lower half of the columns, warps 5-8 (the same TMEM lanes) the upper half, whose lists come
+    // back through the (now idle) operand ring.
     const int c_mid = ((n_pad / 16 + 1) / 2) * 16;
-    const int row = tid;                             // TMEM lane == accumulator row
-    const bool row_valid = row < w.nrows;
-    const float rs = row_valid ? rn[d.patch0 + rowS[row]] : 0.f;
+    const bool lower = warp < 4;
     float v[LCAP];
     int ix[LCAP];
-    if (acc_ok && warp * 32 < w.nrows)
-      epilogue_scan<LCAP>(tmem_base + ((uint32_t)(warp * 32) << 16), 0, c_mid,
-                          col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
-                          t_scale);
+    if (acc_ok && (warp & 3) * 32 < w.nrows)
+      epilogue_scan<LCAP>(tmem_base + ((uint32_t)((warp & 3) * 32) << 16), lower ? 0 : c_mid, lower ? c_mid : n_pad,
+                          col_begin, rs, rnT, v, ix, tSb + min(row, s_stride - 1), s_stride, tT, n_pad, M, gamma, t_scale);
     else {
 #pragma unroll
       for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
     }
-    cta_sync(1, 256);                                // helper lists are in shared memory
-    {
-      const float* hv = reinterpret_cast<const float*>(um_raw + (ring - smem_u32(um_raw)));
-      const int* hi = reinterpret_cast<const int*>(hv + UM * LCAP);
-      #pragma unroll 1                               // rolled: the body is a full insertion
-      for (int e = 0; e < L; ++e) {
-        {
-          float cv = hv[tid * LCAP + e];
-          int ci = hi[tid * LCAP + e];
-          bool shift = ci == INT_MAX;                // empty helper slot: nothing to insert
-          if (!shift) {
-            shift = false;
-#pragma unroll
-            for (int k = 0; k < LCAP; ++k)
-              if (k < L && (shift || toplist_better(cv, ci, v[k], ix[k]))) {
-                const float tv = v[k]; const int ti = ix[k];
-                v[k] = cv; ix[k] = ci; cv = tv; ci = ti;
-                shift = true;
-              }
-          }
-        }
-      }
-    }
-    if (row_valid) {
-      const size_t o = (size_t)d.part0 + ((size_t)(w.r0 + row) * d.nsplit + w.aux) * L;
-#pragma unroll
-      for (int k = 0; k < LCAP; ++k)
-        if (k < L) {
-          part_val[o + k] = v[k];
-          part_idx[o + k] = ix[k] == INT_MAX ? -1 : ix[k];
-        }
-    }
-    } else {
-    // ---------------- epilogue helpers: upper half of the columns --------------------------------
-    const int grp = warp & 3;                          // TMEM lanes this warp may read
-    const int c_mid = ((n_pad / 16 + 1) / 2) * 16;
     float* hv = reinterpret_cast<float*>(um_raw + (ring - smem_u32(um_raw)));
     int* hi = reinterpret_cast<int*>(hv + UM * LCAP);
-    const int row = grp * 32 + lane;
-    const bool row_valid = row < w.nrows;
-    const float rs = row_valid ? rn[d.patch0 + rowS[row]] : 0.f;
-    float v[LCAP];
-    int ix[LCAP];
-    if (acc_ok && grp * 32 < w.nrows)
-      epilogue_scan<LCAP>(tmem_base + ((uint32_t)(grp * 32) << 16), c_mid, n_pad,
-                          col_begin, rs, rnT, v, ix, tSb + row, rows_pad, tT, n_pad, M, gamma,
-                          t_scale);
-    else {
+    if (!lower) {
 #pragma unroll
-      for (int k = 0; k < LCAP; ++k) { v[k] = -CUDART_INF_F; ix[k] = INT_MAX; }
+      for (int k = 0; k < LCAP; ++k) { hv[row * LCAP + k] = v[k]; hi[row * LCAP + k] = ix[k]; }
     }
+    cta_sync(1, 256);                                  // helper lists are in shared memory
+    if (lower) {
+      #pragma unroll 1                               // rolled: the body is a full insertion
+      for (int e = 0; e < L; ++e) {
+        float cv = hv[row * LCAP + e];
+        int ci = hi[row * LCAP + e];
+        bool shift = ci == INT_MAX;                // empty helper slot: nothing to insert
+        if (!shift) {
 #pragma unroll
-    for (int k = 0; k < LCAP; ++k) { hv[row * LCAP + k] = v[k]; hi[row * LCAP + k] = ix[k]; }
-    cta_sync(1, 256);
+          for (int k = 0; k < LCAP; ++k)
+            if (k < L && (shift || toplist_better(cv, ci, v[k], ix[k]))) {
+              const float tv = v[k]; const int ti = ix[k];
+              v[k] = cv; ix[k] = ci; cv = tv; ci = ti;
+              shift = true;
+            }
+        }
+      }
+      if (row_valid) {
+        const size_t o = (size_t)d.part0 + ((size_t)(w.r0 + row) * d.nsplit + w.aux) * L;
+#pragma unroll
+        for (int k = 0; k < LCAP; ++k)
+          if (k < L) {
+            part_val[o + k] = v[k];
+            part_idx[o + k] = ix[k] == INT_MAX ? -1 : ix[k];
+          }
+      }
     }
   } else {
     // ---------------- MMA issuer (the whole warp, one elected lane per instruction) -------------
     const uint32_t idesc = umma_idesc_bf16(n_pad);
-    const uint32_t u_tmem = warp_uniform(tmem_base), u_ring = warp_uniform(ring);
+    const uint32_t u_tmem = warp_uniform(tmem_base);
     const uint32_t kblock_bytes = (uint32_t)stage_bytes / KSUB;
     bool m_ok = true;
     int s = 0;
@@ -440,8 +412,8 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
       tc_fence_after();
 #pragma unroll
       for (int j = 0; j < KSUB; ++j) {
-        if (j > 0 && 2 * kb + 1 >= nk) break;
-        const uint32_t a0 = u_ring + (uint32_t)s * stage_bytes + j * kblock_bytes;
+        if (j > 0 && KSUB * kb + j >= nk) break;
+        const uint32_t a0 = ring + (uint32_t)s * stage_bytes + j * kblock_bytes;
         const uint64_t ad = umma_smem_desc(a0), bd = umma_smem_desc(a0 + (uint32_t)a_bytes);
 #pragma unroll
         for (int k4 = 0; k4 < UKB / 16; ++k4) {
@@ -450,7 +422,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
         }
       }
       umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
-      if (++s == NSTAGE) { s = 0; par ^= 1u; }
+      if (++s == nstage) { s = 0; par ^= 1u; }
     }
     if (m_ok) umma_commit(&acc_bar);   // accumulator complete
     if (lane == 0) {

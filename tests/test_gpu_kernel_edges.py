@@ -78,6 +78,29 @@ def test_correlate_tiles(ctx, dim, n_src, n_tgt):
     run_v(ctx, 93, 2, n // gw, gw, dim, n_tgt)
 
 
+@pytest.mark.parametrize("n_vision,n_text,dim,keep,p", [
+    (65, 1, 64, 1, fo.Params()),                        # one k-block, one text token, one column
+    (130, 3, 1088, 17, fo.Params()),                    # 17 k-blocks: the last stage of four holds one
+    (300, 100, 512, 30, fo.Params(eps=0.5)),            # top lists of 16 entries merged over lanes and splits
+    (272, 100, 64, 271, fo.Params()),                   # one source, two splits, the most text that tiles are planned for
+], ids=["one", "last-stage", "long-lists", "one-source"])
+def test_correlate_text_weights(n_vision, n_text, dim, keep, p):
+    """FiCoCo-L tiles: odd numbers of blocks, little and much text."""
+    c = binding.Context(max_tokens=2 * (n_vision + n_text), max_dim=dim, max_batch=2, max_text=n_text, device=0)
+    try:
+        b = synth.make_l_batch(96, 2, n_vision, n_text, dim, 3, keep)
+        gaps.repair_l(b, p)
+        parity.run_and_compare_l(c, b, p, DEV, what=f"L {n_vision} + {n_text}, {dim}, keep {keep}")
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("eps,keep", [(0.998, 96), (0.9, 96), (0.9, 150)], ids=["2", "11", "16"])
+def test_lists_merged_over_splits(ctx, eps, keep):
+    """One image, whose tiles are split over many CTAs: lists of 2 to 16 entries merged by groups of lanes."""
+    run_v(ctx, 98, 1, 18, 40, 1024, keep, p=fo.Params(eps=eps))
+
+
 @pytest.mark.parametrize("batch,gh,gw,dim", [(149, 7, 7, 64), (170, 10, 10, 256), (3, 44, 44, 512)])
 def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
     """More images than SMs, and images of several pieces."""
