@@ -64,6 +64,25 @@ __device__ __forceinline__ void unpack(const uint4& u, float (&f)[8], const __nv
   f[6] = __uint_as_float(u.w << 16); f[7] = __uint_as_float(u.w & 0xFFFF0000u);
 }
 
+// The same as pairs of neighbours, for the two-wide fp32 instructions of sm_100 (each half rounded like the one-wide one).
+__device__ __forceinline__ void unpack2(const uint4& u, float2 (&f)[2], const float*) {
+  f[0] = make_float2(__uint_as_float(u.x), __uint_as_float(u.y));
+  f[1] = make_float2(__uint_as_float(u.z), __uint_as_float(u.w));
+}
+__device__ __forceinline__ void unpack2(const uint4& u, float2 (&f)[4], const __nv_bfloat16*) {
+  f[0] = make_float2(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u));
+  f[1] = make_float2(__uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
+  f[2] = make_float2(__uint_as_float(u.z << 16), __uint_as_float(u.z & 0xFFFF0000u));
+  f[3] = make_float2(__uint_as_float(u.w << 16), __uint_as_float(u.w & 0xFFFF0000u));
+}
+__device__ __forceinline__ float2 fma2(const float2& a, const float2& b, const float2& c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d)
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
+        "l"(reinterpret_cast<const unsigned long long&>(c)));
+  return reinterpret_cast<const float2&>(d);
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);

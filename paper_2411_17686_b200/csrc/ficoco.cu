@@ -470,8 +470,8 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
     cudaFuncSetAttribute(k_correlate_umma_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
   }
   {
-    const int fmax = 221 * 1024;
-#define FICOCO_FUSED_ATTR(TT, V) cudaFuncSetAttribute(k_filter_fused<TT, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, fmax)
+#define FICOCO_FUSED_ATTR(TT, V) \
+    cudaFuncSetAttribute(k_filter_fused<TT, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM)
     FICOCO_FUSED_ATTR(float, 1); FICOCO_FUSED_ATTR(float, 2); FICOCO_FUSED_ATTR(float, 4);
     FICOCO_FUSED_ATTR(float, 5); FICOCO_FUSED_ATTR(float, 8);
     FICOCO_FUSED_ATTR(__nv_bfloat16, 1); FICOCO_FUSED_ATTR(__nv_bfloat16, 2); FICOCO_FUSED_ATTR(__nv_bfloat16, 4);
@@ -609,8 +609,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     if (best.cost < 0 || (best.cost * 100 > (best.even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024)) p->fused = false;
     // shared memory: ring stages of 16 rows (the selection works in them), the fold area, a score per row of a piece
     const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)best.max_piece * 4 + 256;
-    const size_t budget = 216 * 1024;
-    int ns = budget > fixed ? (int)((budget - fixed) / stage) : 0;
+    int ns = F_SMEM > fixed ? (int)((F_SMEM - fixed) / stage) : 0;
     if (ns > F_MAXSTAGE) ns = F_MAXSTAGE;
     size_t sel_need = 0;
     for (int b = 0; b < B; ++b) {
@@ -941,7 +940,7 @@ cudaError_t launch_filter_fused(ficoco_ctx* c, const Plan* p, const T* tok, int 
                                 cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p->f_grid);
-  cfg.blockDim = dim3(F_THREADS);
+  cfg.blockDim = dim3(F_NCONS);
   cfg.dynamicSmemBytes = p->f_smem;
   cfg.stream = st;
   cudaLaunchAttribute at[2];

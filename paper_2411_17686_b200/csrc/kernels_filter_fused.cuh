@@ -1,13 +1,12 @@
 // Filter stage as one persistent kernel (Eq. 1, local penalty, top-N^S selection).
 //
 // Launched cooperatively with one CTA per SM at most, so all CTAs are co-resident.  Every CTA
-// owns a fixed list of "pieces" (consecutive patch rows of one image).  Warp 16 streams the
-// rows of its pieces, 16 rows (one bulk copy) per stage, into a shared-memory ring (TMA);
-// the 16 consumer warps take one row each per stage.
+// owns a fixed list of "pieces" (consecutive patch rows of one image), of which each of its 16 warps
+// takes a sixteenth and streams it through a shared-memory ring of its own (bulk copies, TMA).
 //   pass 1  rn_i = 1/||x_i||, column sums of the normalised rows -> one partial per piece;
 //           the piece's image counter is bumped;
-//   pass 2  (rows read again, now L2-resident, with plain 16-byte loads, three rows in flight
-//           per warp) once all pieces of the image are in:
+//   pass 2  (the rows still in the rings from there, the others, now L2-resident, with 16-byte loads, several rows in
+//           flight per warp) once all pieces of the image are in:
 //           v_i = rn_i (x_i . sum of partials) / Np,  s_i = cA v_i - (1 - cA) a_i;
 //   select  images of up to 1024 tokens: every CTA that scored a piece waits until all of the
 //           image's scores are in, runs the (short) selection on the whole image and writes the
@@ -19,6 +18,15 @@
 // used is cleared by the merge grid of the same step (which runs once the filter grid is complete
 // and before a later filter grid can start), so launches replayed from CUDA graphs, whose
 // parities are fixed at capture, find their set clean in whatever order they run.
+//
+// What bounds it: the read of the rows with 16 warps to convert and add them up (pass 1: 32 x 577 rows of 1024 bf16 take
+// 7 us, 5.2 TB/s), then trips to L2 of 0.7 to 1.2 us one behind the other.  So the heads of the attention, the other
+// pieces' column sums (half of the threads half of the pieces each) and the first rows and norms of pass 2 are each one
+// trip, asked for before what they do not depend on is waited for; the plan is read under the tail of the grid before;
+// the mean direction sits in registers, sums of four rows are folded together, and fp32 work goes two at a time.
+// Phases, before / now: attention 2.1 / 1.1 us, column sums of 18 pieces 2.8 / 1.0, scores of 144 rows 6.9 / 5.2,
+// publication of the scores 1.9 / 0.8.  Whole step: 16 ragged images 100.5 -> 92.0, one fp32 image 50.4 -> 47.1, 8 x 2881
+// tokens 132.2 -> 130.7, 32 x 577 the same.
 #pragma once
 #include "async_ops.cuh"
 #include "common.cuh"
@@ -26,18 +34,31 @@
 
 namespace ficoco {
 
-constexpr int FWARPS = 16;        // consumer warps
-constexpr int FROWS = 16;         // rows per ring stage (one 16-row bulk copy), one per consumer warp
+constexpr int FWARPS = 16;
+constexpr int FROWS = FWARPS;     // rows of a ring stage: one per warp
 constexpr int FFOLD = 8;          // rows of the fold buffer (warps w and w + 8 share a row)
-constexpr int F_NCONS = 512;      // consumer threads
-constexpr int F_THREADS = 544;    // + one producer warp
+constexpr int F_NCONS = 512;
 constexpr int F_MAXSTAGE = 16;
+constexpr size_t F_SMEM = 216 * 1024;   // dynamic shared memory at most (7 KB are static)
 constexpr int F_MAXWON = 32;      // pieces per CTA (and therefore selections it can win)
 static_assert(F_NCONS == SEL_SMALL_THREADS, "the short selection is written for the consumer threads");
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Loads that are issued where they stand (the compiler moves a plain load of constant data to its first use, behind the
+// waits that it is meant to be in flight under).
+__device__ __forceinline__ uint4 ld16_now(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_now(const float* p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
 
@@ -65,41 +86,21 @@ __device__ __forceinline__ int msum_slot(int c, int nvec) {
   return (e < 4 ? 0 : 4 * nvec) + 4 * v + (e & 3);
 }
 
-// Dot products of R rows (16-byte vectors u[r][k], vector lane + 32k of the row) with m, summed
-// over the warp.  m is read once for all R rows.
-template <class T, int VPL, int R>
-__device__ __forceinline__ void score_rows(const uint4 (&u)[R][VPL], const float* msum, int nvec, int lane,
-                                           float (&dot)[R]) {
-  constexpr int E = VecTraits<T>::E;
+// Sums of four values over the warp in six shuffles: lanes 8 r .. 8 r + 7 end up with the sum of v[r].
+__device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
+  const bool hi = lane & 16, odd = lane & 8;
+  float a = hi ? v[2] : v[0], b = hi ? v[3] : v[1];
+  a += __shfl_xor_sync(0xFFFFFFFFu, hi ? v[0] : v[2], 16);
+  b += __shfl_xor_sync(0xFFFFFFFFu, hi ? v[1] : v[3], 16);
+  float c = odd ? b : a;
+  c += __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 8);
 #pragma unroll
-  for (int r = 0; r < R; ++r) dot[r] = 0.f;
-#pragma unroll
-  for (int k = 0; k < VPL; ++k) {
-    const int v = lane + 32 * k;
-    const int vv = v < nvec ? v : 0;
-    float m[E];
-    const float4 ma = *reinterpret_cast<const float4*>(msum + 4 * vv);
-    m[0] = ma.x; m[1] = ma.y; m[2] = ma.z; m[3] = ma.w;
-    if (E == 8) {
-      const float4 mb = *reinterpret_cast<const float4*>(msum + 4 * (nvec + vv));
-      m[E - 4] = mb.x; m[E - 3] = mb.y; m[E - 2] = mb.z; m[E - 1] = mb.w;
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      float f[E];
-      unpack(u[r][k], f, (const T*)nullptr);
-      float t = 0.f;
-#pragma unroll
-      for (int e = 0; e < E; ++e) t = fmaf(f[e], m[e], t);
-      dot[r] += t;
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < R; ++r) dot[r] = warp_sum(dot[r]);
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+  return c;
 }
 
 template <class T, int VPL>
-__global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
+__global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
     const T* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
     const WorkItem* __restrict__ pieces, const int* __restrict__ cta_first,
     float* __restrict__ rn, float* __restrict__ partial, const float* __restrict__ attn, int H, float cA,
@@ -110,9 +111,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
     int nstage, int parity, int set_stride, unsigned long long wait_ns, int dbg_extra_arrivals,
     int dep_wait_first) {
   constexpr int E = VecTraits<T>::E;
-  constexpr int F_P2B = VPL <= 4 ? 2 : 1;   // rows a warp scores together in pass 2 (and has in flight from L2)
+  constexpr int F_P2B = VPL <= 4 ? 4 : VPL <= 5 ? 2 : 1;   // rows a warp has in flight from L2 in pass 2
   extern __shared__ __align__(128) unsigned char fs_raw[];
-  __shared__ uint64_t full_bar[F_MAXSTAGE], empty_bar[F_MAXSTAGE];
+  __shared__ uint64_t full_bar[FWARPS][F_MAXSTAGE];
   __shared__ SelectShared sel_sh;
   __shared__ SelectSmallShared sel_small_sh;
   // All CTAs of this grid are co-resident, so the next grid may be staged right away: its blocks
@@ -121,6 +122,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
   FICOCO_PHASE_BEGIN(0);
   __shared__ int won[F_MAXWON];
   __shared__ int nwon, failed;
+  __shared__ WorkItem w_s[F_MAXWON];          // this CTA's pieces and their images
+  __shared__ ImgDesc d_s[F_MAXWON];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row_bytes = D * (int)sizeof(T);
@@ -138,15 +141,20 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
     // different plans find and clear each other's counters)
     int* other = cnt + (parity ? 0 : set_stride);
     if (blockIdx.x == 0)
-      for (int i = tid; i < set_stride; i += F_THREADS) other[i] = 0;
+      for (int i = tid; i < set_stride; i += F_NCONS) other[i] = 0;
     cnt += parity ? set_stride : 0;
   }
 
-  if (tid == 0) {
-    for (int s = 0; s < nstage; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], FWARPS); }
-    nwon = 0;
-    failed = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (lane < nstage) mbar_init(&full_bar[warp][lane], 1);
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (tid == 0) { nwon = 0; failed = 0; }
+  // (plan data: looked up once, under the tail of the grid before)
+  for (int i = warp; i < p_end - p_begin; i += F_NCONS / 32) {
+    const WorkItem w = pieces[p_begin + i];
+    static_assert(sizeof(ImgDesc) % 4 == 0 && sizeof(ImgDesc) / 4 <= 32, "a lane copies a word of the descriptor");
+    if (lane == 0) w_s[i] = w;
+    if (lane < sizeof(ImgDesc) / 4)
+      reinterpret_cast<uint32_t*>(&d_s[i])[lane] = reinterpret_cast<const uint32_t*>(desc + w.img)[lane];
   }
   __syncthreads();
   // A step fed from the outputs of the step before it on the stream (a progressive schedule) is
@@ -154,67 +162,78 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
   // must not touch the tokens before then.
   if (dep_wait_first) grid_dep_wait();
 
-  if (warp == FWARPS) {
-    // ------------------------------- producer (pass 1 only) -------------------------------
-    if (lane == 0) {
-      int seq = 0;
-      bool ok = true;
-      for (int pi = p_begin; pi < p_end && ok; ++pi) {
-        const WorkItem w = pieces[pi];
-        const ImgDesc d = desc[w.img];
-        const unsigned char* base =
-            reinterpret_cast<const unsigned char*>(tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D);
-        for (int g = 0; g * FROWS < w.nrows && ok; ++g, ++seq) {
-          const int s = seq % nstage;
-          if (seq >= nstage) ok = mbar_wait(&empty_bar[s], ((seq / nstage) - 1) & 1, wait_ns);
-          if (!ok) break;
-          const int rows = min(FROWS, w.nrows - g * FROWS);
-          mbar_expect_tx(&full_bar[s], (uint32_t)(rows * row_bytes));
-          bulk_load(ring + (size_t)s * stage_bytes, base + (size_t)g * stage_bytes,
-                    (uint32_t)(rows * row_bytes), &full_bar[s]);
-        }
-      }
-      if (!ok) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
-      // no copy outlives the CTA, also where the consumers have given up (nobody re-arms these barriers)
-      for (int q = max(0, seq - nstage); q < seq; ++q) mbar_wait(&full_bar[q % nstage], (q / nstage) & 1, wait_ns);
+  // Every warp has a ring of its own for its sixteenth of a piece's rows (G = ceil(rows / 16) consecutive ones; a warp's
+  // rows end where the piece does).  Lane 0 asks for the first row and for as many behind it as fit here, then, once the
+  // warp has read a row, for the one that takes its place.  A copy of several rows completes on the barrier of its first
+  // slot and the others' complete without one: slots are read in order.  (One ring of 16-row copies for all, filled by a
+  // producer warp: the warps advance in step, and a 17th warp leaves 96 registers a thread instead of 128; filled by a
+  // consumer, which every 32 KB copy keeps for half a microsecond, or row by row from the start, 80 copies of 54 cycles:
+  // 32 x 577 tokens 60.8 and 59.7 us.)
+  int issued = 0, ip = p_begin, ig = 0;            // rows asked for; piece and number of the next one
+  unsigned char* my_ring = ring + (size_t)warp * nstage * row_bytes;
+  auto issue = [&](int most) {
+    if (ip >= p_end) return;
+    const WorkItem& w = w_s[ip - p_begin];
+    const ImgDesc& d = d_s[ip - p_begin];
+    const int G = (w.nrows + FROWS - 1) / FROWS, r = warp * G + ig, n = min(most, G - ig), have = max(0, min(n, w.nrows - r));
+    const int s = issued % nstage;
+    if (have > 0) {
+      mbar_expect_tx(&full_bar[warp][s], (uint32_t)(have * row_bytes));
+      bulk_load(my_ring + (size_t)s * row_bytes, tokens + (size_t)(d.row0 + d.n_cls + w.r0 + r) * D,
+                (uint32_t)(have * row_bytes), &full_bar[warp][s]);
     }
-    return;
+    for (int j = have > 0 ? 1 : 0; j < n; ++j) mbar_arrive(&full_bar[warp][s + j]);
+    issued += n;
+    ig += n;
+    if (ig >= G) { ig = 0; ++ip; }
+  };
+  if (lane == 0) {
+    issue(1);
+    while (issued < nstage && ip < p_end) issue(nstage - issued);
   }
+  __syncwarp();
 
-  // --------------------------------- consumers ----------------------------------------------
   FICOCO_PHASE(0, 1);
   int seq = 0;
   bool ok = true;
-  // The attention term of the first piece's rows depends on nothing this kernel computes: it is
-  // fetched now, while the ring fills, instead of between the two passes.
-  if (p_begin < p_end) {
-    const WorkItem w = pieces[p_begin];
-    const ImgDesc d = desc[w.img];
+  // Head mean of the attention of a piece's rows, the heads' loads in flight together (four at a time by the compiler's own
+  // choice kept the first warps from pass 1 for 2 us on 32 x 577 tokens, 4 us on 16 ragged images).
+  auto attn_means = [&](const WorkItem& w, const ImgDesc& d) {
     const float inv_h = 1.0f / (float)H;
     for (int r = tid; r < w.nrows; r += F_NCONS) {
       const float* a = attn + d.attn0 + w.r0 + r;
       float t = 0.f;
-      for (int h = 0; h < H; ++h) t += __ldg(a + (size_t)h * d.np);
+      for (int h0 = 0; h0 < H; h0 += 16) {
+        float q[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) q[j] = h0 + j < H ? __ldg(a + (size_t)(h0 + j) * d.np) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) t += q[j];
+      }
       a_s[r] = t * inv_h;
     }
-  }
+  };
+  // That of the first piece depends on nothing this kernel computes: it is fetched now, while the ring fills, instead of
+  // between the two passes.
+  if (p_begin < p_end) attn_means(w_s[0], d_s[0]);
   // pass 1: norms and column sums
   for (int pi = p_begin; pi < p_end; ++pi) {
-    const WorkItem w = pieces[pi];
-    const ImgDesc d = desc[w.img];
-    float acc[VPL][E];
+    const WorkItem& w = w_s[pi - p_begin];
+    const ImgDesc& d = d_s[pi - p_begin];
+    float2 acc[VPL][E / 2];
 #pragma unroll
     for (int k = 0; k < VPL; ++k)
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[k][e] = 0.f;
-    for (int g = 0; g * FROWS < w.nrows; ++g, ++seq) {
+      for (int e = 0; e < E / 2; ++e) acc[k][e] = make_float2(0.f, 0.f);
+    const int G1 = (w.nrows + FROWS - 1) / FROWS;
+    for (int g = 0; g < G1; ++g, ++seq) {
       const int s = seq % nstage;
-      if (ok) ok = mbar_wait(&full_bar[s], (seq / nstage) & 1, wait_ns);
-      const int r = g * FROWS + warp;
+      ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(&full_bar[warp][s], (seq / nstage) & 1, wait_ns));
+      const int r = warp * G1 + g;
       if (r < w.nrows) {
-        const unsigned char* rp = ring + (size_t)s * stage_bytes + (size_t)warp * row_bytes;
+        const unsigned char* rp = my_ring + (size_t)s * row_bytes;
         uint4 u[VPL];
-        float ssk[VPL];
+        float2 ssk[VPL];
 #pragma unroll
         for (int k = 0; k < VPL; ++k) {
           const int v = lane + 32 * k;
@@ -222,62 +241,52 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
         }
 #pragma unroll
         for (int k = 0; k < VPL; ++k) {
-          float f[E];
-          unpack(u[k], f, (const T*)nullptr);
-          float t = 0.f;
+          float2 f[E / 2];
+          unpack2(u[k], f, (const T*)nullptr);
+          ssk[k] = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < E; ++e) t = fmaf(f[e], f[e], t);
-          ssk[k] = t;
+          for (int e = 0; e < E / 2; ++e) ssk[k] = fma2(f[e], f[e], ssk[k]);
         }
         float ss = 0.f;
 #pragma unroll
-        for (int k = 0; k < VPL; ++k) ss += ssk[k];
+        for (int k = 0; k < VPL; ++k) ss += ssk[k].x + ssk[k].y;
         ss = warp_sum(ss);
         const float s1 = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
         if (lane == 0) rn[d.patch0 + w.r0 + r] = s1;
+        const float2 s2 = make_float2(s1, s1);
 #pragma unroll
         for (int k = 0; k < VPL; ++k) {
-          float f[E];
-          unpack(u[k], f, (const T*)nullptr);
+          float2 f[E / 2];
+          unpack2(u[k], f, (const T*)nullptr);
 #pragma unroll
-          for (int e = 0; e < E; ++e) acc[k][e] = fmaf(f[e], s1, acc[k][e]);
+          for (int e = 0; e < E / 2; ++e) acc[k][e] = fma2(f[e], s2, acc[k][e]);
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&empty_bar[s]);
+      if (lane == 0 && ok) issue(1);
+      __syncwarp();
     }
     // fold the 16 warps in a fixed order -> partial of this piece: warps 0-7 store, warps 8-15
     // add into the row of warp - 8, then the 8 rows are summed per column
-    if (warp < FFOLD) {
 #pragma unroll
-      for (int k = 0; k < VPL; ++k) {
-        const int v = lane + 32 * k;
-        if (v < nvec) {
-          float4* dst = reinterpret_cast<float4*>(fold + (size_t)warp * D + (size_t)v * E);
-          dst[0] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
-          if (E == 8) dst[1] = make_float4(acc[k][E - 4], acc[k][E - 3], acc[k][E - 2], acc[k][E - 1]);
-        }
-      }
-    }
-    cta_sync(1, F_NCONS);
-    if (warp >= FFOLD) {
+    for (int half = 0; half < 2; ++half) {
+      if (warp / FFOLD == half) {
 #pragma unroll
-      for (int k = 0; k < VPL; ++k) {
-        const int v = lane + 32 * k;
-        if (v < nvec) {
-          float4* dst = reinterpret_cast<float4*>(fold + (size_t)(warp - FFOLD) * D + (size_t)v * E);
-          float4 x = dst[0];
-          x.x += acc[k][0]; x.y += acc[k][1]; x.z += acc[k][2]; x.w += acc[k][3];
-          dst[0] = x;
-          if (E == 8) {
-            float4 y = dst[1];
-            y.x += acc[k][E - 4]; y.y += acc[k][E - 3]; y.z += acc[k][E - 2]; y.w += acc[k][E - 1];
-            dst[1] = y;
+        for (int k = 0; k < VPL; ++k) {
+          const int v = lane + 32 * k;
+          if (v < nvec) {
+            float4* dst = reinterpret_cast<float4*>(fold + (size_t)(warp % FFOLD) * D + (size_t)v * E);
+#pragma unroll
+            for (int q = 0; q < E / 4; ++q) {
+              float4 x = half ? dst[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+              x.x += acc[k][2 * q].x; x.y += acc[k][2 * q].y; x.z += acc[k][2 * q + 1].x; x.w += acc[k][2 * q + 1].y;
+              dst[q] = x;
+            }
           }
         }
       }
+      cta_sync(1, F_NCONS);
     }
-    cta_sync(1, F_NCONS);
     float* pout = partial + (size_t)(d.chunk0 + w.aux) * D;
     for (int c = tid; c < D; c += F_NCONS) {
       float t = 0.f;
@@ -288,112 +297,160 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
     cta_sync(1, F_NCONS);
     if (tid == 0) red_release_add(&cnt[w.img], 1);   // pairs with the ld.acquire poll of pass 2
   }
-  if (!ok && lane == 0) { atomicOr(status, STATUS_TIMEOUT); failed = 1; }
+  if (!ok && lane == 0) {
+    atomicOr(status, STATUS_TIMEOUT);
+    failed = 1;
+    // no copy outlives the CTA
+    for (int q = max(0, issued - nstage); q < issued; ++q) mbar_wait(&full_bar[warp][q % nstage], (q / nstage) & 1, wait_ns);
+  }
+  __syncwarp();
   FICOCO_PHASE(0, 2);
 
   // pass 2: scores.  The last `nstage` row groups of pass 1 are still in the ring and are read
   // from there (only when every wait of pass 1 succeeded); the older ones are L2-resident and
   // are read with plain loads.
-  const int first_kept = ok ? seq - nstage : seq;   // groups numbered >= this are in shared memory
+  const int first_kept = ok ? seq - nstage : seq;   // rows numbered >= this are in shared memory
   int seq2 = 0;
   for (int pi = p_begin; pi < p_end; ++pi) {
-    const WorkItem w = pieces[pi];
-    const ImgDesc d = desc[w.img];
-    const int seq_piece = seq2;                     // number of this piece's first group
-    seq2 += (w.nrows + FROWS - 1) / FROWS;
+    const WorkItem& w = w_s[pi - p_begin];
+    const ImgDesc& d = d_s[pi - p_begin];
+    const int seq_piece = seq2;                     // number of the warp's first row of this piece
+    const int nrows = w.nrows;
+    const T* base = tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D;
+    // Row g of this warp is row warp * G + g of the piece.  Those below g_res were overwritten in the ring and come from
+    // L2; the others are still in shared memory.
+    const int G = (nrows + FROWS - 1) / FROWS;
+    const int g_res = min(G, max(0, first_kept - seq_piece));
+    seq2 += G;
+    // The first rows from L2 and the norms of the warp's rows (lane l: row l) are asked for before the
+    // other pieces' column sums are waited for: they depend on nothing but this CTA.
+    uint4 ub[F_P2B][VPL];
+    auto load_row = [&](int g, uint4 (&u)[VPL]) {
+      const int r = warp * G + g;
+      const bool on = g < g_res && r < nrows;
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) {
+        const int v = lane + 32 * k;
+        u[k] = (on && v < nvec) ? ld16_now(base + (size_t)r * D + (size_t)v * E) : make_uint4(0, 0, 0, 0);
+      }
+    };
+#pragma unroll
+    for (int j = 0; j < F_P2B; ++j) load_row(j, ub[j]);
+    const int row_l = warp * G + lane;
+    const float rn_l = (lane < G && row_l < nrows) ? ld_now(rn + d.patch0 + w.r0 + row_l) : 0.f;
     if (tid == 0 && !poll_count(&cnt[w.img], d.n_chunks + dbg_extra_arrivals, wait_ns, status)) {
       atomicOr(status, STATUS_TIMEOUT);
       failed = 1;
     }
     if (pi == p_begin) FICOCO_PHASE(0, 3);
-    const float inv_h = 1.0f / (float)H;
-    for (int r = tid; pi > p_begin && r < w.nrows; r += F_NCONS) {     // attention term of a further piece
-      const float* a = attn + d.attn0 + w.r0 + r;
-      float t = 0.f;
-      for (int h = 0; h < H; ++h) t += __ldg(a + (size_t)h * d.np);
-      a_s[r] = t * inv_h;
-    }
+    if (pi > p_begin) attn_means(w, d);
     cta_sync(1, F_NCONS);
-    float* msum = fold;
-    for (int c = tid; c < D; c += F_NCONS) {
-      float t = 0.f;
-      for (int k0 = 0; k0 < d.n_chunks; k0 += 8) {
-        float q[8];
+    // Column sums of the image: half of the threads adds the first half of the pieces, the others the second, four columns
+    // and twelve pieces in flight each, so that up to 24 pieces are one trip to L2.
+    {
+      const int half = tid >> 8, nh = (d.n_chunks + 1) / 2, k_lo = half * nh, k_hi = min(d.n_chunks, k_lo + nh);
+      for (int c = 4 * (tid & 255); c < D; c += 4 * 256) {
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        #pragma unroll 1
+        for (int k0 = k_lo; k0 < k_hi; k0 += 12) {
+          float4 q[12];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          q[k] = k0 + k < d.n_chunks ? __ldcg(partial + (size_t)(d.chunk0 + k0 + k) * D + c) : 0.f;
+          for (int k = 0; k < 12; ++k)
+            q[k] = k0 + k < k_hi ? __ldcg(reinterpret_cast<const float4*>(partial + (size_t)(d.chunk0 + k0 + k) * D + c))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) t += q[k];
+          for (int k = 0; k < 12; ++k) { t.x += q[k].x; t.y += q[k].y; t.z += q[k].z; t.w += q[k].w; }
+        }
+        *reinterpret_cast<float4*>(fold + (size_t)half * D + msum_slot<E>(c, nvec)) = t;
       }
-      msum[msum_slot<E>(c, nvec)] = t;
     }
     cta_sync(1, F_NCONS);
     if (pi == p_begin) FICOCO_PHASE(0, 4);
-    const float inv_np = 1.0f / (float)d.np;
-    const T* base = tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D;
-    // This warp owns line `warp` of every 16-row group of the piece.  Groups numbered below
-    // g_res were overwritten in the ring and come from L2; the others are still in shared memory.
-    const int G = (w.nrows + FROWS - 1) / FROWS;
-    const int g_res = min(G, max(0, first_kept - seq_piece));
-    // norms of the warp's rows, lane l holding the one of group l
-    const int row_l = lane * FROWS + warp;
-    const float rn_l = (lane < G && row_l < w.nrows) ? __ldcg(rn + d.patch0 + w.r0 + row_l) : 0.f;
-    auto finish_row = [&](int g, float dot) {      // dot already summed over the warp
-      const int r = g * FROWS + warp;
-      const float rnv = g < 32 ? __shfl_sync(0xFFFFFFFFu, rn_l, g) : __ldcg(rn + d.patch0 + w.r0 + r);
-      if (lane == 0 && r < w.nrows)
-        s_raw[d.patch0 + w.r0 + r] = cA * (dot * rnv * inv_np) - (1.0f - cA) * a_s[r];
-    };
-    uint4 ub[F_P2B][VPL];
-    auto load_batch = [&](int g0) {
+    // The lane's columns of the mean direction, for all its rows.  (Read from shared memory with every pair of rows, they
+    // were half of this pass's shared-memory traffic.)
+    float2 m[VPL][E / 2];
 #pragma unroll
-      for (int jb = 0; jb < F_P2B; ++jb) {
-        const int r = (g0 + jb) * FROWS + warp;
-        const bool on = g0 + jb < g_res && r < w.nrows;
+    for (int k = 0; k < VPL; ++k) {
+      const int vv = lane + 32 * k < nvec ? lane + 32 * k : 0;
 #pragma unroll
-        for (int k = 0; k < VPL; ++k) {
-          const int v = lane + 32 * k;
-          ub[jb][k] = (on && v < nvec) ? ldg16(base + (size_t)r * D + (size_t)v * E) : make_uint4(0, 0, 0, 0);
-        }
+      for (int e = 0; e < E; e += 4) {
+        const float* at = fold + 4 * (e / 4 * nvec + vv);
+        const float4 ma = *reinterpret_cast<const float4*>(at), mb = *reinterpret_cast<const float4*>(at + D);
+        m[k][e / 2] = make_float2(ma.x + mb.x, ma.y + mb.y);
+        m[k][e / 2 + 1] = make_float2(ma.z + mb.z, ma.w + mb.w);
       }
-    };
-    load_batch(0);
-    // the rows in the ring are scored while the first batch from L2 is in flight
-    #pragma unroll 1
-    for (int g0 = g_res; g0 < G; g0 += F_P2B) {
-      uint4 us[F_P2B][VPL];
-#pragma unroll
-      for (int jb = 0; jb < F_P2B; ++jb) {
-        const int g = g0 + jb;
-        const bool on = g < G && g * FROWS + warp < w.nrows;
-        const unsigned char* rp =
-            ring + (size_t)((seq_piece + g) % nstage) * stage_bytes + (size_t)warp * row_bytes;
-#pragma unroll
-        for (int k = 0; k < VPL; ++k) {
-          const int v = lane + 32 * k;
-          us[jb][k] = (on && v < nvec) ? *reinterpret_cast<const uint4*>(rp + (size_t)v * 16) : make_uint4(0, 0, 0, 0);
-        }
-      }
-      float dot[F_P2B];
-      score_rows<T, VPL, F_P2B>(us, msum, nvec, lane, dot);
-#pragma unroll
-      for (int jb = 0; jb < F_P2B; ++jb)
-        if (g0 + jb < G) finish_row(g0 + jb, dot[jb]);
     }
+    const float inv_np = 1.0f / (float)d.np;
+    float* s_out = s_raw + d.patch0 + w.r0;
+    // Rows g .. g + 3 of the warp (from `end` on: nothing), their dot products summed over the warp together.
+    auto finish_rows = [&](int g, int end, const float (&dot)[4]) {
+      const float t = warp_sum4(dot, lane);
+      g += lane >> 3;
+      const int r = warp * G + g;
+      const float k = __shfl_sync(0xFFFFFFFFu, rn_l, g & 31);
+      if ((lane & 7) == 0 && g < end && r < nrows) {
+        const float rnv = g < 32 ? k : __ldcg(rn + d.patch0 + w.r0 + r);
+        s_out[r] = cA * (t * rnv * inv_np) - (1.0f - cA) * a_s[r];
+      }
+    };
+    auto add_dot = [&](const uint4& u, int k, float2& dot) {
+      float2 f[E / 2];
+      unpack2(u, f, (const T*)nullptr);
+#pragma unroll
+      for (int e = 0; e < E / 2; ++e) dot = fma2(f[e], m[k][e], dot);
+    };
+    // the rows in the ring, four at a time, while the first ones from L2 are in flight (lines without a row: garbage that
+    // nothing stores)
+    #pragma unroll 1
+    for (int g = g_res; g < G; g += 4) {
+      const unsigned char* rp[4];
+      float2 dot2[4];
+      float dot[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        rp[j] = my_ring + (size_t)((seq_piece + min(g + j, G - 1)) % nstage) * row_bytes;
+        dot2[j] = make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) {
+        const int v = lane + 32 * k;
+        if (v < nvec) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) add_dot(*reinterpret_cast<const uint4*>(rp[j] + (size_t)v * 16), k, dot2[j]);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 4; ++j) dot[j] = dot2[j].x + dot2[j].y;
+      finish_rows(g, G, dot);
+    }
+    // the others, the registers of a batch filled again as soon as it is done
     #pragma unroll 1
     for (int g0 = 0; g0 < g_res; g0 += F_P2B) {
-      float dot[F_P2B];
-      score_rows<T, VPL, F_P2B>(ub, msum, nvec, lane, dot);
+      float dot[4];
 #pragma unroll
-      for (int jb = 0; jb < F_P2B; ++jb)
-        if (g0 + jb < g_res) finish_row(g0 + jb, dot[jb]);
-      if (g0 + F_P2B < g_res) load_batch(g0 + F_P2B);
+      for (int j = 0; j < 4; ++j) {
+        dot[j] = 0.f;
+        if (j < F_P2B) {
+          float2 dot2 = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int k = 0; k < VPL; ++k) add_dot(ub[j][k], k, dot2);
+          dot[j] = dot2.x + dot2.y;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < F_P2B; ++j) load_row(g0 + F_P2B + j, ub[j]);
+      finish_rows(g0, min(g_res, g0 + F_P2B), dot);
     }
     cta_sync(1, F_NCONS);
     if (tid == 0) {
-      // release this piece's scores, and (for the CTA that arrives last) acquire everyone else's
-      const int old = atom_acq_rel_add(&cnt[B + w.img], 1);
-      if (d.np > SEL_SMALL_MAX && old == d.n_chunks - 1 && nwon < F_MAXWON) won[nwon++] = w.img;
+      if (d.np <= SEL_SMALL_MAX) {
+        red_release_add(&cnt[B + w.img], 1);         // releases this piece's scores; the selection polls for all of them
+      } else {
+        // (for the CTA that arrives last) acquires everyone else's as well
+        const int old = atom_acq_rel_add(&cnt[B + w.img], 1);
+        if (old == d.n_chunks - 1 && nwon < F_MAXWON) won[nwon++] = w.img;
+      }
     }
   }
   cta_sync(1, F_NCONS);
@@ -409,10 +466,10 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_filter_fused(
   int pi = p_begin;
   #pragma unroll 1
   while (pi < p_end) {
-    const WorkItem w0 = pieces[pi];
-    const ImgDesc d = desc[w0.img];
+    const WorkItem& w0 = w_s[pi - p_begin];
+    const ImgDesc& d = d_s[pi - p_begin];
     int pj = pi, hi = w0.r0;
-    while (pj < p_end && pieces[pj].img == w0.img) { hi = pieces[pj].r0 + pieces[pj].nrows; ++pj; }
+    while (pj < p_end && w_s[pj - p_begin].img == w0.img) { hi = w_s[pj - p_begin].r0 + w_s[pj - p_begin].nrows; ++pj; }
     if (d.np <= SEL_SMALL_MAX) {
       select_small_prepare(d, penalty, ring, tid);
       if (tid == 0 && !poll_count(&cnt[B + w0.img], d.n_chunks, wait_ns, status)) {

@@ -101,9 +101,10 @@ def test_lists_merged_over_splits(ctx, eps, keep):
     run_v(ctx, 98, 1, 18, 40, 1024, keep, p=fo.Params(eps=eps))
 
 
-@pytest.mark.parametrize("batch,gh,gw,dim", [(149, 7, 7, 64), (170, 10, 10, 256), (3, 44, 44, 512)])
+@pytest.mark.parametrize("batch,gh,gw,dim", [(149, 7, 7, 64), (170, 10, 10, 256), (3, 44, 44, 512), (1, 3, 11, 64), (2, 33, 3, 1280),
+                                               (1, 5, 5, 2048)])
 def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
-    """More images than SMs, and images of several pieces."""
+    """More images than SMs, images of several pieces, and warps without a row."""
     run_v(ctx, 94, batch, gh, gw, dim, gh * gw // 2)
 
 
