@@ -456,7 +456,8 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   c->plan_slots = b + o_pl;
 
   // kernels that may need more than 48 KB of dynamic shared memory
-  cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaFuncSetAttribute(k_select<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaFuncSetAttribute(k_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   {
     const int um_smem_max = 221 * 1024;
 #define FICOCO_UMMA_ATTR(LC)                                                                                  \
@@ -1062,17 +1063,13 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
         tok, D, p->d_desc, p->d_rows, c->rn, c->msum, attn, attn_rows, cA, c->s_raw);
   c->launches += 2;
   }
-  size_t sel_smem = select_work_bytes(p->max_np, penalty ? p->max_nwin_cells : 0) + 16;
-  if (p->max_np <= SEL_SMALL_MAX) {
-    const size_t small = select_small_bytes(p->max_np, penalty ? p->max_nwin_cells : 0) + 16;
-    if (small > sel_smem) sel_smem = small;
-  }
+  const int sel_cells = penalty ? p->max_nwin_cells : 0;
+  const size_t small_smem = select_small_bytes(std::min(p->max_np, SEL_SMALL_MAX), sel_cells) + 16;
+  const size_t sel_smem = p->max_np <= SEL_SMALL_MAX ? small_smem : std::max(small_smem, select_work_bytes(p->max_np, sel_cells) + 16);
   prof_tick(c, st, "select");
-  // images of up to 1024 tokens: half the threads (two tokens each), cheaper barriers
-  launch_dependent(k_select, dim3(p->key.batch), p->max_np <= 1024 ? 512 : 1024, sel_smem, st,
-      p->d_desc, c->s_raw, pos, window, coef, penalty,
-                                                  c->s_pen, scores_out, c->S_idx, c->T_idx, kept_idx,
-                                                  pos_out, c->status);
+  launch_dependent(p->max_np <= SEL_SMALL_MAX ? k_select<true> : k_select<false>, dim3(p->key.batch), SEL_THREADS, sel_smem,
+                   st, p->d_desc, c->s_raw, pos, window, coef, penalty, c->s_pen, scores_out, c->S_idx, c->T_idx, kept_idx,
+                   pos_out, c->status);
   c->launches += 1;
   }
   if (p->n_corr > 0) {

@@ -4,6 +4,7 @@
 // reads its plan entries, which are constants, then waits for that grid to be complete and only then lets the next
 // one in.  A grid that runs therefore finds everything before its predecessor complete as well.
 #pragma once
+#include <math_constants.h>
 #include "async_ops.cuh"
 #include "common.cuh"
 
@@ -634,186 +635,298 @@ __device__ __forceinline__ void settle_cells(Cell* cell, int cells, const float*
   } while (cta_sync_or(bar, nthr, again));
 }
 
+// Token whose score is largest in window `wdx` of `nwc` per grid row (lower token index on equal scores), -1: none alive.
+// cell: token of every grid cell, NONE where there is none; sc: scores.
+template <class Cell, Cell NONE>
+__device__ __forceinline__ int window_best(const Cell* cell, const float* sc, int gh, int gw, int window, int nwc, int wdx) {
+  const int r0 = (wdx / nwc) * window, c0 = (wdx % nwc) * window;
+  int best = -1;
+  float bs = 0.f;
+  if (window == 2) {                               // the four cells and their scores as two trips, not eight
+    Cell t[4];
+    float v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = r0 + (j >> 1), c = c0 + (j & 1);
+      t[j] = r < gh && c < gw ? cell[r * gw + c] : NONE;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = t[j] != NONE ? sc[t[j]] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (t[j] != NONE && (best < 0 || v[j] > bs || (v[j] == bs && (int)t[j] < best))) { best = t[j]; bs = v[j]; }
+    return best;
+  }
+  const int r1 = min(gh, r0 + window), c1 = min(gw, c0 + window);
+  #pragma unroll 1
+  for (int r = r0; r < r1; ++r)
+    #pragma unroll 1
+    for (int c = c0; c < c1; ++c) {
+      const Cell t = cell[r * gw + c];
+      if (t == NONE) continue;
+      const float v = sc[t];
+      if (best < 0 || v > bs || (v == bs && (int)t < best)) { best = t; bs = v; }
+    }
+  return best;
+}
+
 // ---------------------------------------------------------------------------------------
-// Local penalty + top-N^S selection of one image by 512 or 1024 threads (tid 0..nthr-1) that
-// synchronise on hardware barrier `bar`.
+// Local penalty + top-N^S selection of one image by 512 threads (hardware barrier `bar`).
 //   1. a grid-cell -> token map lets one thread per window pick the window's maximum (lower token index on
 //      equal scores) and multiply it in place;
-//   2. a search over the value range finds the threshold (select_threshold); ties at it go to the lower index;
+//   2. a histogram of the scores over SEL_BINS equal parts of their range finds the part that the threshold lies in (a
+//      few tokens of thousands); its tokens, listed, are ranked among themselves.  Where they are more than the list
+//      takes (scores that are mostly equal, or not finite), a search over the value range takes over;
+//      ties at the threshold go to the lower index;
 //   3. ballots and one scan turn the membership flags into ascending index lists S and T, the kept
 //      row indices and the surviving grid positions.
-// What bounds it is the chain of barriers, not the work.  (Bids for the windows by 64-bit shared-memory maxima, a
-// radix select and runs of tokens per thread: the filter of 16 ragged images of up to 4096 tokens took 60 us, now 56.)
-// The code runs once per image, so it is kept compact (rolled loops, not inlined): a long
-// unrolled body would be paid for in instruction-cache misses.
-// `work` is a shared-memory area of select_work_bytes(np, cells) bytes: the scores and grid
-// positions are read from global memory once and kept there with the keys and the cell map.
+// Only the outputs of tokens w_lo <= i < w_hi are written (plus the CLS / trailing entries of kept_idx when w_lo == 0), so
+// the CTAs that scored an image can each run the selection and write their own slice.  select_image_prepare() clears the
+// work area; a barrier (or any inter-CTA wait that ends in one) must separate it from select_image().
+// What bounds it is the chain of barriers and shared-memory trips, and instruction fetch, as the code runs once: loops are
+// rolled (eight tokens per thread in registers, everything unrolled: 13 us).  2880 tokens, on the CTA that scored the image's last
+// piece alone and with sixteen keys per thread in a search of the value range: 17.6 us, of which threshold 6.5, keys 3.6,
+// windows 2.0, lists 3.2; now 11 (whole step of 8 x 2881 tokens 130.7 -> 123 us, 16 ragged images 92 -> 85.5).
 // ---------------------------------------------------------------------------------------
+constexpr int SEL_THREADS = 512;
+constexpr int SEL_BINS = 4 * SEL_THREADS;
+constexpr int SEL_LIST = 512;      // tokens of one part that are ranked among themselves
+
 __host__ __device__ inline size_t select_work_bytes(int np, int cells) {
-  return (size_t)np * 12 + (size_t)cells * 2 + 32;
+  return (size_t)np * 4 + 16 + SEL_BINS * sizeof(int) + (size_t)cells * 2 + 64;
 }
 
 struct SelectShared {
   int group[MAX_IMG_TOKENS / 32];
+  uint32_t list[SEL_LIST];
+  uint32_t wmin[16], wmax[16];
+  int wsum[16];
   int cnt[192];
-  uint32_t wmin[32], wmax[32];
+  int n_list, part, rest, in_part, need_eq;
+  uint32_t thr;
 };
+
+struct SelectWork {
+  float* sc;             // [np] scores (penalised in place)
+  int* hist;             // [SEL_BINS]
+  unsigned short* cell;  // [gh * gw] token of every grid cell, 0xFFFF: none
+};
+__device__ __forceinline__ SelectWork select_layout(unsigned char* work, int np) {
+  SelectWork w;
+  w.sc = reinterpret_cast<float*>(work);
+  w.hist = reinterpret_cast<int*>((reinterpret_cast<uintptr_t>(work + (size_t)np * 4) + 15) & ~(uintptr_t)15);
+  w.cell = reinterpret_cast<unsigned short*>(w.hist + SEL_BINS);
+  return w;
+}
+
+__device__ __forceinline__ void select_image_prepare(const ImgDesc& d, int penalty, unsigned char* work, SelectShared& sh, int tid) {
+  const SelectWork w = select_layout(work, d.np);
+  *reinterpret_cast<int4*>(w.hist + 4 * tid) = make_int4(0, 0, 0, 0);
+  if (tid == 0) sh.n_list = 0;
+  if (penalty) {
+    const int cells = d.gh * d.gw;
+    #pragma unroll 1
+    for (int i = tid; i < cells; i += SEL_THREADS) w.cell[i] = 0xFFFFu;
+  }
+}
+
+// Threshold by a search over the value range, for images whose scores are mostly equal or not finite.
+__device__ __noinline__ void select_threshold_search(const float* sc, int np, int k, uint32_t kmin, uint32_t kmax,
+                                                     SelectShared& sh, int tid, int bar) {
+  constexpr int KPT = MAX_IMG_TOKENS / SEL_THREADS;
+  uint32_t key[KPT], thr;
+  int need_eq;
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) key[q] = tid + SEL_THREADS * q < np ? max(1u, order_key(sc[tid + SEL_THREADS * q] + 0.0f)) : 0u;
+  select_threshold<KPT>(key, k, kmin, kmax, sh.cnt, tid, SEL_THREADS, bar, thr, need_eq);
+  if (tid == 0) {
+    sh.thr = need_eq < 0 ? thr - 1u : thr;         // all keys > thr - 1, none at the threshold
+    sh.need_eq = max(need_eq, 0);
+  }
+  cta_sync(bar, SEL_THREADS);
+}
 
 __device__ __noinline__ void select_image(
     const ImgDesc& d, const float* s_raw, const int* __restrict__ pos, int window, float coef,
     int penalty, float* __restrict__ s_pen, float* __restrict__ scores_out, int* __restrict__ S_idx,
     int* __restrict__ T_idx, int* __restrict__ kept_idx, int* __restrict__ pos_out,
-    unsigned* __restrict__ status, unsigned char* work, SelectShared& sh, int tid, int nthr, int bar) {
-  constexpr int KPT = MAX_IMG_TOKENS / 512;      // keys a thread holds in the threshold search
+    unsigned* __restrict__ status, unsigned char* work, SelectShared& sh, int tid, int bar, int w_lo, int w_hi) {
+  constexpr int NT = SEL_THREADS;
   const int np = d.np, lane = tid & 31, warp = tid >> 5;
-  uint32_t* keys = reinterpret_cast<uint32_t*>(work);
-  float* sc = reinterpret_cast<float*>(work + (size_t)np * 4);
-  int* pp = reinterpret_cast<int*>(work + (size_t)np * 8);
-  unsigned short* cell = reinterpret_cast<unsigned short*>(work + (size_t)np * 12);   // [gh * gw] token, 0xFFFF: none
-  const int cells = penalty ? d.gh * d.gw : 0;
-
+  const SelectWork wk = select_layout(work, np);
+  float* sc = wk.sc;
+  const int cells = d.gh * d.gw;
   #pragma unroll 1
-  for (int i = tid; i < cells; i += nthr) cell[i] = 0xFFFFu;
-  if (penalty) cta_sync(bar, nthr);
-  #pragma unroll 1
-  for (int i0 = tid; i0 < np; i0 += 4 * nthr) {    // four tokens' loads in flight per thread
-    float a[4];
-    int q[4];
+  for (int i0 = tid; i0 < np; i0 += 8 * NT) {      // eight tokens' loads in flight per thread
+    float a[8];
+    int p[8];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = i0 + j * nthr;
+    for (int j = 0; j < 8; ++j) {
+      const int i = i0 + NT * j;
       a[j] = i < np ? __ldcg(s_raw + d.patch0 + i) : 0.f;
-      q[j] = (i < np && pos) ? pos[d.patch0 + i] : i;
+      p[j] = i < np && pos ? pos[d.patch0 + i] : i;
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = i0 + j * nthr;
-      if (i >= np) continue;
+    for (int j = 0; j < 8; ++j) {
+      const int i = i0 + NT * j;
+      if (i >= np) break;
       sc[i] = a[j];
-      pp[i] = q[j];
       if (penalty) {
-        if (q[j] >= 0 && q[j] < cells) cell[q[j]] = (unsigned short)i;
+        if (p[j] >= 0 && p[j] < cells) wk.cell[p[j]] = (unsigned short)i;
         else atomicOr(status, STATUS_POS_RANGE);
       }
     }
   }
-  cta_sync(bar, nthr);
+  cta_sync(bar, NT);
 
   // ---- local penalty: one thread per window ------------------------------------------------
   if (penalty) {
-    if (pos) settle_cells(cell, cells, sc, [&](int i, int) { return pp[i]; }, np, tid, nthr, bar);
+    if (pos) settle_cells(wk.cell, cells, sc, [&](int i, int) { return pos[d.patch0 + i]; }, np, tid, NT, bar);
     const int nwc = (d.gw + window - 1) / window, nwr = (d.gh + window - 1) / window;
     #pragma unroll 1
-    for (int wdx = tid; wdx < nwc * nwr; wdx += nthr) {
-      const int r0 = (wdx / nwc) * window, c0 = (wdx % nwc) * window;
-      const int r1 = min(d.gh, r0 + window), c1 = min(d.gw, c0 + window);
-      int best = -1;
-      float bs = 0.f;
-      #pragma unroll 1
-      for (int r = r0; r < r1; ++r)
-        #pragma unroll 1
-        for (int c = c0; c < c1; ++c) {
-          const int t = cell[r * d.gw + c];
-          if (t == 0xFFFF) continue;
-          const float v = sc[t];
-          if (best < 0 || v > bs || (v == bs && t < best)) { best = t; bs = v; }
-        }
-      if (best >= 0) sc[best] = bs * coef;         // windows are disjoint: nobody else touches this token
+    for (int wdx = tid; wdx < nwc * nwr; wdx += NT) {
+      const int best = window_best<unsigned short, 0xFFFFu>(wk.cell, sc, d.gh, d.gw, window, nwc, wdx);
+      if (best >= 0) sc[best] *= coef;               // windows are disjoint: nobody else touches this token
     }
-    cta_sync(bar, nthr);
+    cta_sync(bar, NT);
   }
 
-  // ---- keys and their range ----------------------------------------------------------------
-  uint32_t key[KPT];
+  // ---- range of the keys -------------------------------------------------------------------
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-#pragma unroll
-  for (int q = 0; q < KPT; ++q) {
-    const int i = tid + nthr * q;
-    key[q] = 0u;                                   // (behind the image: never counted, thresholds are > 0)
-    if (i < np) {
-      const float s = sc[i] + 0.0f;                // -0 and +0 are one score
+  #pragma unroll 2
+  for (int i = tid; i < np; i += NT) {
+    const float s = sc[i] + 0.0f;                  // -0 and +0 are one score
+    if (i >= w_lo && i < w_hi) {
       s_pen[d.patch0 + i] = s;
       if (scores_out) scores_out[d.patch0 + i] = s;
-      key[q] = max(1u, order_key(s));
-      keys[i] = key[q];
-      kmin = min(kmin, key[q]);
-      kmax = max(kmax, key[q]);
     }
+    const uint32_t key = max(1u, order_key(s));
+    kmin = min(kmin, key);
+    kmax = max(kmax, key);
   }
-  kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
-  kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
-  if (lane == 0) { sh.wmin[warp] = kmin; sh.wmax[warp] = kmax; }
-  cta_sync(bar, nthr);
   const int k = d.n_src;
   uint32_t thr = 0;       // threshold key
-  int need_eq = -1;       // how many keys equal to thr are selected (lowest indices); -1: all
+  int need_eq = 0;        // how many keys equal to thr are selected (lowest indices)
   if (k > 0 && k < np) {
-    kmin = __reduce_min_sync(0xFFFFFFFFu, lane < (nthr >> 5) ? sh.wmin[lane] : 0xFFFFFFFFu);
-    kmax = __reduce_max_sync(0xFFFFFFFFu, lane < (nthr >> 5) ? sh.wmax[lane] : 0u);
-    select_threshold<KPT>(key, k, kmin, kmax, sh.cnt, tid, nthr, bar, thr, need_eq);
+    kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
+    kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
+    if (lane == 0) { sh.wmin[warp] = kmin; sh.wmax[warp] = kmax; }
+    cta_sync(bar, NT);
+    kmin = __reduce_min_sync(0xFFFFFFFFu, sh.wmin[lane & 15]);
+    kmax = __reduce_max_sync(0xFFFFFFFFu, sh.wmax[lane & 15]);
+    // ---- histogram over the value range (the part of a score does not fall as the score rises) ----
+    const float lo = key_score(kmin), range = key_score(kmax) - lo;
+    const float scale = range > 0.f && range < CUDART_MAX_NORMAL_F ? (float)(SEL_BINS - 1) / range : 0.f;
+    auto part_of = [&](float s) { return max(0, min(SEL_BINS - 1, (int)__fmul_rn(__fsub_rn(s + 0.0f, lo), scale))); };
+    #pragma unroll 2
+    for (int i = tid; i < np; i += NT) atomicAdd(&wk.hist[part_of(sc[i])], 1);
+    cta_sync(bar, NT);
+    // thread t: parts SEL_BINS - 1 - 4 t and the three below; running counts from the top
+    const int4 h4 = *reinterpret_cast<const int4*>(wk.hist + SEL_BINS - 4 - 4 * tid);
+    const int h[4] = {h4.w, h4.z, h4.y, h4.x}, sum = h4.x + h4.y + h4.z + h4.w;
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += n;
+    }
+    if (lane == 31) sh.wsum[warp] = inc;
+    cta_sync(bar, NT);
+    int run = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? sh.wsum[lane & 15] : 0) + inc - sum;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (run < k && run + h[j] >= k) { sh.part = SEL_BINS - 1 - 4 * tid - j; sh.rest = k - run; sh.in_part = h[j]; }
+      run += h[j];
+    }
+    cta_sync(bar, NT);
+    const int in_part = sh.in_part, rest = sh.rest, at = sh.part;
+    if (in_part <= SEL_LIST) {
+      #pragma unroll 2
+      for (int i = tid; i < np; i += NT)
+        if (part_of(sc[i]) == at) sh.list[atomicAdd(&sh.n_list, 1)] = max(1u, order_key(sc[i] + 0.0f));
+      cta_sync(bar, NT);
+      // the rest-th largest of the list: every entry counts the ones above it and the ones not below it
+      if (tid < in_part) {
+        const uint32_t mine = sh.list[tid];
+        int above = 0, not_below = 0;
+        #pragma unroll 4
+        for (int j = 0; j < in_part; ++j) {
+          above += sh.list[j] > mine ? 1 : 0;
+          not_below += sh.list[j] >= mine ? 1 : 0;
+        }
+        if (above < rest && not_below >= rest) { sh.thr = mine; sh.need_eq = rest - above; }   // (equal entries: the same)
+      }
+      cta_sync(bar, NT);
+    } else {
+      select_threshold_search(sc, np, k, kmin, kmax, sh, tid, bar);
+    }
+    thr = sh.thr;
+    need_eq = sh.need_eq;
   }
-  if (need_eq < 0) { need_eq = 0; thr = k > 0 && k < np ? thr - 1u : thr; }   // all keys > thr - 1, none at the threshold
 
   // ---- ordered compaction into S and T ------------------------------------------------------
   // 32 tokens per warp and trip: ballots give the members among them, one scan over the groups' packed counts
   // (greater-than in the high half, equal in the low half) what lies before each group.
-  {
-    const int nw = (np + 31) / 32, nwarp = nthr >> 5;
-    #pragma unroll 1
-    for (int g = warp; g < nw; g += nwarp) {
-      const int i = 32 * g + lane;
-      const uint32_t ky = i < np ? keys[i] : 0u;
-      const unsigned gt = __ballot_sync(0xFFFFFFFFu, i < np && (k >= np || (k > 0 && ky > thr)));
-      const unsigned eq = __ballot_sync(0xFFFFFFFFu, i < np && k > 0 && k < np && ky == thr);
-      if (lane == 0) sh.group[g] = __popc(gt) << 16 | __popc(eq);
+  const int nw = (np + 31) / 32;
+  auto members = [&](int g, unsigned& gt, unsigned& eq) {
+    const int i = 32 * g + lane;
+    const uint32_t key = i < np ? max(1u, order_key(sc[i] + 0.0f)) : 0u;
+    gt = __ballot_sync(0xFFFFFFFFu, i < np && (k >= np || (k > 0 && key > thr)));
+    eq = __ballot_sync(0xFFFFFFFFu, i < np && k > 0 && k < np && key == thr);
+  };
+  #pragma unroll 2
+  for (int g = warp; g < nw; g += NT / 32) {
+    unsigned gt, eq;
+    members(g, gt, eq);
+    if (lane == 0) sh.group[g] = __popc(gt) << 16 | __popc(eq);
+  }
+  cta_sync(bar, NT);
+  if (warp == 0) {
+    constexpr int PER = MAX_IMG_TOKENS / 32 / 32;
+    int c[PER], sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) { c[j] = PER * lane + j < nw ? sh.group[PER * lane + j] : 0; sum += c[j]; }
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += n;
     }
-    cta_sync(bar, nthr);
-    if (warp == 0) {
-      constexpr int PER = MAX_IMG_TOKENS / 32 / 32;
-      int c[PER], sum = 0;
+    int run = inc - sum;
 #pragma unroll
-      for (int j = 0; j < PER; ++j) { c[j] = PER * lane + j < nw ? sh.group[PER * lane + j] : 0; sum += c[j]; }
-      int inc = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-        if (lane >= o) inc += n;
-      }
-      int run = inc - sum;
-#pragma unroll
-      for (int j = 0; j < PER; ++j) {
-        if (PER * lane + j < nw) sh.group[PER * lane + j] = run;
-        run += c[j];
-      }
-    }
-    cta_sync(bar, nthr);
-    #pragma unroll 1
-    for (int g = warp; g < nw; g += nwarp) {
-      const int i = 32 * g + lane;
-      const uint32_t ky = i < np ? keys[i] : 0u;
-      const bool is_gt = i < np && (k >= np || (k > 0 && ky > thr)), is_eq = i < np && k > 0 && k < np && ky == thr;
-      const unsigned gt = __ballot_sync(0xFFFFFFFFu, is_gt), eq = __ballot_sync(0xFFFFFFFFu, is_eq);
-      const unsigned lt = (1u << lane) - 1u;
-      const int before = sh.group[g];
-      const int gt_before = (before >> 16) + __popc(gt & lt), eq_before = (before & 0xFFFF) + __popc(eq & lt);
-      const int sel_rank = gt_before + min(eq_before, need_eq);   // selected tokens before i
-      if (i >= np) continue;
-      if (is_gt || (is_eq && eq_before < need_eq)) {
-        S_idx[d.src0 + sel_rank] = i;
-      } else {
-        const int tp = i - sel_rank;
-        T_idx[d.tgt0 + tp] = i;
-        kept_idx[d.out_row0 + d.n_cls + tp] = d.n_cls + i;
-        if (pos_out) pos_out[d.tgt0 + tp] = pp[i];
-      }
+    for (int j = 0; j < PER; ++j) {
+      if (PER * lane + j < nw) sh.group[PER * lane + j] = run;
+      run += c[j];
     }
   }
+  cta_sync(bar, NT);
   #pragma unroll 1
-  for (int i = tid; i < d.n_cls; i += nthr) kept_idx[d.out_row0 + i] = i;
-  #pragma unroll 1
-  for (int i = tid; i < d.n_tail; i += nthr)
-    kept_idx[d.out_row0 + d.n_cls + d.n_tgt + d.n_extra + i] = d.n_cls + np + i;
-  if (tid == 0 && d.n_extra) kept_idx[d.out_row0 + d.n_cls + d.n_tgt] = -1;
+  for (int g = (w_lo >> 5) + warp; 32 * g < w_hi; g += NT / 32) {
+    const int i = 32 * g + lane;
+    unsigned gt, eq;
+    members(g, gt, eq);
+    if (i < w_lo || i >= w_hi) continue;
+    const unsigned lt = (1u << lane) - 1u;
+    const int before = sh.group[g];
+    const int gt_before = (before >> 16) + __popc(gt & lt), eq_before = (before & 0xFFFF) + __popc(eq & lt);
+    const int sel_rank = gt_before + min(eq_before, need_eq);   // selected tokens before i
+    if ((gt >> lane & 1u) || ((eq >> lane & 1u) && eq_before < need_eq)) {
+      S_idx[d.src0 + sel_rank] = i;
+    } else {
+      const int tp = i - sel_rank;
+      T_idx[d.tgt0 + tp] = i;
+      kept_idx[d.out_row0 + d.n_cls + tp] = d.n_cls + i;
+      if (pos_out) pos_out[d.tgt0 + tp] = pos ? pos[d.patch0 + i] : i;
+    }
+  }
+  if (w_lo == 0) {
+    #pragma unroll 1
+    for (int i = tid; i < d.n_cls; i += NT) kept_idx[d.out_row0 + i] = i;
+    #pragma unroll 1
+    for (int i = tid; i < d.n_tail; i += NT)
+      kept_idx[d.out_row0 + d.n_cls + d.n_tgt + d.n_extra + i] = d.n_cls + np + i;
+    if (tid == 0 && d.n_extra) kept_idx[d.out_row0 + d.n_cls + d.n_tgt] = -1;
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -836,7 +949,7 @@ __device__ __noinline__ void select_image(
 // inter-CTA wait that ends in one) must separate it from select_small().
 // ---------------------------------------------------------------------------------------
 constexpr int SEL_SMALL_MAX = 1024;
-constexpr int SEL_SMALL_THREADS = 512;
+constexpr int SEL_SMALL_THREADS = SEL_THREADS;
 
 struct SelectSmallShared {
   uint32_t wmin[16], wmax[16];
@@ -911,20 +1024,8 @@ __device__ __noinline__ void select_small(
     const int nwc = (d.gw + window - 1) / window, nwr = (d.gh + window - 1) / window;
     #pragma unroll 1
     for (int wdx = tid; wdx < nwc * nwr; wdx += NT) {
-      const int r0 = (wdx / nwc) * window, c0 = (wdx % nwc) * window;
-      const int r1 = min(d.gh, r0 + window), c1 = min(d.gw, c0 + window);
-      int best = -1;
-      float bs = 0.f;
-      #pragma unroll 1
-      for (int r = r0; r < r1; ++r)
-        #pragma unroll 1
-        for (int c = c0; c < c1; ++c) {
-          const int t = wk.cell[r * d.gw + c];
-          if (t < 0) continue;
-          const float v = wk.sc[t];
-          if (best < 0 || v > bs || (v == bs && t < best)) { best = t; bs = v; }
-        }
-      if (best >= 0) wk.sc[best] = bs * coef;      // windows are disjoint: nobody else touches this token
+      const int best = window_best<short, -1>(wk.cell, wk.sc, d.gh, d.gw, window, nwc, wdx);
+      if (best >= 0) wk.sc[best] *= coef;            // windows are disjoint: nobody else touches this token
     }
     cta_sync(bar, NT);
   }
@@ -1090,30 +1191,38 @@ __device__ __noinline__ void select_small(
   }
 }
 
-// One CTA (512 or 1024 threads) per image.
-__global__ void __launch_bounds__(1024) k_select(const ImgDesc* __restrict__ desc,
-                                                 const float* __restrict__ s_raw,
-                                                 const int* __restrict__ pos, int window, float coef,
-                                                 int penalty, float* __restrict__ s_pen,
-                                                 float* __restrict__ scores_out,
-                                                 int* __restrict__ S_idx, int* __restrict__ T_idx,
-                                                 int* __restrict__ kept_idx, int* __restrict__ pos_out,
-                                                 unsigned* __restrict__ status) {
-  extern __shared__ unsigned char sm_raw[];
-  __shared__ SelectShared sh;
-  __shared__ SelectSmallShared shs;
+// One CTA per image.  SMALL: no image has more than SEL_SMALL_MAX tokens.
+template <bool SMALL>
+__global__ void __launch_bounds__(SEL_THREADS, 2) k_select(const ImgDesc* __restrict__ desc,
+                                                           const float* __restrict__ s_raw,
+                                                           const int* __restrict__ pos, int window, float coef,
+                                                           int penalty, float* __restrict__ s_pen,
+                                                           float* __restrict__ scores_out,
+                                                           int* __restrict__ S_idx, int* __restrict__ T_idx,
+                                                           int* __restrict__ kept_idx, int* __restrict__ pos_out,
+                                                           unsigned* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
   const ImgDesc d = desc[blockIdx.x];
-  grid_dep_wait();
-  grid_dep_launch();
-  if (d.np <= SEL_SMALL_MAX && blockDim.x == SEL_SMALL_THREADS) {
-    select_small_prepare(d, penalty, sm_raw, threadIdx.x);
+  const int tid = threadIdx.x;
+  if (SMALL || d.np <= SEL_SMALL_MAX) {
+    __shared__ SelectSmallShared shs;
+    select_small_prepare(d, penalty, sm_raw, tid);
+    grid_dep_wait();
+    grid_dep_launch();
     __syncthreads();
     select_small(d, s_raw, pos, window, coef, penalty, s_pen, scores_out, S_idx, T_idx, kept_idx, pos_out,
-                 status, sm_raw, shs, threadIdx.x, 0, 0, d.np);
+                 status, sm_raw, shs, tid, 0, 0, d.np);
     return;
   }
-  select_image(d, s_raw, pos, window, coef, penalty, s_pen, scores_out, S_idx, T_idx, kept_idx, pos_out,
-               status, sm_raw, sh, threadIdx.x, (int)blockDim.x, 0);
+  if constexpr (!SMALL) {
+    __shared__ SelectShared sh;
+    select_image_prepare(d, penalty, sm_raw, sh, tid);
+    grid_dep_wait();
+    grid_dep_launch();
+    __syncthreads();
+    select_image(d, s_raw, pos, window, coef, penalty, s_pen, scores_out, S_idx, T_idx, kept_idx, pos_out,
+                 status, sm_raw, sh, tid, 0, 0, d.np);
+  }
 }
 
 }  // namespace ficoco

@@ -8,10 +8,8 @@
 //   pass 2  (the rows still in the rings from there, the others, now L2-resident, with 16-byte loads, several rows in
 //           flight per warp) once all pieces of the image are in:
 //           v_i = rn_i (x_i . sum of partials) / Np,  s_i = cA v_i - (1 - cA) a_i;
-//   select  images of up to 1024 tokens: every CTA that scored a piece waits until all of the
-//           image's scores are in, runs the (short) selection on the whole image and writes the
-//           outputs of its own tokens; larger images: the CTA that finishes the last piece runs
-//           the selection alone.
+//   select  every CTA that scored a piece waits until all of the image's scores are in, runs the selection on the whole
+//           image and writes the outputs of its own tokens.
 // The inter-CTA waits are polls of per-image counters, bounded by elapsed time (wait_ns).  The
 // counters exist twice; a launch uses the set of its parity and zeroes the other one, so a step
 // that gave up half-way cannot leave counts behind for the step after the next.  The set a launch
@@ -40,8 +38,8 @@ constexpr int FFOLD = 8;          // rows of the fold buffer (warps w and w + 8 
 constexpr int F_NCONS = 512;
 constexpr int F_MAXSTAGE = 16;
 constexpr size_t F_SMEM = 216 * 1024;   // dynamic shared memory at most (7 KB are static)
-constexpr int F_MAXWON = 32;      // pieces per CTA (and therefore selections it can win)
-static_assert(F_NCONS == SEL_SMALL_THREADS, "the short selection is written for the consumer threads");
+constexpr int F_MAXWON = 32;      // pieces per CTA
+static_assert(F_NCONS == SEL_SMALL_THREADS, "the selection is written for the threads of this kernel");
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
@@ -120,8 +118,7 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
   // take over SMs as blocks of this grid exit and park until this grid has completed.
   grid_dep_launch();
   FICOCO_PHASE_BEGIN(0);
-  __shared__ int won[F_MAXWON];
-  __shared__ int nwon, failed;
+  __shared__ int failed;
   __shared__ WorkItem w_s[F_MAXWON];          // this CTA's pieces and their images
   __shared__ ImgDesc d_s[F_MAXWON];
 
@@ -147,7 +144,7 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
 
   if (lane < nstage) mbar_init(&full_bar[warp][lane], 1);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  if (tid == 0) { nwon = 0; failed = 0; }
+  if (tid == 0) failed = 0;
   // (plan data: looked up once, under the tail of the grid before)
   for (int i = warp; i < p_end - p_begin; i += F_NCONS / 32) {
     const WorkItem w = pieces[p_begin + i];
@@ -443,15 +440,7 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
       finish_rows(g0, min(g_res, g0 + F_P2B), dot);
     }
     cta_sync(1, F_NCONS);
-    if (tid == 0) {
-      if (d.np <= SEL_SMALL_MAX) {
-        red_release_add(&cnt[B + w.img], 1);         // releases this piece's scores; the selection polls for all of them
-      } else {
-        // (for the CTA that arrives last) acquires everyone else's as well
-        const int old = atom_acq_rel_add(&cnt[B + w.img], 1);
-        if (old == d.n_chunks - 1 && nwon < F_MAXWON) won[nwon++] = w.img;
-      }
-    }
+    if (tid == 0) red_release_add(&cnt[B + w.img], 1);   // releases this piece's scores; the selection polls for all of them
   }
   cta_sync(1, F_NCONS);
 
@@ -470,28 +459,24 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
     const ImgDesc& d = d_s[pi - p_begin];
     int pj = pi, hi = w0.r0;
     while (pj < p_end && w_s[pj - p_begin].img == w0.img) { hi = w_s[pj - p_begin].r0 + w_s[pj - p_begin].nrows; ++pj; }
-    if (d.np <= SEL_SMALL_MAX) {
-      select_small_prepare(d, penalty, ring, tid);
-      if (tid == 0 && !poll_count(&cnt[B + w0.img], d.n_chunks, wait_ns, status)) {
-        atomicOr(status, STATUS_TIMEOUT);
-        failed = 1;
-      }
-      cta_sync(1, F_NCONS);
-      if (failed) return;
-      FICOCO_PHASE(0, 7);
+    const bool small = d.np <= SEL_SMALL_MAX;
+    if (small) select_small_prepare(d, penalty, ring, tid);
+    else select_image_prepare(d, penalty, ring, sel_sh, tid);
+    if (tid == 0 && !poll_count(&cnt[B + w0.img], d.n_chunks, wait_ns, status)) {
+      atomicOr(status, STATUS_TIMEOUT);
+      failed = 1;
+    }
+    cta_sync(1, F_NCONS);
+    if (failed) return;
+    FICOCO_PHASE(0, 7);
+    // (the counters are not reset here: the next launch zeroes this launch's set, see the top)
+    if (small)
       select_small(d, s_raw, pos, window, coef, penalty, s_pen, scores_out, S_idx, T_idx, kept_idx, pos_out,
                    status, ring, sel_small_sh, tid, 1, w0.r0, hi);
-      // (the counters are not reset here: the next launch zeroes this launch's set, see the top)
-      if (pj < p_end) cta_sync(1, F_NCONS);     // the work area is reused by the next image
-    } else {
-      bool mine = false;
-      for (int k = 0; k < nwon; ++k) mine = mine || won[k] == w0.img;
-      if (mine) {
-        select_image(d, s_raw, pos, window, coef, penalty, s_pen, scores_out, S_idx, T_idx, kept_idx, pos_out,
-                     status, ring, sel_sh, tid, F_NCONS, 1);
-        if (pj < p_end) cta_sync(1, F_NCONS);
-      }
-    }
+    else
+      select_image(d, s_raw, pos, window, coef, penalty, s_pen, scores_out, S_idx, T_idx, kept_idx, pos_out,
+                   status, ring, sel_sh, tid, 1, w0.r0, hi);
+    if (pj < p_end) cta_sync(1, F_NCONS);         // the work area is used again by the next image
     pi = pj;
   }
   FICOCO_PHASE(0, 8);

@@ -63,10 +63,32 @@ def test_most_rows_kept_of_wide_rows(kind, batch, dim, dtype):
         c.close()
 
 
-@pytest.mark.parametrize("gh,gw,keep", [(31, 33, 900), (32, 32, 1), (25, 41, 1024), (25, 41, 4), (48, 45, 40)])
+@pytest.mark.parametrize("gh,gw,keep", [(31, 33, 900), (32, 32, 1), (25, 41, 1024), (25, 41, 4), (48, 45, 40),
+                                         (64, 64, 2000), (17, 241, 4096)])
 def test_selection_sizes(ctx, gh, gw, keep):
-    """1023 and 1024 tokens: two per thread in registers; from 1025 on the search over the score range."""
-    run_v(ctx, 92, 1, gh, gw, 64, keep, cls=False)
+    """1023 and 1024 tokens: two per thread; from 1025 on eight, from 4097 on sixteen (the last: unfused)."""
+    run_v(ctx, 92, 1, gh, gw, 64, keep, cls=False, p=fo.Params(max_targets=0) if gh * gw > 4000 else fo.Params())
+
+
+@pytest.mark.parametrize("fused", [True, False], ids=["fused", "unfused"])
+@pytest.mark.parametrize("n,keep,levels", [(1100, 500, 1), (2000, 1300, 2), (1100, 1099, 2000), (3000, 40, 4), (4100, 2000, 40)])
+def test_selection_of_equal_scores(n, keep, levels, fused):
+    """Scores that take few values (lambda = 0: the attention alone): ties at the threshold go to the lower index whether
+    they fit the list of the part it lies in or not."""
+    dim = 256 if fused else 4096
+    g = torch.Generator(device="cuda").manual_seed(n)
+    a = torch.randint(0, levels, (1, 1, n), generator=g, device="cuda").float() / 4096
+    x = torch.randn((n, dim), generator=g, device="cuda").to(torch.bfloat16)
+    c = binding.Context(max_tokens=n, max_dim=dim, max_batch=1, device=0)
+    try:
+        r = c.ficoco_v_reduce(x, a, keep, n // 50, 50, 1, n_tokens=n,
+                              params=binding.make_params(lam=0.0, has_cls=False, local_penalty=False, max_targets=0))
+        gone = (-a[0, 0]).argsort(descending=True, stable=True)[:n - keep]
+        left = torch.ones(n, dtype=torch.bool, device="cuda")
+        left[gone] = False
+        assert torch.equal(r.kept_idx.long(), left.nonzero()[:, 0])
+    finally:
+        c.close()
 
 
 @pytest.mark.parametrize("dim,n_src,n_tgt", [
