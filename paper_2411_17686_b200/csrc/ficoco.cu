@@ -487,6 +487,17 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   // step 108 us instead of 102).  76 % is the 196 KB setting.
   cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributePreferredSharedMemoryCarveout, 76);
   cudaFuncSetAttribute(k_merge_rows<__nv_bfloat16>, cudaFuncAttributePreferredSharedMemoryCarveout, 76);
+  // The kernels in front of them ask for 100 KB, which suits what they stream and lets them start beside their
+  // neighbours; what the driver picks by itself depends on the neighbours (256 x 577 tokens: column sums 74 or 98 us, the
+  // step 315 or 339; relation map: the step 41.8 or 44.8; 28 and 57 % like 43).
+  {
+    auto carve = [](auto* kernel) { cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 43); };
+#define FICOCO_COLSUM_CARVE(V) carve(k_colsum<float, V, true>); carve(k_colsum<__nv_bfloat16, V, true>)
+    FICOCO_COLSUM_CARVE(1); FICOCO_COLSUM_CARVE(2); FICOCO_COLSUM_CARVE(4); FICOCO_COLSUM_CARVE(5); FICOCO_COLSUM_CARVE(8);
+#undef FICOCO_COLSUM_CARVE
+    carve(k_score_rel); carve(k_correlate_rel<2>); carve(k_correlate_rel<4>); carve(k_correlate_rel<16>);
+    carve(k_select<true>); carve(k_select<false>);
+  }
   cudaFuncSetAttribute(k_score<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   cudaFuncSetAttribute(k_score<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   if (cudaGetLastError() != cudaSuccess) { ficoco_destroy(c); return FICOCO_ERR_CUDA; }
