@@ -95,6 +95,19 @@ __device__ __forceinline__ uint4 pack(const float (&f)[8], const __nv_bfloat16*)
 }
 
 __device__ __forceinline__ uint4 ldg16(const void* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+// Loads that are issued where they stand (the compiler moves a plain load of constant data to its first use, behind the
+// waits that it is meant to be in flight under).
+__device__ __forceinline__ uint4 ld16_now(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_now(const float* p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+
 // Streaming store (st.global.cs) for the output rows.  A step's token rows, read by all three of its kernels, plus its
 // output rows are about as much as L2 keeps.  32 x 577 tokens of 1024, DRAM reads of correlate and merge in the running
 // step: 0.64 and 0.18 MB where inputs are used again, 1.50 and 0.47 with ordinary stores; on cycled inputs 0.3 MB both ways.

@@ -1038,9 +1038,9 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     c->launches += 1;
   } else if (wide) {
     if (nvec <= 512) launch_dependent(k_colsum_wide<T, 2, 8>, dim3(p->n_rows), 256, 0, st,
-      tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
+      tok, D, p->d_desc, p->d_rows, c->rn, c->partial, tmean != nullptr ? 1 : 0);
     else launch_dependent(k_colsum_wide<T, 4, 4>, dim3(p->n_rows), 256, 0, st,
-      tok, D, p->d_desc, p->d_rows, c->rn, c->partial);
+      tok, D, p->d_desc, p->d_rows, c->rn, c->partial, tmean != nullptr ? 1 : 0);
     c->launches += 1;
   } else {
     launch_dependent(k_rownorm<T>, dim3(p->n_rows), 256, 0, st,

@@ -47,19 +47,6 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
   return v;
 }
 
-// Loads that are issued where they stand (the compiler moves a plain load of constant data to its first use, behind the
-// waits that it is meant to be in flight under).
-__device__ __forceinline__ uint4 ld16_now(const void* p) {
-  uint4 v;
-  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ float ld_now(const float* p) {
-  float v;
-  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-
 // Poll until *p >= need.  Gives up after limit_ns, or at once when another CTA has already
 // raised STATUS_TIMEOUT (its pieces will never arrive).  One thread calls this.
 __device__ __forceinline__ bool poll_count(const int* p, int need, unsigned long long limit_ns,
