@@ -75,7 +75,8 @@ struct Plan {
   bool need_finalize = false;   // some image merges nothing: its per-token counts are zeroed by a kernel
   bool umma = false;
   bool um_f32 = false;          // fp32 tokens split into three bf16 terms (k_correlate_umma_f32)
-  int um_b_bytes = 0;
+  bool uf_small = false;        // fp32 tiles of 32 x 32 instead of 128 x 64
+  int um_b_bytes = 0, uf_stg = 0, uf_stg_off = 0;     // slots for fp32 values (k-blocks in flight) and where they lie
   int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1, um_text_off = 0;
   size_t um_smem = 0;
   std::vector<ImgDesc> h_desc;
@@ -466,9 +467,11 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
     cudaFuncSetAttribute(k_correlate_umma<LC, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max)
     FICOCO_UMMA_ATTR(2); FICOCO_UMMA_ATTR(4); FICOCO_UMMA_ATTR(16);
 #undef FICOCO_UMMA_ATTR
-    cudaFuncSetAttribute(k_correlate_umma_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
-    cudaFuncSetAttribute(k_correlate_umma_f32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max);
+#define FICOCO_UF32_ATTR(LC)                                                                                       \
+    cudaFuncSetAttribute(k_correlate_umma_f32<LC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max); \
+    cudaFuncSetAttribute(k_correlate_umma_f32<LC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, um_smem_max)
+    FICOCO_UF32_ATTR(2); FICOCO_UF32_ATTR(4); FICOCO_UF32_ATTR(16);
+#undef FICOCO_UF32_ATTR
   }
   {
 #define FICOCO_FUSED_ATTR(TT, V) \
@@ -544,8 +547,9 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   // fp32 tokens (FiCoCo-V): the same tiling with narrower column tiles, operands split into bf16 terms
   p->um_f32 = key.dtype == FICOCO_FP32 && key.dim % UKB == 0 && key.mode == 0;
   if (p->um_f32) p->umma = true;
+  p->uf_small = false;
   if (key.rel) p->umma = p->um_f32 = false;           // C is read from the supplied matrix, not contracted
-  const int un_max = p->um_f32 ? UF_COLS : UN_MAX;    // accumulator columns per CTA
+  int un_max = p->um_f32 ? UF_COLS : UN_MAX;          // accumulator columns per CTA
   int tile_rows_max = p->umma ? UM : CBM;             // source rows per correlate CTA
   if (key.rel) {
     // a warp of the relation correlate takes one discarded token at a time and is bound by the
@@ -647,7 +651,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   }
 
   // ---- correlate tiling ---------------------------------------------------------------------
-  const int cols_max = p->umma ? un_max : INT_MAX;
+  int cols_max = p->umma ? un_max : INT_MAX;
   auto split_cols = [&](int n_tgt, int ns) {           // columns per split: ns splits, or more if they got too wide
     ns = std::max(ns, (n_tgt - 1) / cols_max + 1);
     return ((n_tgt + ns - 1) / ns + col_granule - 1) / col_granule * col_granule;
@@ -733,12 +737,26 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     }
     tile_rows_max = best_rows;
   } else {
-    // as many splits as give every SM two CTAs (fp32 tiles: the CTA that completes a tile merges nsplit * L entries
-    // per token, one thread each)
+    // As many splits as give every SM two CTAs, no more than eight with fp32 tiles; a grid of fp32 tiles of
+    // 32 x 32 that needs no second CTA on any SM is taken instead (47.0 -> 43.0 us for 64 x 512 entries; twice as many
+    // entries as fit: the larger tiles are ahead).
     long long strips = 0;
     for (int b = 0; b < B; ++b)
       if (p->h_desc[b].list_len > 0) strips += row_tiles(p->h_desc[b].n_src);
     if (strips > 0) want_split = (int)std::min(std::max(2LL * c->num_sms / strips, 1LL), p->um_f32 ? 8LL : (long long)NSPLIT_MAX);
+    long long n_ctas = 0, entries = 0;
+    for (int b = 0; b < B; ++b) {
+      const ImgDesc& d = p->h_desc[b];
+      if (d.list_len == 0) continue;
+      const int ns = (d.n_tgt + UF_SMALL - 1) / UF_SMALL;
+      n_ctas += (long long)((d.n_src + UF_SMALL - 1) / UF_SMALL) * ns;
+      entries += (long long)d.n_src * ns * d.list_len;
+    }
+    if (p->um_f32 && n_ctas <= c->num_sms && n_ctas <= c->cap_corr && entries <= c->cap_part) {
+      p->uf_small = true;
+      tile_rows_max = cols_max = um_a_rows = um_cols = UF_SMALL;     // (full tiles)
+      want_split = 1;
+    }
   }
 
   // Output rows per merge CTA: the fewest that make one wave of two CTAs per SM, or else as many as the shared
@@ -842,13 +860,19 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   p->tot_patch = (int)patch0; p->tot_src = (int)src0; p->tot_tgt = (int)tgt0; p->tot_out_rows = (int)out0;
   p->n_rows = (int)rows.size(); p->n_corr = (int)corr.size(); p->n_out = (int)outw.size();
   if (p->um_f32) {
-    // two stages of three bf16 tiles per operand, 16 KB behind them for the 128-row reads of the last A tile
+    // stages of three bf16 tiles per operand, 16 KB behind them for the 128-row reads of the last A tile
     p->um_a_bytes = um_a_rows * 128;
     p->um_b_bytes = (um_cols + 15) / 16 * 16 * 128;
     p->um_tmem_cols = 32;
     while (p->um_tmem_cols < 6 * (p->um_b_bytes / 128)) p->um_tmem_cols *= 2;   // six partial products per entry
-    p->um_nstage = UF_STAGES;
-    p->um_smem = (size_t)UF_STAGES * 3 * (p->um_a_bytes + p->um_b_bytes) + (size_t)UM * 128 + 2048;
+    p->um_nstage = uf_stages(p->uf_small);
+    p->um_smem = (size_t)uf_stages(p->uf_small) * 3 * (p->um_a_bytes + p->um_b_bytes) + (size_t)UM * 128 + 2048;
+    if (p->uf_small) {                                 // slots for the fp32 values of the next k-blocks
+      const size_t slot = 2 * 8192;
+      p->uf_stg = (int)std::min<size_t>(8, (220 * 1024 - p->um_smem) / slot);
+      p->uf_stg_off = (int)(p->um_smem - 1024);
+      p->um_smem += p->uf_stg * slot;
+    }
     if (um_a_rows > UM || um_cols > UF_COLS || p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
   } else if (p->umma) {
     const UmRing r = um_ring(um_a_rows, um_cols, (long long)corr.size());
@@ -1102,10 +1126,10 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       prof_tick(c, st, "correlate_umma_f32");
       const float* tk = reinterpret_cast<const float*>(tok);
 #define FICOCO_UF32_LAUNCH(LC)                                                                         \
-  launch_dependent(k_correlate_umma_f32<LC>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,               \
+  launch_dependent(p->uf_small ? k_correlate_umma_f32<LC, true> : k_correlate_umma_f32<LC, false>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,                                                                  \
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
       (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status,                 \
-      p->um_a_bytes, p->um_b_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt,        \
+      p->um_a_bytes, p->um_b_bytes, p->uf_stg_off, p->uf_stg, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt, \
       c->e_w, c->e_c, c->wait_ns)
       if (p->max_list <= 2) FICOCO_UF32_LAUNCH(2);
       else if (p->max_list <= 4) FICOCO_UF32_LAUNCH(4);

@@ -18,14 +18,22 @@
 // One CTA: up to 128 discarded tokens x up to 64 preserved tokens of one image, two stages of
 // 64 hidden elements; thread (row r mod 32, 16-byte chunk c) of the 256 producers handles chunk c of
 // rows r, r + 32, ... of both operands and keeps the next k-block's loads in flight while it
-// converts the current one (a third register buffer spilled and was slower).  Every wait is bounded as in the bf16 kernel.
+// converts the current one (a third register buffer spilled and was slower).  A grid that would leave SMs idle takes tiles
+// of 32 x 32 (SMALL): a thread's fp32 values arrive by cp.async in up to eight shared-memory slots of its own, which needs
+// no barrier, and are converted into four stages.  Every wait is bounded as in the bf16 kernel.
+//
+// What bounds it: the producers' instructions per k-block (two barriers, conversion and 48 bytes of stores per eight
+// values).  One image of 576 tokens, 64 x 512 entries: 8 CTAs of 64 x 64 took 0.8 us per k-block; 32 CTAs of 32 x 32
+// 0.5 (whole step 47.0 -> 43.0 us; 288 x 288 entries 43.8 -> 37.7).  Slots with a test for each of six rows per thread:
+// 1.1 us per k-block; staged tiles of 64 x 64: four images of 576 tokens 59 us instead of 45.
 #pragma once
 #include "kernels_correlate_umma.cuh"
 
 namespace ficoco {
 
 constexpr int UF_COLS = 64;      // preserved tokens per CTA (two rows per producer thread)
-constexpr int UF_STAGES = 2;
+constexpr int UF_SMALL = 32;     // rows and columns of a small tile
+__host__ __device__ constexpr int uf_stages(bool small) { return small ? 4 : 2; }   // stages of converted operands
 constexpr int UF_AR = UM / 32;       // A rows per producer thread
 constexpr int UF_BR = UF_COLS / 32;  // B rows per producer thread
 
@@ -83,21 +91,23 @@ __device__ __forceinline__ void epilogue_scan_split(uint32_t tmem_lane, int nb, 
     if (ix[k] != INT_MAX) v[k] *= rs;
 }
 
-// Dynamic shared memory: [1024-aligned] two stages of [A_h | A_m | A_l | B_h | B_m | B_l]; an A tile has
+// Dynamic shared memory: [1024-aligned] stages of [A_h | A_m | A_l | B_h | B_m | B_l]; an A tile has
 // a_bytes (valid rows rounded up to 8, x 128 B), a B tile b_bytes (columns rounded to 16, x 128 B).  An
 // MMA reads 128 A rows: rows past a tile alias the tiles behind it (or the slack the host adds behind
 // the last stage) and only feed accumulator rows that are never read.
-template <int LCAP>
+template <int LCAP, bool SMALL>
 __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
     const float* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
     const WorkItem* __restrict__ work, const float* __restrict__ rn,
     const int* __restrict__ S_idx, const int* __restrict__ T_idx,
     float* __restrict__ part_val, int* __restrict__ part_idx, unsigned* __restrict__ status,
-    int a_bytes, int b_bytes, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
+    int a_bytes, int b_bytes, int stg_off, int n_stg, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
     float* __restrict__ tau_out, int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c,
     unsigned long long wait_ns) {
+  constexpr int NST = uf_stages(SMALL);
+  constexpr int AR = SMALL ? UF_SMALL / 32 : UF_AR, BR = SMALL ? UF_SMALL / 32 : UF_BR;   // rows per producer thread
   extern __shared__ unsigned char uf_raw[];
-  __shared__ uint64_t full_bar[UF_STAGES], empty_bar[UF_STAGES], acc_bar;
+  __shared__ uint64_t full_bar[NST], empty_bar[NST], acc_bar;
   __shared__ uint32_t tmem_base_s;
   __shared__ int rowS[UM], rowT[UF_COLS];
   __shared__ float rnT[UF_COLS];
@@ -117,7 +127,7 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
   const uint32_t ring = (smem_u32(uf_raw) + 1023u) & ~1023u;
 
   if (tid == 0) {
-    for (int s = 0; s < UF_STAGES; ++s) { mbar_init(&full_bar[s], 8); mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < NST; ++s) { mbar_init(&full_bar[s], 8); mbar_init(&empty_bar[s], 1); }
     mbar_init(&acc_bar, 1);
     failed = 0;
     acc_committed = 0;
@@ -161,50 +171,49 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
     const int pt = warp < 4 ? tid : tid - 32;
     const int chunk = pt & 7;
     const int rsub = pt >> 3;           // 0..31
-    size_t offA[UF_AR], offB[UF_BR];
+    size_t offA[AR], offB[BR];
     uint32_t onA = 0, onB = 0;
 #pragma unroll
-    for (int i = 0; i < UF_AR; ++i) {
+    for (int i = 0; i < AR; ++i) {
       const int r = rsub + 32 * i;
-      const bool on = r < w.nrows;
-      offA[i] = on ? (size_t)rowS[r] * (size_t)D : 0;
+      const bool on = SMALL || r < w.nrows;           // (small tiles are full: the last row again)
+      offA[i] = on ? (size_t)rowS[min(r, w.nrows - 1)] * (size_t)D : 0;
       onA |= on ? 1u << i : 0u;
     }
 #pragma unroll
-    for (int i = 0; i < UF_BR; ++i) {
+    for (int i = 0; i < BR; ++i) {
       const int r = rsub + 32 * i;
-      const bool on = r < ncols;
-      offB[i] = on ? (size_t)rowT[r] * (size_t)D : 0;
+      const bool on = SMALL || r < ncols;
+      offB[i] = on ? (size_t)rowT[min(r, ncols - 1)] * (size_t)D : 0;
       onB |= on ? 1u << i : 0u;
     }
     const uint32_t dsw = (uint32_t)((rsub >> 3) * 1024 + (rsub & 7) * 128 + ((chunk ^ (rsub & 7)) << 4));
     const float* tbase = tokens + (size_t)(d.row0 + d.n_cls) * D + chunk * 8;
     bool ok = true;
-    float4 bufA[UF_AR + UF_BR][2], bufB[UF_AR + UF_BR][2];
-    auto load = [&](float4 (&buf)[UF_AR + UF_BR][2], int kb) {
+    auto load = [&](float4 (&buf)[AR + BR][2], int kb) {
       const float* src = tbase + (size_t)kb * UKB;
 #pragma unroll
-      for (int i = 0; i < UF_AR; ++i)
-        if (onA >> i & 1u) {
+      for (int i = 0; i < AR; ++i)
+        if (SMALL || (onA >> i & 1u)) {
           buf[i][0] = __ldg(reinterpret_cast<const float4*>(src + offA[i]));
           buf[i][1] = __ldg(reinterpret_cast<const float4*>(src + offA[i]) + 1);
         }
 #pragma unroll
-      for (int i = 0; i < UF_BR; ++i)
-        if (onB >> i & 1u) {
-          buf[UF_AR + i][0] = __ldg(reinterpret_cast<const float4*>(src + offB[i]));
-          buf[UF_AR + i][1] = __ldg(reinterpret_cast<const float4*>(src + offB[i]) + 1);
+      for (int i = 0; i < BR; ++i)
+        if (SMALL || (onB >> i & 1u)) {
+          buf[AR + i][0] = __ldg(reinterpret_cast<const float4*>(src + offB[i]));
+          buf[AR + i][1] = __ldg(reinterpret_cast<const float4*>(src + offB[i]) + 1);
         }
     };
-    auto store = [&](const float4 (&buf)[UF_AR + UF_BR][2], int kb) {
-      const int s = kb % UF_STAGES;
-      if (kb >= UF_STAGES && ok) ok = mbar_wait(&empty_bar[s], ((kb / UF_STAGES) - 1) & 1, wait_ns);
+    auto store = [&](const float4 (&buf)[AR + BR][2], int kb) {
+      const int s = kb % NST;
+      if (kb >= NST && ok) ok = mbar_wait(&empty_bar[s], ((kb / NST) - 1) & 1, wait_ns);
       if (ok) {
         const uint32_t a0 = ring + (uint32_t)s * stage_bytes + dsw;
         const uint32_t b0 = a0 + 3u * (uint32_t)a_bytes;
 #pragma unroll
-        for (int i = 0; i < UF_AR; ++i)
-          if (onA >> i & 1u) {
+        for (int i = 0; i < AR; ++i)
+          if (SMALL || (onA >> i & 1u)) {
             uint4 h, m, l;
             split3(buf[i][0], buf[i][1], h, m, l);
             st_shared16(a0 + i * 4096, h);
@@ -212,10 +221,10 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
             st_shared16(a0 + 2u * (uint32_t)a_bytes + i * 4096, l);
           }
 #pragma unroll
-        for (int i = 0; i < UF_BR; ++i)
-          if (onB >> i & 1u) {
+        for (int i = 0; i < BR; ++i)
+          if (SMALL || (onB >> i & 1u)) {
             uint4 h, m, l;
-            split3(buf[UF_AR + i][0], buf[UF_AR + i][1], h, m, l);
+            split3(buf[AR + i][0], buf[AR + i][1], h, m, l);
             st_shared16(b0 + i * 4096, h);
             st_shared16(b0 + (uint32_t)b_bytes + i * 4096, m);
             st_shared16(b0 + 2u * (uint32_t)b_bytes + i * 4096, l);
@@ -225,13 +234,50 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
       __syncwarp();
       if (lane == 0) mbar_arrive(&full_bar[s]);
     };
-    load(bufA, 0);
-    for (int kb = 0; kb < nkb; kb += 2) {
-      if (kb + 1 < nkb) load(bufB, kb + 1);
-      store(bufA, kb);
-      if (kb + 1 < nkb) {
-        if (kb + 2 < nkb) load(bufA, kb + 2);
-        store(bufB, kb + 1);
+    if constexpr (SMALL) {
+      // slot (k-block mod n_stg, row chunk i, half): 16 bytes per thread, side by side
+      constexpr uint32_t stage_step = (AR + BR) * 8192;
+      const uint32_t mine = ring + (uint32_t)stg_off + (uint32_t)pt * 16u;
+      const float* next = tbase;
+      auto fetch = [&](int kb, uint32_t to) {
+        if (kb < nkb) {
+#pragma unroll
+          for (int i = 0; i < AR + BR; ++i) {
+            const float* from = next + (i < AR ? offA[i < AR ? i : 0] : offB[i < AR ? 0 : i - AR]);
+            cp_async16(to + (uint32_t)i * 8192u, from);
+            cp_async16(to + (uint32_t)i * 8192u + 4096u, from + 4);
+          }
+          next += UKB;
+        }
+        cp_async_commit();
+      };
+      #pragma unroll 1
+      for (int st = 0; st < n_stg; ++st) fetch(st, mine + (uint32_t)st * stage_step);
+      int st = 0;
+      #pragma unroll 1
+      for (int kb = 0; kb < nkb; ++kb) {
+        cp_async_wait_groups(n_stg - 1);
+        float4 buf[AR + BR][2];
+        const unsigned char* from = uf_raw + (mine - smem_u32(uf_raw)) + (size_t)st * stage_step;
+#pragma unroll
+        for (int i = 0; i < AR + BR; ++i) {
+          buf[i][0] = *reinterpret_cast<const float4*>(from + (size_t)i * 8192);
+          buf[i][1] = *reinterpret_cast<const float4*>(from + (size_t)i * 8192 + 4096);
+        }
+        fetch(kb + n_stg, mine + (uint32_t)st * stage_step);   // (the values are in registers)
+        store(buf, kb);
+        if (++st == n_stg) st = 0;
+      }
+    } else {
+      float4 bufA[AR + BR][2], bufB[AR + BR][2];
+      load(bufA, 0);
+      for (int kb = 0; kb < nkb; kb += 2) {
+        if (kb + 1 < nkb) load(bufB, kb + 1);
+        store(bufA, kb);
+        if (kb + 1 < nkb) {
+          if (kb + 2 < nkb) load(bufA, kb + 2);
+          store(bufB, kb + 1);
+        }
       }
     }
     FICOCO_PHASE(3, 4);
@@ -306,14 +352,14 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
     // ---------------- MMA issuer (the whole warp, one elected lane per instruction): six products per k-step,
     // smallest terms first --------------------------------------------------------------------------
     const uint32_t id3 = umma_idesc_bf16(3 * nb), id2 = umma_idesc_bf16(2 * nb), id1 = umma_idesc_bf16(nb);
-    const uint32_t u_tmem = warp_uniform(tmem_base), u_ring = warp_uniform(ring);
+    const uint32_t u_tmem = warp_uniform(tmem_base);
     bool m_ok = true;
     for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % UF_STAGES;
-      m_ok = __all_sync(0xFFFFFFFFu, mbar_wait(&full_bar[s], (kb / UF_STAGES) & 1, wait_ns));
+      const int s = kb % NST;
+      m_ok = __all_sync(0xFFFFFFFFu, mbar_wait(&full_bar[s], (kb / NST) & 1, wait_ns));
       if (!m_ok) break;
       tc_fence_after();
-      const uint32_t a0 = u_ring + (uint32_t)s * stage_bytes;
+      const uint32_t a0 = ring + (uint32_t)s * stage_bytes;
       const uint64_t ah = umma_smem_desc(a0), am = umma_smem_desc(a0 + (uint32_t)a_bytes),
                      al = umma_smem_desc(a0 + 2u * (uint32_t)a_bytes);
       const uint64_t bh = umma_smem_desc(a0 + 3u * (uint32_t)a_bytes);   // [h' | m' | l'] start here

@@ -123,6 +123,15 @@ def test_lists_merged_over_splits(ctx, eps, keep):
     run_v(ctx, 98, 1, 18, 40, 1024, keep, p=fo.Params(eps=eps))
 
 
+@pytest.mark.parametrize("batch,n_src,n_tgt,dim", [
+    (1, 1, 16, 64), (1, 33, 65, 192), (2, 95, 31, 576), (1, 64, 200, 1024), (3, 100, 300, 320), (8, 128, 257, 128)])
+def test_correlate_fp32_tiles(ctx, batch, n_src, n_tgt, dim):
+    """Tiles of 32 x 32 and 128 x 64 around their edges, fewer and more k-blocks than slots in flight."""
+    n = n_src + n_tgt
+    gw = next(g for g in (16, 11, 9, 7, 5, 4, 3, 2, 1) if n % g == 0)
+    run_v(ctx, 99, batch, n // gw, gw, dim, n_tgt, dtype="fp32")
+
+
 @pytest.mark.parametrize("batch,gh,gw,dim", [(149, 7, 7, 64), (170, 10, 10, 256), (3, 44, 44, 512), (1, 3, 11, 64), (2, 33, 3, 1280),
                                                (1, 5, 5, 2048)])
 def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
