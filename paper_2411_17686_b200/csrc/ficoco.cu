@@ -477,9 +477,10 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
 #define FICOCO_FUSED_ATTR(TT, V) \
     cudaFuncSetAttribute(k_filter_fused<TT, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM)
     FICOCO_FUSED_ATTR(float, 1); FICOCO_FUSED_ATTR(float, 2); FICOCO_FUSED_ATTR(float, 4);
-    FICOCO_FUSED_ATTR(float, 5); FICOCO_FUSED_ATTR(float, 8);
+    FICOCO_FUSED_ATTR(float, 5); FICOCO_FUSED_ATTR(float, 6); FICOCO_FUSED_ATTR(float, 7); FICOCO_FUSED_ATTR(float, 8);
     FICOCO_FUSED_ATTR(__nv_bfloat16, 1); FICOCO_FUSED_ATTR(__nv_bfloat16, 2); FICOCO_FUSED_ATTR(__nv_bfloat16, 4);
-    FICOCO_FUSED_ATTR(__nv_bfloat16, 5); FICOCO_FUSED_ATTR(__nv_bfloat16, 8);
+    FICOCO_FUSED_ATTR(__nv_bfloat16, 5); FICOCO_FUSED_ATTR(__nv_bfloat16, 6); FICOCO_FUSED_ATTR(__nv_bfloat16, 7);
+    FICOCO_FUSED_ATTR(__nv_bfloat16, 8);
 #undef FICOCO_FUSED_ATTR
   }
   cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
@@ -614,15 +615,15 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     f_rc = best.rc;
     f_cap = best.cap;
     // A deal that comes out uneven leaves SMs idle through both passes; from about 64 MB of tokens on three plain
-    // kernels then make up for their launches and the second read.  Both paths forced on 192 uniform batches (257,
-    // 577, 1025 and 2305 tokens, 15 to 340 MB; 768, 1024, 1664, 2048 values in bf16, 768, 1024 in fp32), time of the
-    // whole step fused / unfused:
-    //   rows of up to 256 vectors but no more than 1024 values: uneven and large 1.00 to 1.21 (mean 1.065 of 30),
-    //   uneven but below 64 MB 0.97 to 1.27 (four), even 0.94 to 1.08 (mean 1.003 of 94; the fused path is ahead above
-    //   64 MB, the plain kernels below about 25);
-    //   1664 and 2048 values in bf16, where a warp of the fused kernel holds one row at a time: 1.06 to 1.54, so the
-    //   plain kernels are ahead in all 64 and the rule leaves 6 to 31 % there where the deal is even.
-    if (best.cost < 0 || (best.cost * 100 > (best.even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024)) p->fused = false;
+    // kernels then make up for their launches and the second read.  Whole step, fused / unfused, both paths forced:
+    //   rows of up to 1024 values, uneven and large: 1.00 to 1.20 (768, 1024 in bf16, 85 to 300 images of 256 to 2304
+    //   tokens; 192 batches on the kernels before these: 1.065 in the mean of 30, even ones 1.003 of 94);
+    //   1280 values, uneven and large: 0.97 to 1.07;
+    //   1408 and 1664 values in bf16: 0.87 to 0.98 uneven and large, 0.83 to 1.07 otherwise (the largest for one image);
+    //   2048 values in bf16, where a warp of the fused kernel holds one row at a time and spills: 1.04 to 1.16 of all nine.
+    const bool wide_bf16 = esz == 2 && p->f_vpl >= 6;
+    const bool uneven = best.cost * 100 > (best.even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024;
+    if (best.cost < 0 || (wide_bf16 ? p->f_vpl == 8 : uneven)) p->fused = false;
     // shared memory: ring stages of 16 rows (the selection works in them), the fold area, a score per row of a piece
     const size_t stage = (size_t)FROWS * key.dim * esz, fixed = (size_t)FFOLD * key.dim * 4 + (size_t)best.max_piece * 4 + 256;
     int ns = F_SMEM > fixed ? (int)((F_SMEM - fixed) / stage) : 0;
@@ -1040,6 +1041,8 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     else if (vpl <= 2) FICOCO_FUSED_GO(2);
     else if (vpl <= 4) FICOCO_FUSED_GO(4);
     else if (vpl <= 5) FICOCO_FUSED_GO(5);
+    else if (vpl <= 6) FICOCO_FUSED_GO(6);
+    else if (vpl <= 7) FICOCO_FUSED_GO(7);
     else FICOCO_FUSED_GO(8);
 #undef FICOCO_FUSED_GO
     if (fe != cudaSuccess) { c->last_cuda = (int)fe; return FICOCO_ERR_CUDA; }

@@ -133,7 +133,7 @@ def test_correlate_fp32_tiles(ctx, batch, n_src, n_tgt, dim):
 
 
 @pytest.mark.parametrize("batch,gh,gw,dim", [(149, 7, 7, 64), (170, 10, 10, 256), (3, 44, 44, 512), (1, 3, 11, 64), (2, 33, 3, 1280),
-                                               (1, 5, 5, 2048)])
+                                               (1, 5, 5, 2048), (2, 7, 9, 1408), (2, 7, 9, 1664)])
 def test_pieces_dealt_to_filter_ctas(ctx, batch, gh, gw, dim):
     """More images than SMs, images of several pieces, and warps without a row."""
     run_v(ctx, 94, batch, gh, gw, dim, gh * gw // 2)
