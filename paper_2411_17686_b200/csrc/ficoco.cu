@@ -495,12 +495,16 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   // neighbours; what the driver picks by itself depends on the neighbours (256 x 577 tokens: column sums 74 or 98 us, the
   // step 315 or 339; relation map: the step 41.8 or 44.8; 28 and 57 % like 43).
   {
-    auto carve = [](auto* kernel) { cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 43); };
+    auto carve = [](auto* kernel, int percent = 43) { cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent); };
 #define FICOCO_COLSUM_CARVE(V) carve(k_colsum<float, V, true>); carve(k_colsum<__nv_bfloat16, V, true>)
     FICOCO_COLSUM_CARVE(1); FICOCO_COLSUM_CARVE(2); FICOCO_COLSUM_CARVE(4); FICOCO_COLSUM_CARVE(5); FICOCO_COLSUM_CARVE(8);
 #undef FICOCO_COLSUM_CARVE
     carve(k_score_rel); carve(k_correlate_rel<2>); carve(k_correlate_rel<4>); carve(k_correlate_rel<16>);
     carve(k_select<true>); carve(k_select<false>);
+    // The wide column sums with the head mean have up to 128 KB of loads in flight per SM, which L1 has to hold: as much L1 as
+    // there is (16 FiCoCo-L sequences of 4096 91.7 us, four 51.5; the driver's choice 93.4 and 53.0, 100 KB 101.2 and 57.7).
+    carve(k_colsum_wide<float, 2, 8>, 0); carve(k_colsum_wide<float, 4, 4>, 0);
+    carve(k_colsum_wide<__nv_bfloat16, 2, 8>, 0); carve(k_colsum_wide<__nv_bfloat16, 4, 4>, 0);
   }
   cudaFuncSetAttribute(k_score<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   cudaFuncSetAttribute(k_score<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
@@ -1009,7 +1013,8 @@ template <class T>
 int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* attn, int attn_rows,
              float cA, const int* pos, int window, float coef, int penalty, const float* tmean, int M,
              float gamma, T* out_tokens, int* kept_idx, int* pos_out, float* scores_out,
-             cudaStream_t st, bool back_to_back, const float* rel = nullptr) {
+             cudaStream_t st, bool back_to_back, const float* rel = nullptr, const float* t2v = nullptr,
+             int t2v_heads = 0) {
   constexpr int E = VecTraits<T>::E;
   const int nvec = D / E;
   const int vpl = (nvec + 31) / 32;
@@ -1032,6 +1037,14 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   // reads only once whatever is in front of it on the stream is complete.
   const int overlap_prev = back_to_back && inputs_clear_of_last_outputs(c->device, st, in_spans, 3) ? 1 : 2;
   record_last_outputs(c->device, st, out_spans, N_SPANS);
+  const bool wide = !p->fused && !rel && vpl > 8 && nvec <= 1024;   // rows of 257 .. 1024 16-byte vectors: CTA-wide rows
+  // FiCoCo-L: head mean of the text->vision attention, in the grid of the column sums where rows are CTA-wide
+  const int mn = t2v ? M * p->max_np : 0, head_ctas = p->key.batch * head_mean_parts(mn);
+  if (t2v && !wide) {
+    prof_tick(c, st, "head_mean");
+    launch_dependent(k_head_mean, dim3(head_ctas), 256, 0, st, t2v, t2v_heads, mn, c->tmean);
+    c->launches += 1;
+  }
   if (p->fused) {
     prof_tick(c, st, "filter_fused");
     cudaError_t fe;
@@ -1054,7 +1067,6 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
         rel, p->d_desc, p->d_rows, attn, attn_rows, cA, p->key.rel == 2 ? 1 : 0, c->s_raw);
     c->launches += 1;
   } else {
-  const bool wide = vpl > 8 && nvec <= 1024;   // rows of 257 .. 1024 16-byte vectors: CTA-wide rows
   prof_tick(c, st, (vpl <= 8 || wide) ? "colsum" : "rownorm");
   if (vpl <= 8) {
     if (vpl <= 1) launch_colsum_fused<T, 1>(c, p, tok, D, st);
@@ -1064,10 +1076,12 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     else launch_colsum_fused<T, 8>(c, p, tok, D, st);
     c->launches += 1;
   } else if (wide) {
-    if (nvec <= 512) launch_dependent(k_colsum_wide<T, 2, 8>, dim3(p->n_rows), 256, 0, st,
-      tok, D, p->d_desc, p->d_rows, c->rn, c->partial, tmean != nullptr ? 1 : 0);
-    else launch_dependent(k_colsum_wide<T, 4, 4>, dim3(p->n_rows), 256, 0, st,
-      tok, D, p->d_desc, p->d_rows, c->rn, c->partial, tmean != nullptr ? 1 : 0);
+#define FICOCO_WIDE_GO(NV, RB)                                                                              \
+  launch_dependent(k_colsum_wide<T, NV, RB>, dim3(p->n_rows + head_ctas), 256, 0, st, tok, D, p->d_desc, p->d_rows, \
+                   c->rn, c->partial, p->n_rows, t2v, t2v_heads, mn, c->tmean)
+    if (nvec <= 512) FICOCO_WIDE_GO(2, 8);
+    else FICOCO_WIDE_GO(4, 4);
+#undef FICOCO_WIDE_GO
     c->launches += 1;
   } else {
     launch_dependent(k_rownorm<T>, dim3(p->n_rows), 256, 0, st,
@@ -1412,18 +1426,15 @@ extern "C" int ficoco_l_reduce(ficoco_ctx* c, const ficoco_l_args* a, const fico
   if (rc) return rc;
   c->last_plan = p;
   c->launches = 0;
-  prof_tick(c, st, "head_mean");
-  launch_dependent(k_head_mean, dim3(a->batch * a->n_text), 256, 0, st,
-      a->attn_t2v, a->heads, a->n_text, a->n_vision, c->tmean);
-  c->launches += 1;
   if (a->dtype == FICOCO_BF16)
     return run_step<__nv_bfloat16>(c, p, (const __nv_bfloat16*)a->tokens, a->dim, c->tmean, a->n_text,
                                    (float)prm->beta, nullptr, 1, 1.0f, 0, c->tmean, a->n_text,
                                    (float)prm->gamma, (__nv_bfloat16*)a->out_tokens, a->kept_idx, nullptr,
-                                   a->scores_out, st, false);
+                                   a->scores_out, st, false, nullptr, a->attn_t2v, a->heads);
   return run_step<float>(c, p, (const float*)a->tokens, a->dim, c->tmean, a->n_text, (float)prm->beta,
                          nullptr, 1, 1.0f, 0, c->tmean, a->n_text, (float)prm->gamma,
-                         (float*)a->out_tokens, a->kept_idx, nullptr, a->scores_out, st, false);
+                         (float*)a->out_tokens, a->kept_idx, nullptr, a->scores_out, st, false, nullptr, a->attn_t2v,
+                         a->heads);
 }
 
 extern "C" int ficoco_status(ficoco_ctx* c, void* cuda_stream, int* device_status) {

@@ -357,11 +357,65 @@ __global__ void __launch_bounds__(256) k_score(const T* __restrict__ tokens, int
 }
 
 // ---------------------------------------------------------------------------------------
+// FiCoCo-L: head mean of the text->vision attention, t[b, k, i] = (1/H) sum_h A[b, h, k, i].
+// The M * N values of a sequence are cut into parts of HM_PART, one CTA per part; a thread takes four
+// values, 16 heads in flight, added in head order (16 sequences of 2048, 75 MB of attention: whole step 68.7 us, with
+// eight heads in flight 76.1).
+// ---------------------------------------------------------------------------------------
+constexpr int HM_PART = 1024;
+__host__ __device__ __forceinline__ int head_mean_parts(int MN) { return (MN + HM_PART - 1) / HM_PART; }
+
+__device__ __forceinline__ void head_mean_part(const float* __restrict__ attn, int H, int MN, int part,
+                                               float* __restrict__ t) {
+  const int per_seq = head_mean_parts(MN), b = part / per_seq, i0 = part % per_seq * HM_PART;
+  const float inv_h = 1.0f / (float)H;
+  const float* src = attn + (size_t)b * H * MN;
+  float* dst = t + (size_t)b * MN;
+  if ((MN & 3) == 0 && (reinterpret_cast<uintptr_t>(attn) & 15) == 0 && (reinterpret_cast<uintptr_t>(t) & 15) == 0) {
+    const int i = i0 + 4 * threadIdx.x;
+    if (i >= MN) return;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int h0 = 0; h0 < H; h0 += 16) {
+      float4 a[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        a[q] = h0 + q < H ? __ldg(reinterpret_cast<const float4*>(src + (size_t)(h0 + q) * MN + i))
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) { s.x += a[q].x; s.y += a[q].y; s.z += a[q].z; s.w += a[q].w; }
+    }
+    *reinterpret_cast<float4*>(dst + i) = make_float4(s.x * inv_h, s.y * inv_h, s.z * inv_h, s.w * inv_h);
+    return;
+  }
+  for (int i = i0 + threadIdx.x; i < min(MN, i0 + HM_PART); i += 256) {
+    float s = 0.f;
+    for (int h0 = 0; h0 < H; h0 += 16) {
+      float a[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) a[q] = h0 + q < H ? __ldg(src + (size_t)(h0 + q) * MN + i) : 0.f;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) s += a[q];
+    }
+    dst[i] = s * inv_h;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_head_mean(const float* __restrict__ attn, int H, int MN, float* __restrict__ t) {
+  grid_dep_wait();
+  grid_dep_launch();
+  head_mean_part(attn, H, MN, blockIdx.x, t);
+}
+
+// ---------------------------------------------------------------------------------------
 // Wide rows (more than 256 16-byte vectors: hidden 4096 in bf16): a row no longer fits one
 // warp's registers, so the CTA's 256 threads own the row's column vectors (NV each) and rows
 // go through in batches of RB.  A per-row sum is folded lane -> warp -> the 8 warps in order.
 //   k_colsum_wide: row norms and the chunk's column sums of the normalised rows in one read;
-//                  every thread keeps the sums of its own columns, so there is no fold at the end
+//                  every thread keeps the sums of its own columns, so there is no fold at the end.  FiCoCo-L's head mean,
+//                  which shares nothing with them, is taken by other CTAs of the same grid, so that the two reads of
+//                  memory run into one another (behind one another: 16 sequences of 4096 92.1 us, one 50.4, eight of 3584
+//                  74.9).  As two grids, the second without a wait ahead of its reads, it was 90.9, 45.1 and 68.4, but a
+//                  grid is promised to see what the grid it waits for wrote, not what grids before that one did.
 //   k_score_wide:  Eq. 1 with the image's column sums held in registers; a batch's rows are asked for under the barrier of
 //                  the batch before, the first ones and the attention ahead of everything (16 sequences of 4096: with
 //                  the overlap of head mean and column sums the step 101.3 -> 93.1 us, one sequence 49.4 -> 45.0)
@@ -389,16 +443,22 @@ __global__ void __launch_bounds__(256, 2) k_colsum_wide(const T* __restrict__ to
                                                      const ImgDesc* __restrict__ desc,
                                                      const WorkItem* __restrict__ work,
                                                      float* __restrict__ rn_out, float* __restrict__ partial,
-                                                     int behind_head_mean) {
+                                                     int n_rows, const float* __restrict__ t2v, int H, int MN,
+                                                     float* __restrict__ t) {
   constexpr int E = VecTraits<T>::E;
   __shared__ __align__(16) float red[2][RB][8];
-  const WorkItem w = work[blockIdx.x];
+  // The CTAs behind the first n_rows take the head mean: what takes longest comes first (head mean first: 10 sequences of 4096
+  // 74.0 instead of 70.2 us, 32 164.9 and 161.8, eight of 3584 70.9 and 67.5; only 16 of 4096, whose rows fill the GPU once,
+  // the other way round, 89.0 and 91.7).
+  const bool rows_here = (int)blockIdx.x < n_rows;
+  const WorkItem w = work[rows_here ? blockIdx.x : 0];
   const ImgDesc d = desc[w.img];
-  // Behind k_head_mean, which lets this grid in only when everything before it is complete and writes nothing that is
-  // read here: the rows need not wait for it, so the two reads of memory run into one another.  It is waited for at the
-  // end, so that a grid that finds this one complete finds that one complete too.
-  if (!behind_head_mean) grid_dep_wait();
+  grid_dep_wait();
   grid_dep_launch();
+  if (!rows_here) {
+    head_mean_part(t2v, H, MN, (int)blockIdx.x - n_rows, t);
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nvec = D / E;
   const T* base = tokens + (size_t)(d.row0 + d.n_cls + w.r0) * D;
@@ -453,7 +513,6 @@ __global__ void __launch_bounds__(256, 2) k_colsum_wide(const T* __restrict__ to
         *reinterpret_cast<float4*>(out + (size_t)v * E + e) = make_float4(acc[k][e], acc[k][e + 1], acc[k][e + 2], acc[k][e + 3]);
     }
   }
-  if (behind_head_mean) grid_dep_wait();
 }
 
 template <class T, int NV, int RB>
@@ -519,48 +578,6 @@ __global__ void __launch_bounds__(256) k_score_wide(const T* __restrict__ tokens
 #pragma unroll
     for (int q = 0; q < 8; ++q) s += part[q * w.nrows + r];
     s_raw[d.patch0 + w.r0 + r] = cA * vrow[r] - (1.0f - cA) * (s * inv_h);
-  }
-}
-
-// ---------------------------------------------------------------------------------------
-// FiCoCo-L: head mean of the text->vision attention, t[b, k, i] = (1/H) sum_h A[b, h, k, i].
-// One CTA per (sequence, text row).
-// ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_head_mean(const float* __restrict__ attn, int H, int M,
-                                                   int N, float* __restrict__ t) {
-  grid_dep_wait();
-  grid_dep_launch();
-  const int b = blockIdx.x / M, k = blockIdx.x % M;
-  const float inv_h = 1.0f / (float)H;
-  const float* src = attn + ((size_t)b * H * M + k) * N;
-  float* dst = t + ((size_t)b * M + k) * N;
-  if ((N & 3) == 0 && (reinterpret_cast<uintptr_t>(attn) & 15) == 0 && (reinterpret_cast<uintptr_t>(t) & 15) == 0) {
-    // four tokens per thread, eight heads in flight, added in head order
-    for (int i = threadIdx.x * 4; i < N; i += 1024) {
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int h0 = 0; h0 < H; h0 += 8) {
-        float4 a[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          a[q] = h0 + q < H ? __ldg(reinterpret_cast<const float4*>(src + (size_t)(h0 + q) * M * N + i))
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) { s.x += a[q].x; s.y += a[q].y; s.z += a[q].z; s.w += a[q].w; }
-      }
-      *reinterpret_cast<float4*>(dst + i) = make_float4(s.x * inv_h, s.y * inv_h, s.z * inv_h, s.w * inv_h);
-    }
-    return;
-  }
-  for (int i = threadIdx.x; i < N; i += 256) {
-    float s = 0.f;
-    for (int h0 = 0; h0 < H; h0 += 8) {      // eight heads in flight, added in head order
-      float a[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) a[q] = h0 + q < H ? __ldg(src + (size_t)(h0 + q) * M * N + i) : 0.f;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) s += a[q];
-    }
-    dst[i] = s * inv_h;
   }
 }
 

@@ -117,6 +117,22 @@ def test_correlate_text_weights(n_vision, n_text, dim, keep, p):
         c.close()
 
 
+@pytest.mark.parametrize("n_vision,n_text,dim,heads,dtype", [
+    (37, 3, 2112, 17, "bf16"),         # 111 attention values, no multiple of four; one head more than are in flight
+    (130, 8, 2112, 3, "bf16"),         # 1040: a second part of 16 values
+    (64, 16, 4096, 16, "fp32"),        # 1024: one full part; rows of 16 KB
+    (205, 5, 1032, 2, "fp32"),         # 1025: a second part of one value; rows just past the narrower kernels
+], ids=["scalar", "two-parts", "full-part", "one-value"])
+def test_head_mean_beside_column_sums(n_vision, n_text, dim, heads, dtype):
+    c = binding.Context(max_tokens=3 * (n_vision + n_text), max_dim=dim, max_batch=3, max_text=n_text, device=0)
+    try:
+        b = synth.make_l_batch(100, 3, n_vision, n_text, dim, heads, n_vision // 2, dtype)
+        gaps.repair_l(b, fo.Params())
+        parity.run_and_compare_l(c, b, fo.Params(), DEV, what=f"L {n_vision} + {n_text}, {dim}, {heads} heads")
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("eps,keep", [(0.998, 96), (0.9, 96), (0.9, 150)], ids=["2", "11", "16"])
 def test_lists_merged_over_splits(ctx, eps, keep):
     """One image, whose tiles are split over many CTAs: lists of 2 to 16 entries merged by groups of lanes."""

@@ -461,6 +461,53 @@ def test_step_behind_a_foreign_producer_kernel(ctx):
             assert np.array_equal(a, binding.to_numpy(b))
 
 
+@pytest.mark.parametrize("captured", [False, True], ids=["called", "captured"])
+def test_wide_l_step_behind_a_foreign_producer_kernel(captured):
+    """FiCoCo-L at 4096, whose first grid reads tokens and attention: both are written by other kernels of the same stream
+    right before the step, other bytes every time, and read in stream order."""
+    batches = [packing.pack_l(synth.make_l_batch(98 + i, 4, 320, 24, 4096, 8, 64), DEV) for i in range(2)]
+    p0 = batches[0]
+    c = binding.Context(max_tokens=4 * 344, max_dim=4096, max_batch=4, max_text=24, device=0)
+    try:
+        def step(tok, attn, **kw):
+            return c.ficoco_l_reduce(tok, attn, p0.keep, p0.n_vision, p0.n_text, p0.heads, **kw)
+
+        want = []
+        for pk in batches:
+            r = step(pk.tokens, pk.attn_t2v)
+            torch.cuda.synchronize()
+            want.append([binding.to_numpy(t) for t in (r.out_tokens, r.kept_idx)])
+        tok, attn = torch.zeros_like(p0.tokens), torch.zeros_like(p0.attn_t2v)
+        out = [[torch.zeros_like(r.out_tokens), torch.zeros_like(r.kept_idx)] for _ in batches]
+        st = torch.cuda.Stream()
+
+        def chain():
+            for pk, (o, k) in zip(batches, out):
+                tok.zero_(); attn.zero_()
+                tok.copy_(pk.tokens); attn.copy_(pk.attn_t2v)          # the producers
+                step(tok, attn, out_tokens=o, kept_idx=k, stream=st.cuda_stream)
+
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        if captured:
+            with torch.cuda.graph(g, stream=st):
+                chain()
+        for rep in range(5):
+            for o, k in out:
+                o.zero_(); k.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(st):
+                g.replay() if captured else chain()
+            torch.cuda.synchronize()
+            for got, exp in zip(out, want):
+                for a, b in zip(got, exp):
+                    assert np.array_equal(binding.to_numpy(a), b), f"repetition {rep}"
+        assert c.ficoco_status() == 0
+    finally:
+        del g
+        c.close()
+
+
 def test_planned_ragged_shape_is_captured_into_a_graph():
     """A ragged shape the context has never seen: ficoco_v_plan builds its plan ahead of time, after
     which the reduce step is captured into a CUDA graph (no synchronisation, no allocation inside
