@@ -1189,10 +1189,9 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     c->launches += 1;
   }
   prof_tick(c, st, "merge_compact");
-  const int after_correlate = p->n_corr > 0 ? 1 : 0;   // else the grid before may be the filter itself
   launch_dependent(k_merge_rows<T>, dim3(p->n_out), MTHREADS, p->m_smem, st, tok, D, (const ImgDesc*)p->d_desc,
                    (const WorkItem*)p->d_out, (const int*)c->S_idx, (const int*)c->T_idx,
-                   (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, after_correlate, c->status,
+                   (const int*)c->e_tgt, (const float*)c->e_w, out_tokens, c->status,
                    p->fused ? c->img_cnt + (size_t)c->last_parity * 3 * c->max_batch : (int*)nullptr,
                    p->fused ? 3 * c->max_batch : 0, c->wait_ns);
   c->launches += 1;

@@ -230,8 +230,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
   }
   // Everything above touches only launch-constant plan data and this CTA's own resources, so it
   // may run while the filter grid is still finishing; the index lists and norms it wrote are
-  // read below.  The dependent (merge) grid is released only after this wait, so by the time
-  // any of its blocks starts, the filter grid is complete as well.
+  // read below.
   FICOCO_PHASE(1, 1);
   grid_dep_wait();
   grid_dep_launch();

@@ -2,7 +2,8 @@
 //
 // Every kernel of a step is launched under the tail of the grid before it (programmatic stream serialization): it
 // reads its plan entries, which are constants, then waits for that grid to be complete and only then lets the next
-// one in.  A grid that runs therefore finds everything before its predecessor complete as well.
+// one in.  All else that it reads or writes it touches behind its own wait: nothing promises a grid that what lies before its
+// predecessor is visible to it any earlier.
 #pragma once
 #include <math_constants.h>
 #include <type_traits>

@@ -85,11 +85,13 @@ __device__ __noinline__ void merge_long_list(const unsigned char* own, const uin
 // with many sources lie close together (neighbouring patches look alike), and dealt out like cards they load the
 // CTAs of an image about alike (16 ragged images: the busiest CTA 38 us after its start, 14 in the median, when the
 // rows of a CTA were consecutive).
-//   rows    the input rows of its output rows are fetched into shared memory by bulk copies (TMA) as soon as the
-//           index lists exist, i.e. under the tail of the correlate grid;
+//   rows    the input rows of its output rows are fetched into shared memory by bulk copies (TMA) that the last warp asks
+//           for as soon as the correlate grid is complete, while the others file the entries (asked for under that grid's
+//           tail, ahead of the wait, which nothing promises to be sound: 32 x 577 59.3 us instead of 59.0, relation map 42.2
+//           and 43.2, 16 FiCoCo-L sequences 93.2 and 94.1, 256 x 577 316 and 314; by a warp that files as well: 59.7);
 //   file    the image's (source -> target) entries that hit its rows are filed into per-row lists in shared
 //           memory, ordered by discarded token; no atomics touch floats; one pass over the entries, four loads in
-//           flight per thread;
+//           flight per thread of the other 15 warps;
 //   copies  a row that nothing is folded into leaves by a bulk store from shared memory: no thread touches it;
 //   merge   out_j = (x_j + sum_{i in I_j} alpha_ij x_i) / (1 + sum alpha_ij), rounded once.  A unit is one row and
 //           512 bytes of it, or 128 where its list is long; a warp adds the row's sources, several of them in flight,
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
     const T* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
     const WorkItem* __restrict__ work, const int* __restrict__ S_idx, const int* __restrict__ T_idx,
     const int* __restrict__ e_tgt, const float* __restrict__ e_w, T* __restrict__ out,
-    int index_before_wait, unsigned* __restrict__ status, int* __restrict__ filter_cnt, int n_filter_cnt,
+    unsigned* __restrict__ status, int* __restrict__ filter_cnt, int n_filter_cnt,
     unsigned long long wait_ns) {
   constexpr int E = VecTraits<T>::E;
   extern __shared__ __align__(128) unsigned char stage[];     // [rows][row bytes]
@@ -132,21 +134,31 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
   const int stride = w.aux;                      // row r of the CTA is output row w.r0 + r * stride of the image
   const float inv_stride = 1.0f / (float)stride;
   const int n_ent = d.n_src * L;
-  const T* pbase = tokens + (size_t)(d.row0 + d.n_cls) * D;
-
   if (tid < MROWS) cnt[tid] = 0;
-  if (tid == 0) { n_match = 0; next_unit = MWARPS; }
-  // When the grid before this one is a correlate grid, the filter grid (which wrote T_idx) had
-  // completed before this grid could start, so the rows may be looked up and fetched under that
-  // grid's tail; otherwise wait first.
-  if (!index_before_wait) grid_dep_wait();
-  if (warp == 0) {
+  if (tid == 0) {
+    n_match = 0;
+    next_unit = MWARPS;
+    mbar_init(&row_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  grid_dep_wait();
+  const T* pbase = tokens + (size_t)(d.row0 + d.n_cls) * D;
+  // The filter grid of this step is complete: its per-image counters are cleared for whichever launch
+  // uses that set next (launches replayed from graphs need not alternate between the two sets).  The
+  // stores are fenced and the CTA synchronised before it releases the dependent grid.
+  if (filter_cnt != nullptr && blockIdx.x == 0) {
+    for (int i = tid; i < n_filter_cnt; i += MTHREADS) filter_cnt[i] = 0;
+    __threadfence();
+    __syncthreads();
+  }
+  grid_dep_launch();   // correlate is complete: the next step's filter may stream its rows under our tail
+  FICOCO_PHASE(2, 1);
+  // a step whose filter or correlate grid gave up has no valid index lists: write nothing
+  if (tid == 0) dead = (*reinterpret_cast<const volatile unsigned*>(status) & STATUS_TIMEOUT) ? 1 : 0;
+  if (warp == MWARPS - 1) {
     // input row of every output row (CLS / preserved token / trailing text row; -1: the additional token, which
     // k_convergent_token writes)
-    if (lane == 0) {
-      mbar_init(&row_bar, 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
     int srow[2], n = 0;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -169,25 +181,12 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
         bulk_load(stage + (size_t)(lane + 32 * j) * row_bytes, tokens + (size_t)(d.row0 + srow[j]) * D, (uint32_t)row_bytes,
                   &row_bar);
   }
-  __syncthreads();
-  if (index_before_wait) grid_dep_wait();
-  // The filter grid of this step is complete: its per-image counters are cleared for whichever launch
-  // uses that set next (launches replayed from graphs need not alternate between the two sets).  The
-  // stores are fenced and the CTA synchronised before it releases the dependent grid.
-  if (filter_cnt != nullptr && blockIdx.x == 0) {
-    for (int i = tid; i < n_filter_cnt; i += MTHREADS) filter_cnt[i] = 0;
-    __threadfence();
-    __syncthreads();
-  }
-  grid_dep_launch();   // correlate is complete: the next step's filter may stream its rows under our tail
-  FICOCO_PHASE(2, 1);
-  // a step whose filter or correlate grid gave up has no valid index lists: write nothing
-  if (tid == 0) dead = (*reinterpret_cast<const volatile unsigned*>(status) & STATUS_TIMEOUT) ? 1 : 0;
   // ---- file the entries that hit this CTA's rows ----------------------------------------------------
-  for (int e0 = tid; e0 < n_ent; e0 += 4 * MTHREADS) {
+  constexpr int FILERS = MTHREADS - 32;
+  for (int e0 = tid; e0 < n_ent && tid < FILERS; e0 += 4 * FILERS) {
     int t[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) t[i] = e0 + MTHREADS * i < n_ent ? e_tgt[d.ent0 + e0 + MTHREADS * i] : -1;
+    for (int i = 0; i < 4; ++i) t[i] = e0 + FILERS * i < n_ent ? e_tgt[d.ent0 + e0 + FILERS * i] : -1;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (t[i] >= 0) {
@@ -196,7 +195,7 @@ __global__ void __launch_bounds__(MTHREADS, 2) k_merge_rows(
         if (o < 0 || r * stride != o || r >= w.nrows) continue;
         const int slot = atomicAdd(&cnt[r], 1), k = atomicAdd(&n_match, 1);
         if (k < MLIST) {
-          m_e[k] = e0 + MTHREADS * i;
+          m_e[k] = e0 + FILERS * i;
           m_rs[k] = (unsigned short)(r << 10 | (slot & 1023));
         }
       }
