@@ -992,11 +992,12 @@ cudaError_t launch_filter_fused(ficoco_ctx* c, const Plan* p, const T* tok, int 
   cfg.attrs = at;
   cfg.numAttrs = (c->coop_pdl_ok && overlap_prev) ? 2 : 1;   // 1: inputs independent of the step before; 2: fed by it
   c->last_parity = (int)(c->epoch++ & 1);
+  const size_t set = 3 * (size_t)c->max_batch;
   return cudaLaunchKernelEx(&cfg, k_filter_fused<T, VPL>, tok, D, (const ImgDesc*)p->d_desc,
                             (const WorkItem*)p->d_rows, (const int*)p->d_ctafirst, c->rn, c->partial, attn,
-                            attn_rows, cA, c->s_raw, c->img_cnt, p->key.batch, pos, window, coef, penalty,
-                            c->s_pen, scores_out, c->S_idx, c->T_idx, kept_idx, pos_out, c->status,
-                            p->f_nstage, c->last_parity, 3 * c->max_batch, c->wait_ns,
+                            attn_rows, cA, c->s_raw, c->img_cnt + c->last_parity * set, p->key.batch, pos, window, coef,
+                            penalty, c->s_pen, scores_out, c->S_idx, c->T_idx, kept_idx, pos_out, c->status,
+                            p->f_nstage, c->img_cnt + (1 - c->last_parity) * set, (int)set, c->wait_ns,
                             c->dbg_extra_arrivals, (c->coop_pdl_ok && overlap_prev == 2) ? 1 : 0);
 }
 

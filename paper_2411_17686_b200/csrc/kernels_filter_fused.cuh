@@ -11,8 +11,9 @@
 //   select  every CTA that scored a piece waits until all of the image's scores are in, runs the selection on the whole
 //           image and writes the outputs of its own tokens.
 // The inter-CTA waits are polls of per-image counters, bounded by elapsed time (wait_ns).  The
-// counters exist twice; a launch uses the set of its parity and zeroes the other one, so a step
-// that gave up half-way cannot leave counts behind for the step after the next.  The set a launch
+// counters ([0, B) pieces through pass 1, [B, 2B) pieces scored) exist twice; a launch uses the set of its parity and
+// zeroes the whole other one, whatever its batch, behind its wait, so a step that ended before its merge cannot leave counts
+// behind for the step after the next.  The set a launch
 // used is cleared by the merge grid of the same step (which runs once the filter grid is complete
 // and before a later filter grid can start), so launches replayed from CUDA graphs, whose
 // parities are fixed at capture, find their set clean in whatever order they run.
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
     const int* __restrict__ pos, int window, float coef, int penalty, float* __restrict__ s_pen,
     float* __restrict__ scores_out, int* __restrict__ S_idx, int* __restrict__ T_idx,
     int* __restrict__ kept_idx, int* __restrict__ pos_out, unsigned* __restrict__ status,
-    int nstage, int parity, int set_stride, unsigned long long wait_ns, int dbg_extra_arrivals,
+    int nstage, int* __restrict__ other_cnt, int n_other, unsigned long long wait_ns, int dbg_extra_arrivals,
     int dep_wait_first) {
   constexpr int E = VecTraits<T>::E;
   constexpr int F_P2B = VPL <= 4 ? 4 : VPL <= 5 ? 2 : 1;   // rows a warp has in flight from L2 in pass 2
@@ -117,18 +118,6 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
   float* fold = reinterpret_cast<float*>(fs_raw + (size_t)nstage * stage_bytes);   // [FFOLD][D], msum aliases fold[0]
   float* a_s = fold + (size_t)FFOLD * D;                                            // a float per row of the largest piece
   const int p_begin = cta_first[blockIdx.x], p_end = cta_first[blockIdx.x + 1];
-  // counters of this launch: [0, B) pieces through pass 1, [B, 2B) pieces scored ([2B, 3B) unused).
-  // The other set belongs to the launch before and the one after: it is zeroed here for the latter
-  // (the launch before is complete: the correlate grid between the two waited for it).
-  {
-    // (the sets lie set_stride apart whatever the batch of this launch, so that launches of
-    // different plans find and clear each other's counters)
-    int* other = cnt + (parity ? 0 : set_stride);
-    if (blockIdx.x == 0)
-      for (int i = tid; i < set_stride; i += F_NCONS) other[i] = 0;
-    cnt += parity ? set_stride : 0;
-  }
-
   if (lane < nstage) mbar_init(&full_bar[warp][lane], 1);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   if (tid == 0) failed = 0;
@@ -433,10 +422,13 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
 
   FICOCO_PHASE(0, 5);
   if (failed) return;
-  // Up to here the kernel wrote only scratch that no grid but a filter or correlate grid reads,
-  // and those of the step before were complete before this grid could start.  The index lists
-  // and outputs written below are read by the merge grid of the step before: wait for it.
+  // Without dep_wait_first (the caller states that what sits in front is a step of this library) the kernel has by now
+  // written only scratch that no grid but a filter or correlate grid reads, and those of that step had ended before its
+  // merge let this grid in.  The index lists and outputs written below are read by that merge: wait for it.
   grid_dep_wait();
+  // the counters of the launch before, complete by now, are zeroed for the launch after (see the top)
+  if (blockIdx.x == 0)
+    for (int i = tid; i < n_other; i += F_NCONS) other_cnt[i] = 0;
   FICOCO_PHASE(0, 6);
   // selections (the ring is idle now and serves as work area), image by image over this CTA's pieces
   int pi = p_begin;

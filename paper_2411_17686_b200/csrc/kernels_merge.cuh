@@ -87,8 +87,9 @@ __device__ __noinline__ void merge_long_list(const unsigned char* own, const uin
 // rows of a CTA were consecutive).
 //   rows    the input rows of its output rows are fetched into shared memory by bulk copies (TMA) that the last warp asks
 //           for as soon as the correlate grid is complete, while the others file the entries (asked for under that grid's
-//           tail, ahead of the wait, which nothing promises to be sound: 32 x 577 59.3 us instead of 59.0, relation map 42.2
-//           and 43.2, 16 FiCoCo-L sequences 93.2 and 94.1, 256 x 577 316 and 314; by a warp that files as well: 59.7);
+//           tail, ahead of the wait, which nothing promises to be sound: relation map 42.0 us instead of 43.1, 16 FiCoCo-L
+//           sequences 93.4 and 94.0, but 32 x 577 58.9 and 58.4, 256 x 577 318 and 315; by a warp that files as well:
+//           0.7 and 5 us more on the last two);
 //   file    the image's (source -> target) entries that hit its rows are filed into per-row lists in shared
 //           memory, ordered by discarded token; no atomics touch floats; one pass over the entries, four loads in
 //           flight per thread of the other 15 warps;

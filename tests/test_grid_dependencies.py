@@ -27,12 +27,12 @@ def kernels():
 
 
 KERNELS = list(kernels())
-DEPENDENT = [k for k in KERNELS if "grid_dep_wait" in k[2] and k[0] != "k_filter_fused"]
+DEPENDENT = [k for k in KERNELS if "grid_dep_wait" in k[2]]
 
 
 def test_the_dependent_kernels_are_found():
     names = {k[0] for k in DEPENDENT}
-    assert {"k_colsum_wide", "k_head_mean", "k_score_wide", "k_select", "k_correlate_umma",
+    assert {"k_filter_fused", "k_colsum_wide", "k_head_mean", "k_score_wide", "k_select", "k_correlate_umma",
             "k_correlate_umma_f32", "k_correlate_rel", "k_merge_rows", "k_equivalent_token"} <= names
 
 
