@@ -13,6 +13,7 @@
 
 #include "../../include/ficoco.h"
 #include "common.cuh"
+#include "correlate_plan.h"
 #include "filter_plan.h"
 #include "kernels_correlate.cuh"
 #include "kernels_correlate_umma.cuh"
@@ -29,7 +30,6 @@ namespace {
 constexpr int N_PLANS = 16;
 constexpr int PART_PER_TOKEN = 64;   // partial top-list entries budgeted per token row
 constexpr int OUT_ROWS_PER_CTA = 16;  // the merge kernel's work table is sized for this many (wide rows: fewer)
-constexpr int NSPLIT_MAX = 16;
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -80,13 +80,6 @@ struct Plan {
   int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1, um_text_off = 0;
   size_t um_smem = 0;
   std::vector<ImgDesc> h_desc;
-};
-
-// Shared memory of a CTA of the bf16 tensor-core correlate.
-struct UmRing {
-  int nstage = 0, ksub = 1, stage_bytes = 0;
-  int text_off = 0;             // where FiCoCo-L's text weights lie, behind the ring's start
-  size_t smem = 0;
 };
 
 // ---- what the last step on a stream wrote ------------------------------------------------------
@@ -657,97 +650,26 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
 
   // ---- correlate tiling ---------------------------------------------------------------------
   int cols_max = p->umma ? un_max : INT_MAX;
-  auto split_cols = [&](int n_tgt, int ns) {           // columns per split: ns splits, or more if they got too wide
-    ns = std::max(ns, (n_tgt - 1) / cols_max + 1);
-    return ((n_tgt + ns - 1) / ns + col_granule - 1) / col_granule * col_granule;
-  };
-  auto row_tiles = [&](int n_src) { return (n_src + tile_rows_max - 1) / tile_rows_max; };
-  // Shared memory of the bf16 tensor-core correlate: as many stages as fit, with four k-blocks per stage where that
-  // leaves four stages, else two (a stage costs about 400 cycles besides its copies and MMAs: one FiCoCo-L sequence,
-  // 80 rows per CTA: k-loop 15 us with one, 11 with two, 9 with four); a grid of more CTAs than SMs keeps to what lets
-  // two share an SM.
-  auto um_ring = [&](int a_rows, int cols, long long n_ctas) {
-    UmRing r;
-    cols = (cols + 15) / 16 * 16;
-    const size_t kblock = (size_t)(a_rows + cols) * 128;
-    const size_t text = key.mode == 1 ? (size_t)key.n_text * (a_rows + cols) * 4 : 0;
-    // every MMA reads 128 A rows: behind the last k-block there must be room for the rows past the tile
-    const size_t slack = 1024 + (kblock < (size_t)UM * 128 ? (size_t)UM * 128 - kblock : 0);
-    const size_t most = 220 * 1024, budget = n_ctas > c->num_sms ? 106 * 1024 : most;
-    auto fit = [&](int ksub, int ns, size_t limit) {
-      if (r.nstage || (size_t)ns * ksub * kblock + slack + text > limit) return;
-      r.nstage = ns;
-      r.ksub = ksub;
-      r.stage_bytes = (int)(ksub * kblock);
-      r.text_off = (int)((size_t)ns * ksub * kblock + slack - 1024);
-      r.smem = (size_t)ns * ksub * kblock + slack + text;
-    };
-    const int nk = key.dim / UKB;
-    for (const size_t limit : {budget, most}) {        // (FiCoCo-L with much text: rather one CTA per SM)
-      for (int ns = std::min(UM_STAGES, (nk + 3) / 4); ns >= 4; --ns) fit(4, ns, limit);
-      for (int ksub = 2; ksub >= 1; --ksub)
-        for (int ns = std::max(2, std::min(UM_STAGES, (nk + ksub - 1) / ksub)); ns >= 2; --ns) fit(ksub, ns, limit);
-    }
-    // the epilogue halves hand their lists over through the ring
-    r.smem = std::max(r.smem, 1024 + (size_t)UM * KCAP * 8);
-    if (r.smem > most) r.nstage = 0;
-    return r;
-  };
-  // Tile of the bf16 tensor-core correlate: rows, and column splits, by the least estimated time (ns), fitted to the
-  // kernel's time on eleven batches (one to 32 images of 144 to 2880 tokens of 1024, one to 16 FiCoCo-L sequences of 4096)
-  // under twenty tilings each: a chain of phases and k-blocks that no tiling shortens, the rows that a CTA gathers, the
-  // columns that its epilogue reads (with a text term per text token), a trip through L2 where a tile is split and one for
-  // every four entries per lane when its lists are merged.  A second CTA on the SM costs its rows again, and a grid that
-  // needs more than one round of two is on average half empty in the last.  Tiles below 128 rows serve small grids:
-  // one sequence of 576 + 64 tokens of 4096, 512 x 64 entries: 22.5 us in 16 CTAs of 128 x 16, 15 in 128 of 16 x 16;
-  // 32 x 288 tokens, 144 x 144 entries: 9.25 us in tiles of 72 x 80, 8.75 in 48 x 144 (no split, no counters); 32 x 576
-  // tokens take 13.5 us in tiles of 96 x 96 and 22 to 82 in any that make a second round.
+  auto split_cols = [&](int n_tgt, int ns) { return split_columns(n_tgt, ns, cols_max, col_granule); };
   int want_split = 1;
   if (p->umma && !p->um_f32) {
-    double best = 0;
-    int best_rows = tile_rows_max;
-    const double k_scale = key.dim / 1024.0, text_scale = key.mode == 1 ? 1.0 + key.n_text / 9.5 : 1.0;
-    const long long wave = 2LL * c->num_sms;
-    for (int t : {128, 64, 32, 16}) {
-      tile_rows_max = t;
-      for (int ws = 1; ws <= NSPLIT_MAX; ++ws) {
-        long long n_ctas = 0, rows_gathered = 0, cols = 0, entries = 0;
-        int rows_most = 8, cols_most = 16, list_most = 0;
-        for (int b = 0; b < B; ++b) {
-          const ImgDesc& d = p->h_desc[b];
-          if (d.list_len == 0) continue;
-          const int cps = split_cols(d.n_tgt, ws), ntile = row_tiles(d.n_src), ns = (d.n_tgt + cps - 1) / cps;
-          const int trows = ((d.n_src + ntile - 1) / ntile + 7) / 8 * 8;
-          const long long n = (long long)ntile * ns;
-          n_ctas += n;
-          rows_gathered += n * (trows + cps);
-          cols += n * cps;
-          entries += (long long)d.n_src * ns * d.list_len;
-          rows_most = std::max(rows_most, trows);
-          cols_most = std::max(cols_most, cps);
-          list_most = std::max(list_most, ns * d.list_len);
-        }
-        if (n_ctas == 0) break;
-        if ((ws > 1 || t < UM) && (n_ctas > c->cap_corr || entries > c->cap_part)) break;
-        if (um_ring(rows_most, cols_most, n_ctas).nstage == 0) continue;
-        int lanes = 1;                                 // lanes that share a token when the lists are merged
-        while (lanes < 8 && rows_most * 2 * lanes <= 256) lanes *= 2;
-        const double rows = k_scale * rows_gathered / n_ctas;
-        double cost = 2900.0 + 2270.0 * k_scale + 9.0 * rows + 10.0 * cols / n_ctas * text_scale +
-                      600.0 * ((list_most + 4 * lanes - 1) / (4 * lanes)) + (list_most > p->max_list ? 700.0 : 0.0);
-        if (n_ctas > c->num_sms) cost += 26.0 * rows;
-        if (n_ctas > wave) cost *= 0.5 * ((double)n_ctas / wave + (double)((n_ctas + wave - 1) / wave));
-        if (best == 0 || cost < best) { best = cost; want_split = ws; best_rows = t; }
-      }
+    std::vector<int> n_src(B), n_tgt(B), len(B);
+    for (int b = 0; b < B; ++b) {
+      n_src[b] = p->h_desc[b].n_src;
+      n_tgt[b] = p->h_desc[b].n_tgt;
+      len[b] = p->h_desc[b].list_len;
     }
-    tile_rows_max = best_rows;
+    const Tiling t = best_tiling(distinct_shapes(n_src.data(), n_tgt.data(), len.data(), B), key.dim, tail, c->num_sms,
+                                 c->cap_corr, c->cap_part);
+    tile_rows_max = t.rows;
+    want_split = t.splits;
   } else {
     // As many splits as give every SM two CTAs, no more than eight with fp32 tiles; a grid of fp32 tiles of
     // 32 x 32 that needs no second CTA on any SM is taken instead (47.0 -> 43.0 us for 64 x 512 entries; twice as many
     // entries as fit: the larger tiles are ahead).
     long long strips = 0;
     for (int b = 0; b < B; ++b)
-      if (p->h_desc[b].list_len > 0) strips += row_tiles(p->h_desc[b].n_src);
+      if (p->h_desc[b].list_len > 0) strips += (p->h_desc[b].n_src + tile_rows_max - 1) / tile_rows_max;
     if (strips > 0) want_split = (int)std::min(std::max(2LL * c->num_sms / strips, 1LL), p->um_f32 ? 8LL : (long long)NSPLIT_MAX);
     long long n_ctas = 0, entries = 0;
     for (int b = 0; b < B; ++b) {
@@ -813,9 +735,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
       const int cps = split_cols(d.n_tgt, want_split), ns = (d.n_tgt + cps - 1) / cps;
       d.nsplit = ns; d.cols_per_split = cps;
       // source tiles of equal size (rounded to 8 rows)
-      const int ntile = (d.n_src + tile_rows_max - 1) / tile_rows_max;
-      int trows = (d.n_src + ntile - 1) / ntile;
-      trows = (trows + 7) / 8 * 8;
+      const int trows = tile_height(d.n_src, tile_rows_max);
       if (trows > um_a_rows) um_a_rows = trows;
       if (cps > um_cols) um_cols = cps;
       for (int s0 = 0; s0 < d.n_src; s0 += trows)
@@ -880,7 +800,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     }
     if (um_a_rows > UM || um_cols > UF_COLS || p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
   } else if (p->umma) {
-    const UmRing r = um_ring(um_a_rows, um_cols, (long long)corr.size());
+    const UmRing r = um_ring(um_a_rows, um_cols, (long long)corr.size(), key.dim, tail, c->num_sms);
     if (r.nstage == 0) return FICOCO_ERR_UNSUPPORTED;
     p->um_a_bytes = um_a_rows * 128;
     p->um_tmem_cols = 32;

@@ -30,15 +30,12 @@
 #include <math_constants.h>
 #include "async_ops.cuh"
 #include "common.cuh"
+#include "correlate_plan.h"
 #include "kernels_correlate.cuh"
 
 namespace ficoco {
 
-constexpr int UM = 128;          // accumulator rows per MMA (one TMEM lane each)
-constexpr int UN_MAX = 256;      // accumulator columns per CTA
-constexpr int UKB = 64;          // bf16 elements per k-block (one 128-byte swizzle row)
 constexpr int UTHREADS = 288;    // warps 0-3 and 5-8 gather + epilogue, warp 4 MMA
-constexpr int UM_STAGES = 8;     // most stages of the operand ring
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
