@@ -22,6 +22,7 @@
 #include "kernels_filter_fused.cuh"
 #include "kernels_merge.cuh"
 #include "kernels_relation.cuh"
+#include "plan_tables.h"
 
 using namespace ficoco;
 
@@ -55,7 +56,8 @@ struct Plan {
   bool valid = false;
   unsigned long long stamp = 0;
   PlanKey key;
-  // device tables (inside the slot)
+  // device tables (one behind the other in the slot)
+  size_t table_bytes = 0;
   ImgDesc* d_desc = nullptr;
   WorkItem* d_rows = nullptr;
   WorkItem* d_corr = nullptr;
@@ -187,7 +189,6 @@ struct ficoco_ctx {
   bool coop_pdl_ok = false;  // a cooperative grid may also be a programmatic dependent
   char* plan_slots = nullptr;
   size_t slot_bytes = 0;
-  size_t off_rows = 0, off_corr = 0, off_out = 0, off_ctaf = 0, off_ocu = 0;
   int cap_rows = 0, cap_corr = 0, cap_out = 0;
   long long cap_part = 0;
 
@@ -408,12 +409,8 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   const size_t out_rows = std::min<size_t>(OUT_ROWS_PER_CTA, std::max<size_t>(1, MSTAGE_BYTES / ((size_t)max_dim * 4)));
   c->cap_out = (int)(T / out_rows + B + 2 * c->num_sms);
   c->cap_part = (long long)T * PART_PER_TOKEN;
-  c->off_rows = align_up(B * sizeof(ImgDesc), 256);
-  c->off_corr = c->off_rows + align_up((size_t)c->cap_rows * sizeof(WorkItem), 256);
-  c->off_out = c->off_corr + align_up((size_t)c->cap_corr * sizeof(WorkItem), 256);
-  c->off_ctaf = c->off_out + align_up((size_t)c->cap_out * sizeof(WorkItem), 256);
-  c->off_ocu = c->off_ctaf + align_up((size_t)(c->num_sms + 2) * sizeof(int), 256);
-  c->slot_bytes = c->off_ocu + align_up((B + 1) * sizeof(int), 256);
+  c->slot_bytes = align_up(plan_tables(B * sizeof(ImgDesc), sizeof(WorkItem), c->cap_rows, c->cap_corr, c->cap_out,
+                                       c->num_sms + 2, B + 1).bytes, 256);
 
   size_t off = 0;
   auto carve = [&](size_t bytes) { size_t o = off; off += align_up(bytes, 256); return o; };
@@ -814,21 +811,26 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
 
   char* slot_dev = c->plan_slots + (size_t)slot * c->slot_bytes;
   p->d_desc = (ImgDesc*)slot_dev;
-  p->d_rows = (WorkItem*)(slot_dev + c->off_rows);
-  p->d_corr = (WorkItem*)(slot_dev + c->off_corr);
-  p->d_out = (WorkItem*)(slot_dev + c->off_out);
-  p->d_ctafirst = (int*)(slot_dev + c->off_ctaf);
-  p->d_out_cu = (int*)(slot_dev + c->off_ocu);
+  const PlanTables at = plan_tables(B * sizeof(ImgDesc), sizeof(WorkItem), rows.size(), corr.size(), outw.size(),
+                                    cta_first.size(), B + 1);
+  if (at.bytes > c->slot_bytes) return FICOCO_ERR_WORKSPACE;
+  p->table_bytes = at.bytes;
+  p->d_rows = (WorkItem*)(slot_dev + at.rows);
+  p->d_corr = (WorkItem*)(slot_dev + at.corr);
+  p->d_out = (WorkItem*)(slot_dev + at.out);
+  p->d_ctafirst = (int*)(slot_dev + at.cta_first);
+  p->d_out_cu = (int*)(slot_dev + at.out_cu);
   {
-    int* ocu = (int*)(c->h_stage + c->off_ocu);
+    int* ocu = (int*)(c->h_stage + at.out_cu);
     for (int b = 0; b < B; ++b) ocu[b] = p->h_desc[b].out_row0;
     ocu[B] = p->tot_out_rows;
   }
   p->key = key;
-  if (p->fused) memcpy(c->h_stage + c->off_ctaf, cta_first.data(), cta_first.size() * sizeof(int));
-  memcpy(c->h_stage + c->off_rows, rows.data(), rows.size() * sizeof(WorkItem));
-  memcpy(c->h_stage + c->off_corr, corr.data(), corr.size() * sizeof(WorkItem));
-  memcpy(c->h_stage + c->off_out, outw.data(), outw.size() * sizeof(WorkItem));
+  auto fill = [&](size_t to, const void* from, size_t bytes) { if (bytes) memcpy(c->h_stage + to, from, bytes); };
+  fill(at.cta_first, cta_first.data(), cta_first.size() * sizeof(int));
+  fill(at.rows, rows.data(), rows.size() * sizeof(WorkItem));
+  fill(at.corr, corr.data(), corr.size() * sizeof(WorkItem));
+  fill(at.out, outw.data(), outw.size() * sizeof(WorkItem));
   return FICOCO_OK;
 }
 
@@ -866,7 +868,7 @@ int get_plan(ficoco_ctx* c, const PlanKey& key, long long attn_rows, cudaStream_
   if (rc != FICOCO_OK) return rc;
   for (int b = 0; b < key.batch; ++b) p->h_desc[b].attn0 = attn_rows * p->h_desc[b].patch0;
   memcpy(c->h_stage, p->h_desc.data(), key.batch * sizeof(ImgDesc));
-  CUDA_TRY(c, cudaMemcpyAsync(c->plan_slots + (size_t)slot * c->slot_bytes, c->h_stage, c->slot_bytes,
+  CUDA_TRY(c, cudaMemcpyAsync(c->plan_slots + (size_t)slot * c->slot_bytes, c->h_stage, p->table_bytes,
                               cudaMemcpyHostToDevice, stream));
   CUDA_TRY(c, cudaStreamSynchronize(stream));
   p->valid = true;
