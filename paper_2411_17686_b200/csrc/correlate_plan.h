@@ -20,6 +20,7 @@ constexpr int UN_MAX = 256;      // accumulator columns per CTA
 constexpr int UKB = 64;          // bf16 elements per k-block (one 128-byte swizzle row)
 constexpr int UM_STAGES = 8;     // most stages of the operand ring
 constexpr int NSPLIT_MAX = 16;
+constexpr int UM_TEXT_MAX = 101; // text tokens of a FiCoCo-L sequence
 
 struct TileShape {
   int n_src, n_tgt, list_len;    // discarded tokens, preserved tokens, entries of a top list
@@ -59,37 +60,56 @@ inline std::vector<TileShape> distinct_shapes(const int* n_src, const int* n_tgt
 struct UmRing {
   int nstage = 0, ksub = 1, stage_bytes = 0;
   int text_off = 0;              // where FiCoCo-L's text weights lie, behind the ring's start
+  bool text_late = false;        // gathered into the ring behind the k-loop instead of beside it, ahead of the operands
   size_t smem = 0;
 };
 
+constexpr size_t UM_SMEM_ONE = 220 * 1024, UM_SMEM_TWO = 106 * 1024;    // most for a CTA alone on its SM, for two
+// Entries that a thread's list of the kernel holds, for lists of at most `longest`.
+inline int list_capacity(int longest) { return longest <= 2 ? 2 : longest <= 4 ? 4 : KCAP; }
+
 // As many stages as fit, with four k-blocks per stage where that leaves four stages, else two (a stage costs about 400
 // cycles besides its copies and MMAs: one FiCoCo-L sequence, 80 rows per CTA: k-loop 15 us with one, 11 with two, 9
-// with four); a grid of more CTAs than SMs keeps to what lets two share an SM.  No stages: it does not fit.
-inline UmRing um_ring(int a_rows, int cols, long long n_ctas, int dim, int n_text, int num_sms) {
+// with four).  A grid of more CTAs than SMs keeps to what lets two share an SM, if need be by having the text weights
+// take the ring's place when it is idle, behind the top lists that pass through it (whole step with one CTA per SM and with
+// two: 8 sequences of 4096 + 64 tokens of 4096, a ninth kept, 483 and 396 us; 8 x 2880 + 64 307 and 262; 30 x 864 + 46,
+// 523 kept, 300 and 277; 32 x 1024 + 100 320 and 297); a smaller grid has them beside the ring, ahead of the operands.
+// No stages: it does not fit.
+inline UmRing um_ring(int a_rows, int cols, long long n_ctas, int dim, int n_text, int list_cap, int num_sms) {
   UmRing r;
   cols = (cols + 15) / 16 * 16;
   const size_t kblock = (size_t)(a_rows + cols) * 128;
-  const size_t text = (size_t)n_text * (a_rows + cols) * 4;
+  const size_t text = (size_t)n_text * (a_rows + cols) * 4, lists = (size_t)UM * list_cap * 8;
   // every MMA reads 128 A rows: behind the last k-block there must be room for the rows past the tile
   const size_t slack = 1024 + (kblock < (size_t)UM * 128 ? (size_t)UM * 128 - kblock : 0);
-  const size_t most = 220 * 1024, budget = n_ctas > num_sms ? 106 * 1024 : most;
-  auto fit = [&](int ksub, int ns, size_t limit) {
-    if (r.nstage || (size_t)ns * ksub * kblock + slack + text > limit) return;
+  bool late = false;
+  size_t limit = 0;
+  auto fit = [&](int ksub, int ns) {
+    const size_t ring = (size_t)ns * ksub * kblock + slack;
+    const size_t smem = late ? std::max(ring, 1024 + lists + text) : std::max(ring + text, 1024 + lists);
+    if (r.nstage || smem > limit) return;
     r.nstage = ns;
     r.ksub = ksub;
     r.stage_bytes = (int)(ksub * kblock);
-    r.text_off = (int)((size_t)ns * ksub * kblock + slack - 1024);
-    r.smem = (size_t)ns * ksub * kblock + slack + text;
+    r.text_off = (int)(late ? lists : ring - 1024);
+    r.text_late = late;
+    r.smem = smem;
   };
   const int nk = dim / UKB;
-  for (const size_t limit : {budget, most}) {          // (FiCoCo-L with much text: rather one CTA per SM)
-    for (int ns = std::min(UM_STAGES, (nk + 3) / 4); ns >= 4; --ns) fit(4, ns, limit);
+  auto stages = [&]() {
+    for (int ns = std::min(UM_STAGES, (nk + 3) / 4); ns >= 4; --ns) fit(4, ns);
     for (int ksub = 2; ksub >= 1; --ksub)
-      for (int ns = std::max(2, std::min(UM_STAGES, (nk + ksub - 1) / ksub)); ns >= 2; --ns) fit(ksub, ns, limit);
+      for (int ns = std::max(2, std::min(UM_STAGES, (nk + ksub - 1) / ksub)); ns >= 2; --ns) fit(ksub, ns);
+  };
+  if (n_ctas > num_sms) {
+    limit = UM_SMEM_TWO;
+    stages();
+    late = n_text > 0;
+    if (late) stages();
+    late = false;
   }
-  // the epilogue halves hand their lists over through the ring
-  r.smem = std::max(r.smem, 1024 + (size_t)UM * KCAP * 8);
-  if (r.smem > most) r.nstage = 0;
+  limit = UM_SMEM_ONE;
+  stages();
   return r;
 }
 
@@ -107,7 +127,8 @@ struct Tiling {
 // 32 x 288 tokens, 144 x 144 entries: 9.25 us in tiles of 72 x 80, 8.75 in 48 x 144 (no split, no counters); 32 x 576
 // tokens take 13.5 us in tiles of 96 x 96 and 22 to 82 in any that make a second round.  At other widths (768, 1280, 1664;
 // FiCoCo-L 2048, 3072, 5120), 42 batches of one to 64 images, whole step under up to 40 tilings each: the choice is the best
-// within 0.5 % in 31 of them, within 1.6 % in all.
+// within 0.5 % in 31 of them, within 1.6 % in all.  A grid whose CTAs have an SM each to themselves goes in rounds of one per
+// SM; with 8 to 101 text tokens, 15 batches of 4 to 32 sequences under ten tilings: the best in 14, 1.5 % off in one.
 inline Tiling best_tiling(const std::vector<TileShape>& shapes, int dim, int n_text, int num_sms, long long max_tiles,
                           long long max_entries) {
   constexpr int HEIGHTS[4] = {128, 64, 32, 16};
@@ -141,20 +162,21 @@ inline Tiling best_tiling(const std::vector<TileShape>& shapes, int dim, int n_t
   }
 
   const double k_scale = dim / 1024.0, text_scale = n_text > 0 ? 1.0 + n_text / 9.5 : 1.0;
-  const long long wave = 2LL * num_sms;
   double least = 0;
   for (int t = 0; t < 4; ++t)
     for (int w = 0; w < NSPLIT_MAX; ++w) {
       const long long n_ctas = (long long)ctas[t][w];
       const double cols = cols_all[t][w];
       if ((w > 0 || t > 0) && (n_ctas > max_tiles || entries[w] > (double)max_entries)) break;
-      if (um_ring(rows_most[t], cols_most[w], n_ctas, dim, n_text, num_sms).nstage == 0) continue;
+      const UmRing ring = um_ring(rows_most[t], cols_most[w], n_ctas, dim, n_text, list_capacity(list_longest), num_sms);
+      if (ring.nstage == 0) continue;
       int lanes = 1;                                   // lanes that share a token when the lists are merged
       while (lanes < 8 && rows_most[t] * 2 * lanes <= 256) lanes *= 2;
       const double rows = k_scale * (rows_all[t][w] + cols) / n_ctas;
       double cost = 2900.0 + 2270.0 * k_scale + 9.0 * rows + 10.0 * cols / n_ctas * text_scale +
                     600.0 * ((list_most[w] + 4 * lanes - 1) / (4 * lanes)) + (list_most[w] > list_longest ? 700.0 : 0.0);
-      if (n_ctas > num_sms) cost += 26.0 * rows;
+      const long long wave = ring.smem > UM_SMEM_TWO ? num_sms : 2LL * num_sms;
+      if (n_ctas > num_sms && wave > num_sms) cost += 26.0 * rows;
       if (n_ctas > wave) cost *= 0.5 * ((double)n_ctas / wave + (double)((n_ctas + wave - 1) / wave));
       if (least == 0 || cost < least) { least = cost; best.rows = HEIGHTS[t]; best.splits = w + 1; }
     }

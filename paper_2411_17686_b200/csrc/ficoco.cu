@@ -80,6 +80,7 @@ struct Plan {
   bool uf_small = false;        // fp32 tiles of 32 x 32 instead of 128 x 64
   int um_b_bytes = 0, uf_stg = 0, uf_stg_off = 0;     // slots for fp32 values (k-blocks in flight) and where they lie
   int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1, um_text_off = 0;
+  bool um_text_late = false;
   size_t um_smem = 0;
   std::vector<ImgDesc> h_desc;
 };
@@ -536,9 +537,10 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   p->max_np = p->max_tgt = p->max_src = p->max_rc = p->max_nwin_cells = p->max_list = 0;
   p->need_finalize = false;
   // tensor-core correlate: bf16 tokens, hidden size a multiple of 64.  FiCoCo-L adds its text term
-  // in the epilogue from weights staged in shared memory, 2 KB per text token for the largest tile.
+  // in the epilogue from weights staged in shared memory.  With up to 101 text tokens tiles of 64 x 256, for which the work
+  // tables are sized, leave room for two stages of operands; sequences with more take the SIMT kernel.
   p->umma = key.dtype == FICOCO_BF16 && key.dim % UKB == 0 &&
-            (key.mode == 0 || (size_t)key.n_text * 2048 + 1024 + (size_t)UM * KCAP * 8 <= 220 * 1024);
+            (key.mode == 0 || key.n_text <= UM_TEXT_MAX);
   // fp32 tokens (FiCoCo-V): the same tiling with narrower column tiles, operands split into bf16 terms
   p->um_f32 = key.dtype == FICOCO_FP32 && key.dim % UKB == 0 && key.mode == 0;
   if (p->um_f32) p->umma = true;
@@ -797,7 +799,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     }
     if (um_a_rows > UM || um_cols > UF_COLS || p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
   } else if (p->umma) {
-    const UmRing r = um_ring(um_a_rows, um_cols, (long long)corr.size(), key.dim, tail, c->num_sms);
+    const UmRing r = um_ring(um_a_rows, um_cols, (long long)corr.size(), key.dim, tail, list_capacity(p->max_list), c->num_sms);
     if (r.nstage == 0) return FICOCO_ERR_UNSUPPORTED;
     p->um_a_bytes = um_a_rows * 128;
     p->um_tmem_cols = 32;
@@ -806,6 +808,7 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     p->um_ksub = r.ksub;
     p->um_stage_bytes = r.stage_bytes;
     p->um_text_off = r.text_off;
+    p->um_text_late = r.text_late;
     p->um_smem = r.smem;
   }
 
@@ -1083,7 +1086,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
       (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status, p->um_nstage,    \
       p->um_stage_bytes, p->um_a_bytes, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt, \
-      c->e_w, c->e_c, tmean, M, p->max_np, gamma, p->um_text_off, c->wait_ns)
+      c->e_w, c->e_c, tmean, M, p->max_np, gamma, p->um_text_off, p->um_text_late ? 1 : 0, c->wait_ns)
 #define FICOCO_UMMA_STAGES(LC)                                                                         \
   do {                                                                                                 \
     if (p->um_ksub == 4) FICOCO_UMMA_LAUNCH(LC, 4);                                                     \

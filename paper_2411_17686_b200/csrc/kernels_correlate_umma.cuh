@@ -186,7 +186,8 @@ __device__ __forceinline__ void epilogue_scan(uint32_t tmem_lane, int c_lo, int 
 // valid source rows rounded up to 8, x 128 B) followed by a B tile (column rows x 128 B).  An
 // MMA always reads 128 A rows; rows past a_bytes alias the B tile (or the slack the host adds
 // behind the ring) and only feed accumulator rows that are never read.  FiCoCo-L's text weights lie text_off bytes behind
-// the ring's start and are gathered ahead of the operands.
+// the ring's start and are gathered ahead of the operands; with text_late they lie in the ring, behind the lists that the
+// epilogue hands over there, and are gathered when the accumulator is complete.
 template <int LCAP, int KSUB>
 __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     const __nv_bfloat16* __restrict__ tokens, int D, const ImgDesc* __restrict__ desc,
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     float* __restrict__ part_val, int* __restrict__ part_idx, unsigned* __restrict__ status,
     int nstage, int stage_bytes, int a_bytes, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
     float* __restrict__ tau_out, int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c,
-    const float* __restrict__ tmean, int M, int NV, float gamma, int text_off, unsigned long long wait_ns) {
+    const float* __restrict__ tmean, int M, int NV, float gamma, int text_off, int text_late, unsigned long long wait_ns) {
   extern __shared__ unsigned char um_raw[];
   __shared__ uint64_t full_bar[UM_STAGES], empty_bar[UM_STAGES], acc_bar;
   __shared__ uint32_t tmem_base_s;
@@ -288,11 +289,9 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     // behind the k-loop, eight at a time through registers, and for 128 rows whatever the tile, they took 4 of the 7 us
     // between accumulator and lists: one sequence of 576 + 64 tokens.)
     const int s_stride = (w.nrows + 7) & ~7;
-    float* tT = nullptr;
-    float* tSb = nullptr;
-    if (tmean != nullptr) {
-      tT = reinterpret_cast<float*>(um_raw + (ring - smem_u32(um_raw)) + text_off);
-      tSb = tT + (size_t)M * n_pad;
+    float* tT = tmean != nullptr ? reinterpret_cast<float*>(um_raw + (ring - smem_u32(um_raw)) + text_off) : nullptr;
+    float* tSb = tT + (size_t)M * n_pad;
+    auto gather_text = [&]() {
       const float* tb = tmean + (size_t)w.img * M * NV;
       #pragma unroll 1
       for (int j = lane; j < n_pad + s_stride; j += 32) {       // a column or a row of the tile
@@ -304,7 +303,8 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
         #pragma unroll 4
         for (int k = pt >> 5; k < M; k += 8) cp_async4(to + (uint32_t)k * step, from + (size_t)k * NV);
       }
-    }
+    };
+    if (tmean != nullptr && !text_late) gather_text();
     bool ok = true;
     // Each thread's copies of a stage arrive on its barrier when they have landed, so a producer never waits
     // for its own copies and the whole ring is in flight; the MMA warp orders the two proxies (below).
@@ -341,7 +341,10 @@ __global__ void __launch_bounds__(UTHREADS, 2) k_correlate_umma(
     acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);          // tcgen05.ld below is warp-collective
     tc_fence_after();
     const float t_scale = tmean != nullptr ? (1.0f - gamma) / (float)M : 0.f;
-    if (tmean != nullptr) cp_async_wait_all();
+    if (tmean != nullptr) {
+      if (text_late && acc_ok) gather_text();          // (the accumulator is complete: nothing reads or fills the ring)
+      cp_async_wait_all();
+    }
     cta_sync(1, 256);                                  // norms and text weights are in shared memory
     // ---------------- epilogue: lane = accumulator row ---------------------------------------
     // Warps 0-3 scan the lower half of the columns, warps 5-8 (the same TMEM lanes) the upper half, whose lists come

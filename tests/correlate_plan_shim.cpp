@@ -9,6 +9,12 @@ extern "C" int plan_tiling(const int* n_src, const int* n_tgt, const int* list_l
   *splits = t.splits;
   return (int)shapes.size();
 }
-extern "C" int plan_stages(int a_rows, int cols, long long n_ctas, int dim, int n_text, int num_sms) {
-  return ficoco::um_ring(a_rows, cols, n_ctas, dim, n_text, num_sms).nstage;
+// Stages of the operand ring; out: its bytes, where the text weights lie, whether they take its place, shared memory of a CTA.
+extern "C" int plan_ring(int a_rows, int cols, long long n_ctas, int dim, int n_text, int list_cap, int num_sms, long long* out) {
+  const ficoco::UmRing r = ficoco::um_ring(a_rows, cols, n_ctas, dim, n_text, list_cap, num_sms);
+  out[0] = (long long)r.nstage * r.stage_bytes;
+  out[1] = r.text_off;
+  out[2] = r.text_late;
+  out[3] = (long long)r.smem;
+  return r.nstage;
 }

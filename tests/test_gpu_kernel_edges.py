@@ -117,6 +117,24 @@ def test_correlate_text_weights(n_vision, n_text, dim, keep, p):
         c.close()
 
 
+@pytest.mark.parametrize("batch,n_vision,n_text,dim,keep,eps", [
+    (20, 800, 101, 64, 200, 0.998),                     # 120 x 112 tokens per tile, one k-block, two splits
+    (10, 1500, 101, 320, 300, 0.998),                   # 120 x 80, four splits, five k-blocks in two stages
+    (20, 800, 80, 64, 200, 0.986),                      # lists of four
+    (80, 400, 85, 64, 133, 0.9),                        # lists of 15, 96 x 144, not split
+], ids=["two-splits", "five-blocks", "lists-of-4", "lists-of-15"])
+def test_correlate_text_weights_in_the_ring(batch, n_vision, n_text, dim, keep, eps):
+    """Grids of more than one CTA per SM with much text: the weights take the place of the operand ring."""
+    p = fo.Params(eps=eps)
+    c = binding.Context(max_tokens=batch * (n_vision + n_text), max_dim=dim, max_batch=batch, max_text=n_text, device=0)
+    try:
+        b = synth.make_l_batch(101, batch, n_vision, n_text, dim, 2, keep)
+        gaps.repair_l(b, p)
+        parity.run_and_compare_l(c, b, p, DEV, what=f"L {batch} x {n_vision} + {n_text}, {dim}, keep {keep}")
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("n_vision,n_text,dim,heads,dtype", [
     (37, 3, 2112, 17, "bf16"),         # 111 attention values, no multiple of four; one head more than are in flight
     (130, 8, 2112, 3, "bf16"),         # 1040: a second part of 16 values
