@@ -38,8 +38,12 @@ constexpr int FROWS = FWARPS;     // rows of a ring stage: one per warp
 constexpr int FFOLD = 8;          // rows of the fold buffer (warps w and w + 8 share a row)
 constexpr int F_NCONS = 512;
 constexpr int F_MAXSTAGE = 16;
-constexpr size_t F_SMEM = 216 * 1024;   // dynamic shared memory at most (7 KB are static)
 constexpr int F_MAXWON = 32;      // pieces per CTA
+constexpr size_t F_SMEM = 216 * 1024;   // dynamic shared memory at most
+// what is static beside it: the rings' barriers, the selections' tables, the pieces and their images, a flag
+constexpr size_t F_STATIC = sizeof(uint64_t) * FWARPS * F_MAXSTAGE + sizeof(SelectShared) + sizeof(SelectSmallShared) +
+                            F_MAXWON * (sizeof(WorkItem) + sizeof(ImgDesc)) + 128;
+static_assert(F_SMEM + F_STATIC <= 227 * 1024, "a CTA of the fused filter does not fit an SM: no context could be created");
 static_assert(F_NCONS == SEL_SMALL_THREADS, "the selection is written for the threads of this kernel");
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
