@@ -471,7 +471,6 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
     FICOCO_FUSED_ATTR(float, 5); FICOCO_FUSED_ATTR(float, 6); FICOCO_FUSED_ATTR(float, 7); FICOCO_FUSED_ATTR(float, 8);
     FICOCO_FUSED_ATTR(__nv_bfloat16, 1); FICOCO_FUSED_ATTR(__nv_bfloat16, 2); FICOCO_FUSED_ATTR(__nv_bfloat16, 4);
     FICOCO_FUSED_ATTR(__nv_bfloat16, 5); FICOCO_FUSED_ATTR(__nv_bfloat16, 6); FICOCO_FUSED_ATTR(__nv_bfloat16, 7);
-    FICOCO_FUSED_ATTR(__nv_bfloat16, 8);
 #undef FICOCO_FUSED_ATTR
   }
   cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
@@ -615,8 +614,11 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
     //   rows of up to 1024 values, uneven and large: 1.00 to 1.20 (768, 1024 in bf16, 85 to 300 images of 256 to 2304
     //   tokens; 192 batches on the kernels before these: 1.065 in the mean of 30, even ones 1.003 of 94);
     //   1280 values, uneven and large: 0.97 to 1.07;
-    //   1408 and 1664 values in bf16: 0.87 to 0.98 uneven and large, 0.83 to 1.07 otherwise (the largest for one image);
-    //   2048 values in bf16, where a warp of the fused kernel holds one row at a time and spills: 1.04 to 1.16 of all nine.
+    //   six and seven vectors a lane in bf16 (1344 to 1792 values, 48 batches of one to 256 images): 0.88 to 0.99, for one
+    //   image 1.01 to 1.05;
+    //   eight (1800 to 2048 values, one to 256 images of 576 tokens, four of 2880), where a warp of the fused kernel held one
+    //   row at a time and spilled: 1.00 to 1.16 from 1984 on; 0.955 to 1.00 at 1856 and 1920 from 18 000 tokens on and for
+    //   large images, up to 1.09 below; 0.995 to 1.38 where the hidden size is no multiple of 64.  They have no fused kernel.
     const bool wide_bf16 = esz == 2 && p->f_vpl >= 6;
     const bool uneven = best.cost * 100 > (best.even + F_PIECE_ROWS) * 122LL && total * key.dim * esz > 64LL * 1024 * 1024;
     if (best.cost < 0 || (wide_bf16 ? p->f_vpl == 8 : uneven)) p->fused = false;
@@ -982,7 +984,8 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
     else if (vpl <= 5) FICOCO_FUSED_GO(5);
     else if (vpl <= 6) FICOCO_FUSED_GO(6);
     else if (vpl <= 7) FICOCO_FUSED_GO(7);
-    else FICOCO_FUSED_GO(8);
+    else if constexpr (sizeof(T) == 4) FICOCO_FUSED_GO(8);
+    else return FICOCO_ERR_UNSUPPORTED;                // (never planned)
 #undef FICOCO_FUSED_GO
     if (fe != cudaSuccess) { c->last_cuda = (int)fe; return FICOCO_ERR_CUDA; }
     c->launches += 1;
