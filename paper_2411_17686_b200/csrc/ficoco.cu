@@ -78,7 +78,7 @@ struct Plan {
   bool umma = false;
   bool um_f32 = false;          // fp32 tokens split into three bf16 terms (k_correlate_umma_f32)
   bool uf_small = false;        // fp32 tiles of 32 x 32 instead of 128 x 64
-  int um_b_bytes = 0, uf_stg = 0, uf_stg_off = 0;     // slots for fp32 values (k-blocks in flight) and where they lie
+  int um_b_bytes = 0, uf_stg_off = 0;     // uf_stg_off: where the slots for fp32 values lie
   int um_stage_bytes = 0, um_a_bytes = 0, um_tmem_cols = 0, um_nstage = 0, um_ksub = 1, um_text_off = 0;
   bool um_text_late = false;
   size_t um_smem = 0;
@@ -786,18 +786,14 @@ int build_plan(ficoco_ctx* c, Plan* p, const PlanKey& key, int slot) {
   p->tot_patch = (int)patch0; p->tot_src = (int)src0; p->tot_tgt = (int)tgt0; p->tot_out_rows = (int)out0;
   p->n_rows = (int)rows.size(); p->n_corr = (int)corr.size(); p->n_out = (int)outw.size();
   if (p->um_f32) {
-    // stages of three bf16 tiles per operand, 16 KB behind them for the 128-row reads of the last A tile
     p->um_a_bytes = um_a_rows * 128;
     p->um_b_bytes = (um_cols + 15) / 16 * 16 * 128;
     p->um_tmem_cols = 32;
     while (p->um_tmem_cols < 6 * (p->um_b_bytes / 128)) p->um_tmem_cols *= 2;   // six partial products per entry
-    p->um_nstage = uf_stages(p->uf_small);
-    p->um_smem = (size_t)uf_stages(p->uf_small) * 3 * (p->um_a_bytes + p->um_b_bytes) + (size_t)UM * 128 + 2048;
-    if (p->uf_small) {                                 // slots for the fp32 values of the next k-blocks
-      const size_t slot = 2 * 8192;
-      p->uf_stg = (int)std::min<size_t>(8, (220 * 1024 - p->um_smem) / slot);
+    p->um_smem = uf_smem(p->uf_small, p->um_a_bytes, p->um_b_bytes);
+    if (p->uf_small) {
       p->uf_stg_off = (int)(p->um_smem - 1024);
-      p->um_smem += p->uf_stg * slot;
+      p->um_smem += UF_SLOTS * UF_SLOT;
     }
     if (um_a_rows > UM || um_cols > UF_COLS || p->um_smem > 220 * 1024) return FICOCO_ERR_UNSUPPORTED;
   } else if (p->umma) {
@@ -1075,7 +1071,7 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   launch_dependent(p->uf_small ? k_correlate_umma_f32<LC, true> : k_correlate_umma_f32<LC, false>, dim3(p->n_corr), UTHREADS, p->um_smem, st, tk, D,                                                                  \
       (const ImgDesc*)p->d_desc, (const WorkItem*)p->d_corr, (const float*)c->rn,                       \
       (const int*)c->S_idx, (const int*)c->T_idx, c->part_val, c->part_idx, c->status,                 \
-      p->um_a_bytes, p->um_b_bytes, p->uf_stg_off, p->uf_stg, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt, \
+      p->um_a_bytes, p->um_b_bytes, p->uf_stg_off, p->um_tmem_cols, c->tile_cnt, c->corr_cnt, c->tau, c->e_tgt, \
       c->e_w, c->e_c, c->wait_ns)
       if (p->max_list <= 2) FICOCO_UF32_LAUNCH(2);
       else if (p->max_list <= 4) FICOCO_UF32_LAUNCH(4);

@@ -19,7 +19,7 @@
 // 64 hidden elements; thread (row r mod 32, 16-byte chunk c) of the 256 producers handles chunk c of
 // rows r, r + 32, ... of both operands and keeps the next k-block's loads in flight while it
 // converts the current one (a third register buffer spilled and was slower).  A grid that would leave SMs idle takes tiles
-// of 32 x 32 (SMALL): a thread's fp32 values arrive by cp.async in up to eight shared-memory slots of its own, which needs
+// of 32 x 32 (SMALL): a thread's fp32 values arrive by cp.async in six shared-memory slots of its own, which needs
 // no barrier, and are converted into four stages.  Every wait is bounded as in the bf16 kernel.
 //
 // What bounds it: the producers' instructions per k-block (two barriers, conversion and 48 bytes of stores per eight
@@ -34,6 +34,14 @@ namespace ficoco {
 constexpr int UF_COLS = 64;      // preserved tokens per CTA (two rows per producer thread)
 constexpr int UF_SMALL = 32;     // rows and columns of a small tile
 __host__ __device__ constexpr int uf_stages(bool small) { return small ? 4 : 2; }   // stages of converted operands
+// Shared memory: stages of three bf16 tiles per operand, 16 KB behind them for the 128-row reads of the last A tile, and for
+// small tiles as many slots for the fp32 values of the next k-blocks (both operands) as fit.
+__host__ __device__ constexpr size_t uf_smem(bool small, int a_bytes, int b_bytes) {
+  return (size_t)uf_stages(small) * 3 * (a_bytes + b_bytes) + (size_t)UM * 128 + 2048;
+}
+constexpr size_t UF_SLOT = 2 * UF_SMALL * UKB * sizeof(float);
+constexpr int UF_SLOTS = (int)((220 * 1024 - uf_smem(true, UF_SMALL * 128, UF_SMALL * 128)) / UF_SLOT);
+static_assert(UF_SLOTS == 6, "the comments and figures are of six slots");
 constexpr int UF_AR = UM / 32;       // A rows per producer thread
 constexpr int UF_BR = UF_COLS / 32;  // B rows per producer thread
 
@@ -101,7 +109,7 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
     const WorkItem* __restrict__ work, const float* __restrict__ rn,
     const int* __restrict__ S_idx, const int* __restrict__ T_idx,
     float* __restrict__ part_val, int* __restrict__ part_idx, unsigned* __restrict__ status,
-    int a_bytes, int b_bytes, int stg_off, int n_stg, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
+    int a_bytes, int b_bytes, int stg_off, int tmem_cols, int* __restrict__ img_done, int* __restrict__ corr_cnt,
     float* __restrict__ tau_out, int* __restrict__ e_tgt, float* __restrict__ e_w, float* __restrict__ e_c,
     unsigned long long wait_ns) {
   constexpr int NST = uf_stages(SMALL);
@@ -235,7 +243,7 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
       if (lane == 0) mbar_arrive(&full_bar[s]);
     };
     if constexpr (SMALL) {
-      // slot (k-block mod n_stg, row chunk i, half): 16 bytes per thread, side by side
+      // slot (k-block mod UF_SLOTS, row chunk i, half): 16 bytes per thread, side by side
       constexpr uint32_t stage_step = (AR + BR) * 8192;
       const uint32_t mine = ring + (uint32_t)stg_off + (uint32_t)pt * 16u;
       const float* next = tbase;
@@ -252,11 +260,11 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
         cp_async_commit();
       };
       #pragma unroll 1
-      for (int st = 0; st < n_stg; ++st) fetch(st, mine + (uint32_t)st * stage_step);
+      for (int st = 0; st < UF_SLOTS; ++st) fetch(st, mine + (uint32_t)st * stage_step);
       int st = 0;
       #pragma unroll 1
       for (int kb = 0; kb < nkb; ++kb) {
-        cp_async_wait_groups(n_stg - 1);
+        cp_async_wait_groups<UF_SLOTS - 1>();
         float4 buf[AR + BR][2];
         const unsigned char* from = uf_raw + (mine - smem_u32(uf_raw)) + (size_t)st * stage_step;
 #pragma unroll
@@ -264,9 +272,9 @@ __global__ void __launch_bounds__(UTHREADS, 1) k_correlate_umma_f32(
           buf[i][0] = *reinterpret_cast<const float4*>(from + (size_t)i * 8192);
           buf[i][1] = *reinterpret_cast<const float4*>(from + (size_t)i * 8192 + 4096);
         }
-        fetch(kb + n_stg, mine + (uint32_t)st * stage_step);   // (the values are in registers)
+        fetch(kb + UF_SLOTS, mine + (uint32_t)st * stage_step);   // (the values are in registers)
         store(buf, kb);
-        if (++st == n_stg) st = 0;
+        if (++st == UF_SLOTS) st = 0;
       }
     } else {
       float4 bufA[AR + BR][2], bufB[AR + BR][2];
