@@ -63,11 +63,17 @@ def test_most_rows_kept_of_wide_rows(kind, batch, dim, dtype):
         c.close()
 
 
-@pytest.mark.parametrize("gh,gw,keep", [(31, 33, 900), (32, 32, 1), (25, 41, 1024), (25, 41, 4), (48, 45, 40),
-                                         (64, 64, 2000), (17, 241, 4096)])
-def test_selection_sizes(ctx, gh, gw, keep):
-    """1023 and 1024 tokens: two per thread; from 1025 on eight, from 4097 on sixteen (the last: unfused)."""
-    run_v(ctx, 92, 1, gh, gw, 64, keep, cls=False, p=fo.Params(max_targets=0) if gh * gw > 4000 else fo.Params())
+@pytest.mark.parametrize("gh,gw,dim,keep,fused", [
+    (31, 33, 64, 900, True), (32, 32, 64, 1, True),       # 1023 and 1024 tokens: two per thread in registers
+    (25, 41, 64, 1024, True), (25, 41, 64, 4, True),      # 1025, the fewest of the histogram: 1 and 1021 discarded
+    (48, 45, 64, 40, True),
+    (64, 64, 64, 2000, False), (17, 241, 64, 4096, False),     # the fused filter's ring is too small to work in
+    (64, 64, 256, 2000, True), (17, 241, 256, 4096, True),     # the same by slices, each on the CTA that scored it
+])
+def test_selection_sizes(ctx, gh, gw, dim, keep, fused):
+    """With the local penalty.  Up to 1024 tokens in registers, more by a histogram over the value range."""
+    run_v(ctx, 92, 1, gh, gw, dim, keep, cls=False, p=fo.Params(max_targets=0) if gh * gw > 4000 else fo.Params())
+    assert (ctx.ficoco_last_launch_count() < 6) == fused       # filter in one kernel or in four
 
 
 @pytest.mark.parametrize("fused", [True, False], ids=["fused", "unfused"])
@@ -104,8 +110,10 @@ def test_correlate_tiles(ctx, dim, n_src, n_tgt):
     (65, 1, 64, 1, fo.Params()),                        # one k-block, one text token, one column
     (130, 3, 1088, 17, fo.Params()),                    # 17 k-blocks: the last stage of four holds one
     (300, 100, 512, 30, fo.Params(eps=0.5)),            # top lists of 16 entries merged over lanes and splits
-    (272, 100, 64, 271, fo.Params()),                   # one source, two splits, the most text that tiles are planned for
-], ids=["one", "last-stage", "long-lists", "one-source"])
+    (272, 100, 64, 271, fo.Params()),                   # one source, two splits, much text
+    (140, 101, 128, 60, fo.Params()),                   # the most text that tiles are planned for
+    (140, 102, 128, 60, fo.Params()),                   # one more: the SIMT kernel
+], ids=["one", "last-stage", "long-lists", "one-source", "most-text", "simt"])
 def test_correlate_text_weights(n_vision, n_text, dim, keep, p):
     """FiCoCo-L tiles: odd numbers of blocks, little and much text."""
     c = binding.Context(max_tokens=2 * (n_vision + n_text), max_dim=dim, max_batch=2, max_text=n_text, device=0)
