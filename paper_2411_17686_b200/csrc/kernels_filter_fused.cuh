@@ -425,14 +425,15 @@ __global__ void __launch_bounds__(F_NCONS, 1) k_filter_fused(
   cta_sync(1, F_NCONS);
 
   FICOCO_PHASE(0, 5);
-  if (failed) return;
   // Without dep_wait_first (the caller states that what sits in front is a step of this library) the kernel has by now
   // written only scratch that no grid but a filter or correlate grid reads, and those of that step had ended before its
-  // merge let this grid in.  The index lists and outputs written below are read by that merge: wait for it.
+  // merge let this grid in.  The index lists and outputs written below are read by that merge: wait for it, also after a
+  // wait that ran out, since the grid behind this one waits for this one alone.
   grid_dep_wait();
   // the counters of the launch before, complete by now, are zeroed for the launch after (see the top)
   if (blockIdx.x == 0)
     for (int i = tid; i < n_other; i += F_NCONS) other_cnt[i] = 0;
+  if (failed) return;
   FICOCO_PHASE(0, 6);
   // selections (the ring is idle now and serves as work area), image by image over this CTA's pieces
   int pi = p_begin;

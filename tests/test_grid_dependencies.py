@@ -45,3 +45,22 @@ def test_nothing_is_touched_ahead_of_the_wait(name, params, body):
     pointers = {re.search(r"(\w+)\s*$", p).group(1) for p in params.split(",") if "*" in p}
     touched = {p for p in pointers - PLAN_TABLES if re.search(rf"\b{p}\b", ahead)}
     assert not touched, f"{name} names {sorted(touched)} ahead of its wait"
+
+
+def without_lambdas(body):
+    while m := re.search(r"\[&\]\s*(\([^()]*\))?\s*\{", body):
+        depth, at = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(body[at], 0)
+            at += 1
+        body = body[:m.start()] + body[at:]
+    return body
+
+
+@pytest.mark.parametrize("name,params,body", DEPENDENT, ids=[k[0] for k in DEPENDENT])
+def test_no_way_out_ahead_of_the_wait(name, params, body):
+    """A grid that gave up has waited all the same: the one behind it waits for it alone."""
+    ahead = without_lambdas(body[:body.rindex("grid_dep_wait();")])
+    if name not in OPT_IN:
+        ahead = ahead[:ahead.index("grid_dep_wait();")] if "grid_dep_wait();" in ahead else ahead
+    assert not re.search(r"\breturn\b", ahead), f"{name} can end without having waited"
