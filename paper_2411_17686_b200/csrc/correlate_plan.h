@@ -87,7 +87,7 @@ inline UmRing um_ring(int a_rows, int cols, long long n_ctas, int dim, int n_tex
   auto fit = [&](int ksub, int ns) {
     const size_t ring = (size_t)ns * ksub * kblock + slack;
     const size_t smem = late ? std::max(ring, 1024 + lists + text) : std::max(ring + text, 1024 + lists);
-    if (r.nstage || smem > limit) return;
+    if (smem > limit) return;
     r.nstage = ns;
     r.ksub = ksub;
     r.stage_bytes = (int)(ksub * kblock);
@@ -97,9 +97,9 @@ inline UmRing um_ring(int a_rows, int cols, long long n_ctas, int dim, int n_tex
   };
   const int nk = dim / UKB;
   auto stages = [&]() {
-    for (int ns = std::min(UM_STAGES, (nk + 3) / 4); ns >= 4; --ns) fit(4, ns);
+    for (int ns = std::min(UM_STAGES, (nk + 3) / 4); ns >= 4 && !r.nstage; --ns) fit(4, ns);
     for (int ksub = 2; ksub >= 1; --ksub)
-      for (int ns = std::max(2, std::min(UM_STAGES, (nk + ksub - 1) / ksub)); ns >= 2; --ns) fit(ksub, ns);
+      for (int ns = std::max(2, std::min(UM_STAGES, (nk + ksub - 1) / ksub)); ns >= 2 && !r.nstage; --ns) fit(ksub, ns);
   };
   if (n_ctas > num_sms) {
     limit = UM_SMEM_TWO;
