@@ -729,7 +729,9 @@ __device__ __forceinline__ int window_best(const Cell* cell, const float* sc, in
 // What bounds it is the chain of barriers and shared-memory trips, and instruction fetch, as the code runs once: loops are
 // rolled (eight tokens per thread in registers, everything unrolled: 13 us).  2880 tokens, on the CTA that scored the image's last
 // piece alone and with sixteen keys per thread in a search of the value range: 17.6 us, of which threshold 6.5, keys 3.6,
-// windows 2.0, lists 3.2; now 11 (whole step of 8 x 2881 tokens 130.7 -> 123 us, 16 ragged images 92 -> 85.5).
+// windows 2.0, lists 3.2; now 11 (whole step of 8 x 2881 tokens 130.7 -> 123 us, 16 ragged images 92 -> 85.5).  As a kernel of
+// its own, 512 threads for an image instead of 1024 and the histogram instead of the search: 8 x 2880 tokens 22.2 -> 14.2 us,
+// 8 x 4096 22.6 -> 15.6 (FiCoCo-L); with relation maps the step of 4 x 1152 47.0 -> 37.0, of 2 x 3000 84.1 -> 77.4.
 // ---------------------------------------------------------------------------------------
 constexpr int SEL_THREADS = 512;
 constexpr int SEL_BINS = 4 * SEL_THREADS;
