@@ -359,55 +359,48 @@ __global__ void __launch_bounds__(256) k_score(const T* __restrict__ tokens, int
 
 // ---------------------------------------------------------------------------------------
 // FiCoCo-L: head mean of the text->vision attention, t[b, k, i] = (1/H) sum_h A[b, h, k, i].
-// The M * N values of a sequence are cut into parts of HM_PART, one CTA per part; a thread takes four
-// values, 16 heads in flight, added in head order (16 sequences of 2048, 75 MB of attention: whole step 68.7 us, with
-// eight heads in flight 76.1).
+// The M * N values of a sequence are cut into parts, one CTA per part, 16 heads in flight, added in head order.  Where
+// everything is aligned a thread takes four values and a part is 1024 (16 sequences of 2048, 75 MB of attention: whole step
+// 68.7 us, with eight heads in flight 76.1); else one value, and a part is 256 (12 sequences of 722 + 19 tokens of 2048 57.7 us,
+// four values of 8 heads 61.5, of 16 heads 63.2; 51 of 410 + 1 of 256 37.7, 40.7, 42.4: registers that the grid before still
+// holds are waited for).
 // ---------------------------------------------------------------------------------------
-constexpr int HM_PART = 1024;
-__host__ __device__ __forceinline__ int head_mean_parts(int MN) { return (MN + HM_PART - 1) / HM_PART; }
+__host__ __device__ __forceinline__ int head_mean_values(const float* attn, const float* t, int MN) {   // of a part
+  return ((MN & 3) == 0 && (reinterpret_cast<uintptr_t>(attn) & 15) == 0 && (reinterpret_cast<uintptr_t>(t) & 15) == 0) ? 1024 : 256;
+}
+__host__ __device__ __forceinline__ int head_mean_parts(int MN, int values) { return (MN + values - 1) / values; }
 
 __device__ __forceinline__ void head_mean_part(const float* __restrict__ attn, int H, int MN, int part,
                                                float* __restrict__ t) {
-  const int per_seq = head_mean_parts(MN), b = part / per_seq, i0 = part % per_seq * HM_PART;
+  const int values = head_mean_values(attn, t, MN), per_seq = head_mean_parts(MN, values), b = part / per_seq;
+  const int i = part % per_seq * values + (values / 256) * (int)threadIdx.x;
   const float inv_h = 1.0f / (float)H;
-  const float* src = attn + (size_t)b * H * MN;
-  float* dst = t + (size_t)b * MN;
-  if ((MN & 3) == 0 && (reinterpret_cast<uintptr_t>(attn) & 15) == 0 && (reinterpret_cast<uintptr_t>(t) & 15) == 0) {
-    const int i = i0 + 4 * threadIdx.x;
-    if (i >= MN) return;
+  const float* src = attn + (size_t)b * H * MN + i;
+  float* dst = t + (size_t)b * MN + i;
+  if (i >= MN) return;
+  if (values == 1024) {
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int h0 = 0; h0 < H; h0 += 16) {
       float4 a[16];
 #pragma unroll
       for (int q = 0; q < 16; ++q)
-        a[q] = h0 + q < H ? __ldg(reinterpret_cast<const float4*>(src + (size_t)(h0 + q) * MN + i))
+        a[q] = h0 + q < H ? __ldg(reinterpret_cast<const float4*>(src + (size_t)(h0 + q) * MN))
                           : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int q = 0; q < 16; ++q) { s.x += a[q].x; s.y += a[q].y; s.z += a[q].z; s.w += a[q].w; }
     }
-    *reinterpret_cast<float4*>(dst + i) = make_float4(s.x * inv_h, s.y * inv_h, s.z * inv_h, s.w * inv_h);
+    *reinterpret_cast<float4*>(dst) = make_float4(s.x * inv_h, s.y * inv_h, s.z * inv_h, s.w * inv_h);
     return;
   }
-  // Not a multiple of four: single values, four of the part per thread and eight heads in flight (12 sequences of 722 + 19
-  // tokens of 2048, whole step 84.1 -> 61.6 us; value by value, each behind a test of its own, the kernel alone took 35 us).
-  float s[4] = {};
-  for (int h0 = 0; h0 < H; h0 += 8) {
-    float a[8][4];
+  float s = 0.f;
+  for (int h0 = 0; h0 < H; h0 += 16) {
+    float a[16];
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
+    for (int q = 0; q < 16; ++q) a[q] = ld_now(src + (size_t)min(h0 + q, H - 1) * MN);
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        a[q][j] = ld_now(src + (size_t)min(h0 + q, H - 1) * MN + min(i0 + (int)threadIdx.x + 256 * j, MN - 1));
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[j] += h0 + q < H ? a[q][j] : 0.f;
+    for (int q = 0; q < 16; ++q) s += h0 + q < H ? a[q] : 0.f;
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int i = i0 + (int)threadIdx.x + 256 * j;
-    if (i < MN) dst[i] = s[j] * inv_h;
-  }
+  *dst = s * inv_h;
 }
 
 __global__ void __launch_bounds__(256) k_head_mean(const float* __restrict__ attn, int H, int MN, float* __restrict__ t) {
