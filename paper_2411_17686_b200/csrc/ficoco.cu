@@ -475,6 +475,8 @@ extern "C" int ficoco_create(ficoco_ctx** out, int device, long long max_tokens,
   }
   cudaFuncSetAttribute(k_merge_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
   cudaFuncSetAttribute(k_merge_rows<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTAGE_BYTES);
+  cudaFuncSetAttribute(k_correlate_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SIMT_ALONE_BYTES);
+  cudaFuncSetAttribute(k_correlate_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SIMT_ALONE_BYTES);
   // Two merge CTAs need 184 KB of shared memory.  Left to itself the SM stays at the largest carve-out when the correlate
   // kernel has set it, and the 28 KB of L1 that leaves slow the streaming kernels of the next step, which start beside
   // the merge (16 FiCoCo-L sequences, correlate CTAs of 205 KB: head mean 15.5 -> 17.4 us, column sums 18.9 -> 20.9,
@@ -1099,7 +1101,10 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
 #undef FICOCO_UMMA_LAUNCH
     } else {
       prof_tick(c, st, "correlate_simt");
-      launch_dependent(k_correlate_simt<T>, dim3(p->n_corr), 256, 0, st,
+      // The CTAs are placed while the filter grid still holds most SMs, two to each of the others.  A grid that needs no
+      // second CTA on any SM asks for shared memory that keeps a second one off (4 x 576 tokens of 1000, 100 CTAs: whole step
+      // 116 -> 89 us; 44 FiCoCo-L sequences of 99 + 34 fp32 tokens of 1024, 88 CTAs: 119 -> 90).
+      launch_dependent(k_correlate_simt<T>, dim3(p->n_corr), 256, p->n_corr <= c->num_sms ? SIMT_ALONE_BYTES : 0, st,
       tok, D, p->d_desc, p->d_corr, c->rn, c->S_idx,
                                                      c->T_idx, tmean, M, gamma, c->part_val, c->part_idx,
                                                      c->tile_cnt, c->corr_cnt, c->tau,

@@ -10,6 +10,7 @@ namespace ficoco {
 constexpr int CBM = 64;   // source rows per CTA
 constexpr int CBN = 64;   // target columns per tile
 constexpr int CKC = 16;   // reduction chunk
+constexpr size_t SIMT_ALONE_BYTES = 96 * 1024;   // unused shared memory with which a CTA has its SM to itself
 constexpr int CPG = 4;    // reduction chunks fetched together (one group in flight ahead of the multiply)
 
 // Four consecutive elements of a token row as fp32 (16-byte / 8-byte aligned).
