@@ -965,10 +965,11 @@ int run_step(ficoco_ctx* c, const Plan* p, const T* tok, int D, const float* att
   record_last_outputs(c->device, st, out_spans, N_SPANS);
   const bool wide = !p->fused && !rel && vpl > 8 && nvec <= 1024;   // rows of 257 .. 1024 16-byte vectors: CTA-wide rows
   // FiCoCo-L: head mean of the text->vision attention, in the grid of the column sums where rows are CTA-wide
-  const int mn = t2v ? M * p->max_np : 0, head_ctas = p->key.batch * head_mean_parts(mn, head_mean_values(t2v, c->tmean, mn));
+  const int mn = t2v ? M * p->max_np : 0;
+  const int head_ctas = p->key.batch * head_mean_parts(mn, head_mean_values(t2v, c->tmean, mn), wide ? 256 : HM_THREADS);
   if (t2v && !wide) {
     prof_tick(c, st, "head_mean");
-    launch_dependent(k_head_mean, dim3(head_ctas), 256, 0, st, t2v, t2v_heads, mn, c->tmean);
+    launch_dependent(k_head_mean, dim3(head_ctas), HM_THREADS, 0, st, t2v, t2v_heads, mn, c->tmean);
     c->launches += 1;
   }
   if (p->fused) {

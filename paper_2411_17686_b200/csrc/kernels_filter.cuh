@@ -359,35 +359,38 @@ __global__ void __launch_bounds__(256) k_score(const T* __restrict__ tokens, int
 
 // ---------------------------------------------------------------------------------------
 // FiCoCo-L: head mean of the text->vision attention, t[b, k, i] = (1/H) sum_h A[b, h, k, i].
-// The M * N values of a sequence are cut into parts, one CTA per part, 16 heads in flight, added in head order.  Where
-// everything is aligned a thread takes four values and a part is 1024 (16 sequences of 2048, 75 MB of attention: whole step
-// 68.7 us, with eight heads in flight 76.1); else one value, and a part is 256 (12 sequences of 722 + 19 tokens of 2048 57.7 us,
-// four values of 8 heads 61.5, of 16 heads 63.2; 51 of 410 + 1 of 256 37.7, 40.7, 42.4: registers that the grid before still
-// holds are waited for).
+// The M * N values of a sequence are cut into parts, one CTA per part; heads are added in order, so many at a time that the
+// loads are in flight together.  Where everything is aligned a thread takes four values, else one (12 sequences of 722 + 19
+// tokens of 2048 57.5 us, four single values 61.5).  In a grid of its own (narrow rows) small CTAs of few registers start
+// beside what the grid before still holds: 128 threads and eight heads; whole step, 35 sequences of 214 + 80 of 1024 50.7 us
+// (256 threads and 16 heads 53.3), 32 of 1000 + 100 of 2048 251.6 (257.2).  Beside the column sums, whose registers are taken
+// anyway, 256 threads and 16 heads.
 // ---------------------------------------------------------------------------------------
-__host__ __device__ __forceinline__ int head_mean_values(const float* attn, const float* t, int MN) {   // of a part
-  return ((MN & 3) == 0 && (reinterpret_cast<uintptr_t>(attn) & 15) == 0 && (reinterpret_cast<uintptr_t>(t) & 15) == 0) ? 1024 : 256;
+__host__ __device__ __forceinline__ int head_mean_values(const float* attn, const float* t, int MN) {   // of a thread
+  return ((MN & 3) == 0 && (reinterpret_cast<uintptr_t>(attn) & 15) == 0 && (reinterpret_cast<uintptr_t>(t) & 15) == 0) ? 4 : 1;
 }
-__host__ __device__ __forceinline__ int head_mean_parts(int MN, int values) { return (MN + values - 1) / values; }
+// CTAs of `threads` threads for a sequence
+__host__ __device__ __forceinline__ int head_mean_parts(int MN, int values, int threads) { return (MN + values * threads - 1) / (values * threads); }
 
+template <int NT, int HF>
 __device__ __forceinline__ void head_mean_part(const float* __restrict__ attn, int H, int MN, int part,
                                                float* __restrict__ t) {
-  const int values = head_mean_values(attn, t, MN), per_seq = head_mean_parts(MN, values), b = part / per_seq;
-  const int i = part % per_seq * values + (values / 256) * (int)threadIdx.x;
+  const int values = head_mean_values(attn, t, MN), per_seq = head_mean_parts(MN, values, NT), b = part / per_seq;
+  const int i = (part % per_seq * NT + (int)threadIdx.x) * values;
   const float inv_h = 1.0f / (float)H;
   const float* src = attn + (size_t)b * H * MN + i;
   float* dst = t + (size_t)b * MN + i;
   if (i >= MN) return;
-  if (values == 1024) {
+  if (values == 4) {
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int h0 = 0; h0 < H; h0 += 16) {
-      float4 a[16];
+    for (int h0 = 0; h0 < H; h0 += HF) {
+      float4 a[HF];
 #pragma unroll
-      for (int q = 0; q < 16; ++q)
+      for (int q = 0; q < HF; ++q)
         a[q] = h0 + q < H ? __ldg(reinterpret_cast<const float4*>(src + (size_t)(h0 + q) * MN))
                           : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) { s.x += a[q].x; s.y += a[q].y; s.z += a[q].z; s.w += a[q].w; }
+      for (int q = 0; q < HF; ++q) { s.x += a[q].x; s.y += a[q].y; s.z += a[q].z; s.w += a[q].w; }
     }
     *reinterpret_cast<float4*>(dst) = make_float4(s.x * inv_h, s.y * inv_h, s.z * inv_h, s.w * inv_h);
     return;
@@ -403,10 +406,11 @@ __device__ __forceinline__ void head_mean_part(const float* __restrict__ attn, i
   *dst = s * inv_h;
 }
 
-__global__ void __launch_bounds__(256) k_head_mean(const float* __restrict__ attn, int H, int MN, float* __restrict__ t) {
+constexpr int HM_THREADS = 128;
+__global__ void __launch_bounds__(HM_THREADS) k_head_mean(const float* __restrict__ attn, int H, int MN, float* __restrict__ t) {
   grid_dep_wait();
   grid_dep_launch();
-  head_mean_part(attn, H, MN, blockIdx.x, t);
+  head_mean_part<HM_THREADS, 8>(attn, H, MN, blockIdx.x, t);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -459,7 +463,7 @@ __global__ void __launch_bounds__(256, 2) k_colsum_wide(const T* __restrict__ to
   grid_dep_wait();
   grid_dep_launch();
   if (!rows_here) {
-    head_mean_part(t2v, H, MN, (int)blockIdx.x - n_rows, t);
+    head_mean_part<256, 16>(t2v, H, MN, (int)blockIdx.x - n_rows, t);
     return;
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

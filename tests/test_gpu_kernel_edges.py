@@ -147,9 +147,13 @@ def test_correlate_text_weights_in_the_ring(batch, n_vision, n_text, dim, keep, 
     (37, 3, 2112, 17, "bf16"),         # 111 attention values, no multiple of four; one head more than are in flight
     (130, 8, 2112, 3, "bf16"),         # 1040: a second part of 16 values
     (64, 16, 4096, 16, "fp32"),        # 1024: one full part; rows of 16 KB
-    (205, 5, 1032, 2, "fp32"),         # 1025: a second part of one value; rows just past the narrower kernels
-], ids=["scalar", "two-parts", "full-part", "one-value"])
-def test_head_mean_beside_column_sums(n_vision, n_text, dim, heads, dtype):
+    (205, 5, 1032, 2, "fp32"),         # 1025: parts of 256 and one value; rows just past the narrower kernels
+    (64, 8, 64, 9, "bf16"),            # a kernel of its own: 512 values, one full part; one head more than are in flight
+    (130, 4, 64, 3, "bf16"),           # 520: a second part of 8 values
+    (129, 1, 64, 17, "bf16"),          # 129: a part of 128 single values and one of one
+], ids=["scalar", "two-parts", "full-part", "one-value", "own-full-part", "own-two-parts", "own-one-value"])
+def test_head_mean(n_vision, n_text, dim, heads, dtype):
+    """In the grid of the column sums where rows are wide, else in a grid of its own."""
     c = binding.Context(max_tokens=3 * (n_vision + n_text), max_dim=dim, max_batch=3, max_text=n_text, device=0)
     try:
         b = synth.make_l_batch(100, 3, n_vision, n_text, dim, heads, n_vision // 2, dtype)
